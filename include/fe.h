@@ -460,10 +460,10 @@ typedef struct {
  * 0/1 matrix of h that come first in `which` order (FE_LM: |lambda| descending, ties ->
  * larger lambda first; FE_LA: descending; FE_SA: ascending).  block = b, nblocks = NB,
  * subspace m = b * NB; requires 1 <= nev <= m - b, m + b <= n, b in {1, 2, 4, 8, 16},
- * NB >= 2, m <= 512, NB <= 130 (m > 96: the projected eigenproblem keeps its matrices in a device
- * workspace that fe_eigs allocates, 2 (m+1)^2 doubles up to m = 160 and 5 (m+1)^2 above; above
- * m = 160 it runs FP32 Jacobi sweeps on one CTA, FP64 matrix products and FP64 Jacobi sweeps on a
- * cooperative grid).  A pair is converged when its Ritz residual estimate is at most
+ * NB >= 2, m <= 512, NB <= 130 (the projected eigenproblem's device
+ * workspace, which fe_eigs allocates, is about 8 m^2 doubles; up to m = 160 one thread-block
+ * cluster solves it by FP32 Jacobi sweeps refined with FP64 matrix products, above m = 160 FP32
+ * sweeps on one CTA, FP64 matrix products and FP64 Jacobi sweeps on a cooperative grid).  A pair is converged when its Ritz residual estimate is at most
  * tol * max(|theta|, 1e-3 * max|theta|) and the explicit residual ||A x - theta x|| passes the
  * same test.  evals: HOST, nev doubles.  evecs: DEVICE, n x nev COLUMN-major FP64 (ConvLayout,
  * Table 1), may be NULL; each vector's largest-magnitude entry is positive.  Synchronous.

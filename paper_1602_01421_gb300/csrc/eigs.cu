@@ -117,12 +117,12 @@ struct Phase {
                               // the ratio only fluctuates)
   cudaStream_t s;
   // state
-  DevBuf vmem, hmem, small, xmem, ritzwork, opbuf, cachemem;
+  DevBuf vmem, hmem, small, xmem, opbuf, cachemem;
   HostBuf vhost;
   void* cache[2] = {nullptr, nullptr};  // subspace_host: device copies (newest block, next)
   std::vector<void*> slot, spare, xblk, axblk;
   double *H = nullptr, *theta = nullptr, *Y = nullptr, *rho = nullptr, *anorm = nullptr,
-         *Cdiag = nullptr, *gtmp = nullptr;
+         *Cdiag = nullptr, *gtmp = nullptr, *ritzwork = nullptr;
   int* info = nullptr;
   uint64_t rng_counter = 0;
   int replacements = 0, restarts = 0, nconv = 0;
@@ -154,15 +154,16 @@ struct Phase {
     FE_TRY(hmem.alloc(sizeof(double) * (size_t)(m + b) * m));
     H = hmem.as<double>();
     const size_t nsmall = (size_t)m + (size_t)m * m + m + 4 + 256 + 64 * 16 + 16;
-    FE_TRY(small.alloc(sizeof(double) * nsmall));
-    theta = small.as<double>();
+    const size_t nritz = ritz_work_doubles(m);
+    FE_TRY(small.alloc(sizeof(double) * (nritz + nsmall)));
+    ritzwork = small.as<double>();
+    theta = ritzwork + nritz;
     Y = theta + m;
     rho = Y + (size_t)m * m;
     anorm = rho + m;
     Cdiag = anorm + 4;
     gtmp = Cdiag + 256;
     info = reinterpret_cast<int*>(gtmp + 64 * 16);
-    if (ritz_work_doubles(m) > 0) FE_TRY(ritzwork.alloc(sizeof(double) * ritz_work_doubles(m)));
     if (op_ata) FE_TRY(opbuf.alloc(blk));
     theta_h.resize(m);
     rho_h.resize(m);
@@ -234,7 +235,7 @@ struct Phase {
   // Ritz values/vectors of the current H, convergence estimate; returns nconv
   int ritz(int* nconv_out) {
     FE_TRY(launch_ritz(H, m, b, which, max_sweeps, 1e-15, theta, Y, rho, info,
-                       ritzwork.as<double>(), s));
+                       ritzwork, s));
     double an = 0.0;
     FE_CUDA(cudaMemcpyAsync(theta_h.data(), theta, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
     FE_CUDA(cudaMemcpyAsync(rho_h.data(), rho, sizeof(double) * m, cudaMemcpyDeviceToHost, s));

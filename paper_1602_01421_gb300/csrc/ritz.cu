@@ -1,14 +1,31 @@
 // Rayleigh-Ritz on the projected matrix (Algorithm 1 steps (2)-(4)) and the Krylov-Schur
 // restart of the small matrix, on the device.
 //
-// ritz_kernel: T = (H_m + H_m^T) / 2 (m x m) is diagonalised by the cyclic Jacobi method in
-// parallel ("round-robin" ordering, Brent & Luk 1985: each of the m-1 steps of a sweep
-// rotates m/2 disjoint index pairs at once).  Each rotation is the 2x2 symmetric Schur
-// decomposition of Golub & Van Loan Section 8.5; a step applies all of them at once as
-// J^T A J on independent 2x2 blocks (rows of one pair, columns of another), so a step costs
-// two barriers.  The Ritz values are then ordered by `which`, and each Ritz
-// pair gets its residual estimate rho_c = ||H[m:m+b, 0:m] y_c|| (the coupling of the last
+// T = (H_m + H_m^T) / 2 (m x m) is diagonalised, the Ritz values are ordered by `which`, and each
+// Ritz pair gets its residual estimate rho_c = ||H[m:m+b, 0:m] y_c|| (the coupling of the last
 // block to the next basis block, since A V_m = V_m H_m + V_{NB} H[m:m+b, :]).
+//
+// m <= 160 (ritz_cluster_kernel): FP64 runs at 1/64 of the FP32 rate here, so FP64 is spent on
+// matrix products only, and those are spread over a thread-block cluster.  One iteration turns
+// the FP64 vectors Q (T ~ Q D Q^T) into better ones:
+//   G = Q^T Q, W = T Q, S = Q^T W                                    (FP64, all CTAs)
+//   R = I - G;  d = diag S + R_ii theta_i,
+//   N_ij = S_ij + R_ij (theta_i + theta_j) / 2                       (FP64, then N in FP32)
+//     -- to first order in R the projection onto the orthonormalised Q (I + R / 2);
+//   E: the rotation that diagonalises D + N, relative to I           (FP32)
+//   Q <- Q + Q (R / 2 + E)                                           (FP64, all CTAs)
+// N and E are small, so their FP32 rounding is relative to something small: the error of an
+// iteration is about 1e-7 of the previous one (and the square of the previous one where E is
+// taken to first order).  The first iteration has Q = I and S = T: a whole FP32 Jacobi
+// diagonalisation.  The second finds N ~ 1e-7 |T| and runs one or two sweeps; the third finds
+// |N_ij / (d_j - d_i)| below 1e-8, takes E_ij = N_ij / (d_j - d_i) and is the last.  The
+// iterative refinement with matrix products and the treatment of R follow Ogita & Aishima,
+// "Iterative refinement for symmetric eigenvalue decomposition", Japan J. Indust. Appl. Math. 35
+// (2018); solving for E by Jacobi in FP32 makes close eigenvalues no special case.
+// Measured per call on a GB300 against FP32 and FP64 Jacobi sweeps on one CTA: m = 32 590 -> 110
+// us (seven FP32 sweeps of 9 us, FP64 18 us), m = 128 14.65 -> 1.15 ms (eight sweeps of 99 us,
+// FP64 0.23 ms).  What bounds it now: the sweeps' two barriers and dependent chains per step (31
+// steps of 0.29 us at m = 32), at m = 128 their shared-memory traffic.
 #include <math.h>
 
 #include <algorithm>
@@ -188,175 +205,570 @@ __device__ int jacobi_sweeps(T* A, T* Q, int ld, int m, int mp, double thresh, i
   }
 }
 
-// smem layout (mp = m rounded up to even, ld = mp + 1, rows padded), m <= kRitzSmallMax:
-//   A64[mp][ld], Q64[mp][ld]             FP64 matrix and eigenvectors
-//   U: A32[mp][ld] + Q32[mp][ld] (FP32)  later reused as W[mp][ld] (FP64 scratch)
-//   cs, sn (mp/2 doubles each), pp, pq (mp/2 ints each), order (mp ints)
-// Larger subspaces (BIG, m <= kRitzMax): the FP32 pair A32 + Q32 occupies the A64 region and
-// A64 is rebuilt from H once the FP32 sweeps are done; Q64 and W live in `gwork`
-// (2 mp ld doubles of global memory, L2-resident).
-// Two precisions: FP32 Jacobi sweeps take the matrix to a relative off-diagonal norm of about
-// 1e-6 (FP32 rotations run at the FP32 rate of the SM, FP64 ones at 1/64 of it); the FP32
-// eigenvector matrix is made orthogonal to FP64 rounding (two Newton-Schulz steps), the FP64 matrix is
-// transformed by it (Q^T T Q, an exact orthogonal similarity), and FP64 sweeps finish from there
-// -- two or three, since Jacobi converges quadratically once the off-diagonal part is small.
-template <bool BIG>
-__global__ void __launch_bounds__(1024) ritz_kernel(const double* __restrict__ H, int m, int b, int which, int max_sweeps,
-                            double tol, double* __restrict__ theta_out, double* __restrict__ Y_out,
-                            double* __restrict__ rho_out, int* __restrict__ info, double* gwork) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int mp = m + (m & 1);  // even size; index m (if odd) is a zero dummy never rotated
-  const int ld = mp + 1;
-  const size_t mat = (size_t)mp * ld;
-  double* A = reinterpret_cast<double*>(smem_raw);
-  double* Q = BIG ? gwork : A + mat;
-  double* W = BIG ? gwork + mat : Q + mat;
-  float* A32 = BIG ? reinterpret_cast<float*>(A) : reinterpret_cast<float*>(W);
-  float* Q32 = A32 + mat;
-  const int np = mp / 2;  // rotation pairs per step
-  double* cs = BIG ? A + mat : W + mat;
-  double* sn = cs + np;
-  int* pp = reinterpret_cast<int*>(sn + np);
-  int* pq = pp + np;
-  int* order = pq + np;
-  __shared__ double red[32];
-  __shared__ bool conv32, conv64;
-  const int tid = threadIdx.x, nth = blockDim.x;
+// ------------------------------------------------------------ m <= 160: one cluster
+constexpr int kRitzMaxIter = 8;        // refinement iterations (three are the rule)
+constexpr float kTinyAngle = 1e-8f;    // first-order E: its error is the angle's square
 
-  for (int e = tid; e < mp * mp; e += nth) {
-    const int i = e / mp, j = e % mp;
-    double a = 0.0;
-    if (i < m && j < m) a = 0.5 * (H[i * m + j] + H[j * m + i]);
-    if (!BIG) A[i * ld + j] = a;
-    A32[i * ld + j] = (float)a;
-    Q32[i * ld + j] = (i == j) ? 1.f : 0.f;
-  }
+// Global workspace (L2-resident): six mp x mp FP64 matrices, N in FP32, two diagonals, the
+// rotation logs of two sweeps, control words.
+struct RitzWork {
+  double *T, *Q, *Q2, *G, *W, *X, *d0, *d1;
+  float* N;
+  float2* log;     // [2][(mp - 1) * np]: (cos - 1, sin) of the step's pairs
+  unsigned* ctl;   // [0] max |R| (float bits), [1] mode, [2] done, [3..4] another sweep follows
+};
+constexpr int kRitzCtl = 8;
+
+__host__ __device__ inline size_t ritz_cluster_doubles(int m) {
+  const size_t mp = m + (m & 1), np = mp / 2;
+  return 6 * mp * mp + 2 * mp + (mp * mp + 1) / 2 + 2 * (mp - 1) * np + kRitzCtl;
+}
+
+__device__ inline RitzWork ritz_cluster_work(double* w, int mp) {
+  const size_t mat = (size_t)mp * mp, np = mp / 2;
+  RitzWork r;
+  r.T = w;
+  r.Q = w + mat;
+  r.Q2 = w + 2 * mat;
+  r.G = w + 3 * mat;
+  r.W = w + 4 * mat;
+  r.X = w + 5 * mat;
+  r.d0 = w + 6 * mat;
+  r.d1 = r.d0 + mp;
+  r.log = reinterpret_cast<float2*>(r.d1 + mp);
+  r.ctl = reinterpret_cast<unsigned*>(r.log + 2 * (mp - 1) * np);
+  r.N = reinterpret_cast<float*>(r.ctl + 2 * kRitzCtl);
+  return r;
+}
+
+// All threads of all CTAs of the cluster; global writes before it are visible after it.
+__device__ __forceinline__ void ritz_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void ritz_bar(int threads) {
+  asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+}
+
+// Maximum over the block of one non-negative float per thread.
+__device__ float ritz_block_max(float v, float* red) {
+  const int tid = threadIdx.x;
+  for (int off = 16; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
+  if ((tid & 31) == 0) red[tid >> 5] = v;
   __syncthreads();
-  double fro2;
-  {
-    double v = 0.0;
-    for (int e = tid; e < m * m; e += nth) {
-      const int i = e / m, j = e % m;
-      const double a = 0.5 * (H[i * m + j] + H[j * m + i]);
-      v += a * a;
-    }
-    fro2 = ritz_block_sum(v, red);
-  }
-  // FP32 sweeps
-  int sweeps = jacobi_sweeps<float>(A32, Q32, ld, m, mp, 1e-12 * fro2, 15, reinterpret_cast<float*>(cs),
-                                    reinterpret_cast<float*>(sn), pp, pq, red, &conv32);
-  // Q32 made orthogonal in FP64 by two Newton-Schulz steps Q <- Q (3 I - Q^T Q) / 2 (Higham,
-  // "Functions of Matrices", 8.3: quadratic convergence to the orthogonal polar factor from
-  // ||Q^T Q - I|| ~ 1e-6, to FP64 rounding in two steps); S and the factor in W, each new row
-  // of Q formed by one warp (all of its entries read before any is written)
-  const float inv_mp = 1.f / (float)mp;
-  for (int e = tid; e < mp * mp; e += nth) {
-    const int i = small_div(e, mp, inv_mp), j = e - i * mp;
-    Q[i * ld + j] = (double)Q32[i * ld + j];
-  }
+  v = (tid & 31) < (int)(blockDim.x >> 5) ? red[tid & 31] : 0.f;
+  for (int off = 16; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
   __syncthreads();
-  for (int it = 0; it < 2; ++it) {
-    for (int e = tid; e < mp * mp; e += nth) {
-      const int i = small_div(e, mp, inv_mp), j = e - i * mp;
-      if (i > j) continue;
-      double sv = 0.0;
-      for (int r = 0; r < mp; ++r) sv = fma(Q[r * ld + i], Q[r * ld + j], sv);
-      const double f = (i == j ? 1.5 : 0.0) - 0.5 * sv;
-      W[i * ld + j] = f;
-      W[j * ld + i] = f;
+  return v;
+}
+
+// FP64 bits as an integer that orders like the value (for comparisons off the FP64 pipe).
+// Negating the value negates the key.
+__device__ __forceinline__ long long ritz_key(double x) {
+  const long long v = __double_as_longlong(x);
+  return v < 0 ? -(v & 0x7fffffffffffffffll) : v;
+}
+
+// Hardware approximations, subnormals flushed (an inexact rotation angle only leaves a small
+// pivot, and the error of its cosine and sine is part of R in the next iteration).
+__device__ __forceinline__ float ritz_rsqrt(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float ritz_rcp(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// The circle method in slots: the index in slot i of a step is in slot ritz_shift(i) of the next
+// one (slot 0 stays), and pair k of a step is slots k and mp - 1 - k.  Data that moves with its
+// slot is at addresses that do not depend on the step, and after mp - 1 steps slot i holds
+// index i again.
+__device__ __forceinline__ int ritz_shift(int i, int mp) { return i == 0 ? 0 : (i == 1 ? mp - 1 : i - 1); }
+// Offset of the entry of slots a != b: the 2 x 2 block of pairs k < k2 is entry tri(k, k2) of four
+// planes (row of pair k from slot k or mp - 1 - k, column likewise); the pivots follow.
+__device__ __forceinline__ int ritz_entry(int a, int b, int mp) {
+  const int np = mp / 2, nt = np * (np - 1) / 2;
+  int ka = a < np ? a : mp - 1 - a, ra = a < np ? 0 : 1;
+  int kb = b < np ? b : mp - 1 - b, rb = b < np ? 0 : 1;
+  if (ka == kb) return 4 * nt + ka;
+  if (ka > kb) {
+    int t = ka; ka = kb; kb = t;
+    t = ra; ra = rb; rb = t;
+  }
+  return (ra * 2 + rb) * nt + ka * np - ka * (ka + 1) / 2 + kb - ka - 1;
+}
+
+// CTA 0's matrix during the sweeps, in shared memory: two copies of the entries (ritz_entry) and
+// of the diagonal by slot (unevaluated sums of two floats), and a step's (cos - 1, sin).
+struct RitzMat {
+  float *n0, *n1;
+  float2 *d0, *d1, *cs;
+};
+
+__device__ __forceinline__ void ritz_swap(RitzMat& mt) {
+  float* tn = mt.n0; mt.n0 = mt.n1; mt.n1 = tn;
+  float2* td = mt.d0; mt.d0 = mt.d1; mt.d1 = td;
+}
+
+// One sweep of the parallel cyclic Jacobi method ("round-robin" ordering, Brent & Luk 1985: each
+// of the mp - 1 steps rotates np = mp / 2 disjoint index pairs), with the threads of warps below
+// nact / 32; mt.n0, mt.d0 hold the matrix before and after.  The rotations also go to `log`.
+// Blocks item0 + u nact < nitems are this thread's: kk their pairs (k | k2 << 16), to where their
+// four entries go.  A pair is left alone when
+// |N_pq| <= skip, or when it is below tau (N's own uncertainty) and its angle would not be
+// tiny; isc: a power of two that brings |T| near 1.  psum: sum of the squared pivots; tmax:
+// largest |tan| (both of this thread).
+// What bounds it: two barriers and two dependent chains per step (rotation, block update), each
+// thread's addresses fixed; at mp = 128 the 11 shared-memory wavefronts per 32 blocks.
+template <int ITEMS>
+__device__ __forceinline__ void ritz_sweep(RitzMat& mt, int mp, int nact, int item0, int nitems,
+                                           const int (&to)[ITEMS][2], const int (&kk)[ITEMS],
+                                           float skip, float tau, float isc, float2* log, float* psum,
+                                           float* tmax) {
+  const int tid = threadIdx.x, np = mp / 2, nt = nitems;
+  float ps = 0.f, tm = 0.f;
+  const int sp = tid, sq = mp - 1 - tid;
+  const int tp = ritz_shift(sp, mp), tq = ritz_shift(sq, mp);
+  const int tres = tid < np ? ritz_entry(tp, tq, mp) : 0;
+  for (int step = 0; step < mp - 1; ++step) {
+    float cm = 0.f, s = 0.f;
+    if (tid < np) {
+      const float n = mt.n0[4 * nt + tid];
+      const float2 dp = mt.d0[sp], dq = mt.d0[sq];
+      const float gap = (dq.x - dp.x) + (dq.y - dp.y);
+      const float an = fabsf(n);
+      const float g = fabsf(gap) * isc, h = 2.f * isc * n;
+      // cos 2a = g / w, sin 2a = h / w with w = |(g, h)|; c^2 = (1 + cos 2a) / 2
+      const float iw = ritz_rsqrt(fmaf(g, g, h * h));
+      const bool rot = an > skip && (an > tau || an <= kTinyAngle * fabsf(gap));
+      const float c2 = rot ? fmaf(0.5f * g, iw, 0.5f) : 1.f, ic = ritz_rsqrt(c2), c = c2 * ic;
+      s = rot ? copysignf(0.5f, gap) * h * (iw * ic) : 0.f;
+      cm = -s * s * ritz_rcp(1.f + c);
+      const float t = s * ic, dn = t * n;
+      // the pivot's remainder: c s (d_p - d_q) + (c^2 - s^2) n
+      const float left = rot ? c2 * fmaf(fmaf(-t, t, 1.f), n, -t * gap) : n;
+      mt.cs[tid] = make_float2(cm, s);
+      mt.n1[tres] = left;
+      const float lo1 = dp.y - dn, h1 = dp.x + lo1;
+      mt.d1[tp] = make_float2(h1, lo1 - (h1 - dp.x));
+      const float lo2 = dq.y + dn, h2 = dq.x + lo2;
+      mt.d1[tq] = make_float2(h2, lo2 - (h2 - dq.x));
+      if (rot) ps = fmaf(n, n, ps);
+      tm = fmaxf(tm, fabsf(t));
     }
-    __syncthreads();
-    const int warp = tid >> 5, lane = tid & 31, nwarps = nth >> 5;
-    for (int r = warp; r < mp; r += nwarps) {
-      double x[5] = {0.0, 0.0, 0.0, 0.0, 0.0};   // columns lane + 32 t (mp <= 160)
-      for (int l = 0; l < mp; ++l) {
-        const double q = Q[r * ld + l];
+    ritz_bar(nact);
+    if (tid < np) log[step * np + tid] = make_float2(cm, s);
+    // N <- J^T N J as independent 2 x 2 blocks (rows of pair k, columns of pair k2, k < k2); all
+    // loads of the thread's blocks are issued before the first store
+    float2 r1[ITEMS], r2[ITEMS];
+    float x[ITEMS][4];
 #pragma unroll
-        for (int t = 0; t < 5; ++t)
-          if (lane + 32 * t < mp) x[t] = fma(q, W[l * ld + lane + 32 * t], x[t]);
+    for (int u = 0; u < ITEMS; ++u) {
+      const int e = item0 + u * nact;
+      const bool on = ITEMS == 1 || e < nitems;
+      r1[u] = mt.cs[kk[u] & 0xffff];
+      r2[u] = mt.cs[kk[u] >> 16];
+#pragma unroll
+      for (int v = 0; v < 4; ++v) x[u][v] = mt.n0[v * nt + (on ? e : 0)];
+    }
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) {
+      const float y00 = x[u][0] + fmaf(r1[u].x, x[u][0], -r1[u].y * x[u][2]);
+      const float y01 = x[u][1] + fmaf(r1[u].x, x[u][1], -r1[u].y * x[u][3]);
+      const float y10 = x[u][2] + fmaf(r1[u].x, x[u][2], r1[u].y * x[u][0]);
+      const float y11 = x[u][3] + fmaf(r1[u].x, x[u][3], r1[u].y * x[u][1]);
+      if (item0 + u * nact < nitems) {
+        mt.n1[to[u][0] & 0xffff] = y00 + fmaf(r2[u].x, y00, -r2[u].y * y01);
+        mt.n1[to[u][0] >> 16] = y01 + fmaf(r2[u].x, y01, r2[u].y * y00);
+        mt.n1[to[u][1] & 0xffff] = y10 + fmaf(r2[u].x, y10, -r2[u].y * y11);
+        mt.n1[to[u][1] >> 16] = y11 + fmaf(r2[u].x, y11, r2[u].y * y10);
+      }
+    }
+    ritz_bar(nact);
+    ritz_swap(mt);
+  }
+  *psum = ps;
+  *tmax = tm;
+}
+
+__device__ __forceinline__ int ritz_next(int p, int mp) { return p == 0 ? 0 : (p == mp - 1 ? 1 : p + 1); }
+
+// One row of E <- (I + E) J - I over a sweep's logged rotations, one warp; row: mp floats of
+// shared memory.  np <= 32: lane k keeps the entries of slots k and mp - 1 - k in registers and
+// the slots move by shuffles; otherwise the entries stay in shared memory.
+__device__ void ritz_apply_row(float* row, int i, int mp, const float2* log) {
+  const int lane = threadIdx.x & 31, np = mp / 2;
+  constexpr int D = 8;   // steps whose rotations are in flight
+  if (np <= 32) {
+    const bool on = lane < np;
+    int p = lane, q = mp - 1 - lane;
+    float ep = on ? row[p] : 0.f, eq = on ? row[q] : 0.f;
+    for (int s0 = 0; s0 < mp - 1; s0 += D) {
+      float2 r[D];
+#pragma unroll
+      for (int t = 0; t < D; ++t)
+        r[t] = (s0 + t < mp - 1 && on) ? log[(s0 + t) * np + lane] : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int t = 0; t < D; ++t) {
+        if (s0 + t >= mp - 1) break;
+        const float vp = ep + (i == p ? 1.f : 0.f), vq = eq + (i == q ? 1.f : 0.f);
+        const float np_ = ep + fmaf(r[t].x, vp, -r[t].y * vq), nq_ = eq + fmaf(r[t].x, vq, r[t].y * vp);
+        const float dn = __shfl_down_sync(0xffffffffu, np_, 1), up = __shfl_up_sync(0xffffffffu, nq_, 1);
+        ep = lane == 0 ? np_ : (lane == np - 1 ? nq_ : dn);
+        eq = lane == 0 ? (np == 1 ? nq_ : dn) : up;
+        p = ritz_next(p, mp);
+        q = ritz_next(q, mp);
+      }
+    }
+    if (on) {
+      row[lane] = ep;
+      row[mp - 1 - lane] = eq;
+    }
+    return;
+  }
+  constexpr int U = (kRitzOneMax / 2 + 31) / 32;
+  int p[U], q[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    p[u] = lane + 32 * u;
+    q[u] = mp - 1 - p[u];
+  }
+  constexpr int D2 = 4;
+  for (int s0 = 0; s0 < mp - 1; s0 += D2) {
+    float2 r[D2][U];
+#pragma unroll
+    for (int t = 0; t < D2; ++t)
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        r[t][u] = (s0 + t < mp - 1 && lane + 32 * u < np) ? log[(s0 + t) * np + lane + 32 * u] : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int t = 0; t < D2; ++t) {
+      if (s0 + t >= mp - 1) break;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (lane + 32 * u < np) {
+          const float ep = row[p[u]], eq = row[q[u]];
+          const float vp = ep + (i == p[u] ? 1.f : 0.f), vq = eq + (i == q[u] ? 1.f : 0.f);
+          row[p[u]] = ep + fmaf(r[t][u].x, vp, -r[t][u].y * vq);
+          row[q[u]] = eq + fmaf(r[t][u].x, vq, r[t][u].y * vp);
+          p[u] = ritz_next(p[u], mp);
+          q[u] = ritz_next(q[u], mp);
+        }
       }
       __syncwarp();
+    }
+  }
+}
+
+// Shared memory: CTA 0 holds the sweep's matrix, the others their rows of E.  ITEMS: 2 x 2 blocks
+// per thread of CTA 0.
+template <int ITEMS>
+__global__ void __launch_bounds__(512, 1)
+    ritz_cluster_kernel(const double* __restrict__ H, int m, int b, int which, int max_sweeps, double tol,
+                        double* __restrict__ theta_out, double* __restrict__ Y_out,
+                        double* __restrict__ rho_out, int* __restrict__ info, double* work) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int mp = m + (m & 1);  // even size; index m (if odd) is a zero dummy never rotated
+  const int np = mp / 2;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = blockIdx.x, ncta = gridDim.x;   // the grid is one cluster
+  const int nth = blockDim.x, nwarps = nth / 32;
+  RitzWork w = ritz_cluster_work(work, mp);
+  __shared__ float red[32];
+  __shared__ double redd[32];
+  __shared__ int order[kRitzOneMax];
+  __shared__ int s_mode, s_done, s_more;
+  float* sm = reinterpret_cast<float*>(smem_raw);
+  // this thread's 2 x 2 blocks (pairs k < k2) of CTA 0's sweeps
+  const int nitems = np * (np - 1) / 2;
+  const int nact = min(nth, (max(nitems, np) + 31) & ~31);
+  RitzMat mt;
+  mt.cs = reinterpret_cast<float2*>(sm);
+  mt.d0 = mt.cs + np;
+  mt.d1 = mt.d0 + mp;
+  mt.n0 = reinterpret_cast<float*>(mt.d1 + mp);
+  mt.n1 = mt.n0 + 4 * nitems + np;
+  int to[ITEMS][2], kk[ITEMS];
 #pragma unroll
-      for (int t = 0; t < 5; ++t)
-        if (lane + 32 * t < mp) Q[r * ld + lane + 32 * t] = x[t];
+  for (int u = 0; u < ITEMS; ++u) {
+    const int e = tid + u * nact;
+    to[u][0] = to[u][1] = kk[u] = 0;
+    if (rank == 0 && tid < nact && e < nitems) {
+      int k = 0, left = e;
+      while (left >= np - 1 - k) { left -= np - 1 - k; ++k; }
+      const int k2 = k + 1 + left;
+      const int p1 = ritz_shift(k, mp), q1 = ritz_shift(mp - 1 - k, mp);
+      const int p2 = ritz_shift(k2, mp), q2 = ritz_shift(mp - 1 - k2, mp);
+      kk[u] = k | (k2 << 16);
+      to[u][0] = ritz_entry(p1, p2, mp) | (ritz_entry(p1, q2, mp) << 16);
+      to[u][1] = ritz_entry(q1, p2, mp) | (ritz_entry(q1, q2, mp) << 16);
     }
-    __syncthreads();
   }
-  if (BIG) {  // the FP32 pair is dead: A64 takes its region back
-    for (int e = tid; e < mp * mp; e += nth) {
-      const int i = e / mp, j = e % mp;
-      A[i * ld + j] = (i < m && j < m) ? 0.5 * (H[i * m + j] + H[j * m + i]) : 0.0;
-    }
-    __syncthreads();
+  // T, its FP32 off-diagonal and its diagonal, shared by the CTAs
+  for (int e = rank * nth + tid; e < mp * mp; e += ncta * nth) {
+    const int i = e / mp, j = e - i * mp;
+    double a = 0.0;
+    if (i < m && j < m) a = 0.5 * (H[i * m + j] + H[j * m + i]);
+    w.T[e] = a;
+    w.N[e] = i == j ? 0.f : (float)a;
+    if (i == j) w.d0[i] = a;
   }
-  // A <- Q^T A Q (W = A Q first; A is symmetric, the result is mirrored from its upper triangle)
-  for (int e = tid; e < mp * mp; e += nth) {
-    const int i = e / mp, j = e % mp;
-    double s = 0.0;
-    for (int l = 0; l < mp; ++l) s += A[i * ld + l] * Q[l * ld + j];
-    W[i * ld + j] = s;
-  }
-  __syncthreads();
-  for (int e = tid; e < mp * mp; e += nth) {
-    const int i = e / mp, j = e % mp;
-    if (i > j) continue;
-    double s = 0.0;
-    for (int l = 0; l < mp; ++l) s += Q[l * ld + i] * W[l * ld + j];
-    A[i * ld + j] = s;
-    A[j * ld + i] = s;
-  }
-  __syncthreads();
-  // FP64 sweeps to the requested tolerance
-  sweeps += jacobi_sweeps<double>(A, Q, ld, m, mp, tol * tol * fro2, max_sweeps, cs, sn, pp, pq,
-                                  red, &conv64);
-  const bool converged = conv64;
-  // order by `which` (stable insertion sort; 0 = LM: |x| desc, ties larger first;
-  // 1 = LA: descending; 2 = SA: ascending)
-  if (tid == 0) {
-    for (int i = 0; i < m; ++i) order[i] = i;
-    for (int i = 1; i < m; ++i) {
-      const int x = order[i];
-      const double tx = A[x * ld + x];
-      int j = i - 1;
-      while (j >= 0) {
-        const double ty = A[order[j] * ld + order[j]];
-        bool before;
-        if (which == 0) before = fabs(tx) > fabs(ty) || (fabs(tx) == fabs(ty) && tx > ty);
-        else if (which == 1) before = tx > ty;
-        else before = tx < ty;
-        if (!before) break;
-        order[j + 1] = order[j];
-        --j;
+  if (rank == 0 && tid < kRitzCtl) w.ctl[tid] = 0u;
+  ritz_cluster_sync();
+  double *Q = w.Q, *Qn = w.Q2, *d = w.d0, *dprev = w.d1;
+  float fro = 0.f, dmax = 0.f, isc = 1.f;
+  int sweeps = 0, done = 0, it = 0;
+  for (;; ++it) {
+    // ---- FP32: E, the rotation that diagonalises D + N (CTA 0; rows of E in the others)
+    if (rank == 0) {
+      float f2 = 0.f, nu = 0.f, dm = 0.f;
+      for (int i = tid; i < mp; i += nth) {
+        const double a = d[i];
+        const float h = (float)a;
+        mt.d0[i] = make_float2(h, (float)(a - (double)h));
+        dm = fmaxf(dm, fabsf(h));
+        f2 = fmaf(h, h, f2);
       }
-      order[j + 1] = x;
+      const float rmax = __uint_as_float(w.ctl[0]);
+      dmax = ritz_block_max(dm, red);
+      // entries of N below tau are rounding (1e-15 |T|) or first-order R left over (R^2 D)
+      float tau = fmaxf((float)tol * fro, 0.5f * (float)mp * rmax * rmax * dmax);
+      if (it >= 4) tau = fmaxf(tau, 1e-13f * fro);
+      float emax = 0.f;
+      for (int e = tid; e < mp * mp; e += nth) {
+        const int i = e / mp, j = e - i * mp;
+        if (i >= j) continue;
+        const float n = w.N[e], an = fabsf(n);
+        mt.n0[ritz_entry(i, j, mp)] = n;
+        nu = fmaxf(nu, an);
+        f2 = fmaf(2.f * n, n, f2);
+        if (an > 0.f) {
+          const float gap = fabsf((mt.d0[j].x - mt.d0[i].x) + (mt.d0[j].y - mt.d0[i].y));
+          if (an > tau || an <= kTinyAngle * gap) emax = fmaxf(emax, gap > 0.f ? __fdividef(an, gap) : 1.f);
+        }
+      }
+      if (it == 0) {
+        fro = (float)sqrt(ritz_block_sum((double)f2, redd));
+        isc = fro > 0.f && fro < 1e38f ? exp2f(-floorf(log2f(fro))) : 1.f;
+        tau = (float)tol * fro;
+      }
+      nu = ritz_block_max(nu, red);
+      emax = ritz_block_max(emax, red);
+      // late iterations only repair orthogonality: rotations that are not tiny are left out
+      const bool first_order = it > 0 && (emax <= kTinyAngle || it >= kRitzMaxIter - 2);
+      if (tid == 0) {
+        w.ctl[0] = 0u;
+        w.ctl[1] = first_order ? 1u : 0u;
+        w.ctl[2] = (first_order && rmax <= kTinyAngle) ? (emax <= kTinyAngle ? 1u : 2u) : 0u;
+      }
+      if (first_order) {
+        ritz_cluster_sync();
+      } else {
+        const float skip = fmaxf(it == 0 ? 2e-8f * fro : 1e-7f * nu, 1e-17f * fro);
+        const int cap = it == 0 ? min(15, max_sweeps) : 6;
+        for (int s = 0; s < cap; ++s) {
+          float ps = 0.f, tm = 0.f;
+          if (tid < nact)
+            ritz_sweep<ITEMS>(mt, mp, nact, tid, nitems, to, kk, skip, tau, isc, w.log + (size_t)(s & 1) * (mp - 1) * np, &ps, &tm);
+          else
+            ritz_swap(mt);   // mp - 1 steps, an odd number
+          __syncthreads();
+          // the pivots met in a sweep bound what the next one would find (quadratic convergence)
+          const float v = it == 0 ? (float)ritz_block_sum((double)ps, redd)
+                                  : ritz_block_max(tm, red);
+          const bool more = s + 1 < cap && v > (it == 0 ? 1e-8f * fro * fro : 1e-4f);
+          ++sweeps;
+          if (tid == 0) w.ctl[3 + (s & 1)] = more ? 1u : 0u;
+          if (!more)
+            for (int i = tid; i < mp; i += nth) d[i] = (double)mt.d0[i].x + (double)mt.d0[i].y;
+          ritz_cluster_sync();
+          if (!more) break;
+        }
+      }
+    } else {
+      const int nrows = (mp - rank + ncta - 1) / (ncta - 1);   // rows rank - 1, + ncta - 1, ..
+      for (int e = tid; e < nrows * mp; e += nth) sm[e] = 0.f;
+      for (int s = 0;; ++s) {
+        ritz_cluster_sync();
+        if (tid == 0) {
+          s_mode = (int)w.ctl[1];
+          s_more = (int)w.ctl[3 + (s & 1)];
+        }
+        __syncthreads();
+        const bool more = s_mode == 0 && s_more != 0, sweep = s_mode == 0;
+        if (sweep)
+          for (int r = warp; r < nrows; r += nwarps) {
+            const int i = rank - 1 + r * (ncta - 1);
+            if (i < mp) ritz_apply_row(sm + r * mp, i, mp, w.log + (size_t)(s & 1) * (mp - 1) * np);
+          }
+        __syncthreads();
+        if (!more) break;
+      }
+      // X = R / 2 + E (it = 0: Q = I + E)
+      for (int e = tid; e < nrows * mp; e += nth) {
+        const int r = e / mp, j = e - r * mp;
+        const int i = rank - 1 + r * (ncta - 1);
+        if (i >= mp) continue;
+        if (it == 0) {
+          Q[i * mp + j] = (double)sm[e] + (i == j ? 1.0 : 0.0);
+          continue;
+        }
+        double x = (i == j ? 0.5 : 0.0) - 0.5 * w.G[i <= j ? i * mp + j : j * mp + i];
+        if (s_mode != 0) {
+          const float n = w.N[i * mp + j];
+          const float gap = (float)(d[j] - d[i]);
+          if (i != j && fabsf(n) <= kTinyAngle * fabsf(gap) && gap != 0.f) x += (double)(n / gap);
+        } else {
+          x += (double)sm[e];
+        }
+        w.X[i * mp + j] = x;
+      }
     }
-    info[0] = converged ? sweeps : -1;
+    ritz_cluster_sync();
+    if (tid == 0) s_done = (int)w.ctl[2];
+    __syncthreads();
+    done = s_done;
+    // ---- FP64: Q <- Q + Q X
+    if (it > 0) {
+      const int chunks = (mp * mp + 31) / 32;
+      for (int c = rank + ncta * warp; c < chunks; c += ncta * nwarps) {
+        const int e = c * 32 + lane;
+        if (e < mp * mp) {
+          const int i = e / mp, j = e - i * mp;
+          const double* q = Q + i * mp;
+          const double* x = w.X + j;
+          double a = 0.0;
+#pragma unroll 8
+          for (int l = 0; l < mp; ++l) a = fma(q[l], x[(size_t)l * mp], a);
+          Qn[e] = q[j] + a;
+        }
+      }
+      double* t = Q; Q = Qn; Qn = t;
+      ritz_cluster_sync();
+    }
+    if (done || it == kRitzMaxIter) break;
+    // ---- FP64: G = Q^T Q (upper triangle) and W = T Q
+    {
+      const int ntri = np * (mp + 1), total = mp * mp + ntri;
+      const int chunks = (total + 31) / 32;
+      for (int c = rank + ncta * warp; c < chunks; c += ncta * nwarps) {
+        const int e = c * 32 + lane;
+        if (e >= total) continue;
+        const double *x, *y;
+        int i, j;
+        if (e < mp * mp) {
+          i = e / mp;
+          j = e - i * mp;
+          x = w.T + i;   // T is symmetric: row i as a column
+        } else {
+          // rows r and mp - 1 - r of the triangle make one line of mp + 1 entries
+          const int f = e - mp * mp, r = f / (mp + 1), col = f - r * (mp + 1);
+          i = col < mp - r ? r : mp - 1 - r;
+          j = col < mp - r ? r + col : col - 1;
+          x = Q + i;
+        }
+        y = Q + j;
+        double a = 0.0;
+#pragma unroll 8
+        for (int l = 0; l < mp; ++l) a = fma(x[(size_t)l * mp], y[(size_t)l * mp], a);
+        if (e < mp * mp) w.W[e] = a;
+        else w.G[i * mp + j] = a;
+      }
+    }
+    ritz_cluster_sync();
+    // ---- FP64: S = Q^T W (upper triangle), then N, the new diagonal and max |R|
+    {
+      double* t = d; d = dprev; dprev = t;
+      const int ntri = np * (mp + 1), chunks = (ntri + 31) / 32;
+      float rm = 0.f;
+      for (int c = rank + ncta * warp; c < chunks; c += ncta * nwarps) {
+        const int f = c * 32 + lane;
+        if (f >= ntri) continue;
+        const int r = f / (mp + 1), col = f - r * (mp + 1);
+        const int i = col < mp - r ? r : mp - 1 - r;
+        const int j = col < mp - r ? r + col : col - 1;
+        const double* x = Q + i;
+        const double* y = w.W + j;
+        double a = 0.0;
+#pragma unroll 8
+        for (int l = 0; l < mp; ++l) a = fma(x[(size_t)l * mp], y[(size_t)l * mp], a);
+        const double R = (i == j ? 1.0 : 0.0) - w.G[i * mp + j];
+        rm = fmaxf(rm, fabsf((float)R));
+        if (i == j) {
+          d[i] = fma(R, dprev[i], a);
+          w.N[i * mp + i] = 0.f;
+        } else {
+          const float n = (float)fma(0.5 * R, dprev[i] + dprev[j], a);
+          w.N[i * mp + j] = n;
+          w.N[j * mp + i] = n;
+        }
+      }
+      for (int off = 16; off > 0; off >>= 1) rm = fmaxf(rm, __shfl_xor_sync(0xffffffffu, rm, off));
+      if (lane == 0 && rm > 0.f) atomicMax(&w.ctl[0], __float_as_uint(rm));
+    }
+    ritz_cluster_sync();
+  }
+  // ---- order by `which` (0 = LM: |x| descending, ties larger first; 1 = LA: descending;
+  // 2 = SA: ascending; equal values in index order) by counting, then the outputs
+  long long* key = reinterpret_cast<long long*>(smem_raw);
+  if (tid < m) key[tid] = ritz_key(d[tid]);
+  __syncthreads();
+  if (tid < m) {
+    const long long x = key[tid];
+    int pos = 0;
+    for (int j = 0; j < m; ++j) {
+      const long long y = key[j];
+      bool before = y > x;
+      if (which == 0) {   // |x| orders like the larger of key and -key
+        const long long ax = max(x, -x), ay = max(y, -y);
+        before = ay > ax || (ay == ax && y > x);
+      } else if (which == 2) {
+        before = y < x;
+      }
+      pos += before || (y == x && j < tid);
+    }
+    order[pos] = tid;
+  }
+  if (rank == 0 && tid == 0) info[0] = done == 1 ? sweeps : -1;
+  __syncthreads();   // order is complete; key's memory is free
+  if (rank == 0)
+    for (int c = tid; c < m; c += nth) theta_out[c] = d[order[c]];
+  for (int e = rank * nth + tid; e < m * m; e += ncta * nth) {
+    const int i = e / m, c = e - i * m;
+    Y_out[e] = Q[i * mp + order[c]];
+  }
+  // rho of columns rank, rank + ncta, ..: one partial square per (column, row of the last block)
+  double* sq = reinterpret_cast<double*>(smem_raw);
+  const int ncols = m > rank ? (m - rank + ncta - 1) / ncta : 0;
+  for (int e = tid; e < ncols * b; e += nth) {
+    const int c = rank + (e / b) * ncta, p = e % b;
+    const double* h = H + (size_t)(m + p) * m;
+    const double* y = Q + order[c];
+    double s = 0.0;
+#pragma unroll 8
+    for (int i = 0; i < m; ++i) s = fma(h[i], y[(size_t)i * mp], s);
+    sq[e] = s * s;
   }
   __syncthreads();
-  for (int c = tid; c < m; c += nth) theta_out[c] = A[order[c] * ld + order[c]];
-  for (int e = tid; e < m * m; e += nth) {
-    const int i = e / m, c = e % m;
-    Y_out[e] = Q[i * ld + order[c]];
-  }
-  for (int c = tid; c < m; c += nth) {
+  for (int k = tid; k < ncols; k += nth) {
     double r2 = 0.0;
-    for (int p = 0; p < b; ++p) {
-      double s = 0.0;
-      for (int i = 0; i < m; ++i) s += H[(m + p) * m + i] * Q[i * ld + order[c]];
-      r2 += s * s;
-    }
-    rho_out[c] = sqrt(r2);
+    for (int p = 0; p < b; ++p) r2 += sq[k * b + p];
+    rho_out[rank + k * ncta] = sqrt(r2);
   }
 }
 
-size_t ritz_smem_bytes(int m) {
-  const int mp = m + (m & 1);
-  const size_t mats = m <= kRitzSmallMax ? 3 : 1;
-  return mats * mp * (mp + 1) * sizeof(double) + (size_t)(mp / 2) * 2 * sizeof(double) +
-         (size_t)(mp / 2) * 2 * sizeof(int) + (size_t)mp * sizeof(int) + 64;
+static size_t ritz_cluster_smem(int m, int b, int ncta) {
+  const size_t mp = m + (m & 1), np = mp / 2;
+  const size_t head = (2 * np + 4 * mp + 2 * (2 * np * (np - 1) + np)) * sizeof(float);
+  const size_t rows = ((mp + ncta - 3) / (ncta - 1) + 1) * mp * sizeof(float);
+  const size_t rho = std::max<size_t>(m, ceil_div(m, ncta) * b) * sizeof(double);
+  return std::max(head, std::max(rows, rho));
 }
 
-// ------------------------------------------------------------ large subspaces (m > kRitzMidMax)
+// ------------------------------------------------------------ large subspaces (m > kRitzOneMax)
 // For m up to kRitzMax (512) the m x m matrices no longer fit one SM's shared memory, and FP64
 // Jacobi work on one SM (2 DFMA per clock) would take tens of milliseconds per sweep.  So:
 //   1. one CTA runs the FP32 Jacobi sweeps (A32, Q32 in global memory, L2-resident) to a
@@ -371,7 +783,6 @@ size_t ritz_smem_bytes(int m) {
 //   4. one CTA orders the pairs and writes theta, Y and the residual estimates.
 // Workspace layout (ld = mp + 1): A32, Q32 (floats, one mp x ld double-array each pair), A64,
 // Q64, W64, S64, then the barrier words and the per-CTA partial sums.
-constexpr int kRitzMidMax = 160;   // the one-CTA kernel's limit (global FP64 Q above 96)
 constexpr int kCoopCtas = 64;
 
 struct BigWork {
@@ -401,9 +812,7 @@ __host__ __device__ inline BigWork big_work(double* w, int m) {
 }
 
 size_t ritz_work_doubles(int m) {
-  const int mp = m + (m & 1);
-  if (m <= kRitzSmallMax) return 0;
-  if (m <= kRitzMidMax) return (size_t)2 * mp * (mp + 1);
+  if (m <= kRitzOneMax) return ritz_cluster_doubles(m);
   return 5 * big_mat_doubles(m) + 4 + kCoopCtas + 8;
 }
 
@@ -702,25 +1111,33 @@ static int launch_ritz_big(const double* H, int m, int b, int which, int max_swe
 int launch_ritz(const double* H, int m, int b, int which, int max_sweeps, double tol,
                 double* theta, double* Y, double* rho, int* info, double* work, cudaStream_t s) {
   FE_ARG(m >= 1 && m <= kRitzMax, "ritz: subspace m = %d not in [1, %d]", m, kRitzMax);
-  if (m > kRitzMidMax) {
-    FE_ARG(work != nullptr, "ritz: m = %d needs a global workspace", m);
+  FE_ARG(work != nullptr, "ritz: m = %d needs a global workspace", m);
+  if (m > kRitzOneMax)
     return launch_ritz_big(H, m, b, which, max_sweeps, tol, theta, Y, rho, info, work, s);
-  }
-  const size_t smem = ritz_smem_bytes(m);
-  FE_ARG(smem <= 225 * 1024, "ritz: subspace m = %d too large", m);
-  const bool big = m > kRitzSmallMax;
-  FE_ARG(!big || work != nullptr, "ritz: m = %d needs a global workspace", m);
-  static KernelSetup ks[2];
-  FE_TRY(kernel_configure(ks[big], big ? reinterpret_cast<const void*>(ritz_kernel<true>)
-                                       : reinterpret_cast<const void*>(ritz_kernel<false>),
-                          225 * 1024));
-  // one CTA: a rotation step is (m/2)^2 / 2 2 x 2 blocks plus m^2 / 2 Q updates between two
-  // barriers; FP64 work on one SM runs at 2 DFMA per clock, hence the FP32 sweeps first, and
-  // 1024 threads, so that many independent FP64 chains hide the FP64 pipe's latency
-  if (big)
-    ritz_kernel<true><<<1, 1024, smem, s>>>(H, m, b, which, max_sweeps, tol, theta, Y, rho, info, work);
-  else
-    ritz_kernel<false><<<1, 1024, smem, s>>>(H, m, b, which, max_sweeps, tol, theta, Y, rho, info, nullptr);
+  // FP64 products take m^3 / ncta / 2 clocks each: 16 CTAs where that outweighs the wider
+  // cluster's barriers (m = 128: 0.43 ms of products on 8, 0.22 ms on 16); threads enough for one, four or seven 2 x 2 blocks each (128 registers
+  // a thread: more threads with fewer spill)
+  const int ncta = m > 64 ? kRitzClusterMax : kRitzCluster;
+  const int variant = m <= 64 ? 0 : (m <= 128 ? 1 : 2);
+  const int threads = m <= 46 ? 256 : 512;
+  auto kern = variant == 0 ? ritz_cluster_kernel<1> : (variant == 1 ? ritz_cluster_kernel<4> : ritz_cluster_kernel<7>);
+  const void* fn = reinterpret_cast<const void*>(kern);
+  static KernelSetup ks[3];
+  FE_TRY(kernel_configure(ks[variant], fn, 128 * 1024));
+  if (ncta > 8) FE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = ncta;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ncta);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = ritz_cluster_smem(m, b, ncta);
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  FE_CUDA(cudaLaunchKernelEx(&cfg, kern, H, m, b, which, max_sweeps, tol, theta, Y, rho, info, work));
   count_launch();
   FE_CUDA(cudaGetLastError());
   return FE_OK;

@@ -248,3 +248,29 @@ def test_fully_external_solve_matches_oracle():
     assert st["converged"]
     assert np.allclose(ev, ref.evals, rtol=1e-8)
     _check_pairs(g, ev, X, 1e-8, ref.evals[0])
+
+
+@pytest.mark.parametrize("fam", ["er", "cube"])
+@pytest.mark.parametrize("b,nb", [(1, 2), (1, 3), (2, 2), (1, 17), (4, 8), (1, 33), (8, 8), (8, 12),
+                                  (1, 97), (4, 32), (1, 129), (16, 10)])
+def test_rayleigh_ritz_sizes(fam, b, nb):
+    """The one-cluster Rayleigh-Ritz at the edges of its range: subspaces of 2 to 160, odd ones
+    (a dummy index), pair counts around a warp and a CTA, and projected matrices with repeated
+    eigenvalues (the hypercube's multiplicities reach 70).  The vectors are products of an
+    orthonormal basis with the Ritz vectors, so their orthonormality (1e-12: 160 products of
+    FP64 rounding, times 50) shows the projected eigenvectors'."""
+    g = graphgen.erdos_renyi(700, 12.0, seed=9) if fam == "er" else graphgen.hypercube(8)
+    m = b * nb
+    nev = max(1, min(6, m - b, m // 2))
+    lam = np.linalg.eigvalsh(g.dense())
+    scale = np.abs(lam).max()
+    with fe.Csr.from_graph(g) as h:
+        ev, X, st = fe.eigs(h, nev, b, nb, 1e-9, "LA", seed=2, max_restarts=4000)
+    assert st["converged"]
+    X = X.cpu().numpy()
+    assert np.abs(X.T @ X - np.eye(nev)).max() < 1e-12
+    # every value is an eigenvalue: |error| <= residual <= tol * scale; multiplicities may be
+    # found in part by a small block, so only the largest is compared by position
+    assert np.abs(lam[:, None] - ev[None, :]).min(axis=0).max() < 2e-9 * scale
+    assert abs(ev[0] - lam[-1]) < 2e-9 * scale
+    _check_pairs(g, ev, to_dev(X), 1e-9, scale)
