@@ -74,90 +74,216 @@ __device__ void inv_upper_dev(const double* R, int b, double* Ri) {
   }
 }
 
-// After pass 2.  G1x = [G1; S1] ((k+b) x b), G2x = [G2; S] ((k+b) x b); k may be 0 (then
-// G2x = S).  Writes G (k x b, ldg), Racc = R1, M = R1^{-1}, C = -G2 R1^{-1}; on a failed check
+// Upper-triangular R (row-major B x B) with R^T R = S and Ri = R^{-1}, by one warp (all lanes
+// call it); S, R, Ri in shared memory.  False if a pivot check fails: a pivot d (before its square
+// root) of at most absthr^2 or below (rel * column norm)^2.  Lane c holds column c; the B pivots
+// are a serial chain, one reciprocal square root each (FP64 square roots and divisions take
+// hundreds of clocks on this part), whose square root, quotients and reciprocals get one Newton
+// correction and so keep the accuracy of the divisions.  Diagonals near the ends of FP64's range,
+// where the corrections would overflow or underflow, take the divisions on one lane.
+template <int B>
+__device__ bool chol_inv_warp(const double* S, double rel, double absthr, double* R, double* Ri) {
+  const int lane = threadIdx.x & 31, c = lane < B ? lane : B - 1;
+  const double sd = S[c * B + c];
+  if (__any_sync(0xffffffffu, !(sd < 1e280) || (sd > 0.0 && sd < 1e-260))) {
+    int good = 0;
+    if (lane == 0) {
+      good = chol_upper_dev(S, B, rel, absthr, R) ? 1 : 0;
+      if (good) inv_upper_dev(R, B, Ri);
+    }
+    good = __shfl_sync(0xffffffffu, good, 0);
+    __syncwarp();
+    return good != 0;
+  }
+  double col[B], rd[B], ri[B];
+#pragma unroll
+  for (int i = 0; i < B; ++i) col[i] = S[i * B + c];
+  bool ok = true;
+#pragma unroll
+  for (int j = 0; j < B; ++j) {
+    const double d = __shfl_sync(0xffffffffu, col[j], j);
+    ok = ok && d > 0.0 && d >= rel * rel * fmax(S[j * B + j], 0.0);
+    double r = rsqrt(ok ? d : 1.0);
+    double q = d * r;
+    q = fma(fma(-q, q, d), 0.5 * r, q);   // sqrt(d)
+    r = fma(fma(-r, q, 1.0), r, r);       // 1 / sqrt(d)
+    ok = ok && q > absthr;
+    rd[j] = q;
+    ri[j] = r;
+    double v = col[j] * r;
+    v = fma(fma(-v, q, col[j]), r, v);
+    col[j] = c == j ? q : v;
+#pragma unroll
+    for (int i = j + 1; i < B; ++i) col[i] = fma(-__shfl_sync(0xffffffffu, col[j], i), col[j], col[i]);
+  }
+  if (!ok) return false;
+  if (lane < B) {
+#pragma unroll
+    for (int i = 0; i < B; ++i) R[i * B + c] = i <= c ? col[i] : 0.0;
+  }
+  __syncwarp();
+  // column c of R^{-1} by back substitution
+  double y[B];
+#pragma unroll
+  for (int i = B - 1; i >= 0; --i) {
+    double t = i == c ? 1.0 : 0.0;
+#pragma unroll
+    for (int l = i + 1; l < B; ++l) t = fma(-R[i * B + l], y[l], t);
+    double v = t * ri[i];
+    v = fma(fma(-v, rd[i], t), ri[i], v);
+    y[i] = i <= c ? v : 0.0;
+  }
+  if (lane < B) {
+#pragma unroll
+    for (int i = 0; i < B; ++i) Ri[i * B + c] = y[i];
+  }
+  __syncwarp();
+  return true;
+}
+
+// After pass 2.  G1x = [G1; S1] ((k+B) x B), G2x = [G2; S] ((k+B) x B); k may be 0 (then
+// G2x = S).  Writes G (k x B, ldg), Racc = R1, M = R1^{-1}, C = -G2 R1^{-1}; on a failed check
 // sets *status = 1, G = G1, Racc = I.  status[1] = 1 when max |C| <= kSmallCorrection.
-__global__ void orth_post2_kernel(const double* __restrict__ G1x, const double* __restrict__ G2x,
-                                  int k, int b, double* __restrict__ anorm, int update_anorm,
-                                  double* __restrict__ G, int ldg, double* __restrict__ Racc,
-                                  double* __restrict__ M, double* __restrict__ C,
-                                  int* __restrict__ status) {
-  __shared__ double S[256], R[256], Ri[256];
+// One CTA of kPostThreads, bound by latency (at B = 4, k = 28 25 us with one thread on the factorisation and
+// on max |C|, 8.4 us now; the second factorisation 15.6 -> 6.2 us).
+constexpr int kPostThreads = 256;
+template <int B>
+__global__ void __launch_bounds__(kPostThreads)
+    orth_post2_kernel(const double* __restrict__ G1x, const double* __restrict__ G2x, int k,
+                      double* __restrict__ anorm, int update_anorm, double* __restrict__ G, int ldg,
+                      double* __restrict__ Racc, double* __restrict__ M, double* __restrict__ C,
+                      int* __restrict__ status) {
+  constexpr int BB = B * B, SL = kPostThreads / BB;   // slices of the sum over k
+  __shared__ double part[kPostThreads], S[BB], R[BB], Ri[BB];
   __shared__ int ok;
   const int tid = threadIdx.x;
-  for (int e = tid; e < b * b; e += blockDim.x) {
-    const int p = e / b, q = e % b;
-    double s = G2x[(k + p) * b + q];
-    for (int i = 0; i < k; ++i) s -= G2x[i * b + p] * G2x[i * b + q];
-    S[e] = s;
+  if (tid < SL * BB) {
+    const int e = tid % BB, p = e / B, q = e % B;
+    double x = 0.0;
+#pragma unroll 4
+    for (int i = tid / BB; i < k; i += SL) x = fma(G2x[i * B + p], G2x[i * B + q], x);
+    part[tid] = x;
   }
   __syncthreads();
-  if (tid == 0) {
+  if (tid < BB) {
+    double x = 0.0;
+#pragma unroll
+    for (int t = 0; t < SL; ++t) x += part[t * BB + tid];
+    S[tid] = G2x[k * B + tid] - x;
+  }
+  __syncthreads();
+  if (tid < 32) {
     double a = *anorm;
     if (update_anorm) {
-      for (int p = 0; p < b; ++p) a = fmax(a, sqrt(fmax(G1x[(k + p) * b + p], 0.0)));
-      *anorm = a;
+      double s1 = tid < B ? G1x[(k + tid) * B + tid] : 0.0;
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) s1 = fmax(s1, __shfl_xor_sync(0xffffffffu, s1, off));
+      a = fmax(a, sqrt(fmax(s1, 0.0)));
+      if (tid == 0) *anorm = a;
     }
-    ok = chol_upper_dev(S, b, kRelPivot, kAbsBreakdown * a, R) ? 1 : 0;
-    if (ok) inv_upper_dev(R, b, Ri);
-    else *status = 1;
+    const bool good = chol_inv_warp<B>(S, kRelPivot, kAbsBreakdown * a, R, Ri);
+    if (tid == 0) {
+      ok = good;
+      if (!good) *status = 1;
+    }
   }
   __syncthreads();
-  for (int e = tid; e < k * b; e += blockDim.x) {
-    const int i = e / b, q = e % b;
-    if (ok) {
-      G[i * ldg + q] = G1x[i * b + q] + G2x[i * b + q];
+  const bool good = ok != 0;
+  bool small = true;
+  for (int e = tid; e < k * B; e += kPostThreads) {
+    const int i = e / B, q = e % B;
+    if (good) {
+      G[i * ldg + q] = G1x[e] + G2x[e];
       double c = 0.0;
-      for (int p = 0; p <= q; ++p) c -= G2x[i * b + p] * Ri[p * b + q];
+#pragma unroll
+      for (int p = 0; p < B; ++p) c = fma(-G2x[i * B + p], Ri[p * B + q], c);
       C[e] = c;
+      small = small && fabs(c) <= kSmallCorrection;
     } else {
-      G[i * ldg + q] = G1x[i * b + q];
+      G[i * ldg + q] = G1x[e];
     }
   }
-  for (int e = tid; e < b * b; e += blockDim.x) {
-    if (ok) {
-      Racc[e] = R[e];
-      M[e] = Ri[e];
+  if (tid < BB) {
+    if (good) {
+      Racc[tid] = R[tid];
+      M[tid] = Ri[tid];
     } else {
-      Racc[e] = (e / b == e % b) ? 1.0 : 0.0;
+      Racc[tid] = (tid / B == tid % B) ? 1.0 : 0.0;
     }
   }
-  __syncthreads();
-  if (tid == 0) {
-    double cmax = 0.0;
-    if (ok)
-      for (int e = 0; e < k * b; ++e) cmax = fmax(cmax, fabs(C[e]));
-    status[1] = (ok && cmax <= kSmallCorrection) ? 1 : 0;
-  }
+  small = __syncthreads_and(small) != 0;
+  if (tid == 0) status[1] = (good && small) ? 1 : 0;
 }
 
 // After pass 3: R2 = chol(S2); R = R2 Racc (-> Rout, ldr), M = R2^{-1}; failure -> *status = 2.
-__global__ void orth_post3_kernel(const double* __restrict__ S2, int b,
-                                  const double* __restrict__ Racc, double* __restrict__ M,
-                                  double* __restrict__ Rout, int ldr, int* __restrict__ status) {
-  __shared__ double R2[256], Ri[256];
+// status[2]: R2^{-1} is the identity up to kSmallCorrection.
+template <int B>
+__global__ void __launch_bounds__(kPostThreads)
+    orth_post3_kernel(const double* __restrict__ S2, const double* __restrict__ Racc,
+                      double* __restrict__ M, double* __restrict__ Rout, int ldr, int* __restrict__ status) {
+  constexpr int BB = B * B;
+  __shared__ double S[BB], R1[BB], R2[BB], Ri[BB];
   __shared__ int ok;
   if (*status) return;
   const int tid = threadIdx.x;
-  if (tid == 0) {
-    ok = chol_upper_dev(S2, b, kRelPivot, 0.0, R2) ? 1 : 0;
-    if (ok) inv_upper_dev(R2, b, Ri);
-    else *status = 2;
+  if (tid < BB) {
+    S[tid] = S2[tid];
+    R1[tid] = Racc[tid];
+  }
+  __syncthreads();
+  if (tid < 32) {
+    const bool good = chol_inv_warp<B>(S, kRelPivot, 0.0, R2, Ri);
+    if (tid == 0) {
+      ok = good;
+      if (!good) *status = 2;
+    }
   }
   __syncthreads();
   if (!ok) return;
-  for (int e = tid; e < b * b; e += blockDim.x) {
-    const int p = e / b, q = e % b;
+  bool small = true;
+  if (tid < BB) {
+    const int p = tid / B, q = tid % B;
     double r = 0.0;
-    for (int l = p; l <= q; ++l) r += R2[p * b + l] * Racc[l * b + q];
+#pragma unroll
+    for (int l = 0; l < B; ++l)
+      if (l >= p && l <= q) r = fma(R2[p * B + l], R1[l * B + q], r);
     Rout[p * ldr + q] = r;
-    M[e] = Ri[e];
+    M[tid] = Ri[tid];
+    small = fabs(Ri[tid] - (p == q ? 1.0 : 0.0)) <= kSmallCorrection;
   }
-  if (tid == 0) {  // status[2]: R2^{-1} is the identity up to kSmallCorrection
-    double dmax = 0.0;
-    for (int e = 0; e < b * b; ++e) dmax = fmax(dmax, fabs(Ri[e] - (e / b == e % b ? 1.0 : 0.0)));
-    status[2] = dmax <= kSmallCorrection ? 1 : 0;
+  small = __syncthreads_and(small) != 0;
+  if (tid == 0) status[2] = small ? 1 : 0;
+}
+
+// CALL(B) for the block width b.
+#define FE_ORTH_B(b, CALL)                                             \
+  switch (b) {                                                         \
+    case 1: CALL(1); break;                                            \
+    case 2: CALL(2); break;                                            \
+    case 4: CALL(4); break;                                            \
+    case 8: CALL(8); break;                                            \
+    case 16: CALL(16); break;                                          \
+    default: return set_error(FE_ERR_INVALID, "orth: b = %d", b);      \
   }
+
+static int launch_post2(const double* G1x, const double* G2x, int k, int b, double* anorm, int update_anorm,
+                        double* G, int ldg, double* Racc, double* M, double* C, int* status, cudaStream_t s) {
+#define POST2(B) orth_post2_kernel<B><<<1, kPostThreads, 0, s>>>(G1x, G2x, k, anorm, update_anorm, G, ldg, Racc, M, C, status)
+  FE_ORTH_B(b, POST2)
+#undef POST2
+  count_launch();
+  FE_CUDA(cudaGetLastError());
+  return FE_OK;
+}
+
+static int launch_post3(const double* S2, int b, const double* Racc, double* M, double* Rout, int ldr,
+                        int* status, cudaStream_t s) {
+#define POST3(B) orth_post3_kernel<B><<<1, kPostThreads, 0, s>>>(S2, Racc, M, Rout, ldr, status)
+  FE_ORTH_B(b, POST3)
+#undef POST3
+  count_launch();
+  FE_CUDA(cudaGetLastError());
+  return FE_OK;
 }
 
 // W <- W M for the second CholeskyQR pass (M = R2^{-1}), skipped after a failed check.  After
@@ -408,8 +534,7 @@ int orth_ex(const BlockSet& V, int64_t n, void* W, int b, fe_dtype dt, double* d
     BlockSet Vu = blockset_of(vu, b, b);
     FE_TRY(tc_combine(Vu, n, sG1 + (size_t)v0 * b * b, b, Wset, s, -1.0, 1.0));   // W <- W - V G1
     FE_TRY(tc_gram(Vx, n, static_cast<const double*>(W), b, 1.0, sG2, s));  // [G2; S]
-    orth_post2_kernel<<<1, 256, 0, s>>>(sG1, sG2, k, b, d_anorm, update_anorm, d_G, ldg, sRacc,
-                                        sM, sC, status);
+    FE_TRY(launch_post2(sG1, sG2, k, b, d_anorm, update_anorm, d_G, ldg, sRacc, sM, sC, status, s));
   } else if (V.nv > 0) {
     // W <- W - V G1 and [G2; S] = [V W]^T W in one sweep
     if (fused) {
@@ -418,14 +543,10 @@ int orth_ex(const BlockSet& V, int64_t n, void* W, int b, fe_dtype dt, double* d
       FE_TRY(update(V, n, sG1, -1.0, 1.0, nullptr, W, b, b, dt, s));
       FE_TRY(gram(Vx, n, W, b, b, dt, 1.0, sG2, s));
     }
-    orth_post2_kernel<<<1, 256, 0, s>>>(sG1, sG2, k, b, d_anorm, update_anorm, d_G, ldg, sRacc,
-                                        sM, sC, status);
+    FE_TRY(launch_post2(sG1, sG2, k, b, d_anorm, update_anorm, d_G, ldg, sRacc, sM, sC, status, s));
   } else {
-    orth_post2_kernel<<<1, 256, 0, s>>>(sG1, sG1, 0, b, d_anorm, update_anorm, d_G, ldg, sRacc,
-                                        sM, sC, status);
+    FE_TRY(launch_post2(sG1, sG1, 0, b, d_anorm, update_anorm, d_G, ldg, sRacc, sM, sC, status, s));
   }
-  count_launch();
-  FE_CUDA(cudaGetLastError());
   // W <- (W - V G2) R1^{-1} and S2 = W^T W in one sweep (skipped after a failed pivot check)
   if (fused && b <= 4) {
     // M = R1^{-1} is upper triangular: thread-per-row sweep over its triangle, S2 = W^T W in
@@ -442,9 +563,7 @@ int orth_ex(const BlockSet& V, int64_t n, void* W, int b, fe_dtype dt, double* d
     BlockSet Wonly = blockset_of({W}, b, b);
     FE_TRY(gram(Wonly, n, W, b, b, dt, 1.0, sS2, s));
   }
-  orth_post3_kernel<<<1, 64, 0, s>>>(sS2, b, sRacc, sM, d_R, ldr, status);
-  count_launch();
-  FE_CUDA(cudaGetLastError());
+  FE_TRY(launch_post3(sS2, b, sRacc, sM, d_R, ldr, status, s));
   const int allow32 = (pass1_f32 && dt == FE_F64) ? 1 : 0;
   if (dt == FE_F64) FE_TRY(launch_right_mult(static_cast<double*>(W), n, b, sM, status, allow32, s));
   else FE_TRY(launch_right_mult(static_cast<float*>(W), n, b, sM, status, 0, s));

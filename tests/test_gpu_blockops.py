@@ -187,3 +187,27 @@ def test_combine_many_blocks_matches_oracle(prec, nv, nout, bv):
     ref = Vt @ Y
     rel = {"f32": 6e-8, "f64": 1.2e-16}[prec] * (nv * bv + 2) * 2
     assert np.all(np.abs(got - ref) <= rel * (np.abs(Vt) @ np.abs(Y)) + 1e-300)
+
+
+@pytest.mark.parametrize("n,nv,b,scale", [(5000, 3, 2, 1.0), (5000, 2, 16, 1.0), (2000, 5, 1, 1.0), (4000, 2, 4, 1e-100),
+                                          (4000, 2, 4, 1e120), (4000, 2, 4, 1e-145), (4000, 0, 8, 1e145)])
+def test_orth_factorisation_widths_and_scales(n, nv, b, scale):
+    """The one-warp Cholesky factorisation at every width, and with Gram diagonals (scale^2 n) inside
+    and outside the range of its Newton-corrected square roots.  Everything scales with W, so the
+    bounds are those of scale 1: R is the Cholesky factor of the projected W to 1e-11 (its
+    condition, below 1e2, times FP64 rounding of sums of n terms)."""
+    r = np.random.default_rng(n + b)
+    Vt, _ = np.linalg.qr(r.standard_normal((n, max(nv, 1) * b)))
+    Vt = Vt[:, : nv * b]
+    W = r.standard_normal((n, b))
+    Wd = to_dev(W * scale)
+    V = to_dev(np.stack([Vt[:, j * b:(j + 1) * b] for j in range(nv)])) if nv else None
+    G, R, rep = fe.block_orth(V, Wd, anorm=10.0 * scale)
+    Q, R = Wd.cpu().numpy(), R.cpu().numpy() / scale
+    P = W - Vt @ (Vt.T @ W) if nv else W
+    want = np.linalg.cholesky(P.T @ P).T
+    assert rep == 0
+    assert np.abs(R - want).max() < 1e-11 * np.abs(want).max()
+    assert np.abs(Q.T @ Q - np.eye(b)).max() < 1e-13
+    if nv:
+        assert np.abs(G.cpu().numpy() / scale - Vt.T @ W).max() < 1e-11 * np.abs(want).max()
