@@ -161,3 +161,44 @@ def test_trained_network_gain_on_a_fresh_graph():
     print(f"block SpMMs: random starts {[x['spmm_blocks'] for x in r['random']]}, "
           f"learned start {r['learned']['spmm_blocks']} (+7 feature SpMMs)")
     assert np.allclose(r["learned"]["evals"], r["random"][0]["evals"], rtol=1e-8)
+
+
+@pytest.mark.parametrize("form,n,hidden,b,t", [
+    ("column", 1, 64, 4, 4), ("column", 127, 32, 1, 1), ("subspace", 128, 64, 8, 16), ("column", 129, 64, 16, 16),
+    ("span", 129, 64, 8, 8), ("span", 40, 64, 4, 4), ("span", 128 * 304 + 1, 64, 4, 8), ("column", 128 * 304 + 127, 32, 16, 16)])
+def test_row_tiles(form, n, hidden, b, t):
+    """Forward, loss and gradient at the edges of the 128-row tiles (one row, one short of a tile, a
+    row over, more tiles than CTAs), biases everywhere, features at an odd 4-byte offset.  Bars as
+    above: FP32 rounding of sums of at most 64 terms per unit, FP64 over the rows' tiles."""
+    t_ = torch()
+    r = np.random.default_rng(n + hidden + b)
+    buf = to_dev(np.concatenate([[0.0], np.abs(r.standard_normal(n * omlp.NFEAT))]), t_.float32)
+    F = buf[1:].view(n, omlp.NFEAT)
+    p = learned.init_params(hidden, b, seed=n) + (0.05 * r.standard_normal(omlp.param_count(hidden, b))).astype(np.float32)
+    U = r.standard_normal((n, t)) / np.sqrt(n)
+    U32 = U.astype(np.float32)
+    F64, p64, U64 = F.cpu().numpy().astype(np.float64), p.astype(np.float64), U32.astype(np.float64)
+    Z = fe.mlp_forward(F, to_dev(p), hidden, b).cpu().numpy()
+    Zo, _ = omlp.forward(F64, p64, hidden, b)
+    assert np.allclose(Z, Zo, rtol=1e-5, atol=1e-5 * np.abs(Zo).max())
+    gpu, ora = {"column": (fe.mlp_loss_grad, omlp.loss_and_grad),
+                "subspace": (fe.mlp_subspace_loss_grad, omlp.subspace_loss_and_grad),
+                "span": (fe.mlp_span_loss_grad, omlp.span_loss_and_grad)}[form]
+    L, grad = gpu(F, to_dev(p), hidden, b, to_dev(U32))
+    Lo, go = ora(F64, p64, hidden, b, U64)
+    assert abs(L - Lo) <= 1e-5 * max(1.0, abs(Lo))
+    grad = grad.cpu().numpy().astype(np.float64)
+    # dz is a difference of two terms (target and norm part of the loss) that cancel down to nothing
+    # at n = 1: each is rounded to a few units of 2^-24, and the gradient is linear in dz with the
+    # row's gain (norms of the activations and weights on the way back)
+    W1, _, W2, _, W3, _ = omlp.unpack(p64, hidden, b)
+    _, acts = omlp.forward(F64, p64, hidden, b)
+    h1, h2 = acts[1], acts[3]
+    n3, n2 = np.linalg.norm(W3), np.linalg.norm(W2)
+    gain2 = (1 + (h2 ** 2).sum(1)) + n3 ** 2 * (1 + (h1 ** 2).sum(1)) + (n3 * n2) ** 2 * (1 + (F64 ** 2).sum(1))
+    term2 = 0.0
+    if form == "column":
+        s, q = (Zo * U64).sum(0), (Zo ** 2).sum(0)
+        term2 = ((2 * s / q * U64) ** 2 + (2 * s ** 2 / q ** 2 * Zo) ** 2).sum(1)
+    slack = 8 * 2.0 ** -24 * np.sqrt((term2 * gain2).sum())
+    assert np.linalg.norm(grad - go) <= 1e-4 * np.linalg.norm(go) + slack
