@@ -156,6 +156,7 @@ struct fe_spmm_plan {
   int nbuckets = 0;
   // warp tasks: hub chunks first (partial slots 0..nhub_tasks-1), then mid rows by degree
   int64_t ntasks = 0, nhub_tasks = 0, nhub = 0;
+  int64_t wide4 = 0, wide2 = 0;      // plan_wide
   void* d_tasks = nullptr;           // struct Task[ntasks] (PTask when packed)
   uint32_t* d_tbits = nullptr;       // packed: the task rows' gap bit stream
   int packed = 0;
@@ -220,6 +221,7 @@ struct PlanView {
   int packed;
   const void* tasks;
   int64_t ntasks, nhub_tasks;
+  int64_t wide4, wide2;    // plan_wide
   const int32_t* slice_rows;
   const int32_t* ell;
   int64_t nslices;
@@ -234,6 +236,8 @@ struct PlanView {
 };
 int build_host_plan(const int64_t* rowptr, const int32_t* colidx, int64_t r0, int64_t r1,
                     int tail_max, int hub_min, int hub_chunk, bool packed, HostPlan& hp);
+// Tasks that several warps share: [0, wide4) by four, [wide4, wide2) by two (see spmm.cu).
+void plan_wide(const HostPlan& hp, int64_t ncols, bool streamed, int64_t* wide4, int64_t* wide2);
 // Bytes the column indices of row i take in a plan (ELL slice, plain task indices or packed
 // gaps), for sizing panels.
 size_t plan_row_index_bytes(const int32_t* cols, int64_t d, int tail_max, int hub_chunk, bool packed);

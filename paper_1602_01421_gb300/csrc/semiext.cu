@@ -31,7 +31,7 @@ struct PanelInfo {
   int nbuckets;
   int32_t deg_of_bucket[kMaxBuckets], deg_slice_begin[kMaxBuckets];
   int64_t deg_ell_base[kMaxBuckets];
-  int64_t nslices, ntasks, nhub_tasks, nhub;
+  int64_t nslices, ntasks, nhub_tasks, wide4, wide2, nhub;
 };
 
 struct SemiExt {
@@ -187,6 +187,7 @@ int semiext_create(fe_csr h, const int64_t* rowptr, const int32_t* colidx, const
     pi.nslices = hp.nslices;
     pi.ntasks = hp.ntasks;
     pi.nhub_tasks = hp.nhub_tasks;
+    plan_wide(hp, h->ncols, true, &pi.wide4, &pi.wide2);
     pi.nhub = hp.nhub;
     h->max_degree = std::max(h->max_degree, hp.max_degree);
     h->rows_empty += hp.rows_empty;
@@ -268,6 +269,9 @@ int semiext_spmm(fe_csr h, const void* X, void* Y, int b, fe_dtype dt, cudaStrea
     v.tasks = base + pi.off_tasks;
     v.ntasks = pi.ntasks;
     v.nhub_tasks = pi.nhub_tasks;
+    v.x_rows = h->ncols;
+    v.wide4 = pi.wide4;
+    v.wide2 = pi.wide2;
     v.slice_rows = reinterpret_cast<const int32_t*>(base + pi.off_slice_rows);
     v.ell = reinterpret_cast<const int32_t*>(base + pi.off_ell);
     v.nslices = pi.nslices;

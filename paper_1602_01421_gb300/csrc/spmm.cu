@@ -6,22 +6,23 @@
 // with work stealing; here the same two problems are solved by degree binning):
 //   * tail rows (degree <= tail_max, default 128; 97% of the scale-22 R-MAT rows): grouped by
 //     exact degree into 32-row slices whose column indices are stored transposed
-//     ("SELL-32"): lane l of a warp owns row l of the slice and step t loads ell[t*32 + l],
-//     one coalesced 128-byte load per step and no divergence or masked lane, since all 32
-//     rows of a slice have the same degree;
-//   * mid rows (tail_max < degree <= hub_min): one warp per row (a "task"), 32 consecutive
+//     ("SELL-32"): step t of row l is ell[t*32 + l]; a lane owns a row (above degree 32, two or
+//     four lanes share one, slice_pieces), with coalesced index loads and no divergence or masked
+//     lane, since all 32 rows of a slice have the same degree;
+//   * mid rows (tail_max < degree <= hub_min): one warp per row (a "task"; long ones of smaller
+//     matrices are shared by two or four warps of a CTA, plan_wide), 32 consecutive
 //     column indices per coalesced load, each lane gathering up to 32 bytes of an X row
 //     (one 256-bit load when X is 32-byte aligned), partial sums combined by a
 //     reduce-scatter butterfly;
 //   * hub rows (degree > hub_min): split into tasks of hub_chunk non-zeros; each task writes
-//     a partial row, and a second kernel adds a hub's partials in task order (deterministic,
+//     a partial row, and a second kernel adds a hub's partials in a fixed order (deterministic,
 //     no atomics).
 // Tasks are ordered longest first so the block scheduler handles them like a longest-
 // processing-time list; tail slices follow in the same launch.  The task rows' column
 // indices are stored either as int32 or, in the packed format, as per-task gap fields that a
 // warp decodes with a prefix sum (fewer bytes to stream from host memory).
-// FP32 sums are compensated per lane (Kahan) before the lane tree, and hub chunks are added in
-// compensated FP64, so the FP32 error bound (9 * 2^-24 * A|X| per entry) does not grow with the
+// FP32 sums are compensated per lane (Kahan) before the lane tree, and the warps of a shared task
+// and hub chunks are added in FP64, so the FP32 error bound (9 * 2^-24 * A|X| per entry) does not grow with the
 // degree or depend on the signs of X.
 #include <stdio.h>
 #include <string.h>
@@ -59,18 +60,44 @@ struct SpmmParams {
   const uint32_t* tbits;
   const Task* tasks;
   const PTask* ptasks;
-  int64_t ntasks, nhub_tasks, task_ctas;
+  int64_t ntasks, nhub_tasks;
+  // tasks [0, wide4) run on four warps each, [wide4, wide2) on two, the rest on one; CTA ranges
+  int64_t wide4, wide2, ctas4, ctas2, task_ctas;
   const int32_t* slice_rows;
   const int32_t* ell;
-  int64_t nslices;
-  int nbuckets;
+  int nbuckets, shared;   // shared: lanes share rows of the slices
   int32_t bucket_deg[kMaxBuckets];
   int32_t bucket_slice_begin[kMaxBuckets + 1];
+  int32_t bucket_warp_begin[kMaxBuckets + 1];  // first warp (after the tasks') of each bucket's slices
   int64_t bucket_ell_base[kMaxBuckets];
 };
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWarpsPerCta = 8;
+
+// Warps of a CTA that share a task: a warp takes up to 128 non-zeros a round, so a task of 4096 on
+// one warp is a serial chain of 32 rounds of two dependent loads, 35 to 50 us whatever the size of
+// the graph.  In plans for at most kWideCols columns, and in streamed panels, hub chunks and rows
+// above 2048 take four warps and rows above kWideLen two (R-MAT with 16384 vertices: FP32 b = 4 35
+// -> 14 us, FP64 b = 4 48 -> 19 us; 131072 vertices: 58 -> 27 and 80 -> 70 us).  With more columns
+// there are long rows enough to hide the chain, and four places of X read at once for one row
+// cost locality (4.2 million vertices: FP32 b = 4 446 -> 467 us, b = 16 1.50 -> 1.57 ms; even at a
+// million, 105 -> 109 us).  The rule uses the columns, which the parts of a row partition share with
+// the whole matrix, so that a row's order of summation is the same in both.
+constexpr int64_t kWideCols = 1 << 19;
+constexpr int kWideLen = 1024;
+
+// Lanes that share a row of a slice of degree d, each taking a run of its steps, and warps that
+// share the slice (32 / pieces rows each): one lane per row makes a slice of 128 steps a serial
+// chain of 32 dependent rounds of gathers (and 128 FP64 adds per column), the last thing that a
+// launch waits for (R-MAT with 2^20 vertices, FP32 b = 4: 138 -> 105 us, FP64 b = 1 120 -> 107 us;
+// 1000 vertices, FP64 b = 8 79 -> 29 us).  By the degree only, like the warps per task; FP64 blocks
+// of more than kSharedCols columns keep one lane per row: their adds bind then, and the lanes' sums
+// are more of them (4.2 million vertices, b = 4: 1.08 against 1.11 ms).
+constexpr int64_t kSharedCols = 1 << 20;
+__host__ __device__ __forceinline__ int slice_pieces(int deg, int shared) {
+  return deg <= 32 || !shared ? 1 : (deg <= 64 ? 2 : 4);
+}
 
 // Per-lane running sums.  FP32: Kahan's compensated summation (Kahan 1965; Higham, "Accuracy
 // and Stability of Numerical Algorithms", 2nd ed., Thm. 4.8): c carries the rounding error of
@@ -89,27 +116,42 @@ __device__ __forceinline__ void kahan_add(double& s, double&, double x) { s += x
 __device__ __forceinline__ float kahan_value(float s, float c) { return s - c; }
 __device__ __forceinline__ double kahan_value(double s, double) { return s; }
 
-template <typename T, int B, bool V32, bool PACKED>
-__device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, const T* __restrict__ X,
-                                         T* __restrict__ Y, T* __restrict__ partial, int lane) {
+// Gap field k (w bits) of a packed task's bit stream.
+__device__ __forceinline__ int gap_field(const uint32_t* __restrict__ tb, int k, int w, uint32_t wmask) {
+  const int64_t bit = (int64_t)k * w;
+  const int64_t wi = bit >> 5;
+  return (int)(__funnelshift_r(__ldcs(tb + wi), __ldcs(tb + wi + 1), (int)(bit & 31)) & wmask);
+}
+
+// Task ti on W warps of the CTA (this one takes piece `piece`); W > 1: all warps of the CTA call it
+// (ti past the range: nothing to do but the barriers).
+template <typename T, int B, bool V32, bool PACKED, int W>
+__device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, int64_t tend, const T* __restrict__ X,
+                                         T* __restrict__ Y, T* __restrict__ partial, int warp, int lane, T* red) {
   using G = Geo<T, B, V32>;
-  int64_t start;
-  int row, len;
+  const int piece = warp % W;
+  int64_t start = 0;
+  int row = 0, len = 0;
   int cbase = 0, w = 1;
-  if constexpr (PACKED) {
-    const int4 r0 = __ldg(reinterpret_cast<const int4*>(p.ptasks + ti));
-    const int4 r1 = __ldg(reinterpret_cast<const int4*>(p.ptasks + ti) + 1);
-    start = (int64_t)(uint32_t)r0.x | ((int64_t)r0.y << 32);  // word offset
-    row = r0.z;
-    len = r0.w;
-    cbase = r1.x;
-    w = r1.y;
-  } else {
-    const int4 raw = __ldg(reinterpret_cast<const int4*>(p.tasks + ti));
-    start = (int64_t)(uint32_t)raw.x | ((int64_t)raw.y << 32);
-    row = raw.z;
-    len = raw.w;
+  if (W == 1 || ti < tend) {
+    if constexpr (PACKED) {
+      const int4 r0 = __ldg(reinterpret_cast<const int4*>(p.ptasks + ti));
+      const int4 r1 = __ldg(reinterpret_cast<const int4*>(p.ptasks + ti) + 1);
+      start = (int64_t)(uint32_t)r0.x | ((int64_t)r0.y << 32);  // word offset
+      row = r0.z;
+      len = r0.w;
+      cbase = r1.x;
+      w = r1.y;
+    } else {
+      const int4 raw = __ldg(reinterpret_cast<const int4*>(p.tasks + ti));
+      start = (int64_t)(uint32_t)raw.x | ((int64_t)raw.y << 32);
+      row = raw.z;
+      len = raw.w;
+    }
   }
+  // this warp's entries [k0, len)
+  const int plen = W == 1 ? len : ((len + W - 1) / W + 31) & ~31;
+  const int k0 = min(len, piece * plen), klen = W == 1 ? len : min(len, k0 + plen);
   const int chunk = lane % G::C;
   const int slot = lane / G::C;
   T acc[G::NE], cmp[G::NE];
@@ -119,20 +161,28 @@ __device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, const 
   const uint32_t* __restrict__ tb = p.tbits + start;
   const uint32_t wmask = (1u << w) - 1u;  // 1 <= w <= 31
   int carry = cbase;  // packed: the column reached by the previous round
-  for (int base = 0; base < len; base += 32 * G::UNROLL) {
+  if constexpr (PACKED && W > 1) {
+    // the columns that the earlier pieces cover: every warp adds up its own gaps first
+    __shared__ int span[kWarpsPerCta];
+    int sum = 0;
+#pragma unroll 4
+    for (int k = k0 + lane; k < klen; k += 32) sum += gap_field(tb, k, w, wmask);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(kFull, sum, off);
+    if (lane == 0) span[warp] = sum;
+    __syncthreads();
+    for (int i = 0; i < piece; ++i) carry += span[warp - piece + i];
+  }
+  for (int base = k0; base < klen; base += 32 * G::UNROLL) {
     int cols[G::UNROLL];
 #pragma unroll
     for (int u = 0; u < G::UNROLL; ++u) {
       int k = base + u * 32 + lane;
       if constexpr (PACKED) {
         // field k of w bits, then an inclusive prefix sum of the gaps across the warp
-        if (base + u * 32 < len) {
+        if (base + u * 32 < klen) {
           int g = 0;
-          if (k < len) {
-            const int64_t bit = (int64_t)k * w;
-            const int64_t wi = bit >> 5;
-            g = (int)(__funnelshift_r(__ldcs(tb + wi), __ldcs(tb + wi + 1), (int)(bit & 31)) & wmask);
-          }
+          if (k < klen) g = gap_field(tb, k, w, wmask);
 #pragma unroll
           for (int off = 1; off < 32; off <<= 1) {
             const int y = __shfl_up_sync(kFull, g, off);
@@ -140,12 +190,12 @@ __device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, const 
           }
           const int col = carry + g;
           carry = __shfl_sync(kFull, col, 31);
-          cols[u] = k < len ? col : -1;
+          cols[u] = k < klen ? col : -1;
         } else {
           cols[u] = -1;
         }
       } else {
-        cols[u] = k < len ? __ldcs(ci + k) : -1;
+        cols[u] = k < klen ? __ldcs(ci + k) : -1;
       }
     }
 #pragma unroll
@@ -153,7 +203,7 @@ __device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, const 
 #pragma unroll
       for (int g = 0; g < 32; g += G::P) {
         // rounds whose P slots all lie past the row's end are skipped (warp-uniform test)
-        if (base + u * 32 + g < len) {
+        if (base + u * 32 + g < klen) {
           int col = __shfl_sync(kFull, cols[u], g + slot);
           if (col >= 0) {
             T f[G::NE];
@@ -186,33 +236,51 @@ __device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, const 
   }
 #pragma unroll
   for (int off = 16 >> G::LNE; off >= G::C; off >>= 1) acc[0] += __shfl_xor_sync(kFull, acc[0], off);
-  if ((lane & G::PLAIN_MASK) == 0) {
-    T* dst = ti < p.nhub_tasks ? partial + ti * B : Y + (int64_t)row * B;
-    dst[chunk * G::NE + ebase] = acc[0];
+  T* dst = ti < p.nhub_tasks ? partial + ti * B : Y + (int64_t)row * B;
+  if constexpr (W == 1) {
+    if ((lane & G::PLAIN_MASK) == 0) dst[chunk * G::NE + ebase] = acc[0];
+  } else {
+    // the pieces in order, in FP64: one more rounding to T however many there are
+    if ((lane & G::PLAIN_MASK) == 0) red[warp * B + chunk * G::NE + ebase] = acc[0];
+    __syncthreads();
+    if (piece == 0 && lane < B && ti < tend) {
+      double s = (double)red[warp * B + lane];
+#pragma unroll
+      for (int i = 1; i < W; ++i) s += (double)red[(warp + i) * B + lane];
+      dst[lane] = (T)s;
+    }
   }
 }
 
+// Warp `wi` of the slices.
 template <typename T, int B, bool V32>
-__device__ __forceinline__ void run_slice(const SpmmParams& p, int64_t si, const T* __restrict__ X,
+__device__ __forceinline__ void run_slice(const SpmmParams& p, int wi, const T* __restrict__ X,
                                           T* __restrict__ Y, int lane) {
   using G = Geo<T, B, V32>;
-  // bucket = last one whose first slice is <= si (buckets are non-empty, so strictly increasing)
+  // bucket = last one whose first warp is <= wi (buckets are non-empty, so strictly increasing)
   int lo = 0, hi = p.nbuckets - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (p.bucket_slice_begin[mid] <= si) lo = mid;
+    if (p.bucket_warp_begin[mid] <= wi) lo = mid;
     else hi = mid - 1;
   }
   const int bkt = lo;
   const int deg = p.bucket_deg[bkt];
-  const int64_t off = p.bucket_ell_base[bkt] + (si - p.bucket_slice_begin[bkt]) * 32 * (int64_t)deg;
-  const int row = __ldcs(p.slice_rows + si * 32 + lane);
+  const int pieces = slice_pieces(deg, p.shared), nrows = 32 / pieces;
+  const int unit = wi - p.bucket_warp_begin[bkt];
+  const int in_bucket = unit / pieces, piece = lane / nrows;
+  const int srow = (unit % pieces) * nrows + lane % nrows;   // row of the slice
+  const int64_t si = (int64_t)p.bucket_slice_begin[bkt] + in_bucket;
+  const int64_t off = p.bucket_ell_base[bkt] + in_bucket * 32 * (int64_t)deg;
+  const int len = ((deg + pieces - 1) / pieces + 3) & ~3;    // steps of a piece
+  const int t1 = min(deg, (piece + 1) * len);
+  const int row = __ldcs(p.slice_rows + si * 32 + srow);
   T acc[B], cmp[B];
 #pragma unroll
   for (int e = 0; e < B; ++e) acc[e] = cmp[e] = T(0);
-  const int32_t* __restrict__ e = p.ell + off + lane;
-  int t = 0;
-  for (; t + 4 <= deg; t += 4) {
+  const int32_t* __restrict__ e = p.ell + off + srow;
+  int t = piece * len;
+  for (; t + 4 <= t1; t += 4) {
     int c[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) c[u] = __ldcs(e + (t + u) * 32);
@@ -226,7 +294,7 @@ __device__ __forceinline__ void run_slice(const SpmmParams& p, int64_t si, const
         for (int q = 0; q < G::NE; ++q) kahan_add(acc[ch * G::NE + q], cmp[ch * G::NE + q], f[q]);
       }
   }
-  for (; t < deg; ++t) {
+  for (; t < t1; ++t) {
     int c = __ldcs(e + t * 32);
 #pragma unroll
     for (int ch = 0; ch < G::C; ++ch) {
@@ -238,46 +306,108 @@ __device__ __forceinline__ void run_slice(const SpmmParams& p, int64_t si, const
   }
 #pragma unroll
   for (int q = 0; q < B; ++q) acc[q] = kahan_value(acc[q], cmp[q]);
-  if (row >= 0) {
-    using F = FragOf<T, B>;  // stores in 16-byte pieces
+  if (pieces == 1) {
+    if (row >= 0) {
+      using F = FragOf<T, B>;  // stores in 16-byte pieces
 #pragma unroll
-    for (int ch = 0; ch < F::NCH; ++ch) st_frag<T, F::NE>(Y + (int64_t)row * B + ch * F::NE, acc + ch * F::NE);
+      for (int ch = 0; ch < F::NCH; ++ch) st_frag<T, F::NE>(Y + (int64_t)row * B + ch * F::NE, acc + ch * F::NE);
+    }
+    return;
   }
+  // the pieces' sums: lanes 16 apart, then (four pieces) 8 apart, each level also dividing the
+  // columns between the two lanes while there are two
+  constexpr int H1 = B >= 2 ? B / 2 : 1, H2 = H1 >= 2 ? H1 / 2 : 1;
+  T* y = Y + (int64_t)row * B;
+  bool writer = row >= 0;
+  const bool up1 = (lane & 16) != 0, up2 = (lane & 8) != 0;
+#pragma unroll
+  for (int i = 0; i < H1; ++i) {
+    const T send = B >= 2 && !up1 ? acc[(i + H1) % B] : acc[i];
+    const T keep = B >= 2 && up1 ? acc[(i + H1) % B] : acc[i];
+    acc[i] = keep + __shfl_xor_sync(kFull, send, 16);
+  }
+  if (B >= 2) y += up1 ? H1 : 0;
+  else writer = writer && !up1;
+  if (pieces == 2) {
+    if (writer) st_row<T, H1>(y, acc);
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < H2; ++i) {
+    const T send = H1 >= 2 && !up2 ? acc[(i + H2) % B] : acc[i];
+    const T keep = H1 >= 2 && up2 ? acc[(i + H2) % B] : acc[i];
+    acc[i] = keep + __shfl_xor_sync(kFull, send, 8);
+  }
+  if (H1 >= 2) y += up2 ? H2 : 0;
+  else writer = writer && !up2;
+  if (writer) st_row<T, H2>(y, acc);
 }
 
 template <typename T, int B, bool V32, bool PACKED>
 __global__ void __launch_bounds__(256) spmm_main_kernel(const SpmmParams p, const T* __restrict__ X,
                                                         T* __restrict__ Y, T* __restrict__ partial) {
+  __shared__ T red[kWarpsPerCta * B];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if ((int64_t)blockIdx.x < p.task_ctas) {
-    const int64_t ti = (int64_t)blockIdx.x * kWarpsPerCta + warp;
-    if (ti < p.ntasks) run_task<T, B, V32, PACKED>(p, ti, X, Y, partial, lane);
+  const int64_t cta = blockIdx.x;
+  if (cta < p.ctas4) {
+    run_task<T, B, V32, PACKED, 4>(p, cta * 2 + warp / 4, p.wide4, X, Y, partial, warp, lane, red);
+  } else if (cta < p.ctas2) {
+    run_task<T, B, V32, PACKED, 2>(p, p.wide4 + (cta - p.ctas4) * 4 + warp / 2, p.wide2, X, Y, partial, warp, lane, red);
+  } else if (cta < p.task_ctas) {
+    const int64_t ti = p.wide2 + (cta - p.ctas2) * kWarpsPerCta + warp;
+    if (ti < p.ntasks) run_task<T, B, V32, PACKED, 1>(p, ti, p.ntasks, X, Y, partial, warp, lane, red);
   } else {
-    const int64_t si = ((int64_t)blockIdx.x - p.task_ctas) * kWarpsPerCta + warp;
-    if (si < p.nslices) run_slice<T, B, V32>(p, si, X, Y, lane);
+    const int wi = (int)(blockIdx.x - p.task_ctas) * kWarpsPerCta + warp;
+    if (wi < p.bucket_warp_begin[p.nbuckets]) run_slice<T, B, V32>(p, wi, X, Y, lane);
   }
 }
 
-// Y[hub_rows[h]] = sum of the hub's task partials in task order, in FP64 with Neumaier's
-// compensation (Neumaier 1974: the TwoSum error of every add is collected separately), then
-// one rounding to T: the partials add with an error of at most 2^-53 |sum| + O(k 2^-106) sum
-// |partial| whatever their number k, so a hub adds one rounding of T to its chunks' errors.
+// s + e <- (s + e) + x exactly up to the rounding of e (Neumaier 1974: the TwoSum error of every
+// add is collected separately).
+__device__ __forceinline__ void neumaier_add(double& s, double& e, double x) {
+  const double u = s + x;
+  e += fabs(s) >= fabs(x) ? (s - u) + x : (x - u) + s;
+  s = u;
+}
+
+// Y[hub_rows[h]] = sum of the hub's task partials in FP64, then one rounding to T.  One warp per
+// hub row: lane l adds column l % B of tasks l / B, l / B + 32 / B, .. in order, then the lanes of a
+// column are added in a fixed tree (R-MAT with 2^20 vertices, FP32 b = 4: 8.4 us with a thread per
+// entry over all of a row's partials, 2.4 us now).  Plain adds while a lane has at most kPlainPartials of them (their
+// error is then below 69 * 2^-53, less than a lane's run of a long row may have; FP64 adds are
+// what the kernel's time is made of), compensated ones above, so that the error does not grow with
+// the degree.
+constexpr int kPlainPartials = 64;
 template <typename T, int B>
-__global__ void hub_reduce_kernel(const int32_t* __restrict__ hub_rows,
-                                  const int32_t* __restrict__ hub_task_begin, int64_t nhub,
-                                  const T* __restrict__ partial, T* __restrict__ Y) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nhub * B) return;
-  const int64_t h = i / B;
-  const int c = (int)(i % B);
+__global__ void __launch_bounds__(256) hub_reduce_kernel(const int32_t* __restrict__ hub_rows,
+                                                         const int32_t* __restrict__ hub_task_begin,
+                                                         int64_t nhub, const T* __restrict__ partial,
+                                                         T* __restrict__ Y) {
+  const int64_t h = (int64_t)blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
+  if (h >= nhub) return;
+  const int lane = threadIdx.x & 31, c = lane % B, slot = lane / B;
+  const int t0 = hub_task_begin[h], t1 = hub_task_begin[h + 1];
+  const T* src = partial + (int64_t)t0 * B + lane;   // task t0 + slot, column c
+  const int steps = (t1 - t0 - slot + 32 / B - 1) / (32 / B);
   double s = 0.0, e = 0.0;
-  for (int t = hub_task_begin[h]; t < hub_task_begin[h + 1]; ++t) {
-    const double x = (double)partial[(int64_t)t * B + c];
-    const double u = s + x;
-    e += fabs(s) >= fabs(x) ? (s - u) + x : (x - u) + s;
-    s = u;
+  if (t1 - t0 <= kPlainPartials * (32 / B)) {
+#pragma unroll 4
+    for (int t = 0; t < steps; ++t) s += (double)src[t * 32];
+#pragma unroll
+    for (int off = B; off < 32; off <<= 1) s += __shfl_xor_sync(kFull, s, off);
+  } else {
+#pragma unroll 4
+    for (int t = 0; t < steps; ++t) neumaier_add(s, e, (double)src[(int64_t)t * 32]);
+#pragma unroll
+    for (int off = B; off < 32; off <<= 1) {
+      const double s2 = __shfl_xor_sync(kFull, s, off), e2 = __shfl_xor_sync(kFull, e, off);
+      neumaier_add(s, e, s2);
+      e += e2;
+    }
   }
-  Y[(int64_t)hub_rows[h] * B + c] = (T)(s + e);
+  // an infinite partial makes the error term NaN: the plain sum is the result then
+  const double r = s + e;
+  if (lane < B) Y[(int64_t)hub_rows[h] * B + c] = (T)(r == r ? r : s);
 }
 
 // Window size for an L2 access-policy window over `bytes` of X: the device's largest window,
@@ -314,16 +444,25 @@ static int launch_spmm(const PlanView& pv, const T* X, T* Y, T* partial, cudaStr
   p.nhub_tasks = pv.nhub_tasks;
   p.slice_rows = pv.slice_rows;
   p.ell = pv.ell;
-  p.nslices = pv.nslices;
   p.nbuckets = pv.nbuckets;
+  p.shared = sizeof(T) == 4 || pv.x_rows <= kSharedCols;
+  int64_t warps = 0;
   for (int i = 0; i < pv.nbuckets; ++i) {
     p.bucket_deg[i] = pv.deg_of_bucket[i];
     p.bucket_slice_begin[i] = pv.deg_slice_begin[i];
+    p.bucket_warp_begin[i] = (int32_t)warps;
     p.bucket_ell_base[i] = pv.deg_ell_base[i];
+    const int64_t end = i + 1 < pv.nbuckets ? pv.deg_slice_begin[i + 1] : pv.nslices;
+    warps += (end - pv.deg_slice_begin[i]) * slice_pieces(pv.deg_of_bucket[i], p.shared);
   }
   p.bucket_slice_begin[pv.nbuckets] = (int32_t)pv.nslices;
-  p.task_ctas = ceil_div(pv.ntasks, kWarpsPerCta);
-  const int64_t ctas = p.task_ctas + ceil_div(pv.nslices, kWarpsPerCta);
+  p.bucket_warp_begin[pv.nbuckets] = (int32_t)warps;
+  p.wide4 = pv.wide4;
+  p.wide2 = pv.wide2;
+  p.ctas4 = ceil_div(pv.wide4, 2);
+  p.ctas2 = p.ctas4 + ceil_div(pv.wide2 - pv.wide4, 4);
+  p.task_ctas = p.ctas2 + ceil_div(pv.ntasks - pv.wide2, kWarpsPerCta);
+  const int64_t ctas = p.task_ctas + ceil_div(warps, kWarpsPerCta);
   if (ctas > 0) {
     // 256-bit gathers when an X row spans at least 32 bytes and X is 32-byte aligned
     bool v32 = false;
@@ -363,8 +502,7 @@ static int launch_spmm(const PlanView& pv, const T* X, T* Y, T* partial, cudaStr
     FE_CUDA(cudaGetLastError());
   }
   if (pv.nhub > 0) {
-    const int64_t th = pv.nhub * B;
-    hub_reduce_kernel<T, B><<<(unsigned)ceil_div(th, 256), 256, 0, s>>>(
+    hub_reduce_kernel<T, B><<<(unsigned)ceil_div(pv.nhub, kWarpsPerCta), 256, 0, s>>>(
         pv.hub_rows, pv.hub_task_begin, pv.nhub, partial, Y);
     count_launch();
     FE_CUDA(cudaGetLastError());
@@ -382,6 +520,8 @@ PlanView resident_view(fe_csr h) {
   v.tasks = pl.d_tasks;
   v.ntasks = pl.ntasks;
   v.nhub_tasks = pl.nhub_tasks;
+  v.wide4 = pl.wide4;
+  v.wide2 = pl.wide2;
   v.slice_rows = pl.d_slice_rows;
   v.ell = pl.d_ell;
   v.nslices = pl.nslices;
@@ -513,6 +653,18 @@ static void pack_tasks(HostPlan& hp) {
   hp.packed = true;
 }
 
+void plan_wide(const HostPlan& hp, int64_t ncols, bool streamed, int64_t* wide4, int64_t* wide2) {
+  *wide4 = *wide2 = 0;
+  if (ncols > kWideCols && !streamed) return;
+  // the tasks after the hub chunks are rows by descending degree
+  int64_t t = hp.nhub_tasks;
+  auto len = [&](int64_t i) { return hp.packed ? hp.ptasks[i].len : hp.tasks[i].len; };
+  while (t < hp.ntasks && len(t) > 2 * kWideLen) ++t;
+  *wide4 = t;
+  while (t < hp.ntasks && len(t) > kWideLen) ++t;
+  *wide2 = t;
+}
+
 int build_host_plan(const int64_t* rowptr, const int32_t* colidx, int64_t r0, int64_t r1,
                     int tail_max, int hub_min, int hub_chunk, bool packed, HostPlan& hp) {
   hp = HostPlan();
@@ -545,7 +697,7 @@ int build_host_plan(const int64_t* rowptr, const int32_t* colidx, int64_t r0, in
     nslices += sl;
     ell_total += sl * 32 * d;
   }
-  FE_ARG(nslices < INT32_MAX, "spmm plan: too many tail slices");
+  FE_ARG(nslices < INT32_MAX / 4, "spmm plan: too many tail slices");
   hp.nslices = nslices;
   hp.slice_rows.assign(nslices * 32, -1);
   std::vector<int64_t> cursor(tail_max + 1, 0);
@@ -643,6 +795,7 @@ int spmm_build_plan(fe_csr h, const int64_t* rowptr, const int32_t* colidx_raw, 
   pl.nslices = hp.nslices;
   pl.ntasks = hp.ntasks;
   pl.nhub_tasks = hp.nhub_tasks;
+  plan_wide(hp, h->ncols, false, &pl.wide4, &pl.wide2);
   pl.nhub = hp.nhub;
   if (packed) {
     FE_TRY(dev_upload(h, (void**)&pl.d_tbits, hp.tbits.data(), sizeof(uint32_t) * hp.tbits.size()));

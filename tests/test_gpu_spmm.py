@@ -304,3 +304,31 @@ def test_spmm_l2_window_same_results(graphs, prec):
         X = to_dev(graphgen.normal_block(g.n, b, seed=b, dtype=NP[prec]))
         with fe.Csr.from_graph(g) as h, fe.Csr.from_graph(g, l2_persist=True) as hl:
             assert np.array_equal(fe.spmm(h, X).cpu().numpy(), fe.spmm(hl, X).cpu().numpy())
+
+
+@pytest.mark.parametrize("ncols", [9000, (1 << 19) + 3])
+@pytest.mark.parametrize("fmt", ["plain", "packed"])
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+def test_spmm_shared_rows(prec, fmt, ncols):
+    """Rows at the edges of the sharing rules: 32 | 33 and 64 | 65 steps of a slice (one, two and
+    four lanes a row), 128 | 129, tasks of 1024 | 1025 and 2048 | 2049 entries (one, two and four
+    warps where the matrix has few columns), hub chunks of 4096 with a ragged last one and hubs with
+    more than 64 partials per lane.  Bounds: those of the interface, 9 * 2^-24 and 518 * 2^-53 of
+    A|X|, the exact sums in extended precision."""
+    r = np.random.default_rng(ncols)
+    degs = [0, 1, 3, 4, 31, 32, 33, 35, 63, 64, 65, 66, 97, 127, 128, 129, 1023, 1024, 1025, 1057, 2047, 2048,
+            2049, 2177, 4095, 4096, 4097, 5000, 8192, 8999] * 2
+    cols = [np.sort(r.choice(ncols, d, replace=False)).astype(np.int32) for d in degs]
+    big = np.sort(r.integers(0, ncols, 700000)).astype(np.int32)   # repeated columns
+    cols.append(big)
+    rowptr = np.concatenate([[0], np.cumsum([len(c) for c in cols])]).astype(np.int64)
+    colidx = np.concatenate(cols)
+    with fe.Csr(rowptr, colidx, ncols=ncols, index_format=fmt) as h:
+        for b in (1, 2, 4, 8, 16):
+            X = r.standard_normal((ncols, b)).astype(NP[prec])
+            Y = fe.spmm(h, to_dev(X)).cpu().numpy()
+            for i, c in enumerate(cols):
+                ref = X[c].astype(np.longdouble).sum(0)
+                mag = np.abs(X[c]).astype(np.longdouble).sum(0)
+                bound = (9 * 2.0 ** -24 if prec == "f32" else 518 * 2.0 ** -53) * mag
+                assert np.all(np.abs(Y[i] - ref) <= bound), (len(c), b)
