@@ -39,12 +39,16 @@ namespace fe {
 static_assert(sizeof(Task) == 16, "Task must be 16 bytes");
 static_assert(sizeof(PTask) == 32, "PTask must be 32 bytes");
 
+template <typename T, int B>
+constexpr bool kUseFx = sizeof(T) == 8 && B >= 2;
+template <typename T, int B>
+constexpr int kFxBytes = !kUseFx<T, B> ? 0 : 16;
 // Per (type, b, fragment width) geometry: a lane moves NE elements (<= FB bytes: 16, or 32
 // with 256-bit loads when X is 32-byte aligned) per load; an X row of b elements spans C lanes
 // in a warp task (P = 32 / C rows gathered per warp instruction) and C chunks in a tail lane.
 template <typename T, int B, bool V32>
 struct Geo {
-  static constexpr int FB = V32 ? 32 : 16;
+  static constexpr int FB = kFxBytes<T, B> ? kFxBytes<T, B> : (V32 ? 32 : 16);
   static constexpr int ROWB = B * (int)sizeof(T);
   static constexpr int NE = ROWB <= FB ? B : FB / (int)sizeof(T);
   static constexpr int C = B / NE;
@@ -68,7 +72,7 @@ struct SpmmParams {
   int nbuckets, shared;   // shared: lanes share rows of the slices
   int32_t bucket_deg[kMaxBuckets];
   int32_t bucket_slice_begin[kMaxBuckets + 1];
-  int32_t bucket_warp_begin[kMaxBuckets + 1];  // first warp (after the tasks') of each bucket's slices
+  uint32_t bucket_warp_begin[kMaxBuckets + 1];  // first warp (after the tasks') of each bucket's slices
   int64_t bucket_ell_base[kMaxBuckets];
 };
 
@@ -91,9 +95,9 @@ constexpr int kWideLen = 1024;
 // share the slice (32 / pieces rows each): one lane per row makes a slice of 128 steps a serial
 // chain of 32 dependent rounds of gathers (and 128 FP64 adds per column), the last thing that a
 // launch waits for (R-MAT with 2^20 vertices, FP32 b = 4: 138 -> 105 us, FP64 b = 1 120 -> 107 us;
-// 1000 vertices, FP64 b = 8 79 -> 29 us).  By the degree only, like the warps per task; FP64 blocks
-// of more than kSharedCols columns keep one lane per row: their adds bind then, and the lanes' sums
-// are more of them (4.2 million vertices, b = 4: 1.08 against 1.11 ms).
+// 1000 vertices, FP64 b = 8 79 -> 29 us).  By the degree only, like the warps per task; FP64 b = 1
+// with more than kSharedCols columns keeps one lane per row (its adds are all FP64, and the lanes'
+// sums are more of them; 4.2 million vertices: 416 against 423 us).
 constexpr int64_t kSharedCols = 1 << 20;
 __host__ __device__ __forceinline__ int slice_pieces(int deg, int shared) {
   return deg <= 32 || !shared ? 1 : (deg <= 64 ? 2 : 4);
@@ -115,6 +119,56 @@ __device__ __forceinline__ void kahan_add(float& s, float& c, float x) {
 __device__ __forceinline__ void kahan_add(double& s, double&, double x) { s += x; }
 __device__ __forceinline__ float kahan_value(float s, float c) { return s - c; }
 __device__ __forceinline__ double kahan_value(double s, double) { return s; }
+
+// FP64 sums in integers.  An FP64 add occupies the FP64 pipe of an SM for 16 clocks per warp; the
+// 32-bit integer units take the 15 instructions of an aligned integer add in half of that, beside it.
+// So of every four gathered values one is added in FP64 and three as integers: an Fx holds
+// a * 2^((e >> 20) - 1080), e the largest biased exponent so far (in its place in the high word),
+// and a value's 53-bit significand, shifted left by 5 and right by its distance to e, is added to a.
+// Bits below 2^-57 of the largest value are dropped (floor; also from a when e rises): between two
+// flushes, 24 values (4.6 bits, so a stays within 63) and at most 8 rises of e, an error below 2^-52
+// of the largest value, no more than that of as many FP64 adds.  Values with exponents near the ends
+// of the range (infinities, NaN, below 2^-943) set `bad`, and the sums are formed again with FP64
+// adds.  Measured against FP64 adds alone (R-MAT, X 32-byte aligned): 4.2 million vertices b = 2 585
+// -> 511 us, b = 4 1085 -> 686, b = 8 2068 -> 1319, b = 16 4.18 -> 2.24 ms; a million, b = 4 288 ->
+// 162 us.  The gathers bind then (FP32 b = 8, rows of the same 32 bytes: 615 us).
+struct Fx {
+  long long a;
+  unsigned e;
+};
+constexpr int kFxGroups = 8;   // groups of four values between flushes
+__device__ __forceinline__ long long fx_align(unsigned hi, unsigned lo, unsigned ev, unsigned e) {
+  const unsigned m = (hi & 0xfffffu) | min(ev, 0x100000u);   // implicit bit (0 for zeros, subnormals)
+  unsigned long long t = (((unsigned long long)m << 32) | lo) << 5;
+  asm("shr.u64 %0, %0, %1;" : "+l"(t) : "r"((e - ev) >> 20));   // shifts of 64 and more give 0
+  const long long sign = (int)hi >> 31;
+  return (long long)t ^ sign;
+}
+__device__ __forceinline__ void fx_add3(Fx& f, double x, double y, double z) {
+  const unsigned hx = __double2hiint(x), hy = __double2hiint(y), hz = __double2hiint(z);
+  const unsigned ex = hx & 0x7ff00000u, ey = hy & 0x7ff00000u, ez = hz & 0x7ff00000u;
+  const unsigned e = max(max(ex, ey), max(ez, f.e));
+  asm("shr.s64 %0, %0, %1;" : "+l"(f.a) : "r"((e - f.e) >> 20));
+  f.e = e;
+  f.a += fx_align(hx, __double2loint(x), ex, e) + fx_align(hy, __double2loint(y), ey, e) +
+         fx_align(hz, __double2loint(z), ez, e);
+}
+// s += f, f = 0
+__device__ __forceinline__ void fx_flush(double& s, Fx& f, bool& bad) {
+  bad = bad || f.e >= 0x7d000000u || (f.e < 0x05000000u && f.a != 0);
+  const double v = __ll2double_rn(f.a);
+  const double x = __hiloint2double(__double2hiint(v) + (int)f.e - (1080 << 20), __double2loint(v));
+  s += f.a != 0 ? x : 0.0;
+  f.a = 0;
+  f.e = 0;
+}
+// FP64 blocks whose sums the FP64 adds would bind (b = 1 is bound by its gathers).
+// Lanes of a slice that share a row by its columns, without 256-bit gathers: 16 bytes of it each.
+// With Fx sums a column takes 13 registers (four gathers in flight), and the warps that fit decide
+// (b = 4 at 4.2 million vertices: 950 us with four columns a lane, 80 registers).
+template <typename T, int B, bool V32>
+constexpr int kColLanes = V32 || B * sizeof(T) <= 16 || (sizeof(T) == 8 && !kUseFx<T, B>) ? 1 : B * (int)sizeof(T) / 16;
+constexpr int kFxMinDegree = 12;   // slices of shorter rows: the flush would cost more than it saves
 
 // Gap field k (w bits) of a packed task's bit stream.
 __device__ __forceinline__ int gap_field(const uint32_t* __restrict__ tb, int k, int w, uint32_t wmask) {
@@ -173,47 +227,97 @@ __device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, int64_
     __syncthreads();
     for (int i = 0; i < piece; ++i) carry += span[warp - piece + i];
   }
-  for (int base = k0; base < klen; base += 32 * G::UNROLL) {
-    int cols[G::UNROLL];
+  // the column of entry base + lane (-1 past the end); packed: calls in order, all lanes
+  auto load_col = [&](int base) {
+    const int k = base + lane;
+    if constexpr (PACKED) {
+      // field k of w bits, then an inclusive prefix sum of the gaps across the warp
+      if (base >= klen) return -1;
+      int g = 0;
+      if (k < klen) g = gap_field(tb, k, w, wmask);
 #pragma unroll
-    for (int u = 0; u < G::UNROLL; ++u) {
-      int k = base + u * 32 + lane;
-      if constexpr (PACKED) {
-        // field k of w bits, then an inclusive prefix sum of the gaps across the warp
-        if (base + u * 32 < klen) {
-          int g = 0;
-          if (k < klen) g = gap_field(tb, k, w, wmask);
+      for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(kFull, g, off);
+        if (lane >= off) g += y;
+      }
+      const int col = carry + g;
+      carry = __shfl_sync(kFull, col, 31);
+      return k < klen ? col : -1;
+    } else {
+      return k < klen ? __ldcs(ci + k) : -1;
+    }
+  };
+  auto plain = [&]() {
+    for (int base = k0; base < klen; base += 32 * G::UNROLL) {
+      int cols[G::UNROLL];
 #pragma unroll
-          for (int off = 1; off < 32; off <<= 1) {
-            const int y = __shfl_up_sync(kFull, g, off);
-            if (lane >= off) g += y;
+      for (int u = 0; u < G::UNROLL; ++u) cols[u] = load_col(base + u * 32);
+#pragma unroll
+      for (int u = 0; u < G::UNROLL; ++u) {
+#pragma unroll
+        for (int g = 0; g < 32; g += G::P) {
+          // rounds whose P slots all lie past the row's end are skipped (warp-uniform test)
+          if (base + u * 32 + g < klen) {
+            int col = __shfl_sync(kFull, cols[u], g + slot);
+            if (col >= 0) {
+              T f[G::NE];
+              ld_frag<T, G::NE>(X + (int64_t)col * B + chunk * G::NE, f);
+#pragma unroll
+              for (int e = 0; e < G::NE; ++e) kahan_add(acc[e], cmp[e], f[e]);
+            }
           }
-          const int col = carry + g;
-          carry = __shfl_sync(kFull, col, 31);
-          cols[u] = k < klen ? col : -1;
-        } else {
-          cols[u] = -1;
         }
-      } else {
-        cols[u] = k < klen ? __ldcs(ci + k) : -1;
+      }
+    }
+  };
+  if constexpr (kUseFx<T, B>) {
+    constexpr int PER = 32 / G::P, NG = G::UNROLL * PER;   // gathers of a lane per 32 columns, per round
+    const int carry0 = carry;
+    Fx fa[G::NE];
+    bool bad = false;
+#pragma unroll
+    for (int e = 0; e < G::NE; ++e) fa[e] = Fx{0, 0u};
+    int groups = 0;
+    int cols[G::UNROLL];   // of the coming round, loaded a round ahead
+#pragma unroll
+    for (int u = 0; u < G::UNROLL; ++u) cols[u] = load_col(k0 + u * 32);
+    for (int base = k0; base < klen; base += 32 * G::UNROLL) {
+#pragma unroll
+      for (int v0 = 0; v0 < NG; v0 += 4) {
+        T f[4][G::NE];   // four gathers of the lane (zero past the row's end)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          const int col = __shfl_sync(kFull, cols[(v0 + v) / PER], (v0 + v) % PER * G::P + slot);
+#pragma unroll
+          for (int e = 0; e < G::NE; ++e) f[v][e] = T(0);
+          if (col >= 0) ld_frag<T, G::NE>(X + (int64_t)col * B + chunk * G::NE, f[v]);
+        }
+        if (v0 + 4 == NG) {
+#pragma unroll
+          for (int u = 0; u < G::UNROLL; ++u) cols[u] = load_col(base + (G::UNROLL + u) * 32);
+        }
+#pragma unroll
+        for (int e = 0; e < G::NE; ++e) {
+          acc[e] += f[0][e];
+          fx_add3(fa[e], f[1][e], f[2][e], f[3][e]);
+        }
+      }
+      if (++groups == kFxGroups * 4 / NG) {
+#pragma unroll
+        for (int e = 0; e < G::NE; ++e) fx_flush(acc[e], fa[e], bad);
+        groups = 0;
       }
     }
 #pragma unroll
-    for (int u = 0; u < G::UNROLL; ++u) {
+    for (int e = 0; e < G::NE; ++e) fx_flush(acc[e], fa[e], bad);
+    if (__any_sync(kFull, bad)) {
 #pragma unroll
-      for (int g = 0; g < 32; g += G::P) {
-        // rounds whose P slots all lie past the row's end are skipped (warp-uniform test)
-        if (base + u * 32 + g < klen) {
-          int col = __shfl_sync(kFull, cols[u], g + slot);
-          if (col >= 0) {
-            T f[G::NE];
-            ld_frag<T, G::NE>(X + (int64_t)col * B + chunk * G::NE, f);
-#pragma unroll
-            for (int e = 0; e < G::NE; ++e) kahan_add(acc[e], cmp[e], f[e]);
-          }
-        }
-      }
+      for (int e = 0; e < G::NE; ++e) acc[e] = T(0);
+      carry = carry0;
+      plain();
     }
+  } else {
+    plain();
   }
 #pragma unroll
   for (int e = 0; e < G::NE; ++e) acc[e] = kahan_value(acc[e], cmp[e]);
@@ -254,9 +358,10 @@ __device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, int64_
 
 // Warp `wi` of the slices.
 template <typename T, int B, bool V32>
-__device__ __forceinline__ void run_slice(const SpmmParams& p, int wi, const T* __restrict__ X,
+__device__ __forceinline__ void run_slice(const SpmmParams& p, unsigned wi, const T* __restrict__ X,
                                           T* __restrict__ Y, int lane) {
-  using G = Geo<T, B, V32>;
+  constexpr int SC = kColLanes<T, B, V32>, K = B / SC;   // lanes per row for its columns, columns of each
+  constexpr int NE = Geo<T, B, V32>::NE < K ? Geo<T, B, V32>::NE : K;
   // bucket = last one whose first warp is <= wi (buckets are non-empty, so strictly increasing)
   int lo = 0, hi = p.nbuckets - 1;
   while (lo < hi) {
@@ -266,67 +371,99 @@ __device__ __forceinline__ void run_slice(const SpmmParams& p, int wi, const T* 
   }
   const int bkt = lo;
   const int deg = p.bucket_deg[bkt];
-  const int pieces = slice_pieces(deg, p.shared), nrows = 32 / pieces;
-  const int unit = wi - p.bucket_warp_begin[bkt];
-  const int in_bucket = unit / pieces, piece = lane / nrows;
-  const int srow = (unit % pieces) * nrows + lane % nrows;   // row of the slice
+  const int pieces = slice_pieces(deg, p.shared), nrows = 32 / (pieces * SC);
+  const int unit = (int)(wi - p.bucket_warp_begin[bkt]);
+  const int in_bucket = unit / (pieces * SC), piece = lane / (nrows * SC), cl = lane % SC;
+  const int srow = (unit % (pieces * SC)) * nrows + lane / SC % nrows;   // row of the slice
   const int64_t si = (int64_t)p.bucket_slice_begin[bkt] + in_bucket;
   const int64_t off = p.bucket_ell_base[bkt] + in_bucket * 32 * (int64_t)deg;
   const int len = ((deg + pieces - 1) / pieces + 3) & ~3;    // steps of a piece
   const int t1 = min(deg, (piece + 1) * len);
-  const int row = __ldcs(p.slice_rows + si * 32 + srow);
-  T acc[B], cmp[B];
+  int row = -1;
+  if constexpr (!kUseFx<T, B>) row = __ldcs(p.slice_rows + si * 32 + srow);
+  T acc[K], cmp[K];
 #pragma unroll
-  for (int e = 0; e < B; ++e) acc[e] = cmp[e] = T(0);
+  for (int q = 0; q < K; ++q) acc[q] = cmp[q] = T(0);
   const int32_t* __restrict__ e = p.ell + off + srow;
-  int t = piece * len;
-  for (; t + 4 <= t1; t += 4) {
-    int c[4];
+  const T* __restrict__ x = X + cl * K;
+  auto add_row = [&](int c) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) c[u] = __ldcs(e + (t + u) * 32);
+    for (int ch = 0; ch < K; ch += NE) {
+      T f[NE];
+      ld_frag<T, NE>(x + (int64_t)c * B + ch, f);
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+      for (int q = 0; q < NE; ++q) kahan_add(acc[ch + q], cmp[ch + q], f[q]);
+    }
+  };
+  auto plain = [&](int t) {   // steps [t, t1)
+    for (; t + 4 <= t1; t += 4) {
+      int c[4];
 #pragma unroll
-      for (int ch = 0; ch < G::C; ++ch) {
-        T f[G::NE];
-        ld_frag<T, G::NE>(X + (int64_t)c[u] * B + ch * G::NE, f);
+      for (int u = 0; u < 4; ++u) c[u] = __ldcs(e + (t + u) * 32);
 #pragma unroll
-        for (int q = 0; q < G::NE; ++q) kahan_add(acc[ch * G::NE + q], cmp[ch * G::NE + q], f[q]);
+      for (int u = 0; u < 4; ++u) add_row(c[u]);
+    }
+    for (; t < t1; ++t) add_row(__ldcs(e + t * 32));
+  };
+  bool done = false;
+  if constexpr (kUseFx<T, B>) {
+    if (deg >= kFxMinDegree) {
+      Fx fa[K];
+      bool bad = false;
+#pragma unroll
+      for (int q = 0; q < K; ++q) fa[q] = Fx{0, 0u};
+      int t = piece * len, groups = 0;
+      int c[4];   // the next round's columns, loaded a round ahead
+#pragma unroll
+      for (int u = 0; u < 4; ++u) c[u] = t + 4 <= t1 ? __ldcs(e + (t + u) * 32) : 0;
+      for (; t + 4 <= t1; t += 4) {
+        T f[4][K];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) ld_frag<T, K>(x + (int64_t)c[u] * B, f[u]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) c[u] = t + 8 <= t1 ? __ldcs(e + (t + 4 + u) * 32) : 0;
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+          acc[q] += f[0][q];
+          fx_add3(fa[q], f[1][q], f[2][q], f[3][q]);
+        }
+        if (++groups == kFxGroups) {
+#pragma unroll
+          for (int q = 0; q < K; ++q) fx_flush(acc[q], fa[q], bad);
+          groups = 0;
+        }
       }
-  }
-  for (; t < t1; ++t) {
-    int c = __ldcs(e + t * 32);
+      for (; t < t1; ++t) add_row(__ldcs(e + t * 32));
 #pragma unroll
-    for (int ch = 0; ch < G::C; ++ch) {
-      T f[G::NE];
-      ld_frag<T, G::NE>(X + (int64_t)c * B + ch * G::NE, f);
+      for (int q = 0; q < K; ++q) fx_flush(acc[q], fa[q], bad);
+      done = !bad;
+      if (bad) {
 #pragma unroll
-      for (int q = 0; q < G::NE; ++q) kahan_add(acc[ch * G::NE + q], cmp[ch * G::NE + q], f[q]);
+        for (int q = 0; q < K; ++q) acc[q] = T(0);
+      }
     }
   }
+  if (!done) plain(piece * len);
 #pragma unroll
-  for (int q = 0; q < B; ++q) acc[q] = kahan_value(acc[q], cmp[q]);
+  for (int q = 0; q < K; ++q) acc[q] = kahan_value(acc[q], cmp[q]);
+  if constexpr (kUseFx<T, B>) row = __ldcs(p.slice_rows + si * 32 + srow);   // late: one register less
+  T* y = Y + (int64_t)row * B + cl * K;
   if (pieces == 1) {
-    if (row >= 0) {
-      using F = FragOf<T, B>;  // stores in 16-byte pieces
-#pragma unroll
-      for (int ch = 0; ch < F::NCH; ++ch) st_frag<T, F::NE>(Y + (int64_t)row * B + ch * F::NE, acc + ch * F::NE);
-    }
+    if (row >= 0) st_row<T, K>(y, acc);
     return;
   }
   // the pieces' sums: lanes 16 apart, then (four pieces) 8 apart, each level also dividing the
   // columns between the two lanes while there are two
-  constexpr int H1 = B >= 2 ? B / 2 : 1, H2 = H1 >= 2 ? H1 / 2 : 1;
-  T* y = Y + (int64_t)row * B;
+  constexpr int H1 = K >= 2 ? K / 2 : 1, H2 = H1 >= 2 ? H1 / 2 : 1;
   bool writer = row >= 0;
   const bool up1 = (lane & 16) != 0, up2 = (lane & 8) != 0;
 #pragma unroll
   for (int i = 0; i < H1; ++i) {
-    const T send = B >= 2 && !up1 ? acc[(i + H1) % B] : acc[i];
-    const T keep = B >= 2 && up1 ? acc[(i + H1) % B] : acc[i];
+    const T send = K >= 2 && !up1 ? acc[(i + H1) % K] : acc[i];
+    const T keep = K >= 2 && up1 ? acc[(i + H1) % K] : acc[i];
     acc[i] = keep + __shfl_xor_sync(kFull, send, 16);
   }
-  if (B >= 2) y += up1 ? H1 : 0;
+  if (K >= 2) y += up1 ? H1 : 0;
   else writer = writer && !up1;
   if (pieces == 2) {
     if (writer) st_row<T, H1>(y, acc);
@@ -334,8 +471,8 @@ __device__ __forceinline__ void run_slice(const SpmmParams& p, int wi, const T* 
   }
 #pragma unroll
   for (int i = 0; i < H2; ++i) {
-    const T send = H1 >= 2 && !up2 ? acc[(i + H2) % B] : acc[i];
-    const T keep = H1 >= 2 && up2 ? acc[(i + H2) % B] : acc[i];
+    const T send = H1 >= 2 && !up2 ? acc[(i + H2) % K] : acc[i];
+    const T keep = H1 >= 2 && up2 ? acc[(i + H2) % K] : acc[i];
     acc[i] = keep + __shfl_xor_sync(kFull, send, 8);
   }
   if (H1 >= 2) y += up2 ? H2 : 0;
@@ -343,8 +480,13 @@ __device__ __forceinline__ void run_slice(const SpmmParams& p, int wi, const T* 
   if (writer) st_row<T, H2>(y, acc);
 }
 
+template <typename T, int B>
+constexpr bool kWide = B * sizeof(T) >= 32 && !kUseFx<T, B>;
+// Resident CTAs to compile for.
+template <typename T, int B, bool V32>
+constexpr int kMinCtas = kUseFx<T, B> ? 5 : (B * sizeof(T) <= 16 ? 8 : (B == 8 ? 5 : (V32 ? 3 : 7)));
 template <typename T, int B, bool V32, bool PACKED>
-__global__ void __launch_bounds__(256) spmm_main_kernel(const SpmmParams p, const T* __restrict__ X,
+__global__ void __launch_bounds__(256, (kMinCtas<T, B, V32>)) spmm_main_kernel(const SpmmParams p, const T* __restrict__ X,
                                                         T* __restrict__ Y, T* __restrict__ partial) {
   __shared__ T red[kWarpsPerCta * B];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -357,7 +499,7 @@ __global__ void __launch_bounds__(256) spmm_main_kernel(const SpmmParams p, cons
     const int64_t ti = p.wide2 + (cta - p.ctas2) * kWarpsPerCta + warp;
     if (ti < p.ntasks) run_task<T, B, V32, PACKED, 1>(p, ti, p.ntasks, X, Y, partial, warp, lane, red);
   } else {
-    const int wi = (int)(blockIdx.x - p.task_ctas) * kWarpsPerCta + warp;
+    const unsigned wi = (unsigned)(cta - p.task_ctas) * kWarpsPerCta + warp;
     if (wi < p.bucket_warp_begin[p.nbuckets]) run_slice<T, B, V32>(p, wi, X, Y, lane);
   }
 }
@@ -445,18 +587,25 @@ static int launch_spmm(const PlanView& pv, const T* X, T* Y, T* partial, cudaStr
   p.slice_rows = pv.slice_rows;
   p.ell = pv.ell;
   p.nbuckets = pv.nbuckets;
-  p.shared = sizeof(T) == 4 || pv.x_rows <= kSharedCols;
+  // 256-bit gathers (FP32 rows of at least 32 bytes on a 32-byte boundary): fewer rounds than with
+  // 16-byte fragments (R-MAT with 16384 vertices, b = 16: 23 against 37 us; 4.2 million, b = 8: 0.62
+  // against 0.64 ms); b = 16 with many columns takes the fragments and four lanes per slice row,
+  // whose registers allow seven CTAs instead of three (4.2 million: 1.50 -> 1.03 ms)
+  bool v32 = false;
+  if constexpr (kWide<T, B>) v32 = ((uintptr_t)X % 32) == 0 && (B < 16 || pv.x_rows <= kWideCols);
+  const int col_lanes = v32 ? kColLanes<T, B, true> : kColLanes<T, B, false>;
+  p.shared = B > 1 || sizeof(T) == 4 || pv.x_rows <= kSharedCols;
   int64_t warps = 0;
   for (int i = 0; i < pv.nbuckets; ++i) {
     p.bucket_deg[i] = pv.deg_of_bucket[i];
     p.bucket_slice_begin[i] = pv.deg_slice_begin[i];
-    p.bucket_warp_begin[i] = (int32_t)warps;
+    p.bucket_warp_begin[i] = (uint32_t)warps;
     p.bucket_ell_base[i] = pv.deg_ell_base[i];
     const int64_t end = i + 1 < pv.nbuckets ? pv.deg_slice_begin[i + 1] : pv.nslices;
-    warps += (end - pv.deg_slice_begin[i]) * slice_pieces(pv.deg_of_bucket[i], p.shared);
+    warps += (end - pv.deg_slice_begin[i]) * slice_pieces(pv.deg_of_bucket[i], p.shared) * col_lanes;
   }
   p.bucket_slice_begin[pv.nbuckets] = (int32_t)pv.nslices;
-  p.bucket_warp_begin[pv.nbuckets] = (int32_t)warps;
+  p.bucket_warp_begin[pv.nbuckets] = (uint32_t)warps;
   p.wide4 = pv.wide4;
   p.wide2 = pv.wide2;
   p.ctas4 = ceil_div(pv.wide4, 2);
@@ -464,12 +613,9 @@ static int launch_spmm(const PlanView& pv, const T* X, T* Y, T* partial, cudaStr
   p.task_ctas = p.ctas2 + ceil_div(pv.ntasks - pv.wide2, kWarpsPerCta);
   const int64_t ctas = p.task_ctas + ceil_div(warps, kWarpsPerCta);
   if (ctas > 0) {
-    // 256-bit gathers when an X row spans at least 32 bytes and X is 32-byte aligned
-    bool v32 = false;
-    if constexpr (B * sizeof(T) >= 32) v32 = ((uintptr_t)X % 32) == 0;
     void (*kern)(const SpmmParams, const T*, T*, T*) = nullptr;
     if (v32) {
-      if constexpr (B * sizeof(T) >= 32)
+      if constexpr (kWide<T, B>)
         kern = pv.packed ? spmm_main_kernel<T, B, true, true> : spmm_main_kernel<T, B, true, false>;
     } else {
       kern = pv.packed ? spmm_main_kernel<T, B, false, true> : spmm_main_kernel<T, B, false, false>;

@@ -332,3 +332,69 @@ def test_spmm_shared_rows(prec, fmt, ncols):
                 mag = np.abs(X[c]).astype(np.longdouble).sum(0)
                 bound = (9 * 2.0 ** -24 if prec == "f32" else 518 * 2.0 ** -53) * mag
                 assert np.all(np.abs(Y[i] - ref) <= bound), (len(c), b)
+
+
+@pytest.mark.parametrize("fmt", ["plain", "packed"])
+@pytest.mark.parametrize("b", [2, 4, 8, 16])
+def test_spmm_f64_exponents(b, fmt):
+    """The aligned integer sums of FP64 blocks: columns whose entries span all exponents (2^-1000 to
+    2^1000, rising and falling along a row, so that the common exponent rises at any point), columns
+    of equal sign, zeros of both signs among values, sums that cancel.  Bound of the interface,
+    518 * 2^-53 of A|X| (the sums in extended precision)."""
+    r = np.random.default_rng(b)
+    n = 3000
+    degs = [1, 4, 11, 12, 13, 16, 31, 32, 33, 64, 65, 100, 128, 129, 200, 1025, 2049, 2600]
+    cols = [np.sort(r.choice(n, d, replace=False)).astype(np.int32) for d in degs]
+    rowptr = np.concatenate([[0], np.cumsum([len(c) for c in cols])]).astype(np.int64)
+    with fe.Csr(rowptr, np.concatenate(cols), ncols=n, index_format=fmt) as h:
+        for kind in range(6):
+            v = r.standard_normal((n, b))
+            if kind == 0:
+                v = np.ldexp(v, r.integers(-1000, 1000, (n, b)))
+            elif kind == 1:
+                v = np.ldexp(v, np.arange(n)[:, None] // 3 - 500)       # rises along a row
+            elif kind == 2:
+                v = np.ldexp(v, 500 - np.arange(n)[:, None] // 3)       # falls along a row
+            elif kind == 3:
+                v = np.abs(v) + 1.0
+            elif kind == 4:
+                v = np.where(r.random((n, b)) < 0.7, np.where(r.random((n, b)) < 0.5, 0.0, -0.0), v)
+            else:
+                v = np.round(v * 2.0 ** 20) * 2.0 ** 30 + np.round(r.standard_normal((n, b)) * 8)  # 53 bits
+            Y = fe.spmm(h, to_dev(v)).cpu().numpy()
+            for i, c in enumerate(cols):
+                ref = v[c].astype(np.longdouble).sum(0)
+                mag = np.abs(v[c]).astype(np.longdouble).sum(0)
+                assert np.all(np.abs(Y[i] - ref) <= 518 * 2.0 ** -53 * mag), (kind, len(c))
+
+
+@pytest.mark.parametrize("b", [2, 4, 16])
+def test_spmm_f64_special_values(b):
+    """Infinities, NaN, subnormals, zeros and values near overflow give what FP64 adds give: the
+    integer sums hand such rows back.  One special value per row of otherwise ordinary ones."""
+    n = 2500
+    r = np.random.default_rng(b)
+    degs = [12, 40, 128, 130, 1100, 2100, 2499]
+    cols = [np.arange(d, dtype=np.int32) for d in degs]
+    rowptr = np.concatenate([[0], np.cumsum(degs)]).astype(np.int64)
+    with fe.Csr(rowptr, np.concatenate(cols), ncols=n) as h:
+        for special in (np.inf, -np.inf, np.nan, 1.7e308, -1.7e308):
+            v = r.standard_normal((n, b))
+            v[5, 0] = special
+            Y = fe.spmm(h, to_dev(v)).cpu().numpy()
+            for i, d in enumerate(degs):
+                want = v[:d].sum(0)
+                assert np.array_equal(np.isnan(Y[i]), np.isnan(want))
+                ok = ~np.isnan(want)
+                assert np.allclose(Y[i][ok], want[ok], rtol=1e-12, atol=1e-12)
+        v = np.zeros((n, b))
+        assert np.all(fe.spmm(h, to_dev(v)).cpu().numpy() == 0.0)
+        assert np.all(fe.spmm(h, to_dev(-v)).cpu().numpy() == 0.0)
+        v = r.integers(-1000, 1000, (n, b)) * 5e-324                    # subnormals: exact sums
+        Y = fe.spmm(h, to_dev(v)).cpu().numpy()
+        for i, d in enumerate(degs):
+            assert np.array_equal(Y[i], v[:d].sum(0))
+        v = r.standard_normal((n, b)) * 1e-290
+        Y = fe.spmm(h, to_dev(v)).cpu().numpy()
+        for i, d in enumerate(degs):
+            assert np.all(np.abs(Y[i] - v[:d].sum(0)) <= 518 * 2.0 ** -53 * np.abs(v[:d]).sum(0) * 2)
