@@ -216,6 +216,243 @@ int gram_reduce(const double* partial, int nctas, int nout, double alpha, double
   return launch_gram_reduce(partial, nctas, nout, alpha, G, s);
 }
 
+// ---------------------------------------------------------------- row sweeps
+// G = alpha V^T W, or (UPD) W = beta W + alpha V C and then G = [V; W]^T W, for blocks of one width
+// B in one sweep over the rows: L lanes hold a row, lane t of them blocks t, t + L, .. (at most NB;
+// UPD: index nv is W itself) with their B x B output tiles in registers for the whole launch.
+// A row of V is loaded once, all blocks of it before the first use; an update sums its L partial
+// results by shuffles, so nothing of the sweep goes through shared memory but C.  Every lane's sums
+// are reduced over the warp by a scatter (each level halves what a lane holds) and over the CTA once,
+// at the end: cross-thread sums in FP64, or, for FP32 sums, as unevaluated pairs of floats (TwoSum;
+// 48 bits), because FP64 adds of 8 * NB * B * B values per warp would take as long as the sweep.
+// Loads of V and W rows bound it in FP32 and the FP64 pipe in FP64 (rows_pick has the figures).
+template <typename TC, int B>
+constexpr int kRowBlocks = B >= 8 ? (sizeof(TC) == 4 ? 2 : 1) : (B == 4 ? 4 : 8);   // NB
+constexpr int kRowLanesMax = 8;
+
+template <typename TC>
+struct RowSum {   // s + e
+  TC s, e;
+};
+__device__ __forceinline__ void row_add(RowSum<float>& a, RowSum<float> b) {
+  const float t = a.s + b.s, z = t - a.s;
+  a.e += b.e + ((a.s - (t - z)) + (b.s - z));
+  a.s = t;
+}
+__device__ __forceinline__ void row_add(RowSum<double>& a, RowSum<double> b) { a.s += b.s; }
+__device__ __forceinline__ RowSum<float> row_shfl(RowSum<float> a, int off) {
+  return {__shfl_xor_sync(kFullMask, a.s, off), __shfl_xor_sync(kFullMask, a.e, off)};
+}
+__device__ __forceinline__ RowSum<double> row_shfl(RowSum<double> a, int off) {
+  return {__shfl_xor_sync(kFullMask, a.s, off), 0.0};
+}
+
+template <typename T, typename TC, int B, int L, bool UPD>
+__global__ void __launch_bounds__(256) rows_kernel(const BlockSet V, const double* __restrict__ C,
+                                                   double alpha, double beta, T* W, int64_t n,
+                                                   double* __restrict__ partial) {
+  constexpr int NB = kRowBlocks<TC, B>, BB = B * B, RW = 32 / L;
+  constexpr int kStride = NB * BB + 16 / (int)sizeof(T);   // of a lane's coefficients: other banks
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* sC = reinterpret_cast<T*>(smem_raw);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = lane / RW;
+  if constexpr (UPD) {
+    for (int e = threadIdx.x; e < L * NB * BB; e += blockDim.x) {
+      const int j = e / BB;   // block j: lane j % L, its j / L-th
+      sC[j % L * kStride + j / L * BB + e % BB] = j < V.nv ? (T)(alpha * C[e]) : T(0);
+    }
+    __syncthreads();
+  }
+  const int tiles = V.nv + (UPD ? 1 : 0);
+  const T* vp[NB];
+#pragma unroll
+  for (int i = 0; i < NB; ++i)
+    vp[i] = t + i * L < V.nv ? reinterpret_cast<const T*>(V.blk[t + i * L]) : nullptr;
+  TC acc[NB][B][B];
+#pragma unroll
+  for (int i = 0; i < NB; ++i)
+#pragma unroll
+    for (int p = 0; p < B; ++p)
+#pragma unroll
+      for (int q = 0; q < B; ++q) acc[i][p][q] = TC(0);
+  for (int64_t base = ((int64_t)blockIdx.x * 8 + warp) * RW; base < n; base += (int64_t)gridDim.x * 8 * RW) {
+    const int64_t r = base + lane % RW;
+    const bool on = r < n;
+    T v[NB][B], w[B];
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+#pragma unroll
+      for (int p = 0; p < B; ++p) v[i][p] = T(0);
+      if (on && vp[i]) ld_row<T, B>(vp[i] + r * B, v[i]);
+    }
+#pragma unroll
+    for (int q = 0; q < B; ++q) w[q] = T(0);
+    if (on && (!UPD || beta != 0.0)) ld_row_rw<T, B>(W + r * B, w);
+    if constexpr (UPD) {
+      const T* c = sC + t * kStride;
+      T a[B];
+#pragma unroll
+      for (int q = 0; q < B; ++q) a[q] = T(0);
+#pragma unroll
+      for (int i = 0; i < NB; ++i)
+        if (i * L < V.nv) {
+#pragma unroll
+          for (int p = 0; p < B; ++p)
+#pragma unroll
+            for (int q = 0; q < B; ++q) a[q] = fma(v[i][p], c[(i * B + p) * B + q], a[q]);
+        }
+#pragma unroll
+      for (int off = RW; off < 32; off <<= 1)
+#pragma unroll
+        for (int q = 0; q < B; ++q) a[q] += __shfl_xor_sync(kFullMask, a[q], off);
+#pragma unroll
+      for (int q = 0; q < B; ++q) w[q] = beta != 0.0 ? fma((T)beta, w[q], a[q]) : a[q];
+      if (on && t == 0) st_row<T, B>(W + r * B, w);
+#pragma unroll
+      for (int i = 0; i < NB; ++i)
+        if (t + i * L == V.nv) {
+#pragma unroll
+          for (int p = 0; p < B; ++p) v[i][p] = on ? w[p] : T(0);
+        }
+    }
+    TC wc[B];
+#pragma unroll
+    for (int q = 0; q < B; ++q) wc[q] = to_arith<TC>(w[q]);
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+      if (i * L < tiles) {
+#pragma unroll
+        for (int p = 0; p < B; ++p) {
+          const TC x = to_arith<TC>(v[i][p]);
+#pragma unroll
+          for (int q = 0; q < B; ++q) acc[i][p][q] = fma(x, wc[q], acc[i][p][q]);
+        }
+      }
+  }
+  // over the rows of the warp
+  constexpr int NV = NB * BB;
+  constexpr TC kScale = sizeof(TC) == 4 ? TC(0.015625) : TC(1);   // pairs of floats: 32 of any size add up
+  RowSum<TC> x[NV];
+#pragma unroll
+  for (int e = 0; e < NV; ++e) x[e] = {acc[e / BB][e / B % B][e % B] * kScale, TC(0)};
+  int first = 0, cnt = NV;
+#pragma unroll
+  for (int off = RW / 2; off >= 1; off >>= 1) {
+    const bool up = (lane & off) != 0;
+    const int h = cnt / 2;
+    if (h >= 1) {
+#pragma unroll
+      for (int i = 0; i < NV / 2; ++i)
+        if (i < h) {
+          const RowSum<TC> send = up ? x[i] : x[i + h];
+          x[i] = up ? x[i + h] : x[i];
+          row_add(x[i], row_shfl(send, off));
+        }
+      if (up) first += h;
+      cnt = h;
+    } else {
+      row_add(x[0], row_shfl(x[0], off));
+    }
+  }
+  // over the warps of the CTA
+  __syncthreads();
+  double* red = reinterpret_cast<double*>(smem_raw);   // [8][L * NV]
+#pragma unroll
+  for (int i = 0; i < NV; ++i)
+    if (i < cnt) {
+      const double z = (double)x[i].s + (double)x[i].e;   // e is NaN where s is infinite
+      const int f = first + i;
+      red[warp * L * NV + (t + f / BB * L) * BB + f % BB] = (z == z ? z : (double)x[i].s) * (1.0 / (double)kScale);
+    }
+  __syncthreads();
+  const int nout = tiles * BB;
+  for (int e = threadIdx.x; e < nout; e += blockDim.x) {
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s += red[k * L * NV + e];
+    partial[(int64_t)blockIdx.x * nout + e] = s;
+  }
+}
+
+// Lanes per row: as few as hold the blocks.
+template <typename TC, int B>
+static int row_lanes(int tiles) {
+  int l = 1;
+  while (l * kRowBlocks<TC, B> < tiles) l *= 2;
+  return l;
+}
+
+// Whether the row sweep takes `tiles` blocks.  It is faster than the kernels with a warp per tile
+// (gram_kernel, update_gram_kernel) where loads bind: FP32 at b = 4 and 8 always (4.2 million rows, 7
+// blocks of 4: Gram 175 -> 109 us, update and Gram 263 -> 148 us; 31 blocks at 200003 rows 98 -> 42 and
+// 224 -> 52 us), narrower FP32 blocks for Grams of b = 2 and for updates of more than 16 tiles, which
+// the other kernel reduces after every range.  In FP64, the FMAs bind: it pays where the lanes' blocks
+// divide evenly (idle slots are issued all the same) and the other kernel's tiles do not fit its
+// registers (b = 8: 8 blocks, a million rows 1745 -> 893 us) or are more than 16 (31 blocks of 4: Gram
+// 1289 -> 896 us, update and Gram 2602 -> 2042 us).
+template <typename T, typename TC, int B, bool UPD>
+static bool rows_pick(int tiles) {
+  if (tiles > kRowBlocks<TC, B> * kRowLanesMax) return false;
+  if (sizeof(TC) == 4) {
+    if (B >= 4) return true;
+    return UPD ? tiles > 16 : (B == 2 && tiles <= 16);
+  }
+  const int l = row_lanes<TC, B>(tiles), slots = (tiles + l - 1) / l * l;
+  if (B == 8) return 3 * slots <= 4 * tiles;
+  if (UPD) return B == 4 && tiles > 16;
+  return tiles > 16 || (B == 4 && 10 * slots <= 11 * tiles);
+}
+
+template <typename T, typename TC, int B, int L, bool UPD>
+static int launch_rows_l(const BlockSet& V, int64_t n, const double* C, double alpha, double beta, T* W,
+                         double gscale, double* G, double* scratch, size_t capacity, cudaStream_t s) {
+  constexpr int NV = kRowBlocks<TC, B> * B * B;
+  const size_t smem = (size_t)8 * L * NV * sizeof(double);   // above the coefficients' L (NV + pad)
+  const void* fn = reinterpret_cast<const void*>(rows_kernel<T, TC, B, L, UPD>);
+  static KernelSetup ks;
+  FE_TRY(kernel_configure(ks, fn, (int)smem));
+  int per_sm = 0;
+  FE_TRY(kernel_occupancy(ks, fn, 256, smem, 0, &per_sm));
+  const int nout = (V.nv + (UPD ? 1 : 0)) * B * B;
+  int64_t nctas = std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 8 * (32 / L)), (int64_t)per_sm * num_sms()));
+  double* part = scratch;
+  if (!part) {
+    part = small_scratch(0, (size_t)nctas * nout);
+    if (!part) return FE_ERR_OOM;
+  } else {
+    nctas = std::min<int64_t>(nctas, (int64_t)(capacity / (size_t)nout));
+    FE_ARG(nctas >= 1, "gram: scratch of %zu doubles cannot hold %d outputs", capacity, nout);
+  }
+  rows_kernel<T, TC, B, L, UPD><<<(unsigned)nctas, 256, smem, s>>>(V, C, alpha, beta, W, n, part);
+  count_launch();
+  FE_CUDA(cudaGetLastError());
+  return launch_gram_reduce(part, (int)nctas, nout, gscale, G, s);
+}
+
+template <typename T, typename TC, int B, bool UPD>
+static int launch_rows(const BlockSet& V, int64_t n, const double* C, double alpha, double beta, T* W,
+                       double gscale, double* G, double* scratch, size_t capacity, cudaStream_t s) {
+  switch (row_lanes<TC, B>(V.nv + (UPD ? 1 : 0))) {
+    case 1: return launch_rows_l<T, TC, B, 1, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s);
+    case 2: return launch_rows_l<T, TC, B, 2, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s);
+    case 4: return launch_rows_l<T, TC, B, 4, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s);
+    default: return launch_rows_l<T, TC, B, 8, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s);
+  }
+}
+
+// The row sweep's V^T W for blocks of one width without gaps; *done tells whether it took the call.
+template <typename T, typename TC, int B>
+static int gram_rows(const BlockSet& V, int64_t n, const T* W, int bw, int ldw, double alpha, double* G,
+                     double* scratch, size_t capacity, bool* done, cudaStream_t s) {
+  *done = false;
+  if constexpr (B <= 8) {
+    if (bw != B || V.bv != B || V.ld != B || ldw != B || !rows_pick<T, TC, B, false>(V.nv)) return FE_OK;
+    *done = true;
+    return launch_rows<T, TC, B, false>(V, n, nullptr, 0.0, 0.0, const_cast<T*>(W), alpha, G, scratch, capacity, s);
+  }
+  return FE_OK;
+}
+
 // Launches gram_kernel<T, BV, NQ, TPW> with as many CTAs as fit on the GPU at once (at most one
 // staged range each per pass), then the partial reduction.  scratch == nullptr: partials in
 // the pool's slot 0; otherwise in scratch (capacity doubles), the grid shrunk to fit.
@@ -270,6 +507,9 @@ static int launch_gram(const BlockSet& V, int64_t n, const T* W, int bw, int ldw
 template <typename T, int BV>
 static int gram_bv(const BlockSet& V, int64_t n, const T* W, int bw, int ldw, double alpha,
                    double* G, cudaStream_t s) {
+  bool done = false;
+  FE_TRY((gram_rows<T, T, BV>(V, n, W, bw, ldw, alpha, G, nullptr, 0, &done, s)));
+  if (done) return FE_OK;
   constexpr int QMAX = 32 / BV >= 16 ? 16 : 32 / BV;
   const int nq = std::min(bw, QMAX);
   switch (nq) {
@@ -329,6 +569,14 @@ int gram_f32_arith(const BlockSet& V, int64_t n, const double* W, int b, double 
                    cudaStream_t s) {
   FE_ARG(V.nv >= 1 && V.nv <= kMaxBlocks, "gram: nv = %d out of range", V.nv);
   FE_ARG(V.bv == b, "gram: block width %d != %d", V.bv, b);
+  bool done = false;
+  switch (b) {
+    case 1: FE_TRY((gram_rows<double, float, 1>(V, n, W, b, b, alpha, G, nullptr, 0, &done, s))); break;
+    case 2: FE_TRY((gram_rows<double, float, 2>(V, n, W, b, b, alpha, G, nullptr, 0, &done, s))); break;
+    case 4: FE_TRY((gram_rows<double, float, 4>(V, n, W, b, b, alpha, G, nullptr, 0, &done, s))); break;
+    case 8: FE_TRY((gram_rows<double, float, 8>(V, n, W, b, b, alpha, G, nullptr, 0, &done, s))); break;
+  }
+  if (done) return FE_OK;
   switch (b) {
     case 1: return launch_gram_any<double, 1, 1, float>(V, n, W, b, b, alpha, G, nullptr, 0, s);
     case 2: return launch_gram_any<double, 2, 2, float>(V, n, W, b, b, alpha, G, nullptr, 0, s);
@@ -691,6 +939,9 @@ template <typename T, int BV>
 static int gram_scratch_bv(const BlockSet& V, int64_t n, const T* W, int bw, int ldw,
                            double alpha, double* G, double* scratch, size_t capacity,
                            cudaStream_t s) {
+  bool done = false;
+  FE_TRY((gram_rows<T, T, BV>(V, n, W, bw, ldw, alpha, G, scratch, capacity, &done, s)));
+  if (done) return FE_OK;
   constexpr int QMAX = 32 / BV >= 16 ? 16 : 32 / BV;
   const int nq = std::min(bw, QMAX);
   switch (nq) {
@@ -959,6 +1210,8 @@ template <typename T, int BV, int BW>
 static int launch_update_gram(const BlockSet& V, int64_t n, const double* C, double alpha,
                               double beta, const double* M, T* W, int gram_v, const int* skip,
                               const int* vc32, double* G, cudaStream_t s) {
+  if (gram_v && !M && !skip && !vc32 && rows_pick<T, T, BW, true>(V.nv + 1))
+    return launch_rows<T, T, BW, true>(V, n, C, alpha, beta, W, 1.0, G, nullptr, 0, s);
   constexpr int NR = BV > BW ? BV : BW;
   constexpr int kRegsPerTile = NR * BW * (int)(sizeof(T) / 4);
   const int gblocks = gram_v ? V.nv + 1 : 1;

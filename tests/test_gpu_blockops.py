@@ -211,3 +211,45 @@ def test_orth_factorisation_widths_and_scales(n, nv, b, scale):
     assert np.abs(Q.T @ Q - np.eye(b)).max() < 1e-13
     if nv:
         assert np.abs(G.cpu().numpy() / scale - Vt.T @ W).max() < 1e-11 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+@pytest.mark.parametrize("b", [1, 2, 4, 8])
+@pytest.mark.parametrize("n,nv", [(1, 1), (31, 2), (33, 3), (255, 4), (256, 5), (257, 7), (70001, 8), (3001, 9), (5000, 15),
+                                  (5001, 16), (4099, 17), (4100, 31), (2000, 32), (2000, 33)])
+def test_row_sweeps(prec, b, n, nv):
+    """Gram and update + Gram at the edges of the row sweeps: every number of lanes per row (1, 2, 4,
+    8, the next one falling back to the tile kernels), one row, ragged last rows, more rows than a
+    grid holds at once.  Bounds: sums of k products in FP32 (FP64) have errors of a few
+    sqrt(k) 2^-24 (2^-53) of |V|^T|W|; 32 times that rate allowed for k = n."""
+    r = np.random.default_rng(1000 * b + nv)
+    V = r.standard_normal((nv, n, b)).astype(NP[prec])
+    W = r.standard_normal((n, b)).astype(NP[prec])
+    C = r.standard_normal((nv * b, b)) / np.sqrt(nv * b)
+    V64 = np.concatenate([v.astype(np.float64) for v in V], axis=1)
+    u = {"f32": 2.0 ** -24, "f64": 2.0 ** -53}[prec]
+    G = fe.block_gram(to_dev(V), to_dev(W), alpha=-0.5, engine="fma").cpu().numpy()
+    want, mag = -0.5 * (V64.T @ W.astype(np.float64)), 0.5 * (np.abs(V64).T @ np.abs(W).astype(np.float64))
+    assert np.all(np.abs(G - want) <= 32 * u * mag + 1e-300)
+    Wd = to_dev(W)
+    G = fe.block_update_gram(to_dev(V), to_dev(C), Wd, alpha=1.0, beta=0.5).cpu().numpy()
+    Wn = 0.5 * W.astype(np.float64) + V64 @ C
+    magw = 0.5 * np.abs(W).astype(np.float64) + np.abs(V64) @ np.abs(C)
+    got = Wd.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(got - Wn) <= (nv * b + 8) * u * magw)
+    X = np.concatenate([V64, got], axis=1)
+    assert np.all(np.abs(G - X.T @ got) <= 32 * u * (np.abs(X).T @ np.abs(got)) + 1e-300)
+
+
+def test_row_sweep_large_sums_and_infinities():
+    """FP32 Grams whose sums leave FP32's range are finite in G (FP64), and an infinite entry makes the
+    entries it enters infinite, not NaN."""
+    n = 4096
+    V = np.full((2, n, 4), 3e18, np.float32)
+    W = np.full((n, 4), 3e19, np.float32)
+    G = fe.block_gram(to_dev(V), to_dev(W)).cpu().numpy()
+    want = n * float(np.float32(3e18)) * float(np.float32(3e19))
+    assert np.allclose(G, want, rtol=1e-6)
+    V[1, 77, 2] = np.inf
+    G = fe.block_gram(to_dev(V), to_dev(W)).cpu().numpy()
+    assert np.all(np.isposinf(G[6])) and np.isfinite(G[:6]).all() and np.isfinite(G[7]).all()
