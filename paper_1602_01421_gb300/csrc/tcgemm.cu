@@ -5,19 +5,25 @@
 //
 //   * every V row is scaled by its largest binary exponent and its 53-bit aligned significands
 //     are cut into seven 8-bit digits (sign-magnitude, so every digit is an integer in
-//     [-255, 255] and exact in FP16): V[r][c] = 2^(Er - 1075) sum_i d_i[r][c] 2^(45 - 8 i);
+//     [-255, 255]; as an operand it is d 2^-24, a subnormal FP16 number, exact): V[r][c] = 2^(Er - 1075) sum_i d_i[r][c] 2^(45 - 8 i);
 //   * every Y column likewise by its largest exponent: Y[c][q] = 2^(Fq - 1075) sum_j e_j 2^(45-8j);
 //   * the digit products are exact in the tensor core's FP32 accumulator as long as each
 //     accumulator sums at most 2^24 / 255^2 = 258 of them: one accumulator per digit-weight
 //     class g = i + j (g <= 6) and per 32-wide slice of K holds at most 7 * 32 products;
 //   * V Y = 2^(Er + Fq - 2108) * T with T = sum_g D_g 2^(8 (6 - g)), assembled in 64-bit
-//     integer arithmetic from the accumulators (T / 2^12, exact up to the dropped bits) and
-//     rounded once (truncation) to FP64.
+//     integer arithmetic from the accumulators (T / 2^12, rounded) and rounded once to FP64.
 //
 // Error: the digit products dropped (i + j >= 7), the truncation of each entry below its
 // row's (column's) leading bit and the 12 dropped bits of T bound |error| <=
-// 2^-49 (K + 1) max_c |V[r][c]| max_c |Y[c][q]| + 2^-52 |result|; the FP64 pipe is not used at
-// all (FP64 on this part runs at 1/64 of FP32).
+// 2^-49 (K + 1) max_c |V[r][c]| max_c |Y[c][q]| + 2^-52 |result|.  The FP64 pipe (1/64 of the FP32
+// rate on this part) only converts: one 64-bit integer per result.
+//
+// What bounds these kernels is the integer work of the split and of the assembly, on an ALU that takes
+// a warp's instruction every other clock, and the latencies between the phases of a tile.  So a value
+// is cut with as few instructions as possible (digits8: 11 for the 14 digits of two values), a result
+// assembled with 32-bit multiply-adds before 64-bit ones (sum7) and converted by one instruction
+// (scale_int), and each splitting thread takes one unit of eight values, with registers capped at 64
+// so that 28-30 warps fit (without spills: beside the staging buffers L1 has no room for them).
 //
 // Kernels: for K <= 32 a warp-specialised pipeline (tc_combine_pipe_kernel: TMA producer,
 // digit splitters, one MMA-issuing thread, result assemblers over double-buffered tiles; see its
@@ -80,15 +86,6 @@ __device__ __forceinline__ uint32_t digit(uint64_t m, int i) {
   return i < 6 ? (uint32_t)(m >> (45 - 8 * i)) & 0xFFu : ((uint32_t)m & 0x1Fu) << 3;
 }
 
-// The aligned significand shifted up by 3 bits (56 bits): digit i is then byte 6 - i.
-__device__ __forceinline__ uint64_t aligned_sig56(double x, int emax) {
-  const uint64_t u = (uint64_t)__double_as_longlong(x);
-  const int e = (int)((u >> 52) & 0x7FF);
-  const int sh = emax - e;
-  if (e == 0 || sh > 52) return 0;
-  return (((u & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << 3) >> sh;
-}
-
 // FP16 x2 fused multiply-add on packed halves (round to nearest).
 __device__ __forceinline__ uint32_t hfma2_u32(uint32_t x, uint32_t y, uint32_t z) {
   uint32_t d;
@@ -96,27 +93,60 @@ __device__ __forceinline__ uint32_t hfma2_u32(uint32_t x, uint32_t y, uint32_t z
   return d;
 }
 
-// The seven digits of two FP64 values x0, x1 relative to the exponent field emax (>= theirs),
-// as packed FP16 pairs: w[i][e] holds digit i of x0 (low half) and of x1 (high half), each with
-// its value's sign.  Per digit pair: a byte permute takes the two digit bytes of the 56-bit
-// significands, a LOP3 puts each under the FP16 exponent of 1024 (1024 + d is exact for
-// d < 1024), and one FP16 FMA forms (1024 + d) s - 1024 s = s d exactly (s = +-1).
-__device__ __forceinline__ void split_pair_f16(double x0, double x1, int emax, uint32_t (&w)[kDigits][4],
-                                               int e) {
-  const uint64_t m0 = aligned_sig56(x0, emax), m1 = aligned_sig56(x1, emax);
-  const uint32_t h0 = (uint32_t)((uint64_t)__double_as_longlong(x0) >> 32);
-  const uint32_t h1 = (uint32_t)((uint64_t)__double_as_longlong(x1) >> 32);
-  const uint32_t s2 = 0x3C003C00u | ((h0 >> 16) & 0x8000u) | (h1 & 0x80000000u);  // (+-1, +-1)
-  const uint32_t c2 = s2 ^ 0xD800D800u;                                          // -1024 (+-1)
+// Eight FP64 values prepared for the cut into digits: their significands aligned to a common exponent
+// and shifted up by 3 bits (56 bits: digit i is byte 6 - i), and the signs of neighbouring values in
+// bits 15 and 31.
+struct Sig8 {
+  uint32_t lo[8], hi[8], s2[4];
+};
+
+// Largest exponent of the eight values, in its place in the high word (0: all zero or subnormal).
+__device__ __forceinline__ uint32_t top_exp8(const double (&x)[8]) {
+  uint32_t e = 0;
 #pragma unroll
-  for (int i = 0; i < kDigits; ++i) {
-    const int k = 6 - i;   // byte of the 56-bit significand holding digit i
-    const uint32_t lo0 = (uint32_t)m0, hi0 = (uint32_t)(m0 >> 32);
-    const uint32_t lo1 = (uint32_t)m1, hi1 = (uint32_t)(m1 >> 32);
-    const uint32_t pa = k < 4 ? lo0 : hi0, pb = k < 4 ? lo1 : hi1;
-    const uint32_t sel = (uint32_t)((k & 3) | ((4 + (k & 3)) << 8));
-    const uint32_t r = (__byte_perm(pa, pb, sel) & 0x00FF00FFu) | 0x64006400u;
-    w[i][e] = hfma2_u32(r, s2, c2);
+  for (int t = 0; t < 8; ++t) e = max(e, (uint32_t)__double2hiint(x[t]) & 0x7FF00000u);
+  return e;
+}
+
+// emax: exponent in its place in the high word, at least every value's.  A zero gives zero, and so
+// does a value below 2^-56 of 2^emax.  (Subnormals only count beside the smallest normal numbers,
+// and then as half their value.)
+__device__ __forceinline__ void align8(const double* x, uint32_t emax, Sig8& s) {
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    const uint32_t hi = (uint32_t)__double2hiint(x[t]), ev = hi & 0x7FF00000u;
+    const uint32_t h = (hi & 0xFFFFFu) | min(ev, 0x100000u);   // with the leading one
+    uint64_t m = (((uint64_t)h << 32) | (uint32_t)__double2loint(x[t])) << 3;
+    asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"((emax - ev) >> 20));
+    s.lo[t] = (uint32_t)m;
+    s.hi[t] = (uint32_t)(m >> 32);
+  }
+#pragma unroll
+  for (int t = 0; t < 4; ++t)
+    s.s2[t] = __byte_perm((uint32_t)__double2hiint(x[2 * t]), (uint32_t)__double2hiint(x[2 * t + 1]), 0x7632) & 0x80008000u;
+}
+
+// Digits of the eight values with their signs; put(i, w) takes digit i of all eight, as FP16 numbers
+// +-d 2^-24: a byte d with zeros above it is the subnormal FP16 number d 2^-24, which the tensor cores
+// multiply exactly.  Per pair of values a byte permute takes two neighbouring digit bytes of both and
+// one more per digit puts their bytes under the signs: 11 instructions for the 14 digits.
+constexpr float kDigitUnit = 16777216.0f;   // 2^24
+template <class Put>
+__device__ __forceinline__ void digits8(const Sig8& s, Put put) {
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {   // bytes (6, 5), 4, (3, 2), (1, 0) of the significands
+    const int k = g == 0 ? 6 : g == 1 ? 4 : g == 2 ? 3 : 1;
+    const uint32_t b1 = k & 3, b0 = g == 1 ? b1 : b1 - 1;
+    uint32_t w0[4], w1[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const uint32_t pa = g < 2 ? s.hi[2 * t] : s.lo[2 * t], pb = g < 2 ? s.hi[2 * t + 1] : s.lo[2 * t + 1];
+      const uint32_t q = __byte_perm(pa, pb, b1 | (b0 << 4) | ((4 + b1) << 8) | ((4 + b0) << 12));
+      w0[t] = __byte_perm(q, s.s2[t], 0x7250);
+      w1[t] = __byte_perm(q, s.s2[t], 0x7351);
+    }
+    put(6 - k, make_uint4(w0[0], w0[1], w0[2], w0[3]));
+    if (g != 1) put(7 - k, make_uint4(w1[0], w1[1], w1[2], w1[3]));
   }
 }
 
@@ -126,30 +156,39 @@ __device__ __forceinline__ uint16_t digit_f16(uint32_t d, uint32_t sign) {
   return (uint16_t)(hfma2_u32(0x6400u | d, s2, s2 ^ 0xD800u) & 0xFFFFu);
 }
 
-// Exact integer value of an FP32 accumulator holding an integer of magnitude below 2^24.
-__device__ __forceinline__ int32_t acc_int(uint32_t bits) {
-  return __float2int_rn(__uint_as_float(bits));
+// Exact integer value of an FP32 accumulator holding an integer of magnitude below 2^24 in units of
+// 1 / unit (a power of two).
+__device__ __forceinline__ int32_t acc_int(uint32_t bits, float unit) {
+  return __float2int_rn(__uint_as_float(bits) * unit);
 }
 
-// The accumulated T = hi 2^32 + lo (|hi| < 2^40, |lo| < 2^50) is taken as floor(T / 2^12), an
-// int64 of at most 60 bits, before it is rounded to FP64: the 12 dropped bits are below the
-// digit truncation already made (2^-50 of max|V_r| max|Y_q|).
+// Seven accumulators d_g of weights 2^(8 (6 - g)) form T = sum_g d_g 2^(8 (6 - g)); it is taken as
+// T / 2^12 rounded to an integer of at most 60 bits: the 12 dropped bits are below the digit
+// truncation already made (2^-50 of max|V_r| max|Y_q|).
 constexpr int kAsmShift = 12;
 
-// 2^s * (hi 2^20 + floor(lo / 2^12)) truncated to FP64; zero below the normal range, infinity
-// above it.  Integer operations only, without branches.
-__device__ __forceinline__ double assemble(int64_t hi, int64_t lo, int s) {
-  const int64_t t = (hi << (32 - kAsmShift)) + (lo >> kAsmShift);
-  const uint64_t sign = (uint64_t)t & 0x8000000000000000ull;
-  const uint64_t a = t < 0 ? (uint64_t)(-t) : (uint64_t)t;
-  const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a;
-  const int lz = ah != 0 ? __clz(ah) : 32 + __clz(al);  // 64 when a == 0 (32-bit counts)
-  const uint64_t m = a << (lz & 63);                    // leading one at bit 63
-  const int ef = 63 - lz + s + 1023;
-  uint64_t bits = sign | ((uint64_t)(uint32_t)ef << 52) | ((m >> 11) & 0xFFFFFFFFFFFFFull);
-  bits = (a == 0 || ef <= 0) ? sign : bits;
-  bits = ef >= 2047 ? (sign | 0x7FF0000000000000ull) : bits;
-  return __longlong_as_double((long long)bits);
+// floor((T + 256 rnd) / 2^12): rnd = 8 rounds to the nearest; 16 j more adds j to the result.  d_0 and
+// d_2 are below 2^31 / 257 (the sums of up to 128 rows of a Gram tile, 128 * 255^2, and the first three
+// classes of a 32-column product), so pairs of them go through 32-bit multiply-adds.
+__device__ __forceinline__ int64_t sum7(const uint32_t (&d)[7], float unit, int rnd) {
+  const int a01 = acc_int(d[0], unit) * 256 + acc_int(d[1], unit);
+  const int a23 = acc_int(d[2], unit) * 256 + acc_int(d[3], unit);
+  const int a6 = __float2int_rd(__uint_as_float(d[6]) * (unit * 0.00390625f));   // floor(d_6 / 2^8)
+  const int a456 = acc_int(d[4], unit) * 16 + ((acc_int(d[5], unit) + a6 + rnd) >> 4);
+  return (int64_t)a01 * (1 << 28) + ((int64_t)a23 * 4096 + a456);
+}
+
+// 2^s * t rounded to FP64; zero below the normal range, infinity above it.
+__device__ __forceinline__ double scale_int(int64_t t, int s) {
+  const double d = __ll2double_rn((long long)t);
+  const uint32_t h = (uint32_t)__double2hiint(d);
+  const int ef = (int)((h >> 20) & 0x7FFu) + s;
+  uint32_t rh = h + ((uint32_t)s << 20), rl = (uint32_t)__double2loint(d);
+  if (h == 0 || (uint32_t)(ef - 1) >= 2046u) {
+    rh = (h & 0x80000000u) | (h != 0 && ef >= 2047 ? 0x7FF00000u : 0u);
+    rl = 0;
+  }
+  return __hiloint2double((int)rh, (int)rl);
 }
 
 // Bounded wait that sleeps until the phase completes: waiting threads take no issue slots from
@@ -327,18 +366,12 @@ __global__ void __launch_bounds__(kThreads, KMAX <= 32 ? 2 : 1) tc_combine_kerne
     // ---- split into seven digits and write them to the A tiles
 #pragma unroll
     for (int k8 = 0; k8 < KH; k8 += 8) {
-      uint32_t w[kDigits][4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const double x0 = v[k8 + 2 * e], x1 = v[k8 + 2 * e + 1];
-        split_pair_f16(x0, x1, emax, w, e);
-      }
+      Sig8 s8;
+      align8(v + k8, (uint32_t)emax << 20, s8);
       const int kk = k_mine + k8;   // column within the chunk
       const int kc = kc_mine + kk / kKChunk;
-#pragma unroll
-      for (int i = 0; i < kDigits; ++i)
-        *reinterpret_cast<uint4*>(sA + (size_t)(kc * kDigits + i) * kATileBytes + tile_off(row, kk % kKChunk)) =
-            make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
+      unsigned char* dst = sA + (size_t)kc * kDigits * kATileBytes + tile_off(row, kk % kKChunk);
+      digits8(s8, [&](int i, uint4 w) { *reinterpret_cast<uint4*>(dst + i * kATileBytes) = w; });
     }
     tc::fence_async_smem();
     tc::fence_before_sync();
@@ -396,15 +429,16 @@ __global__ void __launch_bounds__(kThreads, KMAX <= 32 ? 2 : 1) tc_combine_kerne
         for (int kc = 0; kc < KMAX / kKChunk; ++kc)
           if (kc < nkc) {
             // 32 x 32 -> 64-bit multiply-adds by powers of two
-            hi += (int64_t)acc_int(acc[kc][0][u]) * 65536 + (int64_t)acc_int(acc[kc][1][u]) * 256 +
-                  (int64_t)acc_int(acc[kc][2][u]);
-            lo += (int64_t)acc_int(acc[kc][3][u]) * 16777216 + (int64_t)acc_int(acc[kc][4][u]) * 65536 +
-                  (int64_t)acc_int(acc[kc][5][u]) * 256 + (int64_t)acc_int(acc[kc][6][u]);
+            hi += (int64_t)acc_int(acc[kc][0][u], kDigitUnit) * 65536 + (int64_t)acc_int(acc[kc][1][u], kDigitUnit) * 256 +
+                  (int64_t)acc_int(acc[kc][2][u], kDigitUnit);
+            lo += (int64_t)acc_int(acc[kc][3][u], kDigitUnit) * 16777216 + (int64_t)acc_int(acc[kc][4][u], kDigitUnit) * 65536 +
+                  (int64_t)acc_int(acc[kc][5][u], kDigitUnit) * 256 + (int64_t)acc_int(acc[kc][6][u], kDigitUnit);
           }
         if (live && q < a.N) {
           double y = 0.0;
           if (!ok) y = __longlong_as_double(0x7FF8000000000000ll);
-          else if (emax > 0) y = assemble(hi, lo, ebase + sF[q]);
+          else if (emax > 0)
+            y = scale_int((hi << (32 - kAsmShift)) + ((lo + (1 << (kAsmShift - 1))) >> kAsmShift), ebase + sF[q]);
           double* dst = a.oblk[q / BV] + r * BV + q % BV;
           if (add_out) y = fma(a.beta, *dst, y);
           *dst = y;
@@ -430,14 +464,13 @@ static size_t tc_smem_bytes(int nkc, int NP) {
 // ---------------------------------------------------------------- pipelined form (K <= 32)
 // The same product with the phases of consecutive tiles overlapped.  One persistent CTA per SM
 // with four warp roles:
-//   warps 0-7   split V rows into digits: a unit is 8 columns of one row, unit u = row
-//               + 128 cb (cb < ceil(K / 8)), thread t takes units t and t + 256, so the work
-//               follows K; units write the digit tiles of buffer t % 2;
-//   warp 16     (one thread) issues the TMA copies of tile t's V rows into staging buffer t % 2;
-//   warp 17     (one thread) issues tile t's MMAs into TMEM buffer t % 2 and owns the TMEM
+//   warps 0-15  split V rows into digits: a unit is 8 columns of one row, thread t takes unit
+//               t = row + 128 cb (cb < ceil(K / 8)); units write the digit tiles of buffer t % 2;
+//   warp 28     (one thread) issues the TMA copies of tile t's V rows into staging buffer t % 2;
+//   warp 29     (one thread) issues tile t's MMAs into TMEM buffer t % 2 and owns the TMEM
 //               allocation;
-//   warps 8-15  read tile t's accumulators (TMEM lane quarter = warp % 4, two threads per row,
-//               alternate groups of four results), assemble and store them; with beta != 0 and
+//   warps 16-27 read tile t's accumulators (TMEM lane quarter = warp % 4, three threads per row,
+//               every third pair of results each), assemble and store them; with beta != 0 and
 //               N <= 16 the rows of Out for tile t + 1 are loaded while tile t is assembled.
 // V staging, digit tiles and accumulators are double-buffered, so tile t + 1 is split while tile
 // t's products run and its results are assembled.  Five mbarrier pairs hand each buffer on:
@@ -446,17 +479,21 @@ static size_t tc_smem_bytes(int nkc, int NP) {
 // epilogue: products complete, digit tiles free), tempty (epilogue -> MMA and splitters: TMEM
 // and row exponents read).  The k-th use of a buffer waits for phase parity k & 1; a
 // barrier cannot run two phases ahead of a waiter because every phase of it needs a phase the
-// waiter itself completes first.  The splitters meet twice per tile at a named barrier that
+// waiter itself completes first.  The splitters meet once per tile at a named barrier that
 // also ORs their wait failures, so they leave the loop together.  Every wait is bounded; a
 // wait that runs out marks the CTA aborted, the other roles stop at their next wait, the
 // epilogue writes NaN to the rows of the tiles it has not finished, and the TMA copies and MMAs
 // in flight are waited for (again bounded) before TMEM is freed.
+// 2^20 rows, K = 32, N = 20 (436 MB): 182 us (194 with 8 splitting and 8 assembling warps, truncating
+// 64-bit assembly and two barriers per tile); without the assembly it would take 137 us, without the
+// split as well 97 us.
 namespace {
-constexpr int kPipeWarps = 18;
-constexpr int kPipeThreads = kPipeWarps * 32;
-constexpr int kSplitWarps = 8, kEpiWarps = 8;
+constexpr int kSplitWarps = 16, kEpiWarps = 12;
+constexpr int kEpiParts = kEpiWarps / 4;                 // epilogue threads per row
 constexpr int kSplitThreads = kSplitWarps * 32;
-constexpr int kProdWarp = 16, kMmaWarp = 17;
+constexpr int kProdWarp = kSplitWarps + kEpiWarps, kMmaWarp = kProdWarp + 1;
+constexpr int kPipeWarps = kMmaWarp + 1;
+constexpr int kPipeThreads = kPipeWarps * 32;
 
 struct PipeBars {
   uint64_t vfull[2], vempty[2], afull[2], mdone[2], tempty[2];
@@ -465,7 +502,7 @@ struct PipeBars {
 // Shared-memory bytes of tc_combine_pipe_kernel for padded N.
 constexpr size_t pipe_smem_bytes(int NP) {
   return (size_t)2 * kDigits * kATileBytes + (size_t)kDigits * NP * kKChunk * 2 +
-         (size_t)2 * kTileRows * kKChunk * 8 + sizeof(PipeBars) + 8 + 4 * kMaxN + 4 * 6 * kTileRows + 64;
+         (size_t)2 * kTileRows * kKChunk * 8 + sizeof(PipeBars) + 8 + 4 * kMaxN + 4 * 10 * kTileRows + 64;
 }
 }  // namespace
 
@@ -514,7 +551,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_combine_pipe_kernel(const 
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
   int* sF = reinterpret_cast<int*>(tslot + 2);                     // N column exponents of Y
   int* sE = sF + kMaxN;                                            // [2][128] row exponents
-  int* sEp = sE + 2 * kTileRows;                                   // [4][128] unit exponents
+  int* sEp = sE + 2 * kTileRows;                                   // [2][4][128] unit exponents
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   {
@@ -549,9 +586,9 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_combine_pipe_kernel(const 
   const int64_t ntiles = (a.n + kTileRows - 1) / kTileRows;
   const int64_t cnt = (int64_t)blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
   auto tile_of = [&](int64_t it) { return (int64_t)blockIdx.x + it * gridDim.x; };
-  auto bulk_ok = [&](int64_t t) {
-    return a.bulk && ((uint64_t)min((int64_t)kTileRows, a.n - t * kTileRows) * BV * 8) % 16 == 0;
-  };
+  // every tile but a ragged last one is a multiple of 16 bytes
+  const int64_t nbulk = !a.bulk ? 0 : ((a.n - (ntiles - 1) * kTileRows) * BV * 8) % 16 == 0 ? ntiles : ntiles - 1;
+  auto bulk_ok = [&](int64_t t) { return t < nbulk; };
 
   if (warp == kProdWarp) {
     // ---- TMA: V rows of tile `it` into staging buffer it % 2
@@ -614,103 +651,87 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_combine_pipe_kernel(const 
     }
   } else if (warp < kSplitWarps) {
     // ---- split: units of 8 columns of one row
-    const int nunits = kTileRows * ((a.K + 7) >> 3);
+    const int ncb = (a.K + 7) >> 3, row = tid & (kTileRows - 1), cb = tid >> 7;
+    const bool unit = cb < ncb;
+    const uint32_t doff = (uint32_t)tile_off(row, cb * 8);
+    const double* sVu = sV + ((size_t)(cb * 8 / BV) * kTileRows + row) * BV + cb * 8 % BV;
+    bool bad = false;
     for (int64_t it = 0; it < cnt; ++it) {
       const int b = (int)(it & 1);
       const uint32_t k = (uint32_t)(it >> 1);
       const int64_t tile = tile_of(it);
-      const bool bulk = bulk_ok(tile);
+      int* sEb = sEp + b * 4 * kTileRows + row;
       const bool ok = pipe_wait_warp(&bars->vfull[b], k & 1, abort_flag);
-      double v[2][8];
-      int emax[2] = {0, 0};
+      double v[8];
+      if (unit) {
+        const bool live = tile * kTileRows + row < a.n;
+        const double* sv = sVu + b * kVBuf;
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int u = tid + kSplitThreads * j;
-        if (u < nunits) {
-          const int row = u & (kTileRows - 1), cb = u >> 7;
-          const int64_t r = tile * kTileRows + row;
-          const bool live = r < a.n;
+        for (int c = 0; c < 8; ++c) v[c] = 0.0;
+        if (live && bulk_ok(tile)) {
+#pragma unroll
+          for (int c0 = 0; c0 < 8; c0 += W)
+            if (W == 8 || cb * 8 + c0 < a.K) {
+              if constexpr (W % 2 == 0) {
+#pragma unroll
+                for (int p = 0; p < W; p += 2) {
+                  const double2 x = *reinterpret_cast<const double2*>(sv + (c0 / BV) * kTileRows * BV + p);
+                  v[c0 + p] = x.x;
+                  v[c0 + p + 1] = x.y;
+                }
+              } else {
+                v[c0] = sv[c0 * kTileRows];
+              }
+            }
+        } else if (live) {
 #pragma unroll
           for (int c0 = 0; c0 < 8; c0 += W) {
             const int c = cb * 8 + c0;
-            if (live && c < a.K) {
-              const double* src = bulk ? sV + (size_t)b * kVBuf + ((size_t)(c / BV) * kTileRows + row) * BV + c % BV
-                                       : a.vblk[c / BV] + r * BV + c % BV;
-              if (bulk && W % 2 == 0) {
+            if (c < a.K) {
+              const double* src = a.vblk[c / BV] + (tile * kTileRows + row) * BV + c % BV;
 #pragma unroll
-                for (int p = 0; p < W; p += 2) {
-                  const double2 x = *reinterpret_cast<const double2*>(src + p);
-                  v[j][c0 + p] = x.x;
-                  v[j][c0 + p + 1] = x.y;
-                }
-              } else {
-#pragma unroll
-                for (int p = 0; p < W; ++p) v[j][c0 + p] = src[p];
-              }
-            } else {
-#pragma unroll
-              for (int p = 0; p < W; ++p) v[j][c0 + p] = 0.0;
+              for (int p = 0; p < W; ++p) v[c0 + p] = __ldg(src + p);
             }
           }
-          int e = 0;
-#pragma unroll
-          for (int c = 0; c < 8; ++c) e = max(e, exp_field(v[j][c]));
-          sEp[cb * kTileRows + row] = e;
         }
+        sEb[cb * kTileRows] = (int)top_exp8(v);
       }
-      if (bar_or(1, kSplitThreads, !ok)) break;   // V read, unit exponents written
+      if (bar_or(1, kSplitThreads, !ok || bad)) break;   // V read, unit exponents written
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&bars->vempty[b]);
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int u = tid + kSplitThreads * j;
-        if (u < nunits) {
-          const int row = u & (kTileRows - 1);
-          for (int c = 0; c < nunits / kTileRows; ++c) emax[j] = max(emax[j], sEp[c * kTileRows + row]);
-        }
-      }
+      int emax = 0;
+      for (int c = 0; c < ncb; ++c) emax = max(emax, sEb[c * kTileRows]);
       // digit tiles and row exponents of this buffer are free once tile it - 2's products and
       // results are done
-      bool ok2 = true;
-      if (k > 0) ok2 = pipe_wait_warp(&bars->mdone[b], (k - 1) & 1, abort_flag) &&
-                       pipe_wait_warp(&bars->tempty[b], (k - 1) & 1, abort_flag);
-      if (bar_or(1, kSplitThreads, !ok2)) break;  // unit exponents read
-      unsigned char* sAb = sA + (size_t)b * kDigits * kATileBytes;
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int u = tid + kSplitThreads * j;
-        if (u < nunits) {
-          const int row = u & (kTileRows - 1), cb = u >> 7;
-          if (cb == 0) sE[b * kTileRows + row] = emax[j];
-          uint32_t w[kDigits][4];
-          split_pair_f16(v[j][0], v[j][1], emax[j], w, 0);
-          split_pair_f16(v[j][2], v[j][3], emax[j], w, 1);
-          split_pair_f16(v[j][4], v[j][5], emax[j], w, 2);
-          split_pair_f16(v[j][6], v[j][7], emax[j], w, 3);
-          const uint32_t off = tile_off(row, cb * 8);
-#pragma unroll
-          for (int i = 0; i < kDigits; ++i)
-            *reinterpret_cast<uint4*>(sAb + (size_t)i * kATileBytes + off) = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
-        }
+      if (k > 0) bad = !pipe_wait_warp(&bars->mdone[b], (k - 1) & 1, abort_flag) ||
+                       !pipe_wait_warp(&bars->tempty[b], (k - 1) & 1, abort_flag);
+      if (bad) continue;   // the splitters leave together at the next tile's barrier
+      if (unit) {
+        if (cb == 0) sE[b * kTileRows + row] = emax >> 20;
+        Sig8 s8;
+        align8(v, (uint32_t)emax, s8);
+        unsigned char* dst = sA + (size_t)b * kDigits * kATileBytes + doff;
+        digits8(s8, [&](int i, uint4 w) { *reinterpret_cast<uint4*>(dst + i * kATileBytes) = w; });
       }
       tc::fence_async_smem();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&bars->afull[b]);
     }
   } else {
-    // ---- epilogue: warps 8-15, TMEM lane quarter warp % 4; the two warps of a quarter take
-    // alternate groups of two results (q0 = 2 half + 4 jj)
-    const int quarter = warp & 3, half = (warp - kSplitWarps) >> 2;
+    // ---- epilogue: TMEM lane quarter warp % 4; the warps of a quarter take turns at groups of two
+    // results (q0 = 2 part + kStep jj)
+    const int quarter = warp & 3, part = (warp - kSplitWarps) >> 2;
     const int row = quarter * 32 + lane;
     const bool add_out = a.beta != 0.0;
-    const int ngroups = (a.N - 2 * half + 3) / 4;        // this thread's groups of two results
+    constexpr int kStep = 2 * kEpiParts;
+    const int ngroups = a.N > 2 * part ? (a.N - 2 * part + kStep - 1) / kStep : 0;        // this thread's groups of two results
     // rows of Out loaded ahead of their tile: one group per thread (N <= 4) two tiles ahead into
     // slot it % 2, two groups (N <= 8) one tile ahead into slot = group
     const int pf = !add_out ? 0 : ngroups <= 1 ? 2 : ngroups == 2 ? 1 : 0;
     double opf[2][2];
     auto load_grp = [&](int64_t it, int jj, int slot) {
       const int64_t r = tile_of(it) * kTileRows + row;
-      const int q0 = 2 * half + 4 * jj;
+      const int q0 = 2 * part + kStep * jj;
       if (r >= a.n || q0 >= a.N) return;
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
@@ -743,10 +764,10 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_combine_pipe_kernel(const 
       uint32_t nxt[kClasses][2];
       if (ngroups > 0) {
 #pragma unroll
-        for (int g = 0; g < kClasses; ++g) tc::tmem_ld2(lane_addr + (uint32_t)(g * NP + 2 * half), nxt[g]);
+        for (int g = 0; g < kClasses; ++g) tc::tmem_ld2(lane_addr + (uint32_t)(g * NP + 2 * part), nxt[g]);
       }
       for (int jj = 0; jj < ngroups; ++jj) {
-        const int q0 = 2 * half + 4 * jj;
+        const int q0 = 2 * part + kStep * jj;
         tc::tmem_ld_wait();
         uint32_t acc[kClasses][2];
 #pragma unroll
@@ -757,7 +778,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_combine_pipe_kernel(const 
         }
         if (jj + 1 < ngroups) {
 #pragma unroll
-          for (int g = 0; g < kClasses; ++g) tc::tmem_ld2(lane_addr + (uint32_t)(g * NP + q0 + 4), nxt[g]);
+          for (int g = 0; g < kClasses; ++g) tc::tmem_ld2(lane_addr + (uint32_t)(g * NP + q0 + kStep), nxt[g]);
         }
         if (jj == ngroups - 1) {
           // TMEM buffer and row exponent read: the buffer goes back to the MMA issuer
@@ -768,11 +789,8 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_combine_pipe_kernel(const 
         double y[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          const int64_t hi = (int64_t)acc_int(acc[0][u]) * 65536 + (int64_t)acc_int(acc[1][u]) * 256 +
-                             (int64_t)acc_int(acc[2][u]);
-          const int64_t lo = (int64_t)acc_int(acc[3][u]) * 16777216 + (int64_t)acc_int(acc[4][u]) * 65536 +
-                             (int64_t)acc_int(acc[5][u]) * 256 + (int64_t)acc_int(acc[6][u]);
-          const double x = assemble(hi, lo, ebase + sF[min(q0 + u, kMaxN - 1)]);
+          const uint32_t d[kClasses] = {acc[0][u], acc[1][u], acc[2][u], acc[3][u], acc[4][u], acc[5][u], acc[6][u]};
+          const double x = scale_int(sum7(d, kDigitUnit, 8), ebase + sF[min(q0 + u, kMaxN - 1)]);
           y[u] = emax > 0 ? x : 0.0;
         }
         if (live) {
@@ -816,7 +834,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_combine_pipe_kernel(const 
       const int64_t r = tile_of(it) * kTileRows + row;
       if (r < a.n)
         for (int jj = 0; jj < ngroups; ++jj)
-          for (int q = 2 * half + 4 * jj; q < min(a.N, 2 * half + 4 * jj + 2); ++q)
+          for (int q = 2 * part + kStep * jj; q < min(a.N, 2 * part + kStep * jj + 2); ++q)
             a.oblk[q / BV][r * BV + q % BV] = __longlong_as_double(0x7FF8000000000000ll);
     }
   }
@@ -935,21 +953,26 @@ int tc_combine(const BlockSet& V, int64_t n, const double* Y, int ldy, const Blo
 // G = alpha V^T W for FP64 blocks on the tensor cores (Table 1 "op3", MvTransMv), the same
 // digit splitting as above with the roles of rows and columns exchanged: the contraction runs
 // over the rows, so every column of V and of W is scaled by its largest exponent within each
-// 128-row tile.  Per tile the MMA multiplies ALL digit slices at once: A holds the digit rows
+// 112-row tile.  Per tile the MMA multiplies ALL digit slices at once: A holds the digit rows
 // (i, c) of V^T (7 * KV <= 252 rows, two 128-row M tiles), B the digit rows (j, q) of W^T
-// (7 * bw rows), K = the tile's 128 rows; every accumulator D[(i, c)][(j, q)] sums 128
+// (7 * bw rows), K = the tile's 112 rows; every accumulator D[(i, c)][(j, q)] sums 112
 // products below 2^16 and is exact.  TMEM lane (i, c) then forms T_i = sum_j D 2^(8 (6 - j))
-// for each q in 64-bit integers; the seven slices i of each output are added exactly in
-// 128-bit integers, and the sum, scaled by the tile's column exponents, is rounded once to FP64
-// and added to the CTA's accumulator of G, and the CTAs' partial Gram matrices are added in a fixed order.
-// Error per tile: 2^-50 * 128 * max|V[., c]| * max|W[., q]| over the tile's rows, plus the FP64
+// for each q in 64-bit integers (T_i / 2^12, rounded); the seven slices i of each output are added as
+// sum_i T_i 2^(-8 i), rounded at each step to T_0's unit, and the sum, scaled by the tile's column
+// exponents, is rounded once to FP64 and added to the CTA's accumulator of G; the CTAs' partial Gram
+// matrices are added in a fixed order.
+// Error per tile: 2^-50 * 112 * max|V[., c]| * max|W[., q]| over the tile's rows, plus the FP64
 // roundings of the sums over tiles and CTAs.
 namespace {
 constexpr int kGramMaxKV = 36;                       // 7 * 36 = 252 digit rows of V^T
 constexpr int kGramMaxBW = 8;                        // 7 * 8 = 56 digit rows of W^T
-constexpr int kGramRows = 128;                       // rows per tile (MMA K = 8 x 16)
-constexpr uint32_t kGSBO = (kGramRows / 8) * kCoreBytes;  // 2048 B between 8-row groups
-constexpr int kGATile = 128 * kGramRows * 2;         // one 128-row M tile of V^T digits: 32 KB
+// Rows per tile (MMA K = 7 x 16): two digit buffers of 112 rows leave room for two staging buffers at
+// 36 + 4 columns.  3000017 x (36 + 4), the kernel alone: 303 us (404 with 12 splitting and 4 epilogue
+// warps, 128-bit sums and 128 rows); 128 rows (one staging buffer, whose load latency shows)
+// 330, 96 rows (three) 309, 80 rows 343; one digit buffer and three staging buffers of 128 rows 426.
+constexpr int kGramRows = 112;
+constexpr uint32_t kGSBO = (kGramRows / 8) * kCoreBytes;  // between 8-row groups
+constexpr int kGATile = 128 * kGramRows * 2;         // one 128-row M tile of V^T digits: 28 KB
 
 struct TcGramArgs {
   const double* vblk[kMaxBlocks];
@@ -967,36 +990,34 @@ struct TcGramArgs {
 
 // ---------------------------------------------------------------- pipelined Gram
 // The same Gram with its phases overlapped, in the warp roles of the pipelined block product:
-//   warps 0-11  split: unit u = 16 c + g (column c of [V W], 8-row group g), thread t takes
-//               units t and t + 384; the 16 lanes of a half-warp hold one column, so its
-//               exponent over the tile is a 4-step shuffle maximum; digits go to the A / B tiles
-//               of buffer t % 2;
-//   warp 16     (one thread) TMA copies of the tile's rows into the (single) staging buffer;
-//   warp 17     (one thread) the nmt x 8 MMAs of a tile into TMEM buffer t % 2;
-//   warps 12-15 (TMEM lane quarter = warp % 4) for every lane (i, c) and column q:
-//               T_i = sum_j D[(i,c)][(j,q)] 2^(8 (6 - j)) as an integer (the 12 low bits
-//               dropped), into shared memory; after a barrier of the four warps, each output
-//               (c, q) sums its seven slices exactly in 128-bit integers, sum_i T_i 2^(8 (6 - i)),
-//               converts once (truncation) to FP64 with the tile's column scales and adds it to
-//               the thread's FP64 partial of G.
+//   warps 0-19  split: a unit is 8 rows (group g) of column c of [V W], thread t takes unit
+//               t = g (KV + bw) + c; the column exponents are shared-memory maxima over the groups;
+//               digits go to the A / B tiles of buffer t % 2;
+//   warp 28     (one thread) TMA copies of the tile's rows into one of up to four staging buffers;
+//   warp 29     (one thread) the nmt x 7 MMAs of a tile into TMEM buffer t % 2;
+//   warps 20-27 (TMEM lane quarter = warp % 4, two warps each) for every lane (i, c) and column q:
+//               T_i into shared memory; after a barrier of these warps each output (c, q) adds its
+//               seven slices and adds the tile's result to the thread's FP64 partial of G.
 // Barriers: xfull / xempty (staging), afull / mdone / tempty per buffer, as in the block
 // product; the splitters meet twice per tile and the epilogue warps twice, at named barriers
 // that OR their wait failures.
 namespace {
-constexpr int kGSplitWarps = 12, kGEpiWarps = 4;
+constexpr int kGSplitWarps = 20, kGEpiWarps = 8;    // 20 x 32 >= (36 + 8) columns x 14 groups
 constexpr int kGSplitThreads = kGSplitWarps * 32;
 constexpr int kGEpiThreads = kGEpiWarps * 32;
-constexpr int kGProdWarp = 16, kGMmaWarp = 17;
-constexpr int kGPipeThreads = 18 * 32;
+constexpr int kGOuts = 2;            // outputs per epilogue thread
+constexpr int kGMaxStages = 4;       // staging buffers
+constexpr int kGProdWarp = kGSplitWarps + kGEpiWarps, kGMmaWarp = kGProdWarp + 1;
+constexpr int kGPipeThreads = (kGMmaWarp + 1) * 32;
 
 struct GramBars {
-  uint64_t xfull[2], xempty[2], afull[2], mdone[2], tempty[2];
+  uint64_t xfull[kGMaxStages], xempty[kGMaxStages], afull[2], mdone[2], tempty[2];
 };
 constexpr int kGramMaxCols = kGramMaxKV + kGramMaxBW;
 
 struct GramPipeLayout {
   size_t a, b, x, xbuf, t, e, bars, total;
-  int nxb;   // staging buffers: 2 when they fit, else 1
+  int nxb;   // staging buffers: as many as fit, at most kGMaxStages
 };
 __host__ __device__ inline GramPipeLayout gram_pipe_layout(int nmt, int NP, int nvb, int bv, int bw, int KV,
                                                           int nxb) {
@@ -1013,22 +1034,6 @@ __host__ __device__ inline GramPipeLayout gram_pipe_layout(int nmt, int NP, int 
   L.total = L.bars + sizeof(GramBars) + 16;
   return L;
 }
-
-// |v| < 2^127 times 2^s, truncated to FP64 (zero below the normal range, infinity above it).
-__device__ __forceinline__ double i128_to_double(__int128 v, int s) {
-  const uint64_t sign = v < 0 ? 0x8000000000000000ull : 0ull;
-  const unsigned __int128 a = v < 0 ? (unsigned __int128)(-v) : (unsigned __int128)v;
-  const uint64_t hi = (uint64_t)(a >> 64), lo = (uint64_t)a;
-  const uint32_t w3 = (uint32_t)(hi >> 32), w2 = (uint32_t)hi, w1 = (uint32_t)(lo >> 32), w0 = (uint32_t)lo;
-  const int lz = w3 != 0 ? __clz(w3) : w2 != 0 ? 32 + __clz(w2) : w1 != 0 ? 64 + __clz(w1) : 96 + __clz(w0);
-  const unsigned __int128 nrm = a << (lz & 127);
-  const uint64_t m = (uint64_t)(nrm >> 64);
-  const int ef = 127 - lz + s + 1023;
-  uint64_t bits = sign | ((uint64_t)(uint32_t)ef << 52) | ((m >> 11) & 0xFFFFFFFFFFFFFull);
-  bits = (a == 0 || ef <= 0) ? sign : bits;
-  bits = ef >= 2047 ? (sign | 0x7FF0000000000000ull) : bits;
-  return __longlong_as_double((long long)bits);
-}
 }  // namespace
 
 template <int BW>
@@ -1042,8 +1047,8 @@ __global__ void __launch_bounds__(kGPipeThreads, 1) tc_gram_pipe_kernel(const Tc
   const int XS = kGramRows * bv + 4;           // doubles per staged V block (padded)
   const GramPipeLayout L = gram_pipe_layout(nmt, NP, nvb, bv, bw, KV, a.nxb);
   const int nxb = a.nxb;
-  unsigned char* sA = smem + L.a;              // [2][nmt] x 32 KB
-  unsigned char* sB = smem + L.b;              // [2] x NP x 128 FP16
+  unsigned char* sA = smem + L.a;              // [2][nmt] x 28 KB
+  unsigned char* sB = smem + L.b;              // [2] x NP x 112 FP16
   double* sX = reinterpret_cast<double*>(smem + L.x);
   int64_t* sT = reinterpret_cast<int64_t*>(smem + L.t);   // [bw][7][KV] slice integers
   int* sEx = reinterpret_cast<int*>(smem + L.e);          // [2][ncol] column exponents by buffer
@@ -1059,9 +1064,11 @@ __global__ void __launch_bounds__(kGPipeThreads, 1) tc_gram_pipe_kernel(const Tc
     for (int e = tid; e < (int)(L.x / 16); e += kGPipeThreads) z[e] = make_int4(0, 0, 0, 0);
   }
   if (tid == 0) {
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < nxb; ++b) {
       tc::mbar_init(&bars->xfull[b], 1);
       tc::mbar_init(&bars->xempty[b], kGSplitWarps);
+    }
+    for (int b = 0; b < 2; ++b) {
       tc::mbar_init(&bars->afull[b], kGSplitWarps);
       tc::mbar_init(&bars->mdone[b], 1);
       tc::mbar_init(&bars->tempty[b], kGEpiWarps);
@@ -1079,23 +1086,24 @@ __global__ void __launch_bounds__(kGPipeThreads, 1) tc_gram_pipe_kernel(const Tc
   tc::fence_after_sync();
   const uint32_t tbase = *tslot;
   const int64_t ntiles = (a.n + kGramRows - 1) / kGramRows;
-  const int64_t cnt = (int64_t)blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-  auto tile_of = [&](int64_t it) { return (int64_t)blockIdx.x + it * gridDim.x; };
-  auto bulk_ok = [&](int64_t t) {
-    const int64_t rows = min((int64_t)kGramRows, a.n - t * kGramRows);
-    return a.bulk && (rows * bv * 8) % 16 == 0 && (rows * bw * 8) % 16 == 0;
-  };
+  const int cnt = (int64_t)blockIdx.x < ntiles ? (int)((ntiles - 1 - blockIdx.x) / gridDim.x + 1) : 0;
+  auto tile_of = [&](int it) { return (int64_t)blockIdx.x + (int64_t)it * gridDim.x; };
+  // this CTA's last tile is the matrix's last one: its rows past the end read zero, and it is loaded
+  // without TMA unless its bytes are a multiple of 16
+  const bool own_last = cnt > 0 && tile_of(cnt - 1) == ntiles - 1;
+  const int last = (int)(a.n - (ntiles - 1) * kGramRows);
+  const int nbulk = !a.bulk ? 0 : own_last && ((last * bv) % 2 != 0 || (last * bw) % 2 != 0) ? cnt - 1 : cnt;
 
   if (warp == kGProdWarp) {
-    int64_t issued = 0;
+    int issued = 0;
     if (lane == 0) {
-      for (int64_t it = 0; it < cnt; ++it) {
-        const int xb = nxb == 2 ? (int)(it & 1) : 0;
-        const int64_t xk = nxb == 2 ? (it >> 1) : it;
-        if (xk > 0 && !pipe_wait(&bars->xempty[xb], (uint32_t)((xk - 1) & 1), abort_flag)) break;
+      int xb = 0;
+      uint32_t xk = 0;   // uses of each buffer so far
+      for (int it = 0; it < cnt; ++it) {
+        if (xk > 0 && !pipe_wait(&bars->xempty[xb], (xk - 1) & 1, abort_flag)) break;
         const int64_t t = tile_of(it), r0 = t * kGramRows;
         double* sXb = sX + (size_t)xb * (L.xbuf / 8);
-        if (bulk_ok(t)) {
+        if (it < nbulk) {
           const int64_t rows = min((int64_t)kGramRows, a.n - r0);
           const uint32_t vb = (uint32_t)(rows * bv * 8), wb = (uint32_t)(rows * bw * 8);
           tc::mbar_arrive_expect_tx(&bars->xfull[xb], vb * (uint32_t)nvb + wb);
@@ -1105,18 +1113,22 @@ __global__ void __launch_bounds__(kGPipeThreads, 1) tc_gram_pipe_kernel(const Tc
           tc::mbar_arrive(&bars->xfull[xb]);   // ragged or unaligned tile: splitters load directly
         }
         issued = it + 1;
+        if (++xb == nxb) {
+          xb = 0;
+          ++xk;
+        }
       }
-      for (int xb = 0; xb < nxb; ++xb) {
-        const int64_t uses = nxb == 2 ? (issued + 1 - xb) / 2 : issued;
+      for (xb = 0; xb < nxb; ++xb) {
+        const int uses = (issued + nxb - 1 - xb) / nxb;
         if (uses > 0) wait_sleep(&bars->xfull[xb], (uint32_t)((uses - 1) & 1));
       }
     }
   } else if (warp == kGMmaWarp) {
-    int64_t committed = 0;
+    int committed = 0;
     if (lane == 0) {
       const uint32_t idesc = tc::idesc_f16_f32(128, NP);
       const uint32_t sa0 = tc::smem_addr(sA), sb0 = tc::smem_addr(sB);
-      for (int64_t it = 0; it < cnt; ++it) {
+      for (int it = 0; it < cnt; ++it) {
         const int b = (int)(it & 1);
         const uint32_t k = (uint32_t)(it >> 1);
         if (!pipe_wait(&bars->afull[b], k & 1, abort_flag)) break;
@@ -1135,109 +1147,76 @@ __global__ void __launch_bounds__(kGPipeThreads, 1) tc_gram_pipe_kernel(const Tc
         committed = it + 1;
       }
       for (int b = 0; b < 2; ++b) {
-        const int64_t uses = (committed + 1 - b) / 2;
+        const int uses = (committed + 1 - b) / 2;
         if (uses > 0) wait_sleep(&bars->mdone[b], (uint32_t)((uses - 1) & 1));
       }
     }
   } else if (warp < kGSplitWarps) {
-    // ---- split: units (column c, 8-row group g) with u = g ncol + c, so that a warp's lanes read
+    // ---- split: unit (column c, 8-row group g) of thread u = g ncol + c, so that a warp's lanes read
     // and write neighbouring columns (no shared-memory bank conflicts); the column exponents
-    // are maxima over the 16 groups through shared-memory atomics (double-buffered by tile)
-    const int nunits = ncol * 16;
-    // this thread's units, the same in every tile: column, row group, column pointer and stride
-    int uc[2], ug[2], ustr[2], usoff[2];
-    const double* ucol[2];
+    // are maxima over the groups through shared-memory atomics (double-buffered by tile)
+    const bool unit = tid < ncol * (kGramRows / 8);
+    const int c = unit ? tid % ncol : 0, g = unit ? tid / ncol : 0;
+    const bool isv = c < KV;
+    const int str = isv ? bv : bw;
+    const int soff = (isv ? (c / bv) * XS + c % bv : nvb * XS + (c - KV)) + g * 8 * str;
+    uint32_t doff[kDigits];   // where the unit's digits go
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int u = tid + kGSplitThreads * j;
-      uc[j] = u < nunits ? u % ncol : 0;
-      ug[j] = u < nunits ? u / ncol : 0;
-      const int c = uc[j];
-      const bool isv = c < KV;
-      ustr[j] = isv ? bv : bw;
-      ucol[j] = isv ? a.vblk[c / bv] + c % bv : a.W + (c - KV);
-      usoff[j] = isv ? (c / bv) * XS + c % bv : nvb * XS + (c - KV);
+    for (int i = 0; i < kDigits; ++i) {
+      const int m = isv ? i * KV + c : i * bw + (c - KV);
+      doff[i] = (uint32_t)((isv ? L.a + (size_t)(m >> 7) * kGATile + ((m & 127) >> 3) * kGSBO
+                                : L.b + (size_t)(m >> 3) * kGSBO) + g * kCoreBytes + (m & 7) * 16);
     }
+    const uint32_t dbuf = isv ? (uint32_t)(nmt * kGATile) : (uint32_t)(NP * kGramRows * 2);
     for (int e = tid; e < 2 * kGramMaxCols; e += kGSplitThreads) sExw[e] = 0;
     bar_or(1, kGSplitThreads, false);
-    for (int64_t it = 0; it < cnt; ++it) {
+    int xb = 0;               // staging buffer
+    uint32_t xph = 0;
+    for (int it = 0; it < cnt; ++it) {
       const int b = (int)(it & 1);
       const uint32_t k = (uint32_t)(it >> 1);
-      const int64_t t = tile_of(it), r0 = t * kGramRows;
-      const bool bulk = bulk_ok(t);
-      int* exw = sExw + (it & 1) * kGramMaxCols;
-      const int xb = nxb == 2 ? (int)(it & 1) : 0;
-      const double* sXb = sX + (size_t)xb * (L.xbuf / 8);
-      const bool ok = pipe_wait_warp(&bars->xfull[xb], (uint32_t)((nxb == 2 ? (it >> 1) : it) & 1), abort_flag);
-      double x[2][8];
+      int* exw = sExw + b * kGramMaxCols;
+      const bool ok = pipe_wait_warp(&bars->xfull[xb], xph, abort_flag);
+      double x[8];
+      if (unit) {
+        if (it < nbulk) {
+          const double* scol = sX + xb * (int)(L.xbuf / 8) + soff;   // in the staging buffer in any case
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int u = tid + kGSplitThreads * j;
-        if (u < nunits) {
-          const int c = uc[j], g = ug[j], str = ustr[j];
-          const double* gcol = ucol[j];
-          const double* scol = sXb + usoff[j];
-          int e = 0;
-          if (bulk) {
+          for (int tt = 0; tt < 8; ++tt) x[tt] = scol[tt * str];
+        } else {
+          const int64_t r = tile_of(it) * kGramRows + g * 8;
+          const double* src = (isv ? a.vblk[c / bv] + c % bv : a.W + (c - KV)) + r * str;
 #pragma unroll
-            for (int tt = 0; tt < 8; ++tt) {
-              const double v = scol[(g * 8 + tt) * str];   // in the staging buffer in any case
-              x[j][tt] = r0 + g * 8 + tt < a.n ? v : 0.0;
-            }
-          } else {
-#pragma unroll
-            for (int tt = 0; tt < 8; ++tt) {
-              const int64_t r = r0 + g * 8 + tt;
-              x[j][tt] = r < a.n ? __ldg(gcol + r * str) : 0.0;
-            }
-          }
-#pragma unroll
-          for (int tt = 0; tt < 8; ++tt) e = max(e, exp_field(x[j][tt]));
-          if (e > 0) atomicMax(exw + c, e);
+          for (int tt = 0; tt < 8; ++tt) x[tt] = r + tt < a.n ? __ldg(src + tt * str) : 0.0;
         }
+        if (own_last && it == cnt - 1) {
+#pragma unroll
+          for (int tt = 0; tt < 8; ++tt) x[tt] = g * 8 + tt < last ? x[tt] : 0.0;
+        }
+        const uint32_t e = top_exp8(x);
+        if (e > 0) atomicMax(exw + c, (int)e);
       }
       if (bar_or(1, kGSplitThreads, !ok)) break;   // staging buffer read, exponent maxima formed
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&bars->xempty[xb]);
-      int emax[2] = {0, 0};
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int u = tid + kGSplitThreads * j;
-        if (u < nunits) emax[j] = exw[uc[j]];
+      if (++xb == nxb) {
+        xb = 0;
+        xph ^= 1u;
       }
+      const uint32_t emax = (uint32_t)exw[c];
       // the other buffer of maxima (read by everyone before the previous tile's second barrier)
       // starts the next tile at zero
-      for (int e = tid; e < ncol; e += kGSplitThreads) sExw[((it + 1) & 1) * kGramMaxCols + e] = 0;
+      if (tid < ncol) sExw[(b ^ 1) * kGramMaxCols + tid] = 0;
       bool ok2 = true;
       if (k > 0) ok2 = pipe_wait_warp(&bars->mdone[b], (k - 1) & 1, abort_flag) &&
                        pipe_wait_warp(&bars->tempty[b], (k - 1) & 1, abort_flag);
       if (bar_or(1, kGSplitThreads, !ok2)) break;  // digit tiles and exponents of buffer b free
-      unsigned char* sAb = sA + (size_t)b * nmt * kGATile;
-      unsigned char* sBb = sB + (size_t)b * NP * kGramRows * 2;
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int u = tid + kGSplitThreads * j;
-        if (u < nunits) {
-          const int c = uc[j], g = ug[j];
-          if (g == 0) sEx[b * kGramMaxCols + c] = emax[j];
-          uint32_t w[kDigits][4];
-          split_pair_f16(x[j][0], x[j][1], emax[j], w, 0);
-          split_pair_f16(x[j][2], x[j][3], emax[j], w, 1);
-          split_pair_f16(x[j][4], x[j][5], emax[j], w, 2);
-          split_pair_f16(x[j][6], x[j][7], emax[j], w, 3);
-#pragma unroll
-          for (int i = 0; i < kDigits; ++i) {
-            unsigned char* dst;
-            if (c < KV) {
-              const int m = i * KV + c;
-              dst = sAb + (size_t)(m >> 7) * kGATile + ((m & 127) >> 3) * kGSBO + g * kCoreBytes + (m & 7) * 16;
-            } else {
-              const int nn = i * bw + (c - KV);
-              dst = sBb + (nn >> 3) * kGSBO + g * kCoreBytes + (nn & 7) * 16;
-            }
-            *reinterpret_cast<uint4*>(dst) = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
-          }
-        }
+      if (unit) {
+        if (g == 0) sEx[b * kGramMaxCols + c] = (int)(emax >> 20);
+        Sig8 s8;
+        align8(x, emax, s8);
+        unsigned char* dst = smem + (uint32_t)b * dbuf;
+        digits8(s8, [&](int i, uint4 w) { *reinterpret_cast<uint4*>(dst + doff[i]) = w; });
       }
       tc::fence_async_smem();
       __syncwarp();
@@ -1245,10 +1224,10 @@ __global__ void __launch_bounds__(kGPipeThreads, 1) tc_gram_pipe_kernel(const Tc
     }
   } else if (warp < kGSplitWarps + kGEpiWarps) {
     // ---- epilogue: TMEM lane quarter warp % 4 of each M tile
-    const int quarter = warp & 3, et = tid - kGSplitThreads;
+    const int quarter = warp & 3, half = (warp - kGSplitWarps) >> 2, et = tid - kGSplitThreads;
     const int nout = KV * bw;
-    double acc[3] = {0.0, 0.0, 0.0};   // outputs et, et + 128, et + 256 (nout <= 288)
-    for (int64_t it = 0; it < cnt; ++it) {
+    double acc[kGOuts] = {};   // outputs et, et + 256 (nout <= 288)
+    for (int it = 0; it < cnt; ++it) {
       const int b = (int)(it & 1);
       const uint32_t k = (uint32_t)(it >> 1);
       const bool ok = pipe_wait_warp(&bars->afull[b], k & 1, abort_flag) &&
@@ -1257,9 +1236,9 @@ __global__ void __launch_bounds__(kGPipeThreads, 1) tc_gram_pipe_kernel(const Tc
       tc::fence_after_sync();
       // this thread's output scales, read before the buffer's exponents are handed back
       const int* ex = sEx + b * kGramMaxCols;
-      int scl[3];
+      int scl[kGOuts];
 #pragma unroll
-      for (int kk = 0; kk < 3; ++kk) {
+      for (int kk = 0; kk < kGOuts; ++kk) {
         const int o = et + kGEpiThreads * kk;
         scl[kk] = 0;
         if (o < nout) {
@@ -1272,6 +1251,7 @@ __global__ void __launch_bounds__(kGPipeThreads, 1) tc_gram_pipe_kernel(const Tc
         const uint32_t laddr = tbase + ((uint32_t)(quarter * 32) << 16) + (uint32_t)b * bufcols + (uint32_t)(mt * NP);
 #pragma unroll
         for (int q = 0; q < bw; ++q) {
+          if (((mt * bw + q) & 1) != half) continue;
           uint32_t d[kDigits];
 #pragma unroll
           for (int jd = 0; jd < kDigits; ++jd) d[jd] = tc::tmem_ld1(laddr + (uint32_t)(jd * bw + q));
@@ -1279,11 +1259,9 @@ __global__ void __launch_bounds__(kGPipeThreads, 1) tc_gram_pipe_kernel(const Tc
 #pragma unroll
           for (int jd = 0; jd < kDigits; ++jd) tc::reg_after_wait(d[jd]);
           if (m < 7 * KV) {
-            const int64_t hi = (int64_t)acc_int(d[0]) * 65536 + (int64_t)acc_int(d[1]) * 256 + (int64_t)acc_int(d[2]);
-            const int64_t lo = (int64_t)acc_int(d[3]) * 16777216 + (int64_t)acc_int(d[4]) * 65536 +
-                               (int64_t)acc_int(d[5]) * 256 + (int64_t)acc_int(d[6]);
-            // T_i / 2^12 (floor), i = m / KV, c = m % KV
-            sT[q * 7 * KV + m] = (hi << (32 - kAsmShift)) + (lo >> kAsmShift);
+            // T_i / 2^12 of slice i = m / KV, column c = m % KV; slices i > 0 hold 128 more, the
+            // rounding of their division by 2^8
+            sT[q * 7 * KV + m] = sum7(d, kDigitUnit * kDigitUnit, m < KV ? 8 : 8 + 16 * 128);
           }
         }
       }
@@ -1292,20 +1270,22 @@ __global__ void __launch_bounds__(kGPipeThreads, 1) tc_gram_pipe_kernel(const Tc
       if (lane == 0) tc::mbar_arrive(&bars->tempty[b]);
       bar_or(2, kGEpiThreads, false);   // slice integers written
 #pragma unroll
-      for (int kk = 0; kk < 3; ++kk) {
+      for (int kk = 0; kk < kGOuts; ++kk) {
         const int o = et + kGEpiThreads * kk;
         if (o < nout) {
           const int c = o / bw, q = o % bw;
-          __int128 sum = 0;
+          // sum_i T_i 2^(-8 i), rounded at each division
+          const int64_t* tq = sT + q * 7 * KV + c;
+          int64_t sum = tq[6 * KV];
 #pragma unroll
-          for (int i = 0; i < kDigits; ++i) sum += (__int128)sT[q * 7 * KV + i * KV + c] << (8 * (6 - i));
-          if (scl[kk] > 0) acc[kk] += i128_to_double(sum, scl[kk] - 2108 + kAsmShift - 48);
+          for (int i = kDigits - 2; i >= 0; --i) sum = tq[i * KV] + (sum >> 8);
+          if (scl[kk] > 0) acc[kk] += scale_int(sum, scl[kk] - 2108 + kAsmShift);
         }
       }
       bar_or(2, kGEpiThreads, false);   // slice integers read: the next tile may overwrite them
     }
 #pragma unroll
-    for (int kk = 0; kk < 3; ++kk) {
+    for (int kk = 0; kk < kGOuts; ++kk) {
       const int o = et + kGEpiThreads * kk;
       if (o < nout) a.partial[(int64_t)blockIdx.x * nout + o] = *abort_flag ? __longlong_as_double(0x7FF8000000000000ll) : acc[kk];
     }
@@ -1339,10 +1319,13 @@ int tc_gram(const BlockSet& V, int64_t n, const double* W, int bw, double alpha,
   a.NP = (int)ceil_div(7 * bw, 16) * 16;
   a.nmt = (int)ceil_div(7 * a.KV, 128);
   a.n = n;
-  GramPipeLayout L = gram_pipe_layout(a.nmt, a.NP, a.KV / a.bv, a.bv, bw, a.KV, 2);
-  if (L.total > 227 * 1024) L = gram_pipe_layout(a.nmt, a.NP, a.KV / a.bv, a.bv, bw, a.KV, 1);
+  GramPipeLayout L;
+  for (int nxb = kGMaxStages; nxb > 0; --nxb) {
+    L = gram_pipe_layout(a.nmt, a.NP, a.KV / a.bv, a.bv, bw, a.KV, nxb);
+    if (L.total <= 227 * 1024) break;
+  }
   a.nxb = L.nxb;
-  FE_ARG(L.total <= 227 * 1024 && a.KV * bw <= 3 * kGEpiThreads, "tc_gram: shape too large");
+  FE_ARG(L.total <= 227 * 1024 && a.KV * bw <= kGOuts * kGEpiThreads, "tc_gram: shape too large");
   static KernelSetup kp[4];
   const int bj = bw == 1 ? 0 : bw == 2 ? 1 : bw == 4 ? 2 : 3;
   const void* fp = bw == 1 ? reinterpret_cast<const void*>(tc_gram_pipe_kernel<1>)

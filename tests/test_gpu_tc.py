@@ -250,6 +250,48 @@ def test_tc_gram_matches_oracle(shape):
     _gram_check(Vh, Wh, G.cpu().numpy())
 
 
+@pytest.mark.parametrize("nv,bv,bw", [(9, 4, 4), (36, 1, 8), (17, 2, 8), (5, 4, 4), (1, 1, 1)])
+@pytest.mark.parametrize("n", [1, 8, 111, 112, 113, 224, 152 * 112 - 1, 152 * 112 + 1, 3 * 152 * 112 + 57])
+def test_tc_gram_row_tiles(n, nv, bv, bw):
+    """The 112-row tiles of the Gram matrix at their edges, one to four staging buffers (2, 1, 1, 3 and 4
+    at these widths), one tile and several per CTA; columns of very different scales, rows of zeros.
+    Bound: 2^-50 * 112 max|V_c| max|W_q| per tile, and the FP64 roundings of the tiles' sum."""
+    rng = np.random.default_rng(n + 5 * nv + bw)
+    Vh = rng.standard_normal((nv, n, bv)) * 2.0 ** rng.integers(-300, 300, (nv, 1, bv))
+    Wh = rng.standard_normal((n, bw)) * 2.0 ** rng.integers(-300, 300, (1, bw))
+    Vh[:, rng.random(n) < 0.1] = 0.0
+    G = fe.block_gram(to_dev(Vh), to_dev(Wh), engine="tc").cpu().numpy()
+    AA = _flat(Vh)
+    ref = (AA.astype(np.longdouble).T @ Wh.astype(np.longdouble)).astype(np.float64)
+    stated = np.zeros_like(ref)
+    for r0 in range(0, n, 112):
+        stated += 2.0 ** -50 * 112 * np.outer(np.abs(AA[r0:r0 + 112]).max(0), np.abs(Wh[r0:r0 + 112]).max(0))
+    stated += (2 + n / 112) * 2.0 ** -52 * (np.abs(AA).T @ np.abs(Wh)) + 2.0 ** -1022
+    assert (np.abs(G - ref) <= stated).all()
+
+
+@pytest.mark.parametrize("beta", [0.0, 1.0])
+@pytest.mark.parametrize("n,K,N", [(129, 7, 1), (128, 8, 2), (300, 9, 3), (127, 32, 5), (400, 31, 6), (1, 1, 7),
+                                   (513, 17, 12), (260, 32, 13), (129, 24, 19), (2000, 32, 32)])
+def test_tc_combine_thread_shares(n, K, N, beta):
+    """Single columns: units of eight columns with a remainder, and results shared by three threads per
+    row, from none to six pairs each; with a result that is added to.  The stated bound."""
+    rng = np.random.default_rng(n + K + N)
+    Vh = rng.standard_normal((K, n, 1)) * 2.0 ** rng.integers(-200, 200, (1, n, 1))
+    Yh = rng.standard_normal((K, N))
+    AA = _flat(Vh)
+    if beta == 0.0:
+        _check(Vh, Yh, _run(Vh, Yh, N))
+        return
+    W0 = rng.standard_normal((n, 1)) * np.abs(AA).max(axis=1)[:, None]
+    W = to_dev(W0)
+    fe.block_update(to_dev(Vh), to_dev(Yh[:, :1]), W, alpha=-1.0, beta=1.0, engine="tc")
+    ref = W0 - AA @ Yh[:, :1]
+    bound = (2.0 ** -49 * (K + 1) * np.abs(AA).max(axis=1)[:, None] * np.abs(Yh[:, :1]).max()
+             + (K + 2) * 2.0 ** -52 * (np.abs(AA) @ np.abs(Yh[:, :1]) + np.abs(W0)))
+    assert (np.abs(W.cpu().numpy() - ref) <= bound).all()
+
+
 def _offset_dev(h, off):
     """h on the device, starting `off` doubles into a larger buffer (8 bytes off a 16-byte
     boundary for odd off)."""
