@@ -128,7 +128,7 @@ struct Phase {
   int replacements = 0, restarts = 0, nconv = 0;
   int64_t spmm_blocks = 0;
   double anorm_h = 0.0, max_resid = 0.0, worst_ratio = 0.0;
-  std::vector<double> theta_h, rho_h, resid_h;
+  std::vector<double> theta_h, rho_h, resid_h, back_h;
 
   int alloc() {
     const size_t es = dt_size(dt);
@@ -157,9 +157,9 @@ struct Phase {
     const size_t nritz = ritz_work_doubles(m);
     FE_TRY(small.alloc(sizeof(double) * (nritz + nsmall)));
     ritzwork = small.as<double>();
-    theta = ritzwork + nritz;
-    Y = theta + m;
-    rho = Y + (size_t)m * m;
+    Y = ritzwork + nritz;
+    theta = Y + (size_t)m * m;   // theta, rho and anorm: read back as one
+    rho = theta + m;
     anorm = rho + m;
     Cdiag = anorm + 4;
     gtmp = Cdiag + 256;
@@ -167,6 +167,7 @@ struct Phase {
     if (op_ata) FE_TRY(opbuf.alloc(blk));
     theta_h.resize(m);
     rho_h.resize(m);
+    back_h.resize(2 * (size_t)m + 1);
     resid_h.assign(nev, 0.0);
     return FE_OK;
   }
@@ -236,11 +237,11 @@ struct Phase {
   int ritz(int* nconv_out) {
     FE_TRY(launch_ritz(H, m, b, which, max_sweeps, 1e-15, theta, Y, rho, info,
                        ritzwork, s));
-    double an = 0.0;
-    FE_CUDA(cudaMemcpyAsync(theta_h.data(), theta, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
-    FE_CUDA(cudaMemcpyAsync(rho_h.data(), rho, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
-    FE_CUDA(cudaMemcpyAsync(&an, anorm, sizeof(double), cudaMemcpyDeviceToHost, s));
+    FE_CUDA(cudaMemcpyAsync(back_h.data(), theta, sizeof(double) * (2 * (size_t)m + 1), cudaMemcpyDeviceToHost, s));
     FE_CUDA(cudaStreamSynchronize(s));
+    theta_h.assign(back_h.begin(), back_h.begin() + m);
+    rho_h.assign(back_h.begin() + m, back_h.begin() + 2 * m);
+    const double an = back_h[2 * (size_t)m];
     double tmax = 0.0;
     for (int c = 0; c < m; ++c) tmax = std::max(tmax, fabs(theta_h[c]));
     anorm_h = std::max(an, tmax);

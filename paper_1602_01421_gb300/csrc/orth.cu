@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kPostThreads)
     const bool good = chol_inv_warp<B>(S, kRelPivot, kAbsBreakdown * a, R, Ri);
     if (tid == 0) {
       ok = good;
-      if (!good) *status = 1;
+      status[0] = good ? 0 : 1;
     }
   }
   __syncthreads();
@@ -212,7 +212,10 @@ __global__ void __launch_bounds__(kPostThreads)
     }
   }
   small = __syncthreads_and(small) != 0;
-  if (tid == 0) status[1] = (good && small) ? 1 : 0;
+  if (tid == 0) {
+    status[1] = (good && small) ? 1 : 0;
+    status[2] = 0;
+  }
 }
 
 // After pass 3: R2 = chol(S2); R = R2 Racc (-> Rout, ldr), M = R2^{-1}; failure -> *status = 2.
@@ -491,7 +494,6 @@ int orth_ex(const BlockSet& V, int64_t n, void* W, int b, fe_dtype dt, double* d
   if (!sG1 || !sG2 || !sM || !sC || !sRacc || !sS2 || !sStat || !gdummy) return FE_ERR_OOM;
   int* status = reinterpret_cast<int*>(sStat);
   if (!d_G) d_G = gdummy;  // k == 0: nothing is written to G
-  FE_CUDA(cudaMemsetAsync(status, 0, 3 * sizeof(int), s));
   std::vector<const void*> vx(V.blk, V.blk + V.nv);
   vx.push_back(W);
   BlockSet Vx = blockset_of(vx, b, b);
@@ -568,11 +570,12 @@ int orth_ex(const BlockSet& V, int64_t n, void* W, int b, fe_dtype dt, double* d
   if (dt == FE_F64) FE_TRY(launch_right_mult(static_cast<double*>(W), n, b, sM, status, allow32, s));
   else FE_TRY(launch_right_mult(static_cast<float*>(W), n, b, sM, status, 0, s));
   int st = 0;
-  double an = 0.0;
   FE_CUDA(cudaMemcpyAsync(&st, status, sizeof(int), cudaMemcpyDeviceToHost, s));
-  FE_CUDA(cudaMemcpyAsync(&an, d_anorm, sizeof(double), cudaMemcpyDeviceToHost, s));
   FE_CUDA(cudaStreamSynchronize(s));
   if (st == 0) return FE_OK;
+  double an = 0.0;
+  FE_CUDA(cudaMemcpyAsync(&an, d_anorm, sizeof(double), cudaMemcpyDeviceToHost, s));
+  FE_CUDA(cudaStreamSynchronize(s));
   return orth_fallback(V, n, W, b, dt, an, seed, rng_counter, d_G, ldg, sRacc, d_R, ldr,
                        replaced, s);
 }

@@ -205,7 +205,6 @@ struct TcArgs {
   int nkc;                     // K chunks of 32
   const uint16_t* bdig;        // global: [nkc][7][NP x 32] canonical tiles
   const int* fexp;             // global: N column exponent fields of Y
-  int* status;                 // device word: 1 = an MMA wait ran out
   double beta;                 // Out = beta Out + (alpha V Y); beta = 0: Out is not read
   int bulk;                    // 1: every V block is 16-byte aligned (TMA bulk copies allowed)
   int ovec;                    // 1: every output block is 16-byte aligned (vector stores allowed)
@@ -319,7 +318,6 @@ __global__ void __launch_bounds__(kThreads, KMAX <= 32 ? 2 : 1) tc_combine_kerne
   const int cbeg = half * KH;                    // this thread's first V column
   const int kc_mine = cbeg / kKChunk, k_mine = cbeg % kKChunk;
   uint32_t phase = 0, lphase = 0;
-  bool failed = false;
 
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int64_t r = tile * kTileRows + row;
@@ -329,7 +327,6 @@ __global__ void __launch_bounds__(kThreads, KMAX <= 32 ? 2 : 1) tc_combine_kerne
     if (bulk) {
       ok = wait_sleep(lbar, lphase);
       if (!ok) {
-        failed = true;
         wait_sleep(lbar, lphase);  // no copy left in flight
       }
       lphase ^= 1;
@@ -400,7 +397,6 @@ __global__ void __launch_bounds__(kThreads, KMAX <= 32 ? 2 : 1) tc_combine_kerne
     // ---- wait for the products (bounded), then read row `row`'s accumulators
     if (!wait_sleep(bar, phase)) {
       ok = false;
-      failed = true;
       wait_sleep(bar, phase);  // let the MMAs in flight finish before TMEM is reused
     }
     phase ^= 1;
@@ -448,7 +444,6 @@ __global__ void __launch_bounds__(kThreads, KMAX <= 32 ? 2 : 1) tc_combine_kerne
     tc::fence_before_sync();
     __syncthreads();  // TMEM read, A tiles and row exponents free for the next tile
   }
-  if (failed && lane == 0) atomicExch(a.status, 1);
   tc::fence_after_sync();
   if (warp == 0) tc::tmem_dealloc(tbase, ncols);
 }
@@ -841,7 +836,6 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_combine_pipe_kernel(const 
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  if (tid == 0 && *abort_flag) atomicExch(a.status, 1);
   if (warp == kMmaWarp) tc::tmem_dealloc(tbase, 2 * kBufCols);
 }
 
@@ -913,14 +907,12 @@ int tc_combine(const BlockSet& V, int64_t n, const double* Y, int ldy, const Blo
     a.oblk[o] = const_cast<double*>(static_cast<const double*>(Out.blk[o]));
     if (reinterpret_cast<uintptr_t>(Out.blk[o]) % 16) a.ovec = 0;
   }
-  // scratch: B digit tiles, column exponents, status word
+  // scratch: B digit tiles, column exponents
   const size_t bbytes = (size_t)a.nkc * kDigits * a.NP * kKChunk * 2;
-  double* scr = small_scratch(17, bbytes / 8 + kMaxN + 2);
+  double* scr = small_scratch(17, bbytes / 8 + kMaxN);
   if (!scr) return FE_ERR_OOM;
   a.bdig = reinterpret_cast<const uint16_t*>(scr);
   a.fexp = reinterpret_cast<const int*>(scr + bbytes / 8);
-  a.status = reinterpret_cast<int*>(scr + bbytes / 8 + kMaxN);
-  FE_CUDA(cudaMemsetAsync(a.status, 0, sizeof(int), s));
   tc_prep_y_kernel<<<1, 256, 0, s>>>(Y, ldy, alpha, a.K, a.N, a.NP, a.nkc, const_cast<uint16_t*>(a.bdig),
                                      const_cast<int*>(a.fexp));
   count_launch();
@@ -982,7 +974,6 @@ struct TcGramArgs {
   int nmt;               // M tiles of V^T digits (1 or 2)
   int64_t n;
   double* partial;       // [gridDim.x][KV * bw]
-  int* status;
   int bulk;              // 1: V blocks and W 16-byte aligned (TMA bulk copies allowed)
   int nxb;               // staging buffers of the pipelined kernel (1 or 2)
 };
@@ -1293,7 +1284,6 @@ __global__ void __launch_bounds__(kGPipeThreads, 1) tc_gram_pipe_kernel(const Tc
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  if (tid == 0 && *abort_flag) atomicExch(a.status, 1);
   if (warp == kGMmaWarp) tc::tmem_dealloc(tbase, 2 * bufcols);
 }
 
@@ -1336,11 +1326,9 @@ int tc_gram(const BlockSet& V, int64_t n, const double* W, int bw, double alpha,
   const int64_t nt = ceil_div(n, kGramRows);
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(nt, (int64_t)num_sms()));
   const int nout = a.KV * bw;
-  double* scr = small_scratch(18, (size_t)grid * nout + 2);
+  double* scr = small_scratch(18, (size_t)grid * nout);
   if (!scr) return FE_ERR_OOM;
   a.partial = scr;
-  a.status = reinterpret_cast<int*>(scr + (size_t)grid * nout);
-  FE_CUDA(cudaMemsetAsync(a.status, 0, sizeof(int), s));
   switch (bw) {
     case 1: tc_gram_pipe_kernel<1><<<grid, kGPipeThreads, L.total, s>>>(a); break;
     case 2: tc_gram_pipe_kernel<2><<<grid, kGPipeThreads, L.total, s>>>(a); break;
