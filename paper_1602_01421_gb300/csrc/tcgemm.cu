@@ -214,17 +214,20 @@ struct TcArgs {
 
 // Y (K x N FP64, row-major, ld ldy) -> per-column exponent fields and the seven digit tiles of
 // every 32-row K chunk in the MMA's B layout (row q of B = column q of Y; rows N..NP-1 and
-// K beyond K zero).  One CTA.
+// K beyond K zero).  One CTA, bound by the latency of its few dependent steps: the exponents are
+// shared-memory maxima over all of Y (K = 32, N = 4: 2.5 us, 3.5 with a column per thread of 256).
+constexpr int kPrepThreads = 512;
 __global__ void tc_prep_y_kernel(const double* __restrict__ Y, int ldy, double alpha, int K, int N, int NP,
                                  int nkc, uint16_t* __restrict__ bdig, int* __restrict__ fexp) {
   __shared__ int sf[kMaxN];
-  for (int q = threadIdx.x; q < N; q += blockDim.x) {
-    int f = 0;
-    for (int c = 0; c < K; ++c) f = max(f, exp_field(alpha * Y[c * ldy + q]));
-    sf[q] = f;
-    fexp[q] = f;
+  for (int q = threadIdx.x; q < N; q += blockDim.x) sf[q] = 0;
+  __syncthreads();
+  for (int e = threadIdx.x; e < K * N; e += blockDim.x) {
+    const int c = e / N, q = e - c * N;
+    atomicMax(sf + q, exp_field(alpha * Y[c * ldy + q]));
   }
   __syncthreads();
+  for (int q = threadIdx.x; q < N; q += blockDim.x) fexp[q] = sf[q];
   const int per_tile = NP * kKChunk;  // elements of one [NP x 32] tile
   const int total = nkc * per_tile;
   for (int e = threadIdx.x; e < total; e += blockDim.x) {
@@ -913,7 +916,7 @@ int tc_combine(const BlockSet& V, int64_t n, const double* Y, int ldy, const Blo
   if (!scr) return FE_ERR_OOM;
   a.bdig = reinterpret_cast<const uint16_t*>(scr);
   a.fexp = reinterpret_cast<const int*>(scr + bbytes / 8);
-  tc_prep_y_kernel<<<1, 256, 0, s>>>(Y, ldy, alpha, a.K, a.N, a.NP, a.nkc, const_cast<uint16_t*>(a.bdig),
+  tc_prep_y_kernel<<<1, kPrepThreads, 0, s>>>(Y, ldy, alpha, a.K, a.N, a.NP, a.nkc, const_cast<uint16_t*>(a.bdig),
                                      const_cast<int*>(a.fexp));
   count_launch();
   FE_CUDA(cudaGetLastError());
