@@ -205,7 +205,11 @@ __global__ void gram_reduce_kernel(const double* __restrict__ partial, int nctas
 }
 
 static int launch_gram_reduce(const double* part, int nctas, int nout, double alpha, double* G,
-                              cudaStream_t s) {
+                              cudaStream_t s, GramParts* parts = nullptr) {
+  if (parts && nctas <= kPartCtas) {
+    *parts = {part, nctas, nout, alpha};
+    return FE_OK;
+  }
   gram_reduce_kernel<<<(unsigned)ceil_div(nout, 8), 256, 0, s>>>(part, nctas, nout, alpha, G);
   count_launch();
   FE_CUDA(cudaGetLastError());
@@ -405,7 +409,7 @@ static bool rows_pick(int tiles) {
 
 template <typename T, typename TC, int B, int L, bool UPD>
 static int launch_rows_l(const BlockSet& V, int64_t n, const double* C, double alpha, double beta, T* W,
-                         double gscale, double* G, double* scratch, size_t capacity, cudaStream_t s) {
+                         double gscale, double* G, double* scratch, size_t capacity, cudaStream_t s, GramParts* parts) {
   constexpr int NV = kRowBlocks<TC, B> * B * B;
   const size_t smem = (size_t)8 * L * NV * sizeof(double);   // above the coefficients' L (NV + pad)
   const void* fn = reinterpret_cast<const void*>(rows_kernel<T, TC, B, L, UPD>);
@@ -426,29 +430,31 @@ static int launch_rows_l(const BlockSet& V, int64_t n, const double* C, double a
   rows_kernel<T, TC, B, L, UPD><<<(unsigned)nctas, 256, smem, s>>>(V, C, alpha, beta, W, n, part);
   count_launch();
   FE_CUDA(cudaGetLastError());
-  return launch_gram_reduce(part, (int)nctas, nout, gscale, G, s);
+  return launch_gram_reduce(part, (int)nctas, nout, gscale, G, s, parts);
 }
 
 template <typename T, typename TC, int B, bool UPD>
 static int launch_rows(const BlockSet& V, int64_t n, const double* C, double alpha, double beta, T* W,
-                       double gscale, double* G, double* scratch, size_t capacity, cudaStream_t s) {
+                       double gscale, double* G, double* scratch, size_t capacity, cudaStream_t s,
+                       GramParts* parts = nullptr) {
   switch (row_lanes<TC, B>(V.nv + (UPD ? 1 : 0))) {
-    case 1: return launch_rows_l<T, TC, B, 1, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s);
-    case 2: return launch_rows_l<T, TC, B, 2, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s);
-    case 4: return launch_rows_l<T, TC, B, 4, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s);
-    default: return launch_rows_l<T, TC, B, 8, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s);
+    case 1: return launch_rows_l<T, TC, B, 1, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s, parts);
+    case 2: return launch_rows_l<T, TC, B, 2, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s, parts);
+    case 4: return launch_rows_l<T, TC, B, 4, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s, parts);
+    default: return launch_rows_l<T, TC, B, 8, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s, parts);
   }
 }
 
 // The row sweep's V^T W for blocks of one width without gaps; *done tells whether it took the call.
 template <typename T, typename TC, int B>
 static int gram_rows(const BlockSet& V, int64_t n, const T* W, int bw, int ldw, double alpha, double* G,
-                     double* scratch, size_t capacity, bool* done, cudaStream_t s) {
+                     double* scratch, size_t capacity, bool* done, cudaStream_t s, GramParts* parts = nullptr) {
   *done = false;
   if constexpr (B <= 8) {
     if (bw != B || V.bv != B || V.ld != B || ldw != B || !rows_pick<T, TC, B, false>(V.nv)) return FE_OK;
     *done = true;
-    return launch_rows<T, TC, B, false>(V, n, nullptr, 0.0, 0.0, const_cast<T*>(W), alpha, G, scratch, capacity, s);
+    return launch_rows<T, TC, B, false>(V, n, nullptr, 0.0, 0.0, const_cast<T*>(W), alpha, G, scratch, capacity, s,
+                                         parts);
   }
   return FE_OK;
 }
@@ -566,15 +572,15 @@ int gram(const BlockSet& V, int64_t n, const void* W, int bw, int ldw, fe_dtype 
 // for first-pass Gram-Schmidt coefficients, which a second FP64 pass corrects.  V blocks and W
 // are n x b with ld b.
 int gram_f32_arith(const BlockSet& V, int64_t n, const double* W, int b, double alpha, double* G,
-                   cudaStream_t s) {
+                   cudaStream_t s, GramParts* parts) {
   FE_ARG(V.nv >= 1 && V.nv <= kMaxBlocks, "gram: nv = %d out of range", V.nv);
   FE_ARG(V.bv == b, "gram: block width %d != %d", V.bv, b);
   bool done = false;
   switch (b) {
-    case 1: FE_TRY((gram_rows<double, float, 1>(V, n, W, b, b, alpha, G, nullptr, 0, &done, s))); break;
-    case 2: FE_TRY((gram_rows<double, float, 2>(V, n, W, b, b, alpha, G, nullptr, 0, &done, s))); break;
-    case 4: FE_TRY((gram_rows<double, float, 4>(V, n, W, b, b, alpha, G, nullptr, 0, &done, s))); break;
-    case 8: FE_TRY((gram_rows<double, float, 8>(V, n, W, b, b, alpha, G, nullptr, 0, &done, s))); break;
+    case 1: FE_TRY((gram_rows<double, float, 1>(V, n, W, b, b, alpha, G, nullptr, 0, &done, s, parts))); break;
+    case 2: FE_TRY((gram_rows<double, float, 2>(V, n, W, b, b, alpha, G, nullptr, 0, &done, s, parts))); break;
+    case 4: FE_TRY((gram_rows<double, float, 4>(V, n, W, b, b, alpha, G, nullptr, 0, &done, s, parts))); break;
+    case 8: FE_TRY((gram_rows<double, float, 8>(V, n, W, b, b, alpha, G, nullptr, 0, &done, s, parts))); break;
   }
   if (done) return FE_OK;
   switch (b) {
@@ -1322,7 +1328,7 @@ __global__ void __launch_bounds__(256) update_tri_gram_kernel(const BlockSet V, 
 template <typename T>
 static int launch_update_tri_gram(const BlockSet& V, int64_t n, const double* C, double alpha, double beta,
                                   const double* M, T* W, int b, const int* skip, const int* vc32, double* S,
-                                  cudaStream_t s) {
+                                  cudaStream_t s, GramParts* parts) {
   const int k = V.nv * b;
   const int threads = 256;
   const int NS = b * (b + 1) / 2;
@@ -1346,19 +1352,19 @@ static int launch_update_tri_gram(const BlockSet& V, int64_t n, const double* C,
   }
   count_launch();
   FE_CUDA(cudaGetLastError());
-  return launch_gram_reduce(part, nctas, b * b, 1.0, S, s);
+  return launch_gram_reduce(part, nctas, b * b, 1.0, S, s, parts);
 }
 
 // W = beta W M + alpha V C, S = W^T W for n x b blocks of dt, b in {1, 2, 4}, M upper triangular
 // (see update_tri_gram_kernel); S: DEVICE b x b.
 int update_tri_gram(const BlockSet& V, int64_t n, const double* C, double alpha, double beta,
                     const double* M, void* W, int b, fe_dtype dt, const int* skip, const int* vc32, double* S,
-                    cudaStream_t s) {
+                    cudaStream_t s, GramParts* parts) {
   FE_ARG(b == 1 || b == 2 || b == 4, "update_tri_gram: b = %d", b);
   FE_ARG(V.nv == 0 || (V.bv == b && V.ld == b), "update_tri_gram: blocks must be n x b");
   if (dt == FE_F64)
-    return launch_update_tri_gram<double>(V, n, C, alpha, beta, M, static_cast<double*>(W), b, skip, vc32, S, s);
-  return launch_update_tri_gram<float>(V, n, C, alpha, beta, M, static_cast<float*>(W), b, skip, nullptr, S, s);
+    return launch_update_tri_gram<double>(V, n, C, alpha, beta, M, static_cast<double*>(W), b, skip, vc32, S, s, parts);
+  return launch_update_tri_gram<float>(V, n, C, alpha, beta, M, static_cast<float*>(W), b, skip, nullptr, S, s, parts);
 }
 
 // W = beta W M + alpha V C; G = [V; W]^T W (gram_v) or W^T W, rows (j*b + p) then W's b rows.

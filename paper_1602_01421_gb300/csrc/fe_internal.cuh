@@ -113,6 +113,15 @@ int tc_combine(const BlockSet& V, int64_t n, const double* Y, int ldy, const Blo
                cudaStream_t s, double alpha = 1.0, double beta = 0.0);
 // G = alpha V^T W on the tensor cores (FP64 blocks; see tc_gram_supported for the shapes).
 bool tc_gram_supported(const BlockSet& V, int bw, int ldw, fe_dtype dt);
+// Partial sums left for the kernel that reads the Gram matrix next (p = nullptr: G is complete): where
+// the one CTA of that kernel has few to add.  At n = 2^16 (256 partials) a solve took 33.7 ms so against
+// 34.7 with a launch of its own, another at n = 2^18 (up to 1024 partials) 24.0 against 23.6.
+constexpr int kPartCtas = 320;
+struct GramParts {
+  const double* p = nullptr;   // [nctas][nout]
+  int nctas = 0, nout = 0;
+  double alpha = 0.0;
+};
 int tc_gram(const BlockSet& V, int64_t n, const double* W, int bw, double alpha, double* G,
             cudaStream_t s);
 // G[e] = alpha * sum over c < nctas of partial[c * nout + e], fixed order (deterministic).

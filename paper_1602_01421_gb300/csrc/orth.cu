@@ -31,10 +31,10 @@ int update_skip(const BlockSet& V, int64_t n, const double* C, double alpha, dou
                 const double* M, void* W, int bw, int ldw, fe_dtype dt, const int* skip,
                 cudaStream_t s);
 int gram_f32_arith(const BlockSet& V, int64_t n, const double* W, int b, double alpha, double* G,
-                   cudaStream_t s);
+                   cudaStream_t s, GramParts* parts = nullptr);
 int update_tri_gram(const BlockSet& V, int64_t n, const double* C, double alpha, double beta,
                     const double* M, void* W, int b, fe_dtype dt, const int* skip, const int* vc32,
-                    double* S, cudaStream_t s);
+                    double* S, cudaStream_t s, GramParts* parts = nullptr);
 
 constexpr double kRelPivot = 1e-6;      // pivot below 1e-6 * column norm: nearly dependent
 constexpr double kAbsBreakdown = 1e-12; // remainder below 1e-12 * ||A||: breakdown
@@ -141,6 +141,37 @@ __device__ bool chol_inv_warp(const double* S, double rel, double absthr, double
   return true;
 }
 
+// The partial sums of a Gram matrix that the kernel before left, added in gram_reduce's order (lane l of
+// a warp adds partials l, l + 32, ..; then halves) into out, which the whole CTA may read afterwards;
+// NT threads take NT / 32 outputs at a time, neighbouring outputs in neighbouring lanes.  Adding them
+// where they are used saves a launch, and at the solver's sizes a step waits for its launches (n = 2^16,
+// b = 4: 16 outputs 5.9 + 2.9 us -> 8.8, 32 outputs 1.7 + 2.9 -> 4.3, and a gap each).  Not for the
+// 144 outputs of the second pass: one SM's FP64 adds take longer than the launch (8.5 + 2.9 -> 24 us).
+constexpr int kPartThreads = 1024;   // the CTA of a kernel that starts from partial sums
+template <int NT>
+__device__ __forceinline__ void add_parts(const GramParts& g, double* out, double* sh) {
+  constexpr int W = NT / 32, LD = W + 1;
+  const int e = threadIdx.x % W, l = threadIdx.x / W, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int buf = 0;
+  for (int e0 = 0; e0 < g.nout; e0 += W, buf ^= 1) {
+    double* t = sh + buf * 32 * LD;
+    double x = 0.0;
+    if (e0 + e < g.nout) {
+#pragma unroll 8
+      for (int c = l; c < g.nctas; c += 32) x += g.p[(int64_t)c * g.nout + e0 + e];
+    }
+    t[l * LD + e] = x;
+    __syncthreads();
+    double y = t[lane * LD + warp];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) y += __shfl_xor_sync(0xffffffffu, y, off);
+    if (lane == 0 && e0 + warp < g.nout) out[e0 + warp] = g.alpha * y;
+  }
+  __syncthreads();
+}
+template <int NT>
+constexpr int kPartWords = 2 * 32 * (NT / 32 + 1);
+
 // After pass 2.  G1x = [G1; S1] ((k+B) x B), G2x = [G2; S] ((k+B) x B); k may be 0 (then
 // G2x = S).  Writes G (k x B, ldg), Racc = R1, M = R1^{-1}, C = -G2 R1^{-1}; on a failed check
 // sets *status = 1, G = G1, Racc = I.  status[1] = 1 when max |C| <= kSmallCorrection.
@@ -220,15 +251,19 @@ __global__ void __launch_bounds__(kPostThreads)
 
 // After pass 3: R2 = chol(S2); R = R2 Racc (-> Rout, ldr), M = R2^{-1}; failure -> *status = 2.
 // status[2]: R2^{-1} is the identity up to kSmallCorrection.
-template <int B>
-__global__ void __launch_bounds__(kPostThreads)
-    orth_post3_kernel(const double* __restrict__ S2, const double* __restrict__ Racc,
+template <int B, bool PARTS>
+__global__ void __launch_bounds__(PARTS ? kPartThreads : kPostThreads)
+    orth_post3_kernel(double* S2, const GramParts parts, const double* __restrict__ Racc,
                       double* __restrict__ M, double* __restrict__ Rout, int ldr, int* __restrict__ status) {
   constexpr int BB = B * B;
   __shared__ double S[BB], R1[BB], R2[BB], Ri[BB];
   __shared__ int ok;
   if (*status) return;
   const int tid = threadIdx.x;
+  if constexpr (PARTS) {
+    __shared__ double sums[kPartWords<kPartThreads>];
+    add_parts<kPartThreads>(parts, S2, sums);
+  }
   if (tid < BB) {
     S[tid] = S2[tid];
     R1[tid] = Racc[tid];
@@ -279,11 +314,15 @@ static int launch_post2(const double* G1x, const double* G2x, int k, int b, doub
   return FE_OK;
 }
 
-static int launch_post3(const double* S2, int b, const double* Racc, double* M, double* Rout, int ldr,
-                        int* status, cudaStream_t s) {
-#define POST3(B) orth_post3_kernel<B><<<1, kPostThreads, 0, s>>>(S2, Racc, M, Rout, ldr, status)
-  FE_ORTH_B(b, POST3)
+static int launch_post3(double* S2, const GramParts& parts, int b, const double* Racc, double* M, double* Rout,
+                        int ldr, int* status, cudaStream_t s) {
+#define POST3P(B) orth_post3_kernel<(B < 4 ? B : 4), true><<<1, kPartThreads, 0, s>>>(S2, parts, Racc, M, Rout, ldr, status)
+#define POST3(B) orth_post3_kernel<B, false><<<1, kPostThreads, 0, s>>>(S2, parts, Racc, M, Rout, ldr, status)
+  FE_ARG(!parts.p || b <= 4, "orth: partial sums at b = %d", b);
+  if (parts.p) FE_ORTH_B(b, POST3P)
+  else FE_ORTH_B(b, POST3)
 #undef POST3
+#undef POST3P
   count_launch();
   FE_CUDA(cudaGetLastError());
   return FE_OK;
@@ -464,8 +503,11 @@ static int orth_fallback(const BlockSet& V, int64_t n, void* W, int b, fe_dtype 
 // sG1 ((k + b) x b, rows j*b + p for block j's column p, then the b rows of S1): rows of the
 // older blocks from the known coefficients (row r, column q = known[q * ldk + r], blocks below
 // nz_first zero), the newest block's rows and S1 from the local Gram [v_last W]^T W (2b x b).
-__global__ void known_g1_kernel(double* __restrict__ sG1, int k, int b, const double* __restrict__ known,
-                                int ldk, int nz_first, const double* __restrict__ local) {
+__global__ void __launch_bounds__(kPartThreads)
+    known_g1_kernel(double* __restrict__ sG1, int k, int b, const double* __restrict__ known, int ldk,
+                    int nz_first, double* local, const GramParts parts) {
+  __shared__ double sums[kPartWords<kPartThreads>];
+  if (parts.p) add_parts<kPartThreads>(parts, local, sums);
   const int kold = k - b;
   for (int e = threadIdx.x; e < (k + b) * b; e += blockDim.x) {
     const int r = e / b, q = e - (e / b) * b;
@@ -511,11 +553,12 @@ int orth_ex(const BlockSet& V, int64_t n, void* W, int b, fe_dtype dt, double* d
     BlockSet Vl = blockset_of({V.blk[V.nv - 1], W}, b, b);
     double* sLoc = small_scratch(19, (size_t)2 * b * b);
     if (!sLoc) return FE_ERR_OOM;
+    GramParts parts;
     if (pass1_f32 && dt == FE_F64)
-      FE_TRY(gram_f32_arith(Vl, n, static_cast<const double*>(W), b, 1.0, sLoc, s));
+      FE_TRY(gram_f32_arith(Vl, n, static_cast<const double*>(W), b, 1.0, sLoc, s, &parts));
     else
       FE_TRY(gram(Vl, n, W, b, b, dt, 1.0, sLoc, s));
-    known_g1_kernel<<<1, 256, 0, s>>>(sG1, k, b, d_known, ldk, nz_first, sLoc);
+    known_g1_kernel<<<1, parts.p ? kPartThreads : 256, 0, s>>>(sG1, k, b, d_known, ldk, nz_first, sLoc, parts);
     count_launch();
     FE_CUDA(cudaGetLastError());
   } else if (pass1_f32 && dt == FE_F64) {
@@ -550,12 +593,13 @@ int orth_ex(const BlockSet& V, int64_t n, void* W, int b, fe_dtype dt, double* d
     FE_TRY(launch_post2(sG1, sG1, 0, b, d_anorm, update_anorm, d_G, ldg, sRacc, sM, sC, status, s));
   }
   // W <- (W - V G2) R1^{-1} and S2 = W^T W in one sweep (skipped after a failed pivot check)
+  GramParts s2parts;
   if (fused && b <= 4) {
     // M = R1^{-1} is upper triangular: thread-per-row sweep over its triangle, S2 = W^T W in
     // per-thread accumulators; for FP64 blocks the correction V C in FP32 arithmetic when it
     // is tiny
     FE_TRY(update_tri_gram(V, n, sC, 1.0, 1.0, sM, W, b, dt, status,
-                           (pass1_f32 && dt == FE_F64) ? status + 1 : nullptr, sS2, s));
+                           (pass1_f32 && dt == FE_F64) ? status + 1 : nullptr, sS2, s, &s2parts));
   } else if (fused) {
     // the correction V C in FP32 arithmetic when it is tiny (FP64 subspace, pass1_f32 mode)
     FE_TRY(update_gram(V, n, sC, 1.0, 1.0, sM, W, b, dt, 0, status, sS2, s,
@@ -565,7 +609,7 @@ int orth_ex(const BlockSet& V, int64_t n, void* W, int b, fe_dtype dt, double* d
     BlockSet Wonly = blockset_of({W}, b, b);
     FE_TRY(gram(Wonly, n, W, b, b, dt, 1.0, sS2, s));
   }
-  FE_TRY(launch_post3(sS2, b, sRacc, sM, d_R, ldr, status, s));
+  FE_TRY(launch_post3(sS2, s2parts, b, sRacc, sM, d_R, ldr, status, s));
   const int allow32 = (pass1_f32 && dt == FE_F64) ? 1 : 0;
   if (dt == FE_F64) FE_TRY(launch_right_mult(static_cast<double*>(W), n, b, sM, status, allow32, s));
   else FE_TRY(launch_right_mult(static_cast<float*>(W), n, b, sM, status, 0, s));

@@ -189,6 +189,23 @@ def test_combine_many_blocks_matches_oracle(prec, nv, nout, bv):
     assert np.all(np.abs(got - ref) <= rel * (np.abs(Vt) @ np.abs(Y)) + 1e-300)
 
 
+@pytest.mark.parametrize("b", [1, 2, 4])
+@pytest.mark.parametrize("n", [1, 31, 255, 257, 8193, 320 * 256, 320 * 256 + 1])
+def test_orth_partial_sums(n, b):
+    """W^T W of the last pass, added by the factorisation itself from 1 to 320 partial sums and by a
+    kernel of its own beyond: W's columns are orthonormal to 1e-13 and R is the Cholesky factor to
+    1e-11 (conditions below 1e2 times the FP64 rounding of sums of n terms)."""
+    r = np.random.default_rng(n + b)
+    b = min(b, n)   # one row: one column
+    W = r.standard_normal((n, b)) + np.eye(n, b) * 4.0
+    Wd = to_dev(W)
+    G, R, rep = fe.block_orth(None, Wd, anorm=10.0)
+    Q, want = Wd.cpu().numpy(), np.linalg.cholesky(W.T @ W).T
+    assert rep == 0
+    assert np.abs(R.cpu().numpy() - want).max() < 1e-11 * np.abs(want).max()
+    assert np.abs(Q.T @ Q - np.eye(b)).max() < 1e-13
+
+
 @pytest.mark.parametrize("n,nv,b,scale", [(5000, 3, 2, 1.0), (5000, 2, 16, 1.0), (2000, 5, 1, 1.0), (4000, 2, 4, 1e-100),
                                           (4000, 2, 4, 1e120), (4000, 2, 4, 1e-145), (4000, 0, 8, 1e145)])
 def test_orth_factorisation_widths_and_scales(n, nv, b, scale):
