@@ -48,11 +48,9 @@ NEV, BLOCK, NBLOCKS, TOL = 8, 4, 8, 1e-8
 # a run that does not converge
 MAX_RESTARTS = 5000
 NOMINAL_HBM = 8000.0
-# FP64 on GB300: 2 FP64 operations per clock per SM x 152 SMs x 2.07 GHz = 629 G/s (1.26
-# TFLOP/s counting an FMA as two); the FP64 SpMM is bound by its adds, not by HBM.
-FP64_ADD_PEAK_G = 2 * 152 * 2.07
 # dram__bytes_read.sum + dram__bytes_write.sum of one spmm_main_kernel<double,4> launch on
-# R-MAT scale 22 (ncu, the one-launch capture of `bench.py --only spmm1 --prec f64 --b 4`)
+# R-MAT scale 22 (ncu, the one-launch capture of `bench.py --only spmm1 --prec f64 --b 4`, taken
+# before the values were added as integers; the loads are the same)
 SPMM_F64_B4_DRAM_BYTES = 1455201024 + 109192192
 
 
@@ -402,20 +400,19 @@ def run_ours(args):
                               "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                               "frac": round(achieved / hbm_peak, 4), "peak_kind": peak_kind,
                               "bytes_per_launch": spmm_bytes(n, nnz, 4, es)}
-    # dominant kernel of the FP64 solve (launch list: 25.6% of the kernel time), the SpMM with an
-    # FP64 block of 4 columns; bound by FP64 adds (one per non-zero and column), reported against
-    # the nominal FP64 add rate
+    # dominant kernel of the FP64 solve, the SpMM with an FP64 block of 4 columns, against the
+    # measured copy bandwidth on compulsory bytes.  What bounds it is the rate of random gathers and
+    # the integer and FP64 adds of the gathered rows (three of four values as integers)
     t64 = sweep["f64_b4"]["ms"]
     adds = float(nnz) * 4
-    gadds = adds / (t64 / 1000.0) / 1e9
+    hbm64 = spmm_bytes(n, nnz, 4, 8) / (t64 / 1000.0) / 1e9
     roofline = {"kernel": "spmm_main_kernel<double,4> + hub_reduce_kernel (FP64 SpMM, b = 4)",
-                "bound": "alu", "achieved": round(gadds, 1), "peak": FP64_ADD_PEAK_G,
-                "unit": "G FP64 adds/s", "frac": round(gadds / FP64_ADD_PEAK_G, 4),
-                "peak_kind": "nominal FP64 add rate (2 per clock per SM x 152 SMs x 2.07 GHz)",
+                "bound": "hbm", "achieved": round(hbm64, 1), "peak": hbm_peak,
+                "unit": "GB/s", "frac": round(hbm64 / hbm_peak, 4), "peak_kind": peak_kind,
                 "traffic": SPMM_F64_B4_DRAM_BYTES if args.scale == 22 else None,
-                "adds_per_launch": adds, "bytes_per_launch": spmm_bytes(n, nnz, 4, 8),
-                "ms_per_launch": t64, "stream": "torch current stream",
-                "hbm_frac": round(spmm_bytes(n, nnz, 4, 8) / (t64 / 1000.0) / 1e9 / hbm_peak, 4)}
+                "adds_per_launch": adds, "gadds_per_s": round(adds / (t64 / 1000.0) / 1e9, 1),
+                "bytes_per_launch": spmm_bytes(n, nnz, 4, 8),
+                "ms_per_launch": t64, "stream": "torch current stream"}
     # the tensor-core split-product kernels at the solve's shapes, against HBM: the restart
     # product V Y (8 blocks of n x 4 into 5) and the second-pass Gram [V_0..V_7 W]^T W
     roofline_tc = {}

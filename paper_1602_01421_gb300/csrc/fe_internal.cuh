@@ -114,8 +114,9 @@ int tc_combine(const BlockSet& V, int64_t n, const double* Y, int ldy, const Blo
 // G = alpha V^T W on the tensor cores (FP64 blocks; see tc_gram_supported for the shapes).
 bool tc_gram_supported(const BlockSet& V, int bw, int ldw, fe_dtype dt);
 // Partial sums left for the kernel that reads the Gram matrix next (p = nullptr: G is complete): where
-// the one CTA of that kernel has few to add.  At n = 2^16 (256 partials) a solve took 33.7 ms so against
-// 34.7 with a launch of its own, another at n = 2^18 (up to 1024 partials) 24.0 against 23.6.
+// the one CTA of that kernel has few to add.  A solve at n = 2^14 (64 partials) took 34.1 ms so against
+// 35.0 with launches of their own, at n = 81,000 (317) 21.3 against 21.7, at n = 2^18 (up to 1024) 24.0
+// against 23.6.
 constexpr int kPartCtas = 320;
 struct GramParts {
   const double* p = nullptr;   // [nctas][nout]

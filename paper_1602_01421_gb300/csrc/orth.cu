@@ -144,7 +144,7 @@ __device__ bool chol_inv_warp(const double* S, double rel, double absthr, double
 // The partial sums of a Gram matrix that the kernel before left, added in gram_reduce's order (lane l of
 // a warp adds partials l, l + 32, ..; then halves) into out, which the whole CTA may read afterwards;
 // NT threads take NT / 32 outputs at a time, neighbouring outputs in neighbouring lanes.  Adding them
-// where they are used saves a launch, and at the solver's sizes a step waits for its launches (n = 2^16,
+// where they are used saves a launch, and at the solver's sizes a step waits for its launches (n = 2^14,
 // b = 4: 16 outputs 5.9 + 2.9 us -> 8.8, 32 outputs 1.7 + 2.9 -> 4.3, and a gap each).  Not for the
 // 144 outputs of the second pass: one SM's FP64 adds take longer than the launch (8.5 + 2.9 -> 24 us).
 constexpr int kPartThreads = 1024;   // the CTA of a kernel that starts from partial sums
