@@ -482,9 +482,10 @@ static size_t tc_smem_bytes(int nkc, int NP) {
 // wait that runs out marks the CTA aborted, the other roles stop at their next wait, the
 // epilogue writes NaN to the rows of the tiles it has not finished, and the TMA copies and MMAs
 // in flight are waited for (again bounded) before TMEM is freed.
-// 2^20 rows, K = 32, N = 20 (436 MB): 182 us (194 with 8 splitting and 8 assembling warps, truncating
-// 64-bit assembly and two barriers per tile); without the assembly it would take 137 us, without the
-// split as well 97 us.  (8 assembling warps: 195; half of the results converted in integers: 196.)
+// 2^20 rows, K = 32, N = 20 (436 MB): a call takes 182 us (194 with 8 splitting and 8 assembling warps,
+// truncating 64-bit assembly and two barriers per tile).  The kernel alone: 173 us; 137 without the
+// assembly, 97 without the split as well; 186 with 8 assembling warps, 187 with every other result
+// normalised in integers instead of converted.
 namespace {
 constexpr int kSplitWarps = 16, kEpiWarps = 12;
 constexpr int kEpiParts = kEpiWarps / 4;                 // epilogue threads per row
