@@ -76,11 +76,7 @@ constexpr int kMaxTailDegree = 128;
 constexpr int kDefaultTailMax = 128;
 constexpr int kDefaultTailMaxPacked = 16;  // packed plans: most rows in the compressed tasks
 constexpr int kMaxBuckets = kMaxTailDegree + 1;
-// Rayleigh-Ritz: subspaces up to kRitzOneMax are diagonalised by one cluster of 8 or
-// 16 CTAs, up to kRitzMax with FP32 sweeps on one CTA, FP64 products and cooperative FP64 sweeps
-// on the grid.
-constexpr int kRitzOneMax = 160;
-constexpr int kRitzCluster = 8, kRitzClusterMax = 16;
+// Rayleigh-Ritz: subspaces up to kRitzMax (the smaller ones on one cluster, ritz_layout.cuh).
 constexpr int kRitzMax = 512;
 struct BlockSet {
   const void* blk[kMaxBlocks];

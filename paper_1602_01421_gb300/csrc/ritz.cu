@@ -31,6 +31,7 @@
 #include <algorithm>
 
 #include "fe_internal.cuh"
+#include "ritz_layout.cuh"
 
 namespace fe {
 
@@ -282,25 +283,6 @@ __device__ __forceinline__ float ritz_rcp(float x) {
   return y;
 }
 
-// The circle method in slots: the index in slot i of a step is in slot ritz_shift(i) of the next
-// one (slot 0 stays), and pair k of a step is slots k and mp - 1 - k.  Data that moves with its
-// slot is at addresses that do not depend on the step, and after mp - 1 steps slot i holds
-// index i again.
-__device__ __forceinline__ int ritz_shift(int i, int mp) { return i == 0 ? 0 : (i == 1 ? mp - 1 : i - 1); }
-// Offset of the entry of slots a != b: the 2 x 2 block of pairs k < k2 is entry tri(k, k2) of four
-// planes (row of pair k from slot k or mp - 1 - k, column likewise); the pivots follow.
-__device__ __forceinline__ int ritz_entry(int a, int b, int mp) {
-  const int np = mp / 2, nt = np * (np - 1) / 2;
-  int ka = a < np ? a : mp - 1 - a, ra = a < np ? 0 : 1;
-  int kb = b < np ? b : mp - 1 - b, rb = b < np ? 0 : 1;
-  if (ka == kb) return 4 * nt + ka;
-  if (ka > kb) {
-    int t = ka; ka = kb; kb = t;
-    t = ra; ra = rb; rb = t;
-  }
-  return (ra * 2 + rb) * nt + ka * np - ka * (ka + 1) / 2 + kb - ka - 1;
-}
-
 // CTA 0's matrix during the sweeps, in shared memory: two copies of the entries (ritz_entry) and
 // of the diagonal by slot (unevaluated sums of two floats), and a step's (cos - 1, sin).
 struct RitzMat {
@@ -367,12 +349,11 @@ __device__ __forceinline__ void ritz_sweep(RitzMat& mt, int mp, int nact, int it
     float x[ITEMS][4];
 #pragma unroll
     for (int u = 0; u < ITEMS; ++u) {
-      const int e = item0 + u * nact;
-      const bool on = ITEMS == 1 || e < nitems;
+      const int e = ritz_read(item0 + u * nact, nitems);
       r1[u] = mt.cs[kk[u] & 0xffff];
       r2[u] = mt.cs[kk[u] >> 16];
 #pragma unroll
-      for (int v = 0; v < 4; ++v) x[u][v] = mt.n0[v * nt + (on ? e : 0)];
+      for (int v = 0; v < 4; ++v) x[u][v] = mt.n0[v * nt + e];
     }
 #pragma unroll
     for (int u = 0; u < ITEMS; ++u) {
@@ -483,14 +464,14 @@ __global__ void __launch_bounds__(512, 1)
   __shared__ int s_mode, s_done, s_more;
   float* sm = reinterpret_cast<float*>(smem_raw);
   // this thread's 2 x 2 blocks (pairs k < k2) of CTA 0's sweeps
-  const int nitems = np * (np - 1) / 2;
-  const int nact = min(nth, (max(nitems, np) + 31) & ~31);
+  const int nitems = ritz_items(np);
+  const int nact = ritz_active(np, nth);
   RitzMat mt;
   mt.cs = reinterpret_cast<float2*>(sm);
   mt.d0 = mt.cs + np;
   mt.d1 = mt.d0 + mp;
   mt.n0 = reinterpret_cast<float*>(mt.d1 + mp);
-  mt.n1 = mt.n0 + 4 * nitems + np;
+  mt.n1 = mt.n0 + ritz_copy(np);
   int to[ITEMS][2], kk[ITEMS];
 #pragma unroll
   for (int u = 0; u < ITEMS; ++u) {
@@ -758,14 +739,6 @@ __global__ void __launch_bounds__(512, 1)
     for (int p = 0; p < b; ++p) r2 += sq[k * b + p];
     rho_out[rank + k * ncta] = sqrt(r2);
   }
-}
-
-static size_t ritz_cluster_smem(int m, int b, int ncta) {
-  const size_t mp = m + (m & 1), np = mp / 2;
-  const size_t head = (2 * np + 4 * mp + 2 * (2 * np * (np - 1) + np)) * sizeof(float);
-  const size_t rows = ((mp + ncta - 3) / (ncta - 1) + 1) * mp * sizeof(float);
-  const size_t rho = std::max<size_t>(m, ceil_div(m, ncta) * b) * sizeof(double);
-  return std::max(head, std::max(rows, rho));
 }
 
 // ------------------------------------------------------------ large subspaces (m > kRitzOneMax)
@@ -1114,12 +1087,8 @@ int launch_ritz(const double* H, int m, int b, int which, int max_sweeps, double
   FE_ARG(work != nullptr, "ritz: m = %d needs a global workspace", m);
   if (m > kRitzOneMax)
     return launch_ritz_big(H, m, b, which, max_sweeps, tol, theta, Y, rho, info, work, s);
-  // FP64 products take m^3 / ncta / 2 clocks each: 16 CTAs where that outweighs the wider
-  // cluster's barriers (m = 128: 0.43 ms of products on 8, 0.22 ms on 16); threads enough for one, four or seven 2 x 2 blocks each (128 registers
-  // a thread: more threads with fewer spill)
-  const int ncta = m > 64 ? kRitzClusterMax : kRitzCluster;
-  const int variant = m <= 64 ? 0 : (m <= 128 ? 1 : 2);
-  const int threads = m <= 46 ? 256 : 512;
+  const RitzShape sh = ritz_shape(m);
+  const int ncta = sh.ncta, variant = sh.items == 1 ? 0 : (sh.items == 4 ? 1 : 2);
   auto kern = variant == 0 ? ritz_cluster_kernel<1> : (variant == 1 ? ritz_cluster_kernel<4> : ritz_cluster_kernel<7>);
   const void* fn = reinterpret_cast<const void*>(kern);
   static KernelSetup ks[3];
@@ -1132,7 +1101,7 @@ int launch_ritz(const double* H, int m, int b, int which, int max_sweeps, double
   attr[0].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ncta);
-  cfg.blockDim = dim3(threads);
+  cfg.blockDim = dim3(sh.threads);
   cfg.dynamicSmemBytes = ritz_cluster_smem(m, b, ncta);
   cfg.stream = s;
   cfg.attrs = attr;
