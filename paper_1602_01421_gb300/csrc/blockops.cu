@@ -310,13 +310,16 @@ __global__ void __launch_bounds__(256) rows_kernel(const BlockSet V, const doubl
 #pragma unroll
         for (int q = 0; q < B; ++q) a[q] += __shfl_xor_sync(kFullMask, a[q], off);
 #pragma unroll
-      for (int q = 0; q < B; ++q) w[q] = beta != 0.0 ? fma((T)beta, w[q], a[q]) : a[q];
+      for (int q = 0; q < B; ++q) {
+        w[q] = beta != 0.0 ? fma((T)beta, w[q], a[q]) : a[q];
+        if (!on) w[q] = T(0);   // past the end: an infinite coefficient made it NaN
+      }
       if (on && t == 0) st_row<T, B>(W + r * B, w);
 #pragma unroll
       for (int i = 0; i < NB; ++i)
         if (t + i * L == V.nv) {
 #pragma unroll
-          for (int p = 0; p < B; ++p) v[i][p] = on ? w[p] : T(0);
+          for (int p = 0; p < B; ++p) v[i][p] = w[p];
         }
     }
     TC wc[B];

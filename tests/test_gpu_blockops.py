@@ -270,3 +270,21 @@ def test_row_sweep_large_sums_and_infinities():
     V[1, 77, 2] = np.inf
     G = fe.block_gram(to_dev(V), to_dev(W)).cpu().numpy()
     assert np.all(np.isposinf(G[6])) and np.isfinite(G[:6]).all() and np.isfinite(G[7]).all()
+
+
+@pytest.mark.parametrize("n", [1, 33, 257, 5001])
+def test_row_sweep_infinite_coefficients(n):
+    """An infinite coefficient makes W's column infinite and with it the entries of G that W enters: rows
+    past the end of a ragged range (0 times infinity) do not turn them into NaN."""
+    r = np.random.default_rng(n)
+    V = r.random((3, n, 4)).astype(np.float32) + 0.5
+    W = r.random((n, 4)).astype(np.float32) + 0.5
+    C = r.random((12, 4))
+    C[5, 2] = np.inf
+    Wd = to_dev(W)
+    G = fe.block_update_gram(to_dev(V), to_dev(C), Wd, alpha=1.0, beta=0.5).cpu().numpy()
+    got = Wd.cpu().numpy()
+    other = [0, 1, 3]
+    assert np.all(np.isposinf(got[:, 2])) and np.isfinite(got[:, other]).all()
+    assert np.all(np.isposinf(G[:, 2])) and np.all(np.isposinf(G[14, :]))
+    assert np.isfinite(G[np.ix_([i for i in range(16) if i != 14], other)]).all()
