@@ -121,37 +121,39 @@ __device__ __forceinline__ float kahan_value(float s, float c) { return s - c; }
 __device__ __forceinline__ double kahan_value(double s, double) { return s; }
 
 // FP64 sums in integers.  An FP64 add occupies the FP64 pipe of an SM for 16 clocks per warp; the
-// 32-bit integer units take the 15 instructions of an aligned integer add in half of that, beside it.
+// 32-bit integer units take the 16 instructions of an aligned integer add in half of that, beside it.
 // So of every four gathered values one is added in FP64 and three as integers: an Fx holds
 // a * 2^((e >> 20) - 1080), e the largest biased exponent so far (in its place in the high word),
 // and a value's 53-bit significand, shifted left by 5 and right by its distance to e, is added to a.
-// Bits below 2^-57 of the largest value are dropped (floor; also from a when e rises): between two
-// flushes, 24 values (4.6 bits, so a stays within 63) and at most 8 rises of e, an error below 2^-52
-// of the largest value, no more than that of as many FP64 adds.  Values with exponents near the ends
-// of the range (infinities, NaN, below 2^-943) set `bad`, and the sums are formed again with FP64
-// adds.  Measured against FP64 adds alone (R-MAT, X 32-byte aligned): 4.2 million vertices b = 2 585
-// -> 511 us, b = 4 1085 -> 686, b = 8 2068 -> 1319, b = 16 4.18 -> 2.24 ms; a million, b = 4 288 ->
-// 162 us.  The gathers bind then (FP32 b = 8, rows of the same 32 bytes: 615 us).
+// Bits below 2^-57 of the largest value are dropped (of a value towards zero, of a, when e rises,
+// downwards): between two flushes, 24 values (4.6 bits, so a stays within 63) and at most 8 rises of
+// e, an error below 2^-52 of the largest value, no more than that of as many FP64 adds; where no bit
+// is dropped (whole numbers, say) the sum is exact.  Values with exponents near the ends of the range
+// (infinities, NaN, below 2^-943) set `bad`, and the sums are formed again with FP64 adds.  Measured
+// against FP64 adds alone (R-MAT, X 32-byte aligned): 4.2 million vertices b = 2 585 -> 520 us, b = 4
+// 1085 -> 707, b = 8 2068 -> 1352, b = 16 4.18 -> 2.34 ms; a million, b = 4 288 -> 172 us.  The gathers
+// bind then (FP32 b = 8, rows of the same 32 bytes: 615 us).
 struct Fx {
   long long a;
   unsigned e;
 };
 constexpr int kFxGroups = 8;   // groups of four values between flushes
-__device__ __forceinline__ long long fx_align(unsigned hi, unsigned lo, unsigned ev, unsigned e) {
+// t or, for sign = -1, -t - 1: fx_add3 takes the signs off again
+__device__ __forceinline__ long long fx_align(unsigned hi, unsigned lo, unsigned ev, unsigned e, int sign) {
   const unsigned m = (hi & 0xfffffu) | min(ev, 0x100000u);   // implicit bit (0 for zeros, subnormals)
   unsigned long long t = (((unsigned long long)m << 32) | lo) << 5;
   asm("shr.u64 %0, %0, %1;" : "+l"(t) : "r"((e - ev) >> 20));   // shifts of 64 and more give 0
-  const long long sign = (int)hi >> 31;
   return (long long)t ^ sign;
 }
 __device__ __forceinline__ void fx_add3(Fx& f, double x, double y, double z) {
   const unsigned hx = __double2hiint(x), hy = __double2hiint(y), hz = __double2hiint(z);
   const unsigned ex = hx & 0x7ff00000u, ey = hy & 0x7ff00000u, ez = hz & 0x7ff00000u;
   const unsigned e = max(max(ex, ey), max(ez, f.e));
+  const int sx = (int)hx >> 31, sy = (int)hy >> 31, sz = (int)hz >> 31;
   asm("shr.s64 %0, %0, %1;" : "+l"(f.a) : "r"((e - f.e) >> 20));
   f.e = e;
-  f.a += fx_align(hx, __double2loint(x), ex, e) + fx_align(hy, __double2loint(y), ey, e) +
-         fx_align(hz, __double2loint(z), ez, e);
+  f.a += fx_align(hx, __double2loint(x), ex, e, sx) + fx_align(hy, __double2loint(y), ey, e, sy) +
+         fx_align(hz, __double2loint(z), ez, e, sz) - (sx + sy + sz);
 }
 // s += f, f = 0
 __device__ __forceinline__ void fx_flush(double& s, Fx& f, bool& bad) {

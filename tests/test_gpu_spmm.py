@@ -398,3 +398,27 @@ def test_spmm_f64_special_values(b):
         Y = fe.spmm(h, to_dev(v)).cpu().numpy()
         for i, d in enumerate(degs):
             assert np.all(np.abs(Y[i] - v[:d].sum(0)) <= 518 * 2.0 ** -53 * np.abs(v[:d]).sum(0) * 2)
+
+
+@pytest.mark.parametrize("fmt", ["plain", "packed"])
+@pytest.mark.parametrize("b", [1, 2, 4, 8, 16])
+def test_spmm_f64_integers_exact(b, fmt):
+    """Whole numbers of both signs whose sums fit 53 bits come out exact, as FP64 adds give them: +-1,
+    small ones, 40-bit ones, sums that cancel, zeros of both signs, the same scaled by a power of
+    two.  Rows in the slices (12 is the first degree with integer sums), tasks on one to four warps and
+    split hub rows."""
+    r = np.random.default_rng(100 + b)
+    n = 9000
+    degs = [2, 11, 12, 13, 15, 16, 31, 32, 33, 48, 64, 65, 100, 127, 128, 129, 200, 1025, 2049, 4097, 8999] * 3
+    cols = [np.sort(r.choice(n, d, replace=False)).astype(np.int32) for d in degs]
+    rowptr = np.concatenate([[0], np.cumsum([len(c) for c in cols])]).astype(np.int64)
+    sign = np.where(r.random((n, b)) < 0.5, -1.0, 1.0)
+    alternate = np.where(np.arange(n)[:, None] % 2 == 0, 1.0, -1.0) * np.ones((1, b))
+    blocks = [sign, alternate, r.integers(-9, 10, (n, b)).astype(float),
+              r.integers(-2 ** 40, 2 ** 40, (n, b)).astype(float),
+              np.where(r.random((n, b)) < 0.5, -0.0, sign), sign * 2.0 ** -300, sign * 3.0 * 2.0 ** 400]
+    with fe.Csr(rowptr, np.concatenate(cols), ncols=n, index_format=fmt) as h:
+        for k, X in enumerate(blocks):
+            Y = fe.spmm(h, to_dev(X)).cpu().numpy()
+            want = np.array([[float(v) for v in X[c].astype(np.longdouble).sum(0)] for c in cols])
+            assert np.array_equal(Y, want), k
