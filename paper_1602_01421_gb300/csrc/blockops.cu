@@ -223,47 +223,74 @@ int gram_reduce(const double* partial, int nctas, int nout, double alpha, double
 // ---------------------------------------------------------------- row sweeps
 // G = alpha V^T W, or (UPD) W = beta W + alpha V C and then G = [V; W]^T W, for blocks of one width
 // B in one sweep over the rows: L lanes hold a row, lane t of them blocks t, t + L, .. (at most NB;
-// UPD: index nv is W itself) with their B x B output tiles in registers for the whole launch.
-// A row of V is loaded once, all blocks of it before the first use; an update sums its L partial
-// results by shuffles, so nothing of the sweep goes through shared memory but C.  Every lane's sums
-// are reduced over the warp by a scatter (each level halves what a lane holds) and over the CTA once,
-// at the end: cross-thread sums in FP64, or, for FP32 sums, as unevaluated pairs of floats (TwoSum;
-// 48 bits), because FP64 adds of 8 * NB * B * B values per warp would take as long as the sweep.
+// UPD: index nv is W itself) with their B x B output tiles in registers.  A row of V is loaded once,
+// all blocks of it before the first use; an update sums its L partial results by shuffles, so nothing
+// of the sweep itself goes through shared memory but C.
+// FP64 sums stay in the lanes for the whole launch; at the end the warp's lanes add them by a scatter
+// (each level halves what a lane holds).  FP32 sums leave the lanes at the end or after kRowRun rows:
+// they are added over the warp's lanes, 32 entries at a time through shared memory, as unevaluated pairs
+// of floats (TwoSum; 48 bits), because the FP64 adds of 8 * NB * B * B values per warp would take as
+// long as the sweep.  Entries whose sums could leave FP32's range (kPairMax; infinities and NaN among
+// them) are added in FP64 instead.
 // Loads of V and W rows bound it in FP32 and the FP64 pipe in FP64 (rows_pick has the figures).
 template <typename TC, int B>
 constexpr int kRowBlocks = B >= 8 ? (sizeof(TC) == 4 ? 2 : 1) : (B == 4 ? 4 : 8);   // NB
 constexpr int kRowLanesMax = 8;
 
-template <typename TC>
-struct RowSum {   // s + e
-  TC s, e;
+// Rows per lane that an FP32 sum runs over (0: all of them).  The kernels with a warp per tile reduce
+// the shapes that their registers do not hold after every range (update + Gram of b = 8 or of more than
+// 16 tiles: 8 rows per lane; Gram of b = 8 and more than 4 blocks: 16, of more than 16 blocks of 4: 32);
+// a sum here runs no longer.  4.2 million rows, 8 blocks of 8, update + Gram: V^T W off by 7.1e-9 of its
+// norm with one sum per launch (1.04 ms), by 2.4e-10 with sums of 8 rows (1.39 ms).
+template <int B, int L, bool UPD>
+constexpr int kRowRun = UPD ? (B == 8 || L * kRowBlocks<float, B> > 16 ? 8 : 0)
+                            : (B == 8 ? (L > 2 ? 16 : 0) : (L * kRowBlocks<float, B> > 16 ? 32 : 0));
+// Resident CTAs to compile for.  Narrow blocks wait for their loads: update + Gram of b = 1, 20 blocks, 4.2
+// million rows 277 us with two CTAs, 214 with three, 153 with four, 183 with six; of b = 2, 60 blocks (L = 8)
+// 1285 us with two, 1008 with three, but 20 blocks (L = 4) 263 and 311; Gram of b = 2, 15 blocks 126 and 109.
+template <typename T, typename TC, int B, int L>
+constexpr int kRowCtas = sizeof(TC) == 8 || B > 4 ? 1 : (B == 1 ? 4 : (B == 2 && L != 4 && sizeof(T) == 4 ? 3 : 2));
+constexpr float kPairMax = 7.9228163e28f;   // 2^96
+
+// Dynamic shared memory: lanes' coefficients, the warps' FP64 sums [8][L * NV] by output and, for
+// FP32 sums, their pairs [8][L * NV] by lane and the entries on their way [8][CH * 32].
+template <typename T, typename TC, int B, int L, bool UPD>
+struct RowSmem {
+  static constexpr bool kPairs = sizeof(TC) == 4, kRuns = kPairs && kRowRun<B, L, UPD> > 0;
+  static constexpr int NV = kRowBlocks<TC, B> * B * B, RW = 32 / L, CNT = NV / RW, CH = NV < 32 ? NV : 32;
+  static_assert(CH >= RW, "an entry for every lane");
+  static constexpr int STRIDE = NV + 16 / (int)sizeof(T);   // of a lane's coefficients: other banks
+  static constexpr int SUMS = UPD ? (L * STRIDE * (int)sizeof(T) + 15) / 16 * 16 : 0;
+  static constexpr int PAIRS = SUMS + 8 * L * NV * (int)sizeof(double);
+  static constexpr int STAGE = PAIRS + (kRuns ? 8 * L * NV * (int)sizeof(float2) : 0);
+  static constexpr int TOTAL = STAGE + (kPairs ? 8 * CH * 32 * (int)sizeof(float) : 0);
 };
-__device__ __forceinline__ void row_add(RowSum<float>& a, RowSum<float> b) {
-  const float t = a.s + b.s, z = t - a.s;
-  a.e += b.e + ((a.s - (t - z)) + (b.s - z));
-  a.s = t;
-}
-__device__ __forceinline__ void row_add(RowSum<double>& a, RowSum<double> b) { a.s += b.s; }
-__device__ __forceinline__ RowSum<float> row_shfl(RowSum<float> a, int off) {
-  return {__shfl_xor_sync(kFullMask, a.s, off), __shfl_xor_sync(kFullMask, a.e, off)};
-}
-__device__ __forceinline__ RowSum<double> row_shfl(RowSum<double> a, int off) {
-  return {__shfl_xor_sync(kFullMask, a.s, off), 0.0};
-}
 
 template <typename T, typename TC, int B, int L, bool UPD>
-__global__ void __launch_bounds__(256) rows_kernel(const BlockSet V, const double* __restrict__ C,
-                                                   double alpha, double beta, T* W, int64_t n,
-                                                   double* __restrict__ partial) {
-  constexpr int NB = kRowBlocks<TC, B>, BB = B * B, RW = 32 / L;
-  constexpr int kStride = NB * BB + 16 / (int)sizeof(T);   // of a lane's coefficients: other banks
+__global__ void __launch_bounds__(256, (kRowCtas<T, TC, B, L>))
+    rows_kernel(const BlockSet V, const double* __restrict__ C, double alpha, double beta, T* W, int64_t n,
+                double* __restrict__ partial) {
+  using S = RowSmem<T, TC, B, L, UPD>;
+  constexpr int NB = kRowBlocks<TC, B>, BB = B * B, RW = S::RW, NV = S::NV, CNT = S::CNT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sC = reinterpret_cast<T*>(smem_raw);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = lane / RW;
+  double* sums = reinterpret_cast<double*>(smem_raw + S::SUMS);
+  double* own = sums + warp * L * NV;
+  float2* pairs = reinterpret_cast<float2*>(smem_raw + S::PAIRS) + warp * L * NV + lane;
+  // output of entry f of the lane's sums
+  auto place = [&](int f) { return (t + f / BB * L) * BB + f % BB; };
+  if constexpr (S::kRuns) {
+#pragma unroll
+    for (int i = 0; i < CNT; ++i) {
+      pairs[i * 32] = make_float2(0.f, 0.f);
+      own[i * 32 + lane] = 0.0;
+    }
+  }
   if constexpr (UPD) {
     for (int e = threadIdx.x; e < L * NB * BB; e += blockDim.x) {
       const int j = e / BB;   // block j: lane j % L, its j / L-th
-      sC[j % L * kStride + j / L * BB + e % BB] = j < V.nv ? (T)(alpha * C[e]) : T(0);
+      sC[j % L * S::STRIDE + j / L * BB + e % BB] = j < V.nv ? (T)(alpha * C[e]) : T(0);
     }
     __syncthreads();
   }
@@ -272,118 +299,160 @@ __global__ void __launch_bounds__(256) rows_kernel(const BlockSet V, const doubl
 #pragma unroll
   for (int i = 0; i < NB; ++i)
     vp[i] = t + i * L < V.nv ? reinterpret_cast<const T*>(V.blk[t + i * L]) : nullptr;
-  TC acc[NB][B][B];
+  TC acc[NV];
 #pragma unroll
-  for (int i = 0; i < NB; ++i)
+  for (int e = 0; e < NV; ++e) acc[e] = TC(0);
+  // FP32: the lanes' sums to the warp's.  Lane l of a row group takes entries l, l + RW, .. of every CH and
+  // adds the group's lanes in order; entry e of lane k lies at k ^ (e % RW), a bank for every l.
+  auto flush = [&]() {
+    if constexpr (S::kPairs) {
+      float* stage = reinterpret_cast<float*>(smem_raw + S::STAGE) + warp * S::CH * 32;
+      const int l = lane % RW;
 #pragma unroll
-    for (int p = 0; p < B; ++p)
+      for (int c0 = 0; c0 < NV; c0 += S::CH) {
+        __syncwarp();
 #pragma unroll
-      for (int q = 0; q < B; ++q) acc[i][p][q] = TC(0);
-  for (int64_t base = ((int64_t)blockIdx.x * 8 + warp) * RW; base < n; base += (int64_t)gridDim.x * 8 * RW) {
-    const int64_t r = base + lane % RW;
-    const bool on = r < n;
-    T v[NB][B], w[B];
-#pragma unroll
-    for (int i = 0; i < NB; ++i) {
-#pragma unroll
-      for (int p = 0; p < B; ++p) v[i][p] = T(0);
-      if (on && vp[i]) ld_row<T, B>(vp[i] + r * B, v[i]);
-    }
-#pragma unroll
-    for (int q = 0; q < B; ++q) w[q] = T(0);
-    if (on && (!UPD || beta != 0.0)) ld_row_rw<T, B>(W + r * B, w);
-    if constexpr (UPD) {
-      const T* c = sC + t * kStride;
-      T a[B];
-#pragma unroll
-      for (int q = 0; q < B; ++q) a[q] = T(0);
-#pragma unroll
-      for (int i = 0; i < NB; ++i)
-        if (i * L < V.nv) {
-#pragma unroll
-          for (int p = 0; p < B; ++p)
-#pragma unroll
-            for (int q = 0; q < B; ++q) a[q] = fma(v[i][p], c[(i * B + p) * B + q], a[q]);
+        for (int e = 0; e < S::CH; ++e) {
+          stage[e * 32 + (lane ^ e % RW)] = acc[c0 + e];
+          acc[c0 + e] = TC(0);
         }
+        __syncwarp();
 #pragma unroll
-      for (int off = RW; off < 32; off <<= 1)
+        for (int i = 0; i < S::CH / RW; ++i) {
+          const float* x = stage + (i * RW + l) * 32 + t * RW;
+          float s = 0.f, e = 0.f;
+          if constexpr (S::kRuns) {
+            const float2 p = pairs[(c0 / RW + i) * 32];
+            s = p.x;
+            e = p.y;
+          }
 #pragma unroll
-        for (int q = 0; q < B; ++q) a[q] += __shfl_xor_sync(kFullMask, a[q], off);
-#pragma unroll
-      for (int q = 0; q < B; ++q) {
-        w[q] = beta != 0.0 ? fma((T)beta, w[q], a[q]) : a[q];
-        if (!on) w[q] = T(0);   // past the end: an infinite coefficient made it NaN
-      }
-      if (on && t == 0) st_row<T, B>(W + r * B, w);
-#pragma unroll
-      for (int i = 0; i < NB; ++i)
-        if (t + i * L == V.nv) {
-#pragma unroll
-          for (int p = 0; p < B; ++p) v[i][p] = w[p];
-        }
-    }
-    TC wc[B];
-#pragma unroll
-    for (int q = 0; q < B; ++q) wc[q] = to_arith<TC>(w[q]);
-#pragma unroll
-    for (int i = 0; i < NB; ++i)
-      if (i * L < tiles) {
-#pragma unroll
-        for (int p = 0; p < B; ++p) {
-          const TC x = to_arith<TC>(v[i][p]);
-#pragma unroll
-          for (int q = 0; q < B; ++q) acc[i][p][q] = fma(x, wc[q], acc[i][p][q]);
+          for (int k = 0; k < RW; ++k) {
+            const float y = x[k ^ l], u = s + y, z = u - s;
+            e += (s - (u - z)) + (y - z);
+            s = u;
+          }
+          double& o = own[place(c0 + i * RW + l)];
+          if (!(fabsf(s) + fabsf(e) < kPairMax)) {
+            double z = 0.0;
+            for (int k = 0; k < RW; ++k) z += (double)x[k ^ l];
+            if constexpr (S::kRuns) o += z;
+            else o = z;
+          } else if constexpr (S::kRuns) {
+            pairs[(c0 / RW + i) * 32] = make_float2(s, e);
+          } else {
+            o = (double)s + (double)e;
+          }
         }
       }
-  }
-  // over the rows of the warp
-  constexpr int NV = NB * BB;
-  constexpr TC kScale = sizeof(TC) == 4 ? TC(0.015625) : TC(1);   // pairs of floats: 32 of any size add up
-  RowSum<TC> x[NV];
+    }
+  };
+  const int64_t step = (int64_t)gridDim.x * 8 * RW;
+  int64_t base = ((int64_t)blockIdx.x * 8 + warp) * RW;
+  auto rows = [&](int64_t stop) {
+    for (; base < stop; base += step) {
+      const int64_t r = base + lane % RW;
+      const bool on = r < n;
+      T v[NB][B], w[B];
 #pragma unroll
-  for (int e = 0; e < NV; ++e) x[e] = {acc[e / BB][e / B % B][e % B] * kScale, TC(0)};
-  int first = 0, cnt = NV;
+      for (int i = 0; i < NB; ++i) {
 #pragma unroll
-  for (int off = RW / 2; off >= 1; off >>= 1) {
-    const bool up = (lane & off) != 0;
-    const int h = cnt / 2;
-    if (h >= 1) {
+        for (int p = 0; p < B; ++p) v[i][p] = T(0);
+        if (on && vp[i]) ld_row<T, B>(vp[i] + r * B, v[i]);
+      }
+#pragma unroll
+      for (int q = 0; q < B; ++q) w[q] = T(0);
+      if (on && (!UPD || beta != 0.0)) ld_row_rw<T, B>(W + r * B, w);
+      if constexpr (UPD) {
+        const T* c = sC + t * S::STRIDE;
+        T a[B];
+#pragma unroll
+        for (int q = 0; q < B; ++q) a[q] = T(0);
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+          if (i * L < V.nv) {
+#pragma unroll
+            for (int p = 0; p < B; ++p)
+#pragma unroll
+              for (int q = 0; q < B; ++q) a[q] = fma(v[i][p], c[(i * B + p) * B + q], a[q]);
+          }
+#pragma unroll
+        for (int off = RW; off < 32; off <<= 1)
+#pragma unroll
+          for (int q = 0; q < B; ++q) a[q] += __shfl_xor_sync(kFullMask, a[q], off);
+#pragma unroll
+        for (int q = 0; q < B; ++q) {
+          w[q] = beta != 0.0 ? fma((T)beta, w[q], a[q]) : a[q];
+          if (!on) w[q] = T(0);   // past the end: an infinite coefficient made it NaN
+        }
+        if (on && t == 0) st_row<T, B>(W + r * B, w);
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+          if (t + i * L == V.nv) {
+#pragma unroll
+            for (int p = 0; p < B; ++p) v[i][p] = w[p];
+          }
+      }
+      TC wc[B];
+#pragma unroll
+      for (int q = 0; q < B; ++q) wc[q] = to_arith<TC>(w[q]);
+#pragma unroll
+      for (int i = 0; i < NB; ++i)
+        if (i * L < tiles) {
+#pragma unroll
+          for (int p = 0; p < B; ++p) {
+            const TC x = to_arith<TC>(v[i][p]);
+#pragma unroll
+            for (int q = 0; q < B; ++q) acc[(i * B + p) * B + q] = fma(x, wc[q], acc[(i * B + p) * B + q]);
+          }
+        }
+    }
+  };
+  if constexpr (S::kRuns) {
+    while (base < n) {
+      rows(n - base > kRowRun<B, L, UPD> * step ? base + kRowRun<B, L, UPD> * step : n);
+      flush();
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < CNT; ++i) {
+      const float2 p = pairs[i * 32];
+      own[place(i * RW + lane % RW)] += (double)p.x + (double)p.y;
+    }
+  } else if constexpr (S::kPairs) {
+    rows(n);
+    flush();
+  } else {
+    rows(n);
+    int first = 0;   // the lane's entries after the scatter
+#pragma unroll
+    for (int off = RW / 2, h = NV / 2; off >= 1; off >>= 1, h >>= 1) {
+      const bool up = (lane & off) != 0;
 #pragma unroll
       for (int i = 0; i < NV / 2; ++i)
         if (i < h) {
-          const RowSum<TC> send = up ? x[i] : x[i + h];
-          x[i] = up ? x[i + h] : x[i];
-          row_add(x[i], row_shfl(send, off));
+          const TC send = up ? acc[i] : acc[i + h];
+          acc[i] = (up ? acc[i + h] : acc[i]) + __shfl_xor_sync(kFullMask, send, off);
         }
-      if (up) first += h;
-      cnt = h;
-    } else {
-      row_add(x[0], row_shfl(x[0], off));
+      first += up ? h : 0;
     }
+#pragma unroll
+    for (int i = 0; i < CNT; ++i) own[place(first + i)] = (double)acc[i];
   }
   // over the warps of the CTA
-  __syncthreads();
-  double* red = reinterpret_cast<double*>(smem_raw);   // [8][L * NV]
-#pragma unroll
-  for (int i = 0; i < NV; ++i)
-    if (i < cnt) {
-      const double z = (double)x[i].s + (double)x[i].e;   // e is NaN where s is infinite
-      const int f = first + i;
-      red[warp * L * NV + (t + f / BB * L) * BB + f % BB] = (z == z ? z : (double)x[i].s) * (1.0 / (double)kScale);
-    }
   __syncthreads();
   const int nout = tiles * BB;
   for (int e = threadIdx.x; e < nout; e += blockDim.x) {
     double s = 0.0;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) s += red[k * L * NV + e];
+    for (int k = 0; k < 8; ++k) s += sums[k * L * NV + e];
     partial[(int64_t)blockIdx.x * nout + e] = s;
   }
 }
 
 // Lanes per row: as few as hold the blocks.
 template <typename TC, int B>
-static int row_lanes(int tiles) {
+constexpr int row_lanes(int tiles) {
   int l = 1;
   while (l * kRowBlocks<TC, B> < tiles) l *= 2;
   return l;
@@ -391,30 +460,31 @@ static int row_lanes(int tiles) {
 
 // Whether the row sweep takes `tiles` blocks.  It is faster than the kernels with a warp per tile
 // (gram_kernel, update_gram_kernel) where loads bind: FP32 at b = 4 and 8 always (4.2 million rows, 7
-// blocks of 4: Gram 175 -> 109 us, update and Gram 263 -> 148 us; 31 blocks at 200003 rows 98 -> 42 and
-// 224 -> 52 us), narrower FP32 blocks for Grams of b = 2 and for updates of more than 16 tiles, which
+// blocks of 4: Gram 185 -> 120 us, update and Gram 267 -> 152 us; 8 blocks of 8
+// 1.92 -> 0.43 and 6.37 -> 1.39 ms; 31 blocks of 4, a million rows 320 -> 175 us and 1010 -> 222 us), narrower FP32 blocks for Grams of b = 2 and for updates of more than 16 tiles, which
 // the other kernel reduces after every range.  In FP64, the FMAs bind: it pays where the lanes' blocks
 // divide evenly (idle slots are issued all the same) and the other kernel's tiles do not fit its
 // registers (b = 8: 8 blocks, a million rows 1745 -> 893 us) or are more than 16 (31 blocks of 4: Gram
 // 1289 -> 896 us, update and Gram 2602 -> 2042 us).
+template <typename TC, int B, bool UPD>
+constexpr int kRowTilesMin = sizeof(TC) == 4   // the fewest and most tiles ever picked; 0: none are
+                                 ? (B >= 4 ? 1 : (UPD ? 17 : (B == 2 ? 1 : 0)))
+                                 : (B == 8 ? 1 : (UPD ? (B == 4 ? 17 : 0) : (B == 4 ? 1 : 17)));
+template <typename TC, int B, bool UPD>
+constexpr int kRowTilesMax = sizeof(TC) == 4 && B == 2 && !UPD ? 16 : kRowBlocks<TC, B> * kRowLanesMax;
 template <typename T, typename TC, int B, bool UPD>
 static bool rows_pick(int tiles) {
-  if (tiles > kRowBlocks<TC, B> * kRowLanesMax) return false;
-  if (sizeof(TC) == 4) {
-    if (B >= 4) return true;
-    return UPD ? tiles > 16 : (B == 2 && tiles <= 16);
-  }
+  if (tiles < kRowTilesMin<TC, B, UPD> || tiles > kRowTilesMax<TC, B, UPD>) return false;
+  if (sizeof(TC) == 4) return true;
   const int l = row_lanes<TC, B>(tiles), slots = (tiles + l - 1) / l * l;
   if (B == 8) return 3 * slots <= 4 * tiles;
-  if (UPD) return B == 4 && tiles > 16;
-  return tiles > 16 || (B == 4 && 10 * slots <= 11 * tiles);
+  return tiles > 16 || 10 * slots <= 11 * tiles;
 }
 
 template <typename T, typename TC, int B, int L, bool UPD>
 static int launch_rows_l(const BlockSet& V, int64_t n, const double* C, double alpha, double beta, T* W,
                          double gscale, double* G, double* scratch, size_t capacity, cudaStream_t s, GramParts* parts) {
-  constexpr int NV = kRowBlocks<TC, B> * B * B;
-  const size_t smem = (size_t)8 * L * NV * sizeof(double);   // above the coefficients' L (NV + pad)
+  const size_t smem = RowSmem<T, TC, B, L, UPD>::TOTAL;
   const void* fn = reinterpret_cast<const void*>(rows_kernel<T, TC, B, L, UPD>);
   static KernelSetup ks;
   FE_TRY(kernel_configure(ks, fn, (int)smem));
@@ -440,12 +510,17 @@ template <typename T, typename TC, int B, bool UPD>
 static int launch_rows(const BlockSet& V, int64_t n, const double* C, double alpha, double beta, T* W,
                        double gscale, double* G, double* scratch, size_t capacity, cudaStream_t s,
                        GramParts* parts = nullptr) {
-  switch (row_lanes<TC, B>(V.nv + (UPD ? 1 : 0))) {
-    case 1: return launch_rows_l<T, TC, B, 1, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s, parts);
-    case 2: return launch_rows_l<T, TC, B, 2, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s, parts);
-    case 4: return launch_rows_l<T, TC, B, 4, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s, parts);
-    default: return launch_rows_l<T, TC, B, 8, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s, parts);
-  }
+  constexpr int LMIN = row_lanes<TC, B>(kRowTilesMin<TC, B, UPD>), LMAX = row_lanes<TC, B>(kRowTilesMax<TC, B, UPD>);
+#define FE_ROWS_L(L)                                                                                            \
+  if constexpr (L >= LMIN && L <= LMAX)                                                                         \
+    if (row_lanes<TC, B>(V.nv + (UPD ? 1 : 0)) == L)                                                            \
+      return launch_rows_l<T, TC, B, L, UPD>(V, n, C, alpha, beta, W, gscale, G, scratch, capacity, s, parts);
+  FE_ROWS_L(1)
+  FE_ROWS_L(2)
+  FE_ROWS_L(4)
+  FE_ROWS_L(8)
+#undef FE_ROWS_L
+  return set_error(FE_ERR_INVALID, "internal: %d blocks of %d in a row sweep", V.nv, B);
 }
 
 // The row sweep's V^T W for blocks of one width without gaps; *done tells whether it took the call.
@@ -453,7 +528,7 @@ template <typename T, typename TC, int B>
 static int gram_rows(const BlockSet& V, int64_t n, const T* W, int bw, int ldw, double alpha, double* G,
                      double* scratch, size_t capacity, bool* done, cudaStream_t s, GramParts* parts = nullptr) {
   *done = false;
-  if constexpr (B <= 8) {
+  if constexpr (B <= 8 && kRowTilesMin<TC, B, false> > 0) {
     if (bw != B || V.bv != B || V.ld != B || ldw != B || !rows_pick<T, TC, B, false>(V.nv)) return FE_OK;
     *done = true;
     return launch_rows<T, TC, B, false>(V, n, nullptr, 0.0, 0.0, const_cast<T*>(W), alpha, G, scratch, capacity, s,
@@ -1219,8 +1294,9 @@ template <typename T, int BV, int BW>
 static int launch_update_gram(const BlockSet& V, int64_t n, const double* C, double alpha,
                               double beta, const double* M, T* W, int gram_v, const int* skip,
                               const int* vc32, double* G, cudaStream_t s) {
-  if (gram_v && !M && !skip && !vc32 && rows_pick<T, T, BW, true>(V.nv + 1))
-    return launch_rows<T, T, BW, true>(V, n, C, alpha, beta, W, 1.0, G, nullptr, 0, s);
+  if constexpr (kRowTilesMin<T, BW, true> > 0)
+    if (gram_v && !M && !skip && !vc32 && rows_pick<T, T, BW, true>(V.nv + 1))
+      return launch_rows<T, T, BW, true>(V, n, C, alpha, beta, W, 1.0, G, nullptr, 0, s);
   constexpr int NR = BV > BW ? BV : BW;
   constexpr int kRegsPerTile = NR * BW * (int)(sizeof(T) / 4);
   const int gblocks = gram_v ? V.nv + 1 : 1;

@@ -288,3 +288,28 @@ def test_row_sweep_infinite_coefficients(n):
     assert np.all(np.isposinf(got[:, 2])) and np.isfinite(got[:, other]).all()
     assert np.all(np.isposinf(G[:, 2])) and np.all(np.isposinf(G[14, :]))
     assert np.isfinite(G[np.ix_([i for i in range(16) if i != 14], other)]).all()
+
+
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -62, 2.0 ** 56])
+@pytest.mark.parametrize("b,nv,n", [(8, 8, 1 << 20), (8, 15, 600011), (8, 2, 1 << 21), (4, 31, 1 << 21), (4, 16, 1 << 20),
+                                    (2, 20, 1 << 21), (2, 60, 600011), (1, 20, 1 << 21), (1, 60, 1 << 20)])
+def test_row_sweep_long_sums(b, nv, n, scale):
+    """FP32 sums of the shapes that a launch does not keep in one accumulator run over 8 rows (update +
+    Gram of b = 8 or more than 16 tiles), 16 (Gram of b = 8, more than 4 blocks) or 32 (more than 16 blocks
+    of 4): whatever n, the error is at most that many units of 2^-24, and one for the rest, which is as
+    good as FP64.  The two constants' products round the same way in every addition: a sum of 200 is
+    48 units off.  Also with products near the smallest normal number (2^-122) and with sums that leave
+    FP32's range (2^113 each)."""
+    t = __import__("torch")
+    v, w = np.float32(1.4888460636138916), np.float32(1.9886953830718994)
+    V = t.full((nv, n, b), float(v) * scale, dtype=t.float32, device="cuda")
+    W = t.full((n, b), float(w) * scale, dtype=t.float32, device="cuda")
+    vw, ww = n * float(v) * float(w) * scale ** 2, n * float(w) ** 2 * scale ** 2
+    u = 2.0 ** -24
+    G = fe.block_update_gram(V, t.zeros(nv * b, b, dtype=t.float64, device="cuda"), W, alpha=1.0, beta=1.0).cpu().numpy()
+    assert np.abs(G[:nv * b] / vw - 1).max() <= 9 * u and np.abs(G[nv * b:] / ww - 1).max() <= 9 * u
+    assert np.array_equal(G[nv * b:], G[nv * b:].T)
+    run = 16 if b == 8 and nv > 4 else 32 if b == 4 and nv > 16 else 0
+    if run:
+        G = fe.block_gram(V, W, engine="fma").cpu().numpy()
+        assert np.abs(G / vw - 1).max() <= (run + 1) * u
