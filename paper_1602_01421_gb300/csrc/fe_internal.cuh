@@ -228,6 +228,7 @@ struct PlanView {
   const void* tasks;
   int64_t ntasks, nhub_tasks;
   int64_t wide4, wide2;    // plan_wide
+  int tail_max;
   const int32_t* slice_rows;
   const int32_t* ell;
   int64_t nslices;

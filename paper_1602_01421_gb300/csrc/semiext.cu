@@ -270,6 +270,7 @@ int semiext_spmm(fe_csr h, const void* X, void* Y, int b, fe_dtype dt, cudaStrea
     v.ntasks = pi.ntasks;
     v.nhub_tasks = pi.nhub_tasks;
     v.x_rows = h->ncols;
+    v.tail_max = h->plan.tail_max;
     v.wide4 = pi.wide4;
     v.wide2 = pi.wide2;
     v.slice_rows = reinterpret_cast<const int32_t*>(base + pi.off_slice_rows);

@@ -170,6 +170,11 @@ __device__ __forceinline__ void fx_flush(double& s, Fx& f, bool& bad) {
 // (b = 4 at 4.2 million vertices: 950 us with four columns a lane, 80 registers).
 template <typename T, int B, bool V32>
 constexpr int kColLanes = V32 || B * sizeof(T) <= 16 || (sizeof(T) == 8 && !kUseFx<T, B>) ? 1 : B * (int)sizeof(T) / 16;
+// Plans with shorter slice rows than this (packed ones, by default 16) take FP64 adds at b = 2: most of their
+// tasks are rows of few entries a lane, whose flushes cost more than the adds, and a packed task's decoding
+// takes the integer units too (packed, 4.2 million vertices: 813 us with FP64 adds, 1042 with Fx; a million 209
+// and 258).  By tail_max, so that both index formats of one split give the same sums.
+constexpr int kFxTailMax = 64;
 constexpr int kFxMinDegree = 12;   // slices of shorter rows: the flush would cost more than it saves
 
 // Gap field k (w bits) of a packed task's bit stream.
@@ -181,7 +186,7 @@ __device__ __forceinline__ int gap_field(const uint32_t* __restrict__ tb, int k,
 
 // Task ti on W warps of the CTA (this one takes piece `piece`); W > 1: all warps of the CTA call it
 // (ti past the range: nothing to do but the barriers).
-template <typename T, int B, bool V32, bool PACKED, int W>
+template <typename T, int B, bool V32, bool PACKED, bool FX, int W>
 __device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, int64_t tend, const T* __restrict__ X,
                                          T* __restrict__ Y, T* __restrict__ partial, int warp, int lane, T* red) {
   using G = Geo<T, B, V32>;
@@ -272,7 +277,7 @@ __device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, int64_
       }
     }
   };
-  if constexpr (kUseFx<T, B>) {
+  if constexpr (FX) {
     constexpr int PER = 32 / G::P, NG = G::UNROLL * PER;   // gathers of a lane per 32 columns, per round
     const int carry0 = carry;
     Fx fa[G::NE];
@@ -359,7 +364,7 @@ __device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, int64_
 }
 
 // Warp `wi` of the slices.
-template <typename T, int B, bool V32>
+template <typename T, int B, bool V32, bool FX>
 __device__ __forceinline__ void run_slice(const SpmmParams& p, unsigned wi, const T* __restrict__ X,
                                           T* __restrict__ Y, int lane) {
   constexpr int SC = kColLanes<T, B, V32>, K = B / SC;   // lanes per row for its columns, columns of each
@@ -382,7 +387,7 @@ __device__ __forceinline__ void run_slice(const SpmmParams& p, unsigned wi, cons
   const int len = ((deg + pieces - 1) / pieces + 3) & ~3;    // steps of a piece
   const int t1 = min(deg, (piece + 1) * len);
   int row = -1;
-  if constexpr (!kUseFx<T, B>) row = __ldcs(p.slice_rows + si * 32 + srow);
+  if constexpr (!FX) row = __ldcs(p.slice_rows + si * 32 + srow);
   T acc[K], cmp[K];
 #pragma unroll
   for (int q = 0; q < K; ++q) acc[q] = cmp[q] = T(0);
@@ -408,7 +413,7 @@ __device__ __forceinline__ void run_slice(const SpmmParams& p, unsigned wi, cons
     for (; t < t1; ++t) add_row(__ldcs(e + t * 32));
   };
   bool done = false;
-  if constexpr (kUseFx<T, B>) {
+  if constexpr (FX) {
     if (deg >= kFxMinDegree) {
       Fx fa[K];
       bool bad = false;
@@ -448,7 +453,7 @@ __device__ __forceinline__ void run_slice(const SpmmParams& p, unsigned wi, cons
   if (!done) plain(piece * len);
 #pragma unroll
   for (int q = 0; q < K; ++q) acc[q] = kahan_value(acc[q], cmp[q]);
-  if constexpr (kUseFx<T, B>) row = __ldcs(p.slice_rows + si * 32 + srow);   // late: one register less
+  if constexpr (FX) row = __ldcs(p.slice_rows + si * 32 + srow);   // late: one register less
   T* y = Y + (int64_t)row * B + cl * K;
   if (pieces == 1) {
     if (row >= 0) st_row<T, K>(y, acc);
@@ -484,25 +489,28 @@ __device__ __forceinline__ void run_slice(const SpmmParams& p, unsigned wi, cons
 
 template <typename T, int B>
 constexpr bool kWide = B * sizeof(T) >= 32 && !kUseFx<T, B>;
-// Resident CTAs to compile for.
-template <typename T, int B, bool V32>
-constexpr int kMinCtas = kUseFx<T, B> ? 5 : (B * sizeof(T) <= 16 ? 8 : (B == 8 ? 5 : (V32 ? 3 : 7)));
-template <typename T, int B, bool V32, bool PACKED>
-__global__ void __launch_bounds__(256, (kMinCtas<T, B, V32>)) spmm_main_kernel(const SpmmParams p, const T* __restrict__ X,
-                                                        T* __restrict__ Y, T* __restrict__ partial) {
+// Resident CTAs to compile for.  Packed tasks decode besides: FP32 b = 4 spills 144 bytes at 8 CTAs, 24 at
+// 6 (4.2 million vertices 879 and 801 us, a million 216 and 192).
+template <typename T, int B, bool V32, bool PACKED, bool FX>
+constexpr int kMinCtas = FX ? 5
+                         : B * sizeof(T) <= 16 ? (PACKED && sizeof(T) == 4 && B == 4 ? 6 : 8)
+                                               : (B == 8 ? 5 : (V32 ? 3 : 7));
+template <typename T, int B, bool V32, bool PACKED, bool FX>
+__global__ void __launch_bounds__(256, (kMinCtas<T, B, V32, PACKED, FX>))
+    spmm_main_kernel(const SpmmParams p, const T* __restrict__ X, T* __restrict__ Y, T* __restrict__ partial) {
   __shared__ T red[kWarpsPerCta * B];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t cta = blockIdx.x;
   if (cta < p.ctas4) {
-    run_task<T, B, V32, PACKED, 4>(p, cta * 2 + warp / 4, p.wide4, X, Y, partial, warp, lane, red);
+    run_task<T, B, V32, PACKED, FX, 4>(p, cta * 2 + warp / 4, p.wide4, X, Y, partial, warp, lane, red);
   } else if (cta < p.ctas2) {
-    run_task<T, B, V32, PACKED, 2>(p, p.wide4 + (cta - p.ctas4) * 4 + warp / 2, p.wide2, X, Y, partial, warp, lane, red);
+    run_task<T, B, V32, PACKED, FX, 2>(p, p.wide4 + (cta - p.ctas4) * 4 + warp / 2, p.wide2, X, Y, partial, warp, lane, red);
   } else if (cta < p.task_ctas) {
     const int64_t ti = p.wide2 + (cta - p.ctas2) * kWarpsPerCta + warp;
-    if (ti < p.ntasks) run_task<T, B, V32, PACKED, 1>(p, ti, p.ntasks, X, Y, partial, warp, lane, red);
+    if (ti < p.ntasks) run_task<T, B, V32, PACKED, FX, 1>(p, ti, p.ntasks, X, Y, partial, warp, lane, red);
   } else {
     const unsigned wi = (unsigned)(cta - p.task_ctas) * kWarpsPerCta + warp;
-    if (wi < p.bucket_warp_begin[p.nbuckets]) run_slice<T, B, V32>(p, wi, X, Y, lane);
+    if (wi < p.bucket_warp_begin[p.nbuckets]) run_slice<T, B, V32, FX>(p, wi, X, Y, lane);
   }
 }
 
@@ -618,9 +626,13 @@ static int launch_spmm(const PlanView& pv, const T* X, T* Y, T* partial, cudaStr
     void (*kern)(const SpmmParams, const T*, T*, T*) = nullptr;
     if (v32) {
       if constexpr (kWide<T, B>)
-        kern = pv.packed ? spmm_main_kernel<T, B, true, true> : spmm_main_kernel<T, B, true, false>;
+        kern = pv.packed ? spmm_main_kernel<T, B, true, true, false> : spmm_main_kernel<T, B, true, false, false>;
     } else {
-      kern = pv.packed ? spmm_main_kernel<T, B, false, true> : spmm_main_kernel<T, B, false, false>;
+      constexpr bool FX = kUseFx<T, B>;
+      kern = pv.packed ? spmm_main_kernel<T, B, false, true, FX> : spmm_main_kernel<T, B, false, false, FX>;
+      if constexpr (FX && B == 2)
+        if (pv.tail_max < kFxTailMax)
+          kern = pv.packed ? spmm_main_kernel<T, B, false, true, false> : spmm_main_kernel<T, B, false, false, false>;
     }
     if (pv.l2_persist) {
       // L2 access-policy window on X: its lines are kept (persisting) while the streamed index
@@ -668,6 +680,7 @@ PlanView resident_view(fe_csr h) {
   v.tasks = pl.d_tasks;
   v.ntasks = pl.ntasks;
   v.nhub_tasks = pl.nhub_tasks;
+  v.tail_max = pl.tail_max;
   v.wide4 = pl.wide4;
   v.wide2 = pl.wide2;
   v.slice_rows = pl.d_slice_rows;

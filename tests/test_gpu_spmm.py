@@ -422,3 +422,24 @@ def test_spmm_f64_integers_exact(b, fmt):
             Y = fe.spmm(h, to_dev(X)).cpu().numpy()
             want = np.array([[float(v) for v in X[c].astype(np.longdouble).sum(0)] for c in cols])
             assert np.array_equal(Y, want), k
+
+
+@pytest.mark.parametrize("tail_max", [8, 63, 64, 128])
+def test_spmm_f64_b2_split(tail_max):
+    """FP64 b = 2 on both sides of the rule that chooses plain adds or integer sums by the plan's
+    tail_max: both index formats of one split agree bit for bit, and either is within the interface's
+    bound (518 * 2^-53 of A|X|, the sums in extended precision)."""
+    r = np.random.default_rng(tail_max)
+    n = 6000
+    degs = [1, 7, 8, 9, 12, 30, 63, 64, 65, 127, 128, 129, 500, 1025, 2049, 5000] * 3
+    cols = [np.sort(r.choice(n, d, replace=False)).astype(np.int32) for d in degs]
+    rowptr = np.concatenate([[0], np.cumsum([len(c) for c in cols])]).astype(np.int64)
+    X = r.standard_normal((n, 2))
+    Y = []
+    for fmt in ("plain", "packed"):
+        with fe.Csr(rowptr, np.concatenate(cols), ncols=n, index_format=fmt, tail_max=tail_max) as h:
+            Y.append(fe.spmm(h, to_dev(X)).cpu().numpy())
+    assert np.array_equal(Y[0], Y[1])
+    for i, c in enumerate(cols):
+        ref, mag = X[c].astype(np.longdouble).sum(0), np.abs(X[c]).astype(np.longdouble).sum(0)
+        assert np.all(np.abs(Y[0][i] - ref) <= 518 * 2.0 ** -53 * mag)
