@@ -184,10 +184,13 @@ int fe_csr_get_info(fe_csr h, fe_csr_info* info);
  *         of at most 5 levels, and the chunks of a split hub row are added in compensated
  *         FP64 and rounded once, so |error| <= 9 * 2^-24 * (A|X|)_ij (about 5.4e-7, plus
  *         terms of order degree * 2^-48);
- *   FP64: |error| <= (m + 6) * 2^-53 * (A|X|)_ij, m the longest run one lane adds: m <= tail_max
+ *   FP64: |error| <= (m + 9) * 2^-53 * (A|X|)_ij, m the longest run one lane adds: m <= tail_max
  *         for rows in the slices, m <= 512 for longer rows (1024 at b = 16), so below 6e-14
- *         (1.2e-13).  For b > 1 three of four values are added as 64-bit integers aligned to
- *         the run's largest exponent, which keeps 57 bits below it, the others in FP64.
+ *         (1.2e-13).  The 9 are the tree over the lanes (5), a row's or chunk's four warps (3) and a
+ *         split hub row's compensated sum and rounding (2), less the run's first addition.  For b > 1
+ *         three of four values are added as 64-bit integers aligned to the run's largest exponent,
+ *         which keeps 57 bits below it (exact where no bits are lost, as for whole numbers), the
+ *         others in FP64; b = 2 with tail_max below 64 adds all in FP64.
  * Both pointers must be 16-byte aligned.  Errors: FE_ERR_INVALID (null/unaligned pointer, unsupported b),
  * FE_ERR_CUDA, FE_ERR_TIMEOUT (semi-external copy wait).  Asynchronous when resident.
  */

@@ -22,7 +22,7 @@
 // indices are stored either as int32 or, in the packed format, as per-task gap fields that a
 // warp decodes with a prefix sum (fewer bytes to stream from host memory).
 // FP32 sums are compensated per lane (Kahan) before the lane tree, and the warps of a shared task
-// and hub chunks are added in FP64, so the FP32 error bound (9 * 2^-24 * A|X| per entry) does not grow with the
+// and (compensated) hub chunks are added in FP64, so the FP32 error bound (9 * 2^-24 * A|X| per entry) does not grow with the
 // degree or depend on the signs of X.
 #include <stdio.h>
 #include <string.h>
@@ -514,22 +514,22 @@ __global__ void __launch_bounds__(256, (kMinCtas<T, B, V32, PACKED, FX>))
   }
 }
 
-// s + e <- (s + e) + x exactly up to the rounding of e (Neumaier 1974: the TwoSum error of every
-// add is collected separately).
+// s + e <- (s + e) + x exactly up to the rounding of e (Neumaier 1974: the error of every add is
+// collected separately).  The larger one by the high words: equal ones have one exponent, which is all
+// that the error's formula needs, and the FP64 pipe is spared a comparison.
 __device__ __forceinline__ void neumaier_add(double& s, double& e, double x) {
   const double u = s + x;
-  e += fabs(s) >= fabs(x) ? (s - u) + x : (x - u) + s;
+  const bool up = (__double2hiint(x) & 0x7fffffff) > (__double2hiint(s) & 0x7fffffff);
+  const double a = up ? x : s, b = up ? s : x;
+  e += (a - u) + b;
   s = u;
 }
 
-// Y[hub_rows[h]] = sum of the hub's task partials in FP64, then one rounding to T.  One warp per
-// hub row: lane l adds column l % B of tasks l / B, l / B + 32 / B, .. in order, then the lanes of a
-// column are added in a fixed tree (R-MAT with 2^20 vertices, FP32 b = 4: 8.4 us with a thread per
-// entry over all of a row's partials, 2.4 us now).  Plain adds while a lane has at most kPlainPartials of them (their
-// error is then below 69 * 2^-53, less than a lane's run of a long row may have; FP64 adds are
-// what the kernel's time is made of), compensated ones above, so that the error does not grow with
-// the degree.
-constexpr int kPlainPartials = 64;
+// Y[hub_rows[h]] = sum of the hub's task partials in compensated FP64, then one rounding to T: an error
+// of about 2^-53 |sum| + O(k 2^-106) sum |partial| for any number k of partials, so a hub adds one
+// rounding to its chunks' errors.  One warp per hub row: lane l adds column l % B of tasks l / B, l / B +
+// 32 / B, .. in order, then the lanes of a column are added in a fixed tree (R-MAT with 2^20 vertices,
+// FP32 b = 4: 8.4 us with a thread per entry over all of a row's partials, 3.1 us now).
 template <typename T, int B>
 __global__ void __launch_bounds__(256) hub_reduce_kernel(const int32_t* __restrict__ hub_rows,
                                                          const int32_t* __restrict__ hub_task_begin,
@@ -541,21 +541,14 @@ __global__ void __launch_bounds__(256) hub_reduce_kernel(const int32_t* __restri
   const int t0 = hub_task_begin[h], t1 = hub_task_begin[h + 1];
   const T* src = partial + (int64_t)t0 * B + lane;   // task t0 + slot, column c
   const int steps = (t1 - t0 - slot + 32 / B - 1) / (32 / B);
-  double s = 0.0, e = 0.0;
-  if (t1 - t0 <= kPlainPartials * (32 / B)) {
+  double s = steps > 0 ? (double)src[0] : 0.0, e = 0.0;
 #pragma unroll 4
-    for (int t = 0; t < steps; ++t) s += (double)src[t * 32];
+  for (int t = 1; t < steps; ++t) neumaier_add(s, e, (double)src[(int64_t)t * 32]);
 #pragma unroll
-    for (int off = B; off < 32; off <<= 1) s += __shfl_xor_sync(kFull, s, off);
-  } else {
-#pragma unroll 4
-    for (int t = 0; t < steps; ++t) neumaier_add(s, e, (double)src[(int64_t)t * 32]);
-#pragma unroll
-    for (int off = B; off < 32; off <<= 1) {
-      const double s2 = __shfl_xor_sync(kFull, s, off), e2 = __shfl_xor_sync(kFull, e, off);
-      neumaier_add(s, e, s2);
-      e += e2;
-    }
+  for (int off = B; off < 32; off <<= 1) {
+    const double s2 = __shfl_xor_sync(kFull, s, off), e2 = __shfl_xor_sync(kFull, e, off);
+    neumaier_add(s, e, s2);
+    e += e2;
   }
   // an infinite partial makes the error term NaN: the plain sum is the result then
   const double r = s + e;

@@ -443,3 +443,25 @@ def test_spmm_f64_b2_split(tail_max):
     for i, c in enumerate(cols):
         ref, mag = X[c].astype(np.longdouble).sum(0), np.abs(X[c]).astype(np.longdouble).sum(0)
         assert np.all(np.abs(Y[0][i] - ref) <= 518 * 2.0 ** -53 * mag)
+
+
+@pytest.mark.parametrize("fmt", ["plain", "packed"])
+@pytest.mark.parametrize("b", [1, 2, 4, 8])
+def test_spmm_f64_hub_chunks(b, fmt):
+    """A hub row of many small chunks, 64 for every lane that adds them: their sum is compensated and adds
+    no more than its rounding, whatever their number.  The interface's bound, (m + 9) 2^-53 of A|X| with
+    at most m = 64 / (32 / max(1, b / 2)) entries a lane in a chunk of 64, on a constant whose chunk sums round
+    the same way in every addition (plain adds of 64 of them are 16 units off)."""
+    c, ncols, chunks = float.fromhex("0x1.f1e4b2c84ce60p+0"), 4096, 64 * (32 // b)
+    m = 64 // (32 // max(1, b // 2))
+    deg = 64 * chunks
+    cols = np.sort(np.arange(deg) % ncols).astype(np.int32)
+    rowptr = np.array([0, deg, deg + 3], dtype=np.int64)
+    X = np.full((ncols, b), c)
+    with fe.Csr(rowptr, np.concatenate([cols, np.arange(3, dtype=np.int32)]), ncols=ncols, hub_min=128, hub_chunk=64,
+                index_format=fmt) as h:
+        assert h.info()["hub_chunks"] == chunks
+        Y = fe.spmm(h, to_dev(X)).cpu().numpy()
+    want = deg * np.longdouble(c)
+    assert np.all(np.abs(Y[0] - want) <= (m + 9) * 2.0 ** -53 * want)
+    assert np.all(np.abs(Y[1] - 3 * np.longdouble(c)) <= 3 * 2.0 ** -53 * 3 * c)
