@@ -382,10 +382,10 @@ __global__ void __launch_bounds__(kThr, 2) mlp_stats_kernel(const float* __restr
     const int rows = (int)min((int64_t)kTile, n - r0);
     for (int e = threadIdx.x; e < rows * B; e += kThr) {
       const int r = e % rows, j = e / rows;
-      zd[j * LDD + r] = f32_to_f64_flush(sm[S::Z + j * kLd + r]);
+      zd[j * LDD + r] = f32_to_f64(sm[S::Z + j * kLd + r]);
     }
     for (int e = threadIdx.x; e < rows * NU; e += kThr)
-      ud[(e % NU) * LDD + e / NU] = f32_to_f64_flush(U[r0 * NU + e]);
+      ud[(e % NU) * LDD + e / NU] = f32_to_f64(U[r0 * NU + e]);
     __syncthreads();
     if (sl < SL) {
       double a = 0.0;

@@ -109,6 +109,11 @@ __device__ __forceinline__ double f32_to_f64_flush(float f) {
   return __longlong_as_double((long long)bits);
 }
 
+// The same with subnormal inputs exact too (by the conversion instruction, where there are any).
+__device__ __forceinline__ double f32_to_f64(float f) {
+  return (__float_as_uint(f) & 0x7f800000u) != 0u ? f32_to_f64_flush(f) : (double)f;
+}
+
 // Conversion of a block element to the Gram's arithmetic type: FP64 -> FP32 by integer
 // truncation (f64_to_f32_trunc), otherwise a plain cast.
 template <typename TC, typename T>

@@ -202,3 +202,24 @@ def test_row_tiles(form, n, hidden, b, t):
         term2 = ((2 * s / q * U64) ** 2 + (2 * s ** 2 / q ** 2 * Zo) ** 2).sum(1)
     slack = 8 * 2.0 ** -24 * np.sqrt((term2 * gain2).sum())
     assert np.linalg.norm(grad - go) <= 1e-4 * np.linalg.norm(go) + slack
+
+
+
+def test_loss_of_subnormal_outputs():
+    """Network outputs below FP32's normal range enter the FP64 loss statistics with their values: the
+    loss is that of the outputs as the forward pass gives them, to the rounding of 300 FP64 terms (1e-12)."""
+    n, hidden, b = 300, 64, 4
+    t_ = torch()
+    r = np.random.default_rng(11)
+    F = np.abs(r.standard_normal((n, omlp.NFEAT))).astype(np.float32)
+    p = learned.init_params(hidden, b, seed=5)
+    Z = omlp.forward(F.astype(np.float64), p.astype(np.float64), hidden, b)[0]
+    U = (Z / np.linalg.norm(Z, axis=0) + 0.2 * r.standard_normal((n, b)) / np.sqrt(n)).astype(np.float32)
+    p[-(hidden * b + b):] *= np.float32(2.0 ** -132)
+    F, p, Ud = to_dev(F, t_.float32), to_dev(p, t_.float32), to_dev(U, t_.float32)
+    Z = fe.mlp_forward(F, p, hidden, b).cpu().numpy()
+    assert (np.abs(Z) < 2.0 ** -126).all() and (Z != 0).any()
+    Z = Z.astype(np.float64)
+    want = b - ((Z * U.astype(np.float64)).sum(0) ** 2 / (Z ** 2).sum(0)).sum()
+    L, _ = fe.mlp_loss_grad(F, p, hidden, b, Ud)
+    assert want < 0.9 * b and abs(L - want) < 1e-12
