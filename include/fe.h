@@ -415,7 +415,8 @@ typedef struct {
                              b = block), for FE_START_LEARNED; features use `seed` */
   int mlp_hidden;         /* hidden width of that MLP: 32 or 64 (64) */
   double mixed_tol;       /* FP32-phase tolerance in mixed mode (5e-6) */
-  int max_sweeps;         /* Jacobi sweeps per Rayleigh-Ritz (60) */
+  int max_sweeps;         /* Jacobi sweeps per Rayleigh-Ritz after the FP32 ones that start it (15
+                             up to subspace 160, 20 above): they bring FP32 accuracy to FP64 (60) */
   int orth_pass1;         /* FP64 subspace, first Gram-Schmidt pass: 0 = its Gram in FP32
                              arithmetic (the FP64 second pass restores full orthogonality, and
                              the coefficients actually subtracted enter H, so the Krylov

@@ -501,7 +501,7 @@ __global__ void __launch_bounds__(512, 1)
   ritz_cluster_sync();
   double *Q = w.Q, *Qn = w.Q2, *d = w.d0, *dprev = w.d1;
   float fro = 0.f, dmax = 0.f, isc = 1.f;
-  int sweeps = 0, done = 0, it = 0;
+  int sweeps = 0, left = max_sweeps, done = 0, it = 0;
   for (;; ++it) {
     // ---- FP32: E, the rotation that diagonalises D + N (CTA 0; rows of E in the others)
     if (rank == 0) {
@@ -538,8 +538,9 @@ __global__ void __launch_bounds__(512, 1)
       }
       nu = ritz_block_max(nu, red);
       emax = ritz_block_max(emax, red);
-      // late iterations only repair orthogonality: rotations that are not tiny are left out
-      const bool first_order = it > 0 && (emax <= kTinyAngle || it >= kRitzMaxIter - 2);
+      // late iterations, and those after the last sweep allowed, only repair orthogonality: rotations
+      // that are not tiny are left out
+      const bool first_order = it > 0 && (emax <= kTinyAngle || it >= kRitzMaxIter - 2 || left == 0);
       if (tid == 0) {
         w.ctl[0] = 0u;
         w.ctl[1] = first_order ? 1u : 0u;
@@ -549,7 +550,7 @@ __global__ void __launch_bounds__(512, 1)
         ritz_cluster_sync();
       } else {
         const float skip = fmaxf(it == 0 ? 2e-8f * fro : 1e-7f * nu, 1e-17f * fro);
-        const int cap = it == 0 ? min(15, max_sweeps) : 6;
+        const int cap = ritz_sweep_cap(it, left);
         for (int s = 0; s < cap; ++s) {
           float ps = 0.f, tm = 0.f;
           if (tid < nact)
@@ -562,6 +563,7 @@ __global__ void __launch_bounds__(512, 1)
                                   : ritz_block_max(tm, red);
           const bool more = s + 1 < cap && v > (it == 0 ? 1e-8f * fro * fro : 1e-4f);
           ++sweeps;
+          if (it > 0) --left;
           if (tid == 0) w.ctl[3 + (s & 1)] = more ? 1u : 0u;
           if (!more)
             for (int i = tid; i < mp; i += nth) d[i] = (double)mt.d0[i].x + (double)mt.d0[i].y;

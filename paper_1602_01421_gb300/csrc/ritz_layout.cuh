@@ -21,6 +21,13 @@ inline RitzShape ritz_shape(int m) {
   return {m > 64 ? kRitzClusterMax : kRitzCluster, m <= 64 ? 1 : (m <= 128 ? 4 : 7), m <= 46 ? 256 : 512};
 }
 
+// Most sweeps of iteration `it`: kRitzFirstSweeps FP32 ones of the projected matrix itself, then, over all later
+// iterations, as many as the caller's max_sweeps (`left` of them are left), at most six at a time.
+constexpr int kRitzFirstSweeps = 15;
+__host__ __device__ __forceinline__ int ritz_sweep_cap(int it, int left) {
+  return it == 0 ? kRitzFirstSweeps : (left < 6 ? left : 6);
+}
+
 // 2 x 2 blocks (pairs k < k2 of np), and the threads that take part in a sweep.
 __host__ __device__ __forceinline__ int ritz_items(int np) { return np * (np - 1) / 2; }
 __host__ __device__ __forceinline__ int ritz_active(int np, int threads) {

@@ -28,5 +28,14 @@ int main() {
     printf("%d %d %d %d %d %d %ld %zu %d\n", m, sh.threads, nact, sh.items, top, ritz_copy(np), end,
            ritz_cluster_smem(m, 1, sh.ncta), once && (size_t)mp * (mp - 1) / 2 == hit.size() ? 1 : 0);
   }
+  for (int max_sweeps : {1, 2, 5, 6, 7, 60}) {   // "sweeps max_sweeps: first, then all later ones" if every cap is used
+    int left = max_sweeps, later = 0;
+    for (int it = 1; it < 40; ++it) {
+      const int cap = ritz_sweep_cap(it, left);
+      later += cap;
+      left -= cap;
+    }
+    printf("sweeps %d %d %d\n", max_sweeps, ritz_sweep_cap(0, max_sweeps), later);
+  }
   return 0;
 }

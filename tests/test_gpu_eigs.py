@@ -274,3 +274,31 @@ def test_rayleigh_ritz_sizes(fam, b, nb):
     assert np.abs(lam[:, None] - ev[None, :]).min(axis=0).max() < 2e-9 * scale
     assert abs(ev[0] - lam[-1]) < 2e-9 * scale
     _check_pairs(g, ev, to_dev(X), 1e-9, scale)
+
+
+def _eigs_few_sweeps(h, nev, b, nb, tol, max_sweeps):
+    """fe_eigs_ex with the option that the Python function leaves at its default."""
+    import ctypes
+    from paper_1602_01421_gb300 import _lib
+    o = _lib.EigsOpts()
+    fe.load().fe_eigs_opts_default(ctypes.byref(o))
+    o.seed, o.max_restarts, o.max_sweeps = 2, 4000, max_sweeps
+    ev = np.zeros(nev)
+    X = __import__("torch").empty((nev, h.n), dtype=__import__("torch").float64, device="cuda")
+    _lib.check(fe.load().fe_eigs_ex(h.handle, nev, b, nb, tol, _lib.WHICH["LA"], ctypes.byref(o),
+                                    ev.ctypes.data_as(ctypes.c_void_p), ctypes.c_void_p(X.data_ptr()), None))
+    return ev, X.t().cpu().numpy()
+
+
+@pytest.mark.parametrize("max_sweeps", [1, 2])
+@pytest.mark.parametrize("b,nb", [(1, 5), (4, 8), (4, 24), (4, 40)])
+def test_rayleigh_ritz_few_sweeps(b, nb, max_sweeps):
+    """Few sweeps allowed after the FP32 ones: the pairs pass the same tests, also where the projected
+    matrix has multiple eigenvalues."""
+    g = graphgen.hypercube(8) if b == 4 else graphgen.erdos_renyi(700, 12.0, seed=9)
+    lam = np.linalg.eigvalsh(g.dense())
+    with fe.Csr.from_graph(g) as h:
+        ev, X = _eigs_few_sweeps(h, 3, b, nb, 1e-9, max_sweeps)
+    assert np.abs(X.T @ X - np.eye(3)).max() < 1e-12
+    assert np.abs(lam[:, None] - ev[None, :]).min(axis=0).max() < 2e-9 * np.abs(lam).max()
+    assert abs(ev[0] - lam[-1]) < 2e-9 * np.abs(lam).max()
