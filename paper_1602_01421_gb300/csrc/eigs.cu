@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "fe_internal.cuh"
+#include "ritz_layout.cuh"
 
 namespace fe {
 
@@ -40,7 +41,7 @@ int orth_ex(const BlockSet& V, int64_t n, void* W, int b, fe_dtype dt, double* d
             double* d_R, int ldr, int* replaced, cudaStream_t s, int pass1_f32, int engine,
             const double* d_known = nullptr, int ldk = 0, int nz_first = 0);
 int launch_ritz(const double* H, int m, int b, int which, int max_sweeps, double tol,
-                double* theta, double* Y, double* rho, int* info, double* work, cudaStream_t s);
+                double* theta, double* Y, double* rho, int* info, double* work, bool grid, cudaStream_t s);
 size_t ritz_work_doubles(int m);
 int launch_restart_h(double* H, int m, int b, int k, const double* theta, const double* Y,
                      cudaStream_t s);
@@ -158,16 +159,16 @@ struct Phase {
     FE_TRY(small.alloc(sizeof(double) * (nritz + nsmall)));
     ritzwork = small.as<double>();
     Y = ritzwork + nritz;
-    theta = Y + (size_t)m * m;   // theta, rho and anorm: read back as one
+    theta = Y + (size_t)m * m;   // theta, rho, anorm and info: read back as one
     rho = theta + m;
     anorm = rho + m;
+    info = reinterpret_cast<int*>(anorm + 1);
     Cdiag = anorm + 4;
     gtmp = Cdiag + 256;
-    info = reinterpret_cast<int*>(gtmp + 64 * 16);
     if (op_ata) FE_TRY(opbuf.alloc(blk));
     theta_h.resize(m);
     rho_h.resize(m);
-    back_h.resize(2 * (size_t)m + 1);
+    back_h.resize(2 * (size_t)m + 2);
     resid_h.assign(nev, 0.0);
     return FE_OK;
   }
@@ -235,10 +236,19 @@ struct Phase {
 
   // Ritz values/vectors of the current H, convergence estimate; returns nconv
   int ritz(int* nconv_out) {
-    FE_TRY(launch_ritz(H, m, b, which, max_sweeps, 1e-15, theta, Y, rho, info,
-                       ritzwork, s));
-    FE_CUDA(cudaMemcpyAsync(back_h.data(), theta, sizeof(double) * (2 * (size_t)m + 1), cudaMemcpyDeviceToHost, s));
-    FE_CUDA(cudaStreamSynchronize(s));
+    // a projected matrix that the one-cluster kernel leaves unfinished (info -1) goes to the sweeps on
+    // the grid; what max_sweeps leaves of those is used as it is
+    for (int grid = 0; grid < 2; ++grid) {
+      FE_TRY(launch_ritz(H, m, b, which, max_sweeps, 1e-15, theta, Y, rho, info, ritzwork, grid != 0, s));
+      FE_CUDA(cudaMemcpyAsync(back_h.data(), theta, sizeof(double) * back_h.size(), cudaMemcpyDeviceToHost, s));
+      FE_CUDA(cudaStreamSynchronize(s));
+      int sweeps = 0;
+      memcpy(&sweeps, &back_h[2 * (size_t)m + 1], sizeof(sweeps));
+      if (sweeps < -1) return set_error(FE_ERR_TIMEOUT, "ritz: a grid barrier timed out (m = %d)", m);
+      if (trace_on() && sweeps < 0)
+        fprintf(stderr, "[fe] ritz m=%d restart %d: not converged%s\n", m, restarts, grid ? " on the grid" : "");
+      if (sweeps >= 0 || m > kRitzOneMax) break;
+    }
     theta_h.assign(back_h.begin(), back_h.begin() + m);
     rho_h.assign(back_h.begin() + m, back_h.begin() + 2 * m);
     const double an = back_h[2 * (size_t)m];

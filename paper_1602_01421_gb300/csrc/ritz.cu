@@ -787,8 +787,8 @@ __host__ __device__ inline BigWork big_work(double* w, int m) {
 }
 
 size_t ritz_work_doubles(int m) {
-  if (m <= kRitzOneMax) return ritz_cluster_doubles(m);
-  return 5 * big_mat_doubles(m) + 4 + kCoopCtas + 8;
+  const size_t grid = 5 * big_mat_doubles(m) + 4 + kCoopCtas + 8;
+  return m <= kRitzOneMax ? std::max(ritz_cluster_doubles(m), grid) : grid;
 }
 
 // 1. FP32 sweeps (one CTA) and the FP64 copies of T and Q32.
@@ -1083,11 +1083,13 @@ static int launch_ritz_big(const double* H, int m, int b, int which, int max_swe
   return FE_OK;
 }
 
+// info[0]: the sweeps run, -1 where the projected matrix is not diagonal to tol, -2 after a barrier that timed
+// out.  grid: the sweeps on the grid whatever m is (m <= kRitzOneMax: the second attempt after a -1).
 int launch_ritz(const double* H, int m, int b, int which, int max_sweeps, double tol,
-                double* theta, double* Y, double* rho, int* info, double* work, cudaStream_t s) {
+                double* theta, double* Y, double* rho, int* info, double* work, bool grid, cudaStream_t s) {
   FE_ARG(m >= 1 && m <= kRitzMax, "ritz: subspace m = %d not in [1, %d]", m, kRitzMax);
   FE_ARG(work != nullptr, "ritz: m = %d needs a global workspace", m);
-  if (m > kRitzOneMax)
+  if (grid || m > kRitzOneMax)
     return launch_ritz_big(H, m, b, which, max_sweeps, tol, theta, Y, rho, info, work, s);
   const RitzShape sh = ritz_shape(m);
   const int ncta = sh.ncta, variant = sh.items == 1 ? 0 : (sh.items == 4 ? 1 : 2);

@@ -276,16 +276,16 @@ def test_rayleigh_ritz_sizes(fam, b, nb):
     _check_pairs(g, ev, to_dev(X), 1e-9, scale)
 
 
-def _eigs_few_sweeps(h, nev, b, nb, tol, max_sweeps):
+def _eigs_few_sweeps(h, nev, b, nb, tol, max_sweeps, max_restarts=4000, which="LA"):
     """fe_eigs_ex with the option that the Python function leaves at its default."""
     import ctypes
     from paper_1602_01421_gb300 import _lib
     o = _lib.EigsOpts()
     fe.load().fe_eigs_opts_default(ctypes.byref(o))
-    o.seed, o.max_restarts, o.max_sweeps = 2, 4000, max_sweeps
+    o.seed, o.max_restarts, o.max_sweeps = 2, max_restarts, max_sweeps
     ev = np.zeros(nev)
     X = __import__("torch").empty((nev, h.n), dtype=__import__("torch").float64, device="cuda")
-    _lib.check(fe.load().fe_eigs_ex(h.handle, nev, b, nb, tol, _lib.WHICH["LA"], ctypes.byref(o),
+    _lib.check(fe.load().fe_eigs_ex(h.handle, nev, b, nb, tol, _lib.WHICH[which], ctypes.byref(o),
                                     ev.ctypes.data_as(ctypes.c_void_p), ctypes.c_void_p(X.data_ptr()), None))
     return ev, X.t().cpu().numpy()
 
@@ -302,3 +302,20 @@ def test_rayleigh_ritz_few_sweeps(b, nb, max_sweeps):
     assert np.abs(X.T @ X - np.eye(3)).max() < 1e-12
     assert np.abs(lam[:, None] - ev[None, :]).min(axis=0).max() < 2e-9 * np.abs(lam).max()
     assert abs(ev[0] - lam[-1]) < 2e-9 * np.abs(lam).max()
+
+
+def test_unfinished_rayleigh_ritz_is_noticed():
+    """Two sweeps after the FP32 ones do not finish the projected matrices of the hypercube with 1024
+    vertices (multiplicities up to 252) at subspace 64: the solver sees that, and hands them to the
+    sweeps on the grid.  The trace says so (in a process of its own: it is switched on at the start)."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    code = ("import graphgen, paper_1602_01421_gb300 as fe; from tests.test_gpu_eigs import _eigs_few_sweeps\n"
+            "with fe.Csr.from_graph(graphgen.hypercube(10)) as h:\n"
+            "    try: _eigs_few_sweeps(h, 3, 8, 8, 1e-9, 2, 12, 'LM')\n"
+            "    except Exception: pass\n")
+    out = subprocess.run([sys.executable, "-c", code], cwd=root, env={**os.environ, "FE_TRACE": "1"},
+                         capture_output=True, text=True, timeout=300).stderr
+    assert "nconv" in out and "ritz m=64" in out and ": not converged\n" in out
