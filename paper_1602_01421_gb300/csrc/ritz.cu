@@ -29,6 +29,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <mutex>
 
 #include "fe_internal.cuh"
 #include "ritz_layout.cuh"
@@ -1091,25 +1092,43 @@ int launch_ritz(const double* H, int m, int b, int which, int max_sweeps, double
   FE_ARG(work != nullptr, "ritz: m = %d needs a global workspace", m);
   if (grid || m > kRitzOneMax)
     return launch_ritz_big(H, m, b, which, max_sweeps, tol, theta, Y, rho, info, work, s);
-  const RitzShape sh = ritz_shape(m);
-  const int ncta = sh.ncta, variant = sh.items == 1 ? 0 : (sh.items == 4 ? 1 : 2);
-  auto kern = variant == 0 ? ritz_cluster_kernel<1> : (variant == 1 ? ritz_cluster_kernel<4> : ritz_cluster_kernel<7>);
-  const void* fn = reinterpret_cast<const void*>(kern);
   static KernelSetup ks[3];
-  FE_TRY(kernel_configure(ks[variant], fn, 128 * 1024));
-  if (ncta > 8) FE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = ncta;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ncta);
-  cfg.blockDim = dim3(sh.threads);
-  cfg.dynamicSmemBytes = ritz_cluster_smem(m, b, ncta);
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  auto shape = [&](const RitzShape& sh) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = sh.ncta;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(sh.ncta);
+    cfg.blockDim = dim3(sh.threads);
+    cfg.dynamicSmemBytes = ritz_cluster_smem(m, b, sh.ncta);
+  };
+  const RitzShape sh = ritz_shape(m, true);
+  const int variant = sh.items == 1 ? 0 : (sh.items == 4 ? 1 : 2);
+  auto kern = variant == 0 ? ritz_cluster_kernel<1> : (variant == 1 ? ritz_cluster_kernel<4> : ritz_cluster_kernel<7>);
+  const void* fn = reinterpret_cast<const void*>(kern);
+  FE_TRY(kernel_configure(ks[variant], fn, 128 * 1024));
+  shape(sh);
+  if (sh.ncta > kRitzCluster) {
+    // asked once per device and kernel: whether the device takes the cluster at all
+    static std::mutex mu;
+    static signed char wide[3][kMaxDevices];   // 0: not asked, 1: yes, -1: no
+    const int dev = cur_device();
+    if (dev < 0) return dev;
+    std::lock_guard<std::mutex> lock(mu);
+    if (wide[variant][dev] == 0) {
+      int clusters = 0;
+      const bool ok = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                      cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters > 0;
+      if (!ok) cudaGetLastError();   // not an error: the smaller cluster does
+      wide[variant][dev] = ok ? 1 : -1;
+    }
+    if (wide[variant][dev] < 0) shape(ritz_shape(m, false));
+  }
   FE_CUDA(cudaLaunchKernelEx(&cfg, kern, H, m, b, which, max_sweeps, tol, theta, Y, rho, info, work));
   count_launch();
   FE_CUDA(cudaGetLastError());

@@ -17,8 +17,9 @@ constexpr int kRitzCluster = 8, kRitzClusterMax = 16;
 struct RitzShape {
   int ncta, items, threads;
 };
-inline RitzShape ritz_shape(int m) {
-  return {m > 64 ? kRitzClusterMax : kRitzCluster, m <= 64 ? 1 : (m <= 128 ? 4 : 7), m <= 46 ? 256 : 512};
+// wide: clusters of kRitzClusterMax can be launched (more than 8 CTAs is a non-portable size).
+inline RitzShape ritz_shape(int m, bool wide) {
+  return {m > 64 && wide ? kRitzClusterMax : kRitzCluster, m <= 64 ? 1 : (m <= 128 ? 4 : 7), m <= 46 ? 256 : 512};
 }
 
 // Most sweeps of iteration `it`: kRitzFirstSweeps FP32 ones of the projected matrix itself, then, over all later

@@ -1,5 +1,6 @@
-// Test helper (host code only): for every subspace m up to 160, the shared-memory reads of the
-// one-cluster Rayleigh-Ritz sweep by the kernel's own index functions.  One line per m:
+// Test helper (host code only): for every subspace m up to 160, on clusters of 8 and of 16, the
+// shared-memory reads of the one-cluster Rayleigh-Ritz sweep by the kernel's own index functions.  One
+// line each:
 //   m  threads  active  items  highest float index read in a copy  floats of a copy
 //   bytes the layout ends at  bytes asked for (b = 1)  entries hit exactly once (1 or 0)
 #include <cstdio>
@@ -10,8 +11,9 @@
 using namespace fe;
 
 int main() {
-  for (int m = 1; m <= kRitzOneMax; ++m) {
-    const RitzShape sh = ritz_shape(m);
+  for (int k = 0; k < 2 * kRitzOneMax; ++k) {
+    const int m = k / 2 + 1;
+    const RitzShape sh = ritz_shape(m, k % 2 != 0);
     const int mp = m + (m & 1), np = mp / 2, nitems = ritz_items(np), nact = ritz_active(np, sh.threads);
     int top = 4 * nitems + np - 1;   // the pivots
     for (int tid = 0; tid < nact; ++tid)
