@@ -39,16 +39,16 @@ namespace fe {
 static_assert(sizeof(Task) == 16, "Task must be 16 bytes");
 static_assert(sizeof(PTask) == 32, "PTask must be 32 bytes");
 
+// FP64 blocks whose sums the FP64 adds would bind (b = 1 is bound by its gathers): they are added in
+// integers for the most part (Fx below) and gathered 16 bytes a lane.
 template <typename T, int B>
 constexpr bool kUseFx = sizeof(T) == 8 && B >= 2;
-template <typename T, int B>
-constexpr int kFxBytes = !kUseFx<T, B> ? 0 : 16;
 // Per (type, b, fragment width) geometry: a lane moves NE elements (<= FB bytes: 16, or 32
 // with 256-bit loads when X is 32-byte aligned) per load; an X row of b elements spans C lanes
 // in a warp task (P = 32 / C rows gathered per warp instruction) and C chunks in a tail lane.
 template <typename T, int B, bool V32>
 struct Geo {
-  static constexpr int FB = kFxBytes<T, B> ? kFxBytes<T, B> : (V32 ? 32 : 16);
+  static constexpr int FB = V32 && !kUseFx<T, B> ? 32 : 16;
   static constexpr int ROWB = B * (int)sizeof(T);
   static constexpr int NE = ROWB <= FB ? B : FB / (int)sizeof(T);
   static constexpr int C = B / NE;
@@ -159,12 +159,12 @@ __device__ __forceinline__ void fx_add3(Fx& f, double x, double y, double z) {
 __device__ __forceinline__ void fx_flush(double& s, Fx& f, bool& bad) {
   bad = bad || f.e >= 0x7d000000u || (f.e < 0x05000000u && f.a != 0);
   const double v = __ll2double_rn(f.a);
-  const double x = __hiloint2double(__double2hiint(v) + (int)f.e - (1080 << 20), __double2loint(v));
+  const unsigned hi = (unsigned)__double2hiint(v) + f.e - (1080u << 20);   // the exponent's change, modulo 2^32
+  const double x = __hiloint2double((int)hi, __double2loint(v));
   s += f.a != 0 ? x : 0.0;
   f.a = 0;
   f.e = 0;
 }
-// FP64 blocks whose sums the FP64 adds would bind (b = 1 is bound by its gathers).
 // Lanes of a slice that share a row by its columns, without 256-bit gathers: 16 bytes of it each.
 // With Fx sums a column takes 13 registers (four gathers in flight), and the warps that fit decide
 // (b = 4 at 4.2 million vertices: 950 us with four columns a lane, 80 registers).
