@@ -316,11 +316,18 @@ static int launch_post2(const double* G1x, const double* G2x, int k, int b, doub
 
 static int launch_post3(double* S2, const GramParts& parts, int b, const double* Racc, double* M, double* Rout,
                         int ldr, int* status, cudaStream_t s) {
-#define POST3P(B) orth_post3_kernel<(B < 4 ? B : 4), true><<<1, kPartThreads, 0, s>>>(S2, parts, Racc, M, Rout, ldr, status)
 #define POST3(B) orth_post3_kernel<B, false><<<1, kPostThreads, 0, s>>>(S2, parts, Racc, M, Rout, ldr, status)
-  FE_ARG(!parts.p || b <= 4, "orth: partial sums at b = %d", b);
-  if (parts.p) FE_ORTH_B(b, POST3P)
-  else FE_ORTH_B(b, POST3)
+#define POST3P(B) orth_post3_kernel<B, true><<<1, kPartThreads, 0, s>>>(S2, parts, Racc, M, Rout, ldr, status)
+  if (!parts.p) {
+    FE_ORTH_B(b, POST3)
+  } else {   // left by update_tri_gram only, which takes b <= 4
+    switch (b) {
+      case 1: POST3P(1); break;
+      case 2: POST3P(2); break;
+      case 4: POST3P(4); break;
+      default: return set_error(FE_ERR_INVALID, "orth: partial sums at b = %d", b);
+    }
+  }
 #undef POST3
 #undef POST3P
   count_launch();

@@ -252,10 +252,10 @@ __global__ void tc_prep_y_kernel(const double* __restrict__ Y, int ldy, double a
 // Row r of a 128-row tile is handled by two threads (warps w and w + 4 address the same TMEM
 // lane quarter): each loads and splits half of the row's K values, and each assembles half of
 // the row's N results.
-// K <= 32: two CTAs per SM (256 TMEM columns each); K <= 64: one (512 columns).
-template <int BV, int KMAX>
-__global__ void __launch_bounds__(kThreads, KMAX <= 32 ? 2 : 1) tc_combine_kernel(const TcArgs a) {
-  constexpr int KH = KMAX / 2;  // V values per thread
+// 32 < K <= 64 (fewer columns take the pipeline below); 256 TMEM columns up to N = 16, else 512.
+template <int BV>
+__global__ void __launch_bounds__(kThreads, 1) tc_combine_kernel(const TcArgs a) {
+  constexpr int KMAX = kMaxK, KH = KMAX / 2;  // V values per thread
   extern __shared__ __align__(1024) unsigned char smem[];
   const int nkc = a.nkc, NP = a.NP;
   unsigned char* sA = smem;                                        // [nkc][7] x 8 KB
@@ -468,8 +468,9 @@ static size_t tc_smem_bytes(int nkc, int NP) {
 //   warp 29     (one thread) issues tile t's MMAs into TMEM buffer t % 2 and owns the TMEM
 //               allocation;
 //   warps 16-27 read tile t's accumulators (TMEM lane quarter = warp % 4, three threads per row,
-//               every third pair of results each), assemble and store them; with beta != 0 and
-//               N <= 16 the rows of Out for tile t + 1 are loaded while tile t is assembled.
+//               every third pair of results each), assemble and store them; with beta != 0 a
+//               thread with at most two pairs (N <= 12: all of them) loads its rows of Out for
+//               the next tiles while tile t is assembled.
 // V staging, digit tiles and accumulators are double-buffered, so tile t + 1 is split while tile
 // t's products run and its results are assembled.  Five mbarrier pairs hand each buffer on:
 // vfull (TMA -> splitters), vempty (splitters -> TMA), afull (splitters -> MMA and
@@ -724,8 +725,8 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_combine_pipe_kernel(const 
     const bool add_out = a.beta != 0.0;
     constexpr int kStep = 2 * kEpiParts;
     const int ngroups = a.N > 2 * part ? (a.N - 2 * part + kStep - 1) / kStep : 0;        // this thread's groups of two results
-    // rows of Out loaded ahead of their tile: one group per thread (N <= 4) two tiles ahead into
-    // slot it % 2, two groups (N <= 8) one tile ahead into slot = group
+    // rows of Out loaded ahead of their tile: by a thread with one group (all of them: N <= 6) two tiles
+    // ahead into slot it % 2, with two groups (N <= 12) one tile ahead into slot = group
     const int pf = !add_out ? 0 : ngroups <= 1 ? 2 : ngroups == 2 ? 1 : 0;
     double opf[2][2];
     auto load_grp = [&](int64_t it, int jj, int slot) {
@@ -869,23 +870,17 @@ bool tc_combine_supported(const BlockSet& V, const BlockSet& Out, fe_dtype dt) {
          N >= 1 && N <= kMaxN && V.bv >= 1 && V.bv <= 16;
 }
 
-template <int BV, int KMAX>
+template <int BV>
 static int launch_tc_combine(const TcArgs& a, size_t smem, bool two_per_sm, cudaStream_t s) {
   static KernelSetup ks;
-  const void* fn = reinterpret_cast<const void*>(tc_combine_kernel<BV, KMAX>);
+  const void* fn = reinterpret_cast<const void*>(tc_combine_kernel<BV>);
   FE_TRY(kernel_configure(ks, fn, 227 * 1024));
   const int64_t ntiles = ceil_div(a.n, kTileRows);
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ntiles, (int64_t)(two_per_sm ? 2 : 1) * num_sms()));
-  tc_combine_kernel<BV, KMAX><<<(unsigned)grid, kThreads, smem, s>>>(a);
+  tc_combine_kernel<BV><<<(unsigned)grid, kThreads, smem, s>>>(a);
   count_launch();
   FE_CUDA(cudaGetLastError());
   return FE_OK;
-}
-
-template <int BV>
-static int launch_tc_combine_k(const TcArgs& a, size_t smem, bool two_per_sm, cudaStream_t s) {
-  if (a.K <= 32) return launch_tc_combine<BV, 32>(a, smem, two_per_sm, s);
-  return launch_tc_combine<BV, 64>(a, smem, two_per_sm, s);
 }
 
 // Out = V Y on the tensor cores (FP64 blocks; see tc_combine_supported for the shapes).
@@ -935,11 +930,11 @@ int tc_combine(const BlockSet& V, int64_t n, const double* Y, int ldy, const Blo
   const bool two = a.nkc * kClasses * a.NP <= 256;
   const size_t smem = std::max(tc_smem_bytes(a.nkc, a.NP), two ? (size_t)100 * 1024 : (size_t)120 * 1024);
   switch (BV) {
-    case 1: return launch_tc_combine_k<1>(a, smem, two, s);
-    case 2: return launch_tc_combine_k<2>(a, smem, two, s);
-    case 4: return launch_tc_combine_k<4>(a, smem, two, s);
-    case 8: return launch_tc_combine_k<8>(a, smem, two, s);
-    case 16: return launch_tc_combine_k<16>(a, smem, two, s);
+    case 1: return launch_tc_combine<1>(a, smem, two, s);
+    case 2: return launch_tc_combine<2>(a, smem, two, s);
+    case 4: return launch_tc_combine<4>(a, smem, two, s);
+    case 8: return launch_tc_combine<8>(a, smem, two, s);
+    case 16: return launch_tc_combine<16>(a, smem, two, s);
   }
   return set_error(FE_ERR_INVALID, "tc_combine: block width %d", BV);
 }
