@@ -188,7 +188,7 @@ __device__ __forceinline__ int gap_field(const uint32_t* __restrict__ tb, int k,
 // (ti past the range: nothing to do but the barriers).
 template <typename T, int B, bool V32, bool PACKED, bool FX, int W>
 __device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, int64_t tend, const T* __restrict__ X,
-                                         T* __restrict__ Y, T* __restrict__ partial, int warp, int lane, T* red) {
+                                         T* __restrict__ Y, double* __restrict__ partial, int warp, int lane, T* red) {
   using G = Geo<T, B, V32>;
   const int piece = warp % W;
   int64_t start = 0;
@@ -347,9 +347,19 @@ __device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, int64_
   }
 #pragma unroll
   for (int off = 16 >> G::LNE; off >= G::C; off >>= 1) acc[0] += __shfl_xor_sync(kFull, acc[0], off);
-  T* dst = ti < p.nhub_tasks ? partial + ti * B : Y + (int64_t)row * B;
+  // column c of the row, or of a hub chunk: its sum stays in FP64 until the hub's chunks are added
+  auto put = [&](int c, auto v) {
+    if constexpr (sizeof(T) == 8) {
+      T* dst = ti < p.nhub_tasks ? partial + ti * B : Y + (int64_t)row * B;
+      dst[c] = v;
+    } else if (ti < p.nhub_tasks) {
+      partial[ti * B + c] = (double)v;
+    } else {
+      Y[(int64_t)row * B + c] = (T)v;
+    }
+  };
   if constexpr (W == 1) {
-    if ((lane & G::PLAIN_MASK) == 0) dst[chunk * G::NE + ebase] = acc[0];
+    if ((lane & G::PLAIN_MASK) == 0) put(chunk * G::NE + ebase, acc[0]);
   } else {
     // the pieces in order, in FP64: one more rounding to T however many there are
     if ((lane & G::PLAIN_MASK) == 0) red[warp * B + chunk * G::NE + ebase] = acc[0];
@@ -358,7 +368,7 @@ __device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, int64_
       double s = (double)red[warp * B + lane];
 #pragma unroll
       for (int i = 1; i < W; ++i) s += (double)red[(warp + i) * B + lane];
-      dst[lane] = (T)s;
+      put(lane, s);
     }
   }
 }
@@ -497,7 +507,7 @@ constexpr int kMinCtas = FX ? 5
                                                : (B == 8 ? 5 : (V32 ? 3 : 7));
 template <typename T, int B, bool V32, bool PACKED, bool FX>
 __global__ void __launch_bounds__(256, (kMinCtas<T, B, V32, PACKED, FX>))
-    spmm_main_kernel(const SpmmParams p, const T* __restrict__ X, T* __restrict__ Y, T* __restrict__ partial) {
+    spmm_main_kernel(const SpmmParams p, const T* __restrict__ X, T* __restrict__ Y, double* __restrict__ partial) {
   __shared__ T red[kWarpsPerCta * B];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t cta = blockIdx.x;
@@ -526,24 +536,24 @@ __device__ __forceinline__ void neumaier_add(double& s, double& e, double x) {
 }
 
 // Y[hub_rows[h]] = sum of the hub's task partials in compensated FP64, then one rounding to T: an error
-// of about 2^-53 |sum| + O(k 2^-106) sum |partial| for any number k of partials, so a hub adds one
-// rounding to its chunks' errors.  One warp per hub row: lane l adds column l % B of tasks l / B, l / B +
+// of about 2^-53 |sum| + O(k 2^-106) sum |partial| for any number k of partials (FP64 in both types),
+// so a hub adds one rounding to its chunks' errors.  One warp per hub row: lane l adds column l % B of tasks l / B, l / B +
 // 32 / B, .. in order, then the lanes of a column are added in a fixed tree (R-MAT with 2^20 vertices,
 // FP32 b = 4: 8.4 us with a thread per entry over all of a row's partials, 3.1 us now).
 template <typename T, int B>
 __global__ void __launch_bounds__(256) hub_reduce_kernel(const int32_t* __restrict__ hub_rows,
                                                          const int32_t* __restrict__ hub_task_begin,
-                                                         int64_t nhub, const T* __restrict__ partial,
+                                                         int64_t nhub, const double* __restrict__ partial,
                                                          T* __restrict__ Y) {
   const int64_t h = (int64_t)blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
   if (h >= nhub) return;
   const int lane = threadIdx.x & 31, c = lane % B, slot = lane / B;
   const int t0 = hub_task_begin[h], t1 = hub_task_begin[h + 1];
-  const T* src = partial + (int64_t)t0 * B + lane;   // task t0 + slot, column c
+  const double* src = partial + (int64_t)t0 * B + lane;   // task t0 + slot, column c
   const int steps = (t1 - t0 - slot + 32 / B - 1) / (32 / B);
-  double s = steps > 0 ? (double)src[0] : 0.0, e = 0.0;
+  double s = steps > 0 ? src[0] : 0.0, e = 0.0;
 #pragma unroll 4
-  for (int t = 1; t < steps; ++t) neumaier_add(s, e, (double)src[(int64_t)t * 32]);
+  for (int t = 1; t < steps; ++t) neumaier_add(s, e, src[(int64_t)t * 32]);
 #pragma unroll
   for (int off = B; off < 32; off <<= 1) {
     const double s2 = __shfl_xor_sync(kFull, s, off), e2 = __shfl_xor_sync(kFull, e, off);
@@ -578,7 +588,7 @@ static int l2_window_bytes(size_t bytes, size_t* win) {
 }
 
 template <typename T, int B>
-static int launch_spmm(const PlanView& pv, const T* X, T* Y, T* partial, cudaStream_t s) {
+static int launch_spmm(const PlanView& pv, const T* X, T* Y, double* partial, cudaStream_t s) {
   SpmmParams p;
   memset(&p, 0, sizeof(p));
   p.colidx = pv.colidx;
@@ -616,7 +626,7 @@ static int launch_spmm(const PlanView& pv, const T* X, T* Y, T* partial, cudaStr
   p.task_ctas = p.ctas2 + ceil_div(pv.ntasks - pv.wide2, kWarpsPerCta);
   const int64_t ctas = p.task_ctas + ceil_div(warps, kWarpsPerCta);
   if (ctas > 0) {
-    void (*kern)(const SpmmParams, const T*, T*, T*) = nullptr;
+    void (*kern)(const SpmmParams, const T*, T*, double*) = nullptr;
     if (v32) {
       if constexpr (kWide<T, B>)
         kern = pv.packed ? spmm_main_kernel<T, B, true, true, false> : spmm_main_kernel<T, B, true, false, false>;
@@ -698,7 +708,7 @@ int spmm_view(const PlanView& v, const void* X, void* Y, void* partial, int b, f
   if (dt == FE_F32) {
     const float* x = static_cast<const float*>(X);
     float* y = static_cast<float*>(Y);
-    float* pa = static_cast<float*>(partial);
+    double* pa = static_cast<double*>(partial);
     switch (b) {
       case 1: return launch_spmm<float, 1>(v, x, y, pa, s);
       case 2: return launch_spmm<float, 2>(v, x, y, pa, s);

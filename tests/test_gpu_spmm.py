@@ -465,3 +465,23 @@ def test_spmm_f64_hub_chunks(b, fmt):
     want = deg * np.longdouble(c)
     assert np.all(np.abs(Y[0] - want) <= (m + 9) * 2.0 ** -53 * want)
     assert np.all(np.abs(Y[1] - 3 * np.longdouble(c)) <= 3 * 2.0 ** -53 * 3 * c)
+
+
+@pytest.mark.parametrize("fmt", ["plain", "packed"])
+@pytest.mark.parametrize("deg,W", [(700, 1), (1500, 2), (5000, 4), (20 * 3000 + 17, 4)])
+def test_spmm_f32_rounds_once(deg, W, fmt):
+    """FP32 sums of one column, bit for bit as the summation restated on the CPU gives them: a warp's
+    lanes compensated and added by a tree, the warps that share a task and a hub row's chunks of 3000 in
+    FP64, rounded to FP32 once."""
+    from tests.test_spmm_f32_summation import hub_sum, shared_task_sum, task_sum
+    ncols, chunk = 70000, 3000
+    r = np.random.default_rng(deg)
+    cols = np.sort(r.choice(ncols, deg, replace=False)).astype(np.int32)
+    rowptr = np.array([0, deg], dtype=np.int64)
+    with fe.Csr(rowptr, cols, ncols=ncols, hub_min=10000, hub_chunk=chunk, index_format=fmt) as h:
+        for X in (r.random(ncols) + 1.0, r.standard_normal(ncols)):
+            X = X.astype(np.float32)
+            Y = fe.spmm(h, to_dev(X[:, None])).cpu().numpy()
+            want = (hub_sum(X[cols], chunk, 32, 1, W) if deg > 10000 else
+                    np.float32(shared_task_sum(X[cols], 32, W) if W > 1 else task_sum(X[cols], 32)))
+            assert Y[0, 0] == want

@@ -10,11 +10,17 @@ The summation restated:
   for b = 8 and 16 or 8 for b = 16, by the load width); every slot adds its terms in order with Kahan's compensation (s, c) and ends with
   s - c; the P slot values are added by a balanced tree (slot s with slot s + P/2, then + P/4,
   ...), one FP32 add per level;
-* a slice row (the low-degree tail): one lane adds the row's terms in order, compensated;
-* a split hub row: its chunks' task results are added in FP64 with Neumaier's compensation in
-  task order and rounded once to FP32.
+  where a row's tasks are few columns or streamed, two or four warps share a long task, each taking a
+  run of whole rounds of 32 terms, and their sums are added in order in FP64 and rounded once;
+* a slice row (the low-degree tail): one lane adds the row's terms in order, compensated; above degree
+  32 two lanes share it and above 64 four, each a run of steps (a multiple of 4), their sums added
+  by a tree;
+* a split hub row: its chunks' task results are added in FP64 with Neumaier's compensation by the
+  lanes of a warp (32 / b of them: lane l tasks l, l + 32 / b, .. in order), the lanes by a compensated
+  tree, and rounded once to FP32.
 Bound: 3 u per slot (2 u + O(m u^2) for the compensated sum, Higham Thm. 4.8, plus the rounding
-of s - c), u per tree level (at most 5), u for the hub's final rounding: 9 u with u = 2^-24.
+of s - c), u per tree level (at most 5), u for the one rounding of what is added in FP64: 9 u with
+u = 2^-24.
 """
 import math
 
@@ -56,15 +62,55 @@ def task_sum(terms, P, slot=slot_sum):
     return part[0]
 
 
-def hub_sum(terms, task_len, P):
-    """A split hub row: task results in FP64 with Neumaier's compensation, rounded once."""
-    s = e = 0.0
-    for t0 in range(0, len(terms), task_len):
-        x = float(task_sum(terms[t0:t0 + task_len], P))
-        u = s + x
-        e += (s - u) + x if abs(s) >= abs(x) else (x - u) + s
-        s = u
-    return F(s + e)
+def shared_task_sum(terms, P, W):
+    """One task on W warps: runs of whole rounds, the warps' sums in order in FP64 (rounded once, to the
+    row or with a hub's other chunks)."""
+    run = ((len(terms) + W - 1) // W + 31) // 32 * 32
+    total = 0.0
+    for w in range(W):
+        total += float(task_sum(terms[w * run:(w + 1) * run], P)) if len(terms[w * run:(w + 1) * run]) else 0.0
+    return total
+
+
+def slice_row_sum(terms):
+    """A slice row on one, two or four lanes."""
+    deg = len(terms)
+    pieces = 1 if deg <= 32 else 2 if deg <= 64 else 4
+    run = ((deg + pieces - 1) // pieces + 3) // 4 * 4
+    part = [slot_sum(terms[k * run:(k + 1) * run]) for k in range(pieces)]
+    while len(part) > 1:
+        h = len(part) // 2
+        part = [F(part[k] + part[k + h]) for k in range(h)]
+    return part[0]
+
+
+def _neumaier(s, e, x):
+    u = s + x
+    a, b = (s, x) if abs(s) >= abs(x) else (x, s)
+    return u, e + ((a - u) + b)
+
+
+def hub_sum(terms, task_len, P, b, W=1):
+    """A split hub row of a block of b columns: 32 / b lanes add the tasks' results with compensation,
+    then a compensated tree, rounded once."""
+    lanes = 32 // b
+    tasks = [shared_task_sum(terms[t0:t0 + task_len], P, W) if W > 1 else float(task_sum(terms[t0:t0 + task_len], P))
+             for t0 in range(0, len(terms), task_len)]
+    acc = []
+    for lane in range(lanes):
+        mine = tasks[lane::lanes]
+        s, e = (mine[0] if mine else 0.0), 0.0
+        for x in mine[1:]:
+            s, e = _neumaier(s, e, x)
+        acc.append((s, e))
+    while len(acc) > 1:
+        h = [None] * (len(acc) // 2)
+        for k in range(len(h)):
+            (s, e), (s2, e2) = acc[2 * k], acc[2 * k + 1]
+            s, e = _neumaier(s, e, s2)
+            h[k] = (s, e + e2)
+        acc = h
+    return F(acc[0][0] + acc[0][1])
 
 
 def rel_err(got, terms):
@@ -103,20 +149,30 @@ def test_warp_task_within_bound(P, deg):
         assert err <= BOUND, (name, P, deg, err / U)
 
 
-@pytest.mark.parametrize("deg", [1, 2, 17, 69, 127, 128])
+@pytest.mark.parametrize("deg", [1, 2, 17, 32, 33, 64, 65, 69, 127, 128])
 def test_slice_row_within_bound(deg):
     rng = np.random.default_rng(deg)
     for name, terms in adversarial_rows(rng, deg).items():
-        err = rel_err(slot_sum(terms), terms)
+        err = rel_err(slice_row_sum(terms), terms)
         assert err <= BOUND, (name, deg, err / U)
 
 
+@pytest.mark.parametrize("W", [2, 4])
 @pytest.mark.parametrize("P", [32, 8])
-def test_split_hub_row_within_bound(P):
-    rng = np.random.default_rng(7 + P)
-    deg, task_len = 20000, 4096                                 # five chunks, the last ragged
+@pytest.mark.parametrize("deg", [1025, 2049, 4096])
+def test_shared_task_within_bound(P, W, deg):
+    rng = np.random.default_rng(deg + P)
     for name, terms in adversarial_rows(rng, deg).items():
-        err = rel_err(hub_sum(terms, task_len, P), terms)
+        err = rel_err(F(shared_task_sum(terms, P, W)), terms)
+        assert err <= BOUND, (name, P, W, err / U)
+
+
+@pytest.mark.parametrize("P,b,task_len,W", [(32, 1, 4096, 1), (8, 16, 4096, 1), (32, 4, 4096, 4), (32, 4, 64, 1)])
+def test_split_hub_row_within_bound(P, b, task_len, W):
+    rng = np.random.default_rng(7 + P)
+    deg = 20000                                                 # the last chunk ragged
+    for name, terms in adversarial_rows(rng, deg).items():
+        err = rel_err(hub_sum(terms, task_len, P, b, W), terms)
         assert err <= BOUND, (name, P, err / U)
 
 
