@@ -119,6 +119,18 @@ __device__ __forceinline__ void kahan_add(float& s, float& c, float x) {
 __device__ __forceinline__ void kahan_add(double& s, double&, double x) { s += x; }
 __device__ __forceinline__ float kahan_value(float s, float c) { return s - c; }
 __device__ __forceinline__ double kahan_value(double s, double) { return s; }
+// The sum of this lane's (s, c), `keep`, and its partner's, `send` of the lane `off` away (TwoSum: the sums
+// of lanes that share a row are compensated too).
+__device__ __forceinline__ void kahan_merge(float keep, float ckeep, float send, float csend, int off, float& s, float& c) {
+  const float x = __shfl_xor_sync(0xffffffffu, send, off), cx = __shfl_xor_sync(0xffffffffu, csend, off);
+  const float t = keep + x, z = t - keep;
+  const float d = (ckeep + cx) - ((keep - (t - z)) + (x - z));
+  c = d == d ? d : 0.f;   // an infinite sum has no error term
+  s = t;
+}
+__device__ __forceinline__ void kahan_merge(double keep, double, double send, double, int off, double& s, double&) {
+  s = keep + __shfl_xor_sync(0xffffffffu, send, off);
+}
 
 // FP64 sums in integers.  An FP64 add occupies the FP64 pipe of an SM for 16 clocks per warp; the
 // 32-bit integer units take the 16 instructions of an aligned integer add in half of that, beside it.
@@ -188,7 +200,7 @@ __device__ __forceinline__ int gap_field(const uint32_t* __restrict__ tb, int k,
 // (ti past the range: nothing to do but the barriers).
 template <typename T, int B, bool V32, bool PACKED, bool FX, int W>
 __device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, int64_t tend, const T* __restrict__ X,
-                                         T* __restrict__ Y, double* __restrict__ partial, int warp, int lane, T* red) {
+                                         T* __restrict__ Y, double* __restrict__ partial, int warp, int lane, double* red) {
   using G = Geo<T, B, V32>;
   const int piece = warp % W;
   int64_t start = 0;
@@ -326,11 +338,15 @@ __device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, int64_
   } else {
     plain();
   }
-#pragma unroll
-  for (int e = 0; e < G::NE; ++e) acc[e] = kahan_value(acc[e], cmp[e]);
   // Sum the P slot partials of each chunk.  The first LNE butterfly levels (offsets 16, 8, ..)
   // also scatter the NE elements -- a lane keeps half of what it holds and adds its partner's
-  // copy of that half -- so every level after them adds one value per lane.
+  // copy of that half -- so every level after them adds one value per lane.  Where warps share the
+  // task the lanes' sums stay compensated, so that the warps' add no more than the last rounding.
+  constexpr bool kPairs = sizeof(T) == 4 && W > 1;
+  if constexpr (!kPairs) {
+#pragma unroll
+    for (int e = 0; e < G::NE; ++e) acc[e] = kahan_value(acc[e], cmp[e]);
+  }
   int ebase = 0;
 #pragma unroll
   for (int lvl = 0; lvl < G::LNE; ++lvl) {
@@ -341,12 +357,16 @@ __device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, int64_
     for (int i = 0; i < (G::NE >> (lvl + 1)); ++i) {
       const T send = up ? acc[i] : acc[i + h];
       const T keep = up ? acc[i + h] : acc[i];
-      acc[i] = keep + __shfl_xor_sync(kFull, send, off);
+      if constexpr (kPairs) kahan_merge(keep, up ? cmp[i + h] : cmp[i], send, up ? cmp[i] : cmp[i + h], off, acc[i], cmp[i]);
+      else acc[i] = keep + __shfl_xor_sync(kFull, send, off);
     }
     if (up) ebase += h;
   }
 #pragma unroll
-  for (int off = 16 >> G::LNE; off >= G::C; off >>= 1) acc[0] += __shfl_xor_sync(kFull, acc[0], off);
+  for (int off = 16 >> G::LNE; off >= G::C; off >>= 1) {
+    if constexpr (kPairs) kahan_merge(acc[0], cmp[0], acc[0], cmp[0], off, acc[0], cmp[0]);
+    else acc[0] += __shfl_xor_sync(kFull, acc[0], off);
+  }
   // column c of the row, or of a hub chunk: its sum stays in FP64 until the hub's chunks are added
   auto put = [&](int c, auto v) {
     if constexpr (sizeof(T) == 8) {
@@ -362,12 +382,13 @@ __device__ __forceinline__ void run_task(const SpmmParams& p, int64_t ti, int64_
     if ((lane & G::PLAIN_MASK) == 0) put(chunk * G::NE + ebase, acc[0]);
   } else {
     // the pieces in order, in FP64: one more rounding to T however many there are
-    if ((lane & G::PLAIN_MASK) == 0) red[warp * B + chunk * G::NE + ebase] = acc[0];
+    if ((lane & G::PLAIN_MASK) == 0)
+      red[warp * B + chunk * G::NE + ebase] = kPairs ? (double)acc[0] - (double)cmp[0] : (double)acc[0];
     __syncthreads();
     if (piece == 0 && lane < B && ti < tend) {
-      double s = (double)red[warp * B + lane];
+      double s = red[warp * B + lane];
 #pragma unroll
-      for (int i = 1; i < W; ++i) s += (double)red[(warp + i) * B + lane];
+      for (int i = 1; i < W; ++i) s += red[(warp + i) * B + lane];
       put(lane, s);
     }
   }
@@ -461,12 +482,14 @@ __device__ __forceinline__ void run_slice(const SpmmParams& p, unsigned wi, cons
     }
   }
   if (!done) plain(piece * len);
-#pragma unroll
-  for (int q = 0; q < K; ++q) acc[q] = kahan_value(acc[q], cmp[q]);
   if constexpr (FX) row = __ldcs(p.slice_rows + si * 32 + srow);   // late: one register less
   T* y = Y + (int64_t)row * B + cl * K;
   if (pieces == 1) {
-    if (row >= 0) st_row<T, K>(y, acc);
+    if (row >= 0) {
+#pragma unroll
+      for (int q = 0; q < K; ++q) acc[q] = kahan_value(acc[q], cmp[q]);
+      st_row<T, K>(y, acc);
+    }
     return;
   }
   // the pieces' sums: lanes 16 apart, then (four pieces) 8 apart, each level also dividing the
@@ -476,25 +499,31 @@ __device__ __forceinline__ void run_slice(const SpmmParams& p, unsigned wi, cons
   const bool up1 = (lane & 16) != 0, up2 = (lane & 8) != 0;
 #pragma unroll
   for (int i = 0; i < H1; ++i) {
-    const T send = K >= 2 && !up1 ? acc[(i + H1) % K] : acc[i];
-    const T keep = K >= 2 && up1 ? acc[(i + H1) % K] : acc[i];
-    acc[i] = keep + __shfl_xor_sync(kFull, send, 16);
+    const int j = (i + H1) % K;   // i for a single column, which both lanes keep
+    kahan_merge(up1 ? acc[j] : acc[i], up1 ? cmp[j] : cmp[i], up1 ? acc[i] : acc[j], up1 ? cmp[i] : cmp[j], 16, acc[i], cmp[i]);
   }
   if (K >= 2) y += up1 ? H1 : 0;
   else writer = writer && !up1;
   if (pieces == 2) {
-    if (writer) st_row<T, H1>(y, acc);
+    if (writer) {
+#pragma unroll
+      for (int q = 0; q < H1; ++q) acc[q] = kahan_value(acc[q], cmp[q]);
+      st_row<T, H1>(y, acc);
+    }
     return;
   }
 #pragma unroll
   for (int i = 0; i < H2; ++i) {
-    const T send = H1 >= 2 && !up2 ? acc[(i + H2) % K] : acc[i];
-    const T keep = H1 >= 2 && up2 ? acc[(i + H2) % K] : acc[i];
-    acc[i] = keep + __shfl_xor_sync(kFull, send, 8);
+    const int j = (i + H2) % H1;
+    kahan_merge(up2 ? acc[j] : acc[i], up2 ? cmp[j] : cmp[i], up2 ? acc[i] : acc[j], up2 ? cmp[i] : cmp[j], 8, acc[i], cmp[i]);
   }
   if (H1 >= 2) y += up2 ? H2 : 0;
   else writer = writer && !up2;
-  if (writer) st_row<T, H2>(y, acc);
+  if (writer) {
+#pragma unroll
+    for (int q = 0; q < H2; ++q) acc[q] = kahan_value(acc[q], cmp[q]);
+    st_row<T, H2>(y, acc);
+  }
 }
 
 template <typename T, int B>
@@ -508,7 +537,7 @@ constexpr int kMinCtas = FX ? 5
 template <typename T, int B, bool V32, bool PACKED, bool FX>
 __global__ void __launch_bounds__(256, (kMinCtas<T, B, V32, PACKED, FX>))
     spmm_main_kernel(const SpmmParams p, const T* __restrict__ X, T* __restrict__ Y, double* __restrict__ partial) {
-  __shared__ T red[kWarpsPerCta * B];
+  __shared__ double red[kWarpsPerCta * B];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t cta = blockIdx.x;
   if (cta < p.ctas4) {

@@ -468,20 +468,39 @@ def test_spmm_f64_hub_chunks(b, fmt):
 
 
 @pytest.mark.parametrize("fmt", ["plain", "packed"])
-@pytest.mark.parametrize("deg,W", [(700, 1), (1500, 2), (5000, 4), (20 * 3000 + 17, 4)])
+@pytest.mark.parametrize("deg,W", [(9, 0), (40, 0), (64, 0), (65, 0), (127, 0), (700, 1), (1500, 2), (5000, 4),
+                                   (20 * 3000 + 17, 4)])
 def test_spmm_f32_rounds_once(deg, W, fmt):
-    """FP32 sums of one column, bit for bit as the summation restated on the CPU gives them: a warp's
-    lanes compensated and added by a tree, the warps that share a task and a hub row's chunks of 3000 in
-    FP64, rounded to FP32 once."""
-    from tests.test_spmm_f32_summation import hub_sum, shared_task_sum, task_sum
+    """FP32 sums of one column, bit for bit as the summation restated on the CPU gives them: slice rows of
+    one, two and four lanes (W = 0), a warp's lanes compensated and added by a tree, the warps that share a
+    task and a hub row's chunks of 3000 in FP64, rounded to FP32 once."""
+    from tests.test_spmm_f32_summation import hub_sum, shared_task_sum, slice_row_sum, task_sum
     ncols, chunk = 70000, 3000
     r = np.random.default_rng(deg)
     cols = np.sort(r.choice(ncols, deg, replace=False)).astype(np.int32)
     rowptr = np.array([0, deg], dtype=np.int64)
-    with fe.Csr(rowptr, cols, ncols=ncols, hub_min=10000, hub_chunk=chunk, index_format=fmt) as h:
+    with fe.Csr(rowptr, cols, ncols=ncols, tail_max=128, hub_min=10000, hub_chunk=chunk, index_format=fmt) as h:
         for X in (r.random(ncols) + 1.0, r.standard_normal(ncols)):
             X = X.astype(np.float32)
             Y = fe.spmm(h, to_dev(X[:, None])).cpu().numpy()
-            want = (hub_sum(X[cols], chunk, 32, 1, W) if deg > 10000 else
+            want = (hub_sum(X[cols], chunk, 32, 1, W) if deg > 10000 else slice_row_sum(X[cols]) if W == 0 else
                     np.float32(shared_task_sum(X[cols], 32, W) if W > 1 else task_sum(X[cols], 32)))
             assert Y[0, 0] == want
+
+
+def test_spmm_f32_no_error_growth_from_sharing():
+    """A row that lanes or warps share is as accurate as one lane's compensated sum: over 300 rows each of
+    degree 40 (two lanes), 100 (four) and 3000 (four warps) of values in [1, 2) the error stays within
+    half a unit in the last place of the sum, what one rounding makes, and 2^-40 of it for the rest."""
+    ncols = 9000
+    r = np.random.default_rng(3)
+    degs = [40] * 300 + [100] * 300 + [3000] * 300
+    cols = [np.sort(r.choice(ncols, d, replace=False)).astype(np.int32) for d in degs]
+    rowptr = np.concatenate([[0], np.cumsum(degs)]).astype(np.int64)
+    X = (r.random((ncols, 4)) + 1.0).astype(np.float32)
+    with fe.Csr(rowptr, np.concatenate(cols), ncols=ncols) as h:
+        Y = fe.spmm(h, to_dev(X)).cpu().numpy().astype(np.float64)
+    for i, c in enumerate(cols):
+        ref = X[c].astype(np.float64).sum(0)
+        half_ulp = np.spacing(ref.astype(np.float32)).astype(np.float64) / 2
+        assert np.all(np.abs(Y[i] - ref) <= half_ulp + 2.0 ** -40 * ref), degs[i]

@@ -7,17 +7,18 @@ up (one sign, constant values, wide exponent ranges, near-total cancellation).
 The summation restated:
 * a warp task (rows of degree above the slice limit, and every chunk of a split hub row):
   term k of the task goes to slot k mod P (P = 32 / chunks per row: 32 for b <= 4, 32 or 16
-  for b = 8 and 16 or 8 for b = 16, by the load width); every slot adds its terms in order with Kahan's compensation (s, c) and ends with
-  s - c; the P slot values are added by a balanced tree (slot s with slot s + P/2, then + P/4,
-  ...), one FP32 add per level;
-  where a row's tasks are few columns or streamed, two or four warps share a long task, each taking a
-  run of whole rounds of 32 terms, and their sums are added in order in FP64 and rounded once;
+  for b = 8 and 16 or 8 for b = 16, by the load width); every slot adds its terms in order with Kahan's
+  compensation (s, c) and ends with s - c; the P slot values are added by a balanced tree (slot s with
+  slot s + P/2, then + P/4, ...), one FP32 add per level.  Where the matrix has few columns or is
+  streamed, two or four warps share a long task, each taking a run of whole rounds of 32 terms: their
+  slots' pairs (s, c) are merged by the tree (TwoSum), and the warps' s - c are added in order in FP64
+  and rounded once;
 * a slice row (the low-degree tail): one lane adds the row's terms in order, compensated; above degree
-  32 two lanes share it and above 64 four, each a run of steps (a multiple of 4), their sums added
+  32 two lanes share it and above 64 four, each a run of steps (a multiple of 4), their pairs merged
   by a tree;
-* a split hub row: its chunks' task results are added in FP64 with Neumaier's compensation by the
-  lanes of a warp (32 / b of them: lane l tasks l, l + 32 / b, .. in order), the lanes by a compensated
-  tree, and rounded once to FP32.
+* a split hub row: its chunks' task results (not rounded where warps share them) are added in FP64 with
+  Neumaier's compensation by the lanes of a warp (32 / b of them: lane l tasks l, l + 32 / b, .. in
+  order), the lanes by a compensated tree, and rounded once to FP32.
 Bound: 3 u per slot (2 u + O(m u^2) for the compensated sum, Higham Thm. 4.8, plus the rounding
 of s - c), u per tree level (at most 5), u for the one rounding of what is added in FP64: 9 u with
 u = 2^-24.
@@ -32,8 +33,8 @@ U = 2.0 ** -24
 BOUND = 9 * U
 
 
-def slot_sum(terms):
-    """Kahan's compensated sum of float32 terms in order, then s - c (float32 throughout)."""
+def slot_pair(terms):
+    """Kahan's compensated sum of float32 terms in order: (s, c), the sum being s - c (float32)."""
     s = F(0.0)
     c = F(0.0)
     for x in terms:
@@ -41,7 +42,27 @@ def slot_sum(terms):
         t = F(s + y)
         c = F((t - s) - y)
         s = t
+    return s, c
+
+
+def slot_sum(terms):
+    s, c = slot_pair(terms)
     return F(s - c)
+
+
+def merge(p, q):
+    """Two lanes' pairs: TwoSum of the sums, its error with the compensations."""
+    (s, c), (s2, c2) = p, q
+    t = F(s + s2)
+    z = F(t - s)
+    return t, F(F(c + c2) - F(F(s - F(t - z)) + F(s2 - z)))
+
+
+def merge_tree(part):
+    while len(part) > 1:
+        h = len(part) // 2
+        part = [merge(part[k], part[k + h]) for k in range(h)]
+    return part[0]
 
 
 def plain_slot_sum(terms):
@@ -68,7 +89,9 @@ def shared_task_sum(terms, P, W):
     run = ((len(terms) + W - 1) // W + 31) // 32 * 32
     total = 0.0
     for w in range(W):
-        total += float(task_sum(terms[w * run:(w + 1) * run], P)) if len(terms[w * run:(w + 1) * run]) else 0.0
+        mine = terms[w * run:(w + 1) * run]
+        s, c = merge_tree([slot_pair(mine[k::P]) for k in range(P)])
+        total += float(s) - float(c)
     return total
 
 
@@ -77,11 +100,8 @@ def slice_row_sum(terms):
     deg = len(terms)
     pieces = 1 if deg <= 32 else 2 if deg <= 64 else 4
     run = ((deg + pieces - 1) // pieces + 3) // 4 * 4
-    part = [slot_sum(terms[k * run:(k + 1) * run]) for k in range(pieces)]
-    while len(part) > 1:
-        h = len(part) // 2
-        part = [F(part[k] + part[k + h]) for k in range(h)]
-    return part[0]
+    s, c = merge_tree([slot_pair(terms[k * run:(k + 1) * run]) for k in range(pieces)])
+    return F(s - c)
 
 
 def _neumaier(s, e, x):
