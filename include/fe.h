@@ -216,7 +216,10 @@ int fe_spmm_t(fe_csr h, const void* X, void* Y, int b, fe_dtype dt);
  * V: DEVICE, nv blocks of n x bv (block j at element j*n*bv), so V^T W is (nv*bv) x bw.
  * W: DEVICE, n x bw row-major.  G: DEVICE, FP64 row-major (nv*bv) x bw, overwritten.
  * 1 <= nv <= 128, bv and bw in {1, 2, 4, 8, 16}; V and W may alias (W = one of V's blocks).
- * FP32 inputs: products and per-thread sums in FP32, cross-thread sums in FP64.  FP64 inputs:
+ * FP32 inputs: products and per-thread sums in FP32 (shapes whose output tiles a warp's registers do
+ * not hold, such as b = 8 with more than 4 blocks, over at most 8 to 32 rows at a time); sums over
+ * threads in FP64, or where the row sweeps run (blocks of 2, 4 and 8) over a warp's rows as unevaluated
+ * pairs of FP32 numbers (48 bits; FP64 where those would overflow) and FP64 from there.  FP64 inputs:
  * tensor-core split products or FP64 FMA, as fe_block_gram_ex with FE_ENGINE_AUTO.
  * Errors: FE_ERR_INVALID, FE_ERR_OOM (scratch), FE_ERR_CUDA.
  */
@@ -226,12 +229,13 @@ int fe_block_gram(const void* V, int64_t n, int nv, int bv, const void* W, int b
 /*
  * fe_block_gram with a choice of arithmetic (fe_engine).  fe_block_gram is this call with
  * FE_ENGINE_AUTO.  For FP64 blocks with nv*bv <= 36 and bw in {1, 2, 4, 8}, FE_ENGINE_TC, and
- * FE_ENGINE_AUTO when nv*bv >= 16 (where it is the faster kernel), run on the tensor cores: within every 128-row tile each column of V and W is cut,
+ * FE_ENGINE_AUTO when nv*bv >= 16 (where it is the faster kernel), run on the tensor cores: within every 112-row tile each column of V and W is cut,
  * relative to its largest exponent in the tile, into seven 8-bit digits; one MMA per 16 rows
- * forms every digit product (exact FP16 x FP16 -> FP32 sums of 128 terms), and the tile's
+ * forms every digit product (exact FP16 x FP16 -> FP32 sums of 112 terms), and the tile's
  * products are assembled in integer arithmetic and added in FP64, so that the error of a tile's
- * contribution is at most 2^-50 * 128 * max|V[., c]| * max|W[., q]| over its rows (plus the
- * FP64 roundings of the sums over tiles); entries must be finite, subnormals are read as zero.
+ * contribution is at most 2^-50 * 112 * max|V[., c]| * max|W[., q]| over its rows (plus the
+ * FP64 roundings of the sums over tiles); entries must be finite, and a column of subnormals in a
+ * tile counts as zero.
  * Otherwise, and with FE_ENGINE_FMA, the FMA kernels of fe_block_gram.  FE_ENGINE_TC with an
  * unsupported shape or FP32 blocks: FE_ERR_INVALID.
  */

@@ -170,8 +170,9 @@ struct MlpParams {
 // The network runs on tiles of kTile rows per CTA of kThr threads, as products of shared-memory
 // operands with register accumulators.  Activations lie transposed (unit, row), kLd floats per
 // unit: a thread's output tile is 8 rows (two runs of four) x H / 16 units, read with two 16-byte
-// loads of activations and one of weights per inner index for 8 H / 16 FMAs, so that FP32 FMA
-// issue (128 per clock per SM) bounds the products, not shared memory.
+// loads of activations and one of weights per inner index for 8 H / 16 FMAs.  Shared-memory bandwidth
+// bounds the products all the same (H = 64, the gradient kernel: its data pipe 79% busy, the FMA pipes
+// 46%, issue 59%).
 constexpr int kTile = 128, kThr = 256, kLd = kTile + 4;   // kLd: units 4 banks apart
 
 struct TileMap {   // the thread's rows r0 .. r0 + 3, r0 + 64 .. r0 + 67 and units c0 ..
@@ -410,8 +411,8 @@ __global__ void __launch_bounds__(kThr, 2) mlp_stats_kernel(const float* __restr
 //   gW3 = h2^T dz, dh2 = (dz W3^T) [h2 > 0], gW2 = h1^T dh2, dh1 = (dh2 W2^T) [h1 > 0],
 //   gW1 = F^T dh1 and the bias sums,
 // with h2's memory reused for dh2 and then dh1.  A gradient entry belongs to one thread, which
-// sums a tile in one accumulator and the tiles in another (deterministic).  FP32 FMA issue bounds
-// it: 3 H^2 of the (3 (8 H + H B) + 3 H^2) FMAs per row are the three products above.
+// sums a tile in one accumulator and the tiles in another (FP32; deterministic).  Shared-memory
+// bandwidth bounds it: 3 H^2 of the (3 (8 H + H B) + 3 H^2) FMAs per row are the three products above.
 // Measured at n = 262141, H = 64, b = 4, t = 8 against one row per thread with shared-memory
 // operands (loss and gradient, all kernels): 1.98 -> 0.37 ms, of which this
 // kernel 1.07 -> 0.21 ms and the statistics 0.20 -> 0.09 ms.

@@ -12,7 +12,7 @@
 //   R = I - G;  d = diag S + R_ii theta_i,
 //   N_ij = S_ij + R_ij (theta_i + theta_j) / 2                       (FP64, then N in FP32)
 //     -- to first order in R the projection onto the orthonormalised Q (I + R / 2);
-//   E: the rotation that diagonalises D + N, relative to I           (FP32)
+//   E: the rotation that diagonalises D + N, relative to I           (FP32, one CTA)
 //   Q <- Q + Q (R / 2 + E)                                           (FP64, all CTAs)
 // N and E are small, so their FP32 rounding is relative to something small: the error of an
 // iteration is about 1e-7 of the previous one (and the square of the previous one where E is

@@ -169,7 +169,8 @@ def test_trained_network_gain_on_a_fresh_graph():
 def test_row_tiles(form, n, hidden, b, t):
     """Forward, loss and gradient at the edges of the 128-row tiles (one row, one short of a tile, a
     row over, more tiles than CTAs), biases everywhere, features at an odd 4-byte offset.  Bars as
-    above: FP32 rounding of sums of at most 64 terms per unit, FP64 over the rows' tiles."""
+    above: FP32 rounding of sums of at most 64 terms per unit; gradients in FP32 over a tile's rows and
+    over the few tiles of a CTA (two at most here), FP64 over the CTAs."""
     t_ = torch()
     r = np.random.default_rng(n + hidden + b)
     buf = to_dev(np.concatenate([[0.0], np.abs(r.standard_normal(n * omlp.NFEAT))]), t_.float32)
