@@ -306,6 +306,18 @@ def test_spmm_l2_window_same_results(graphs, prec):
             assert np.array_equal(fe.spmm(h, X).cpu().numpy(), fe.spmm(hl, X).cpu().numpy())
 
 
+def _f64_bound(deg, b, fmt):
+    """The interface's FP64 bound for a row: (m + 9) 2^-53 of A|X|, m the longest run that a lane adds --
+    in the slices (degree up to 128, packed 16) the row's steps over the lanes that share it, in multiples
+    of 4; else the entries of a task of at most 4096 over the lanes that gather whole X rows."""
+    if deg <= (128 if fmt == "plain" else 16):
+        pieces = 1 if deg <= 32 else 2 if deg <= 64 else 4
+        m = min(deg, (-(-deg // pieces) + 3) // 4 * 4)
+    else:
+        m = -(-min(deg, 4096) // (32 // max(1, b // 2)))
+    return (m + 9) * 2.0 ** -53
+
+
 @pytest.mark.parametrize("ncols", [9000, (1 << 19) + 3])
 @pytest.mark.parametrize("fmt", ["plain", "packed"])
 @pytest.mark.parametrize("prec", ["f32", "f64"])
@@ -313,7 +325,7 @@ def test_spmm_shared_rows(prec, fmt, ncols):
     """Rows at the edges of the sharing rules: 32 | 33 and 64 | 65 steps of a slice (one, two and
     four lanes a row), 128 | 129, tasks of 1024 | 1025 and 2048 | 2049 entries (one, two and four
     warps where the matrix has few columns), hub chunks of 4096 with a ragged last one and hubs with
-    more than 64 partials per lane.  Bounds: those of the interface, 9 * 2^-24 and 518 * 2^-53 of
+    more than 64 partials per lane.  Bounds: those of the interface, 9 * 2^-24 and _f64_bound of
     A|X|, the exact sums in extended precision."""
     r = np.random.default_rng(ncols)
     degs = [0, 1, 3, 4, 31, 32, 33, 35, 63, 64, 65, 66, 97, 127, 128, 129, 1023, 1024, 1025, 1057, 2047, 2048,
@@ -330,7 +342,7 @@ def test_spmm_shared_rows(prec, fmt, ncols):
             for i, c in enumerate(cols):
                 ref = X[c].astype(np.longdouble).sum(0)
                 mag = np.abs(X[c]).astype(np.longdouble).sum(0)
-                bound = (9 * 2.0 ** -24 if prec == "f32" else 518 * 2.0 ** -53) * mag
+                bound = (9 * 2.0 ** -24 if prec == "f32" else _f64_bound(len(c), b, fmt)) * mag
                 assert np.all(np.abs(Y[i] - ref) <= bound), (len(c), b)
 
 
@@ -339,8 +351,8 @@ def test_spmm_shared_rows(prec, fmt, ncols):
 def test_spmm_f64_exponents(b, fmt):
     """The aligned integer sums of FP64 blocks: columns whose entries span all exponents (2^-1000 to
     2^1000, rising and falling along a row, so that the common exponent rises at any point), columns
-    of equal sign, zeros of both signs among values, sums that cancel.  Bound of the interface,
-    518 * 2^-53 of A|X| (the sums in extended precision)."""
+    of equal sign, zeros of both signs among values, sums that cancel.  Bound of the interface
+    (_f64_bound of A|X|, the sums in extended precision)."""
     r = np.random.default_rng(b)
     n = 3000
     degs = [1, 4, 11, 12, 13, 16, 31, 32, 33, 64, 65, 100, 128, 129, 200, 1025, 2049, 2600]
@@ -365,7 +377,7 @@ def test_spmm_f64_exponents(b, fmt):
             for i, c in enumerate(cols):
                 ref = v[c].astype(np.longdouble).sum(0)
                 mag = np.abs(v[c]).astype(np.longdouble).sum(0)
-                assert np.all(np.abs(Y[i] - ref) <= 518 * 2.0 ** -53 * mag), (kind, len(c))
+                assert np.all(np.abs(Y[i] - ref) <= _f64_bound(len(c), b, fmt) * mag), (kind, len(c))
 
 
 @pytest.mark.parametrize("b", [2, 4, 16])
