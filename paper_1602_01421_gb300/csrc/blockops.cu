@@ -460,25 +460,37 @@ constexpr int row_lanes(int tiles) {
 
 // Whether the row sweep takes `tiles` blocks.  It is faster than the kernels with a warp per tile
 // (gram_kernel, update_gram_kernel) where loads bind: FP32 at b = 4 and 8 always (4.2 million rows, 7
-// blocks of 4: Gram 185 -> 120 us, update and Gram 267 -> 152 us; 8 blocks of 8
-// 1.92 -> 0.43 and 6.37 -> 1.39 ms; 31 blocks of 4, a million rows 320 -> 175 us and 1010 -> 222 us), narrower FP32 blocks for Grams of b = 2 and for updates of more than 16 tiles, which
-// the other kernel reduces after every range.  In FP64, the FMAs bind: it pays where the lanes' blocks
-// divide evenly (idle slots are issued all the same) and the other kernel's tiles do not fit its
-// registers (b = 8: 8 blocks, a million rows 1745 -> 893 us) or are more than 16 (31 blocks of 4: Gram
-// 1289 -> 896 us, update and Gram 2602 -> 2042 us).
+// blocks of 4: Gram 185 -> 120 us, update and Gram 267 -> 152 us; 8 blocks of 8 1.92 -> 0.43 and 6.37 ->
+// 1.39 ms; 31 blocks of 4, a million rows 320 -> 175 us and 1010 -> 222 us), narrower FP32 blocks for
+// Grams of b = 2 and for updates of more than 16 tiles, which the other kernel reduces after every
+// range.  In FP64, the FMAs bind, and a lane issues its idle slots too (cap: the slots of the lanes that
+// a row takes).  It pays
+//   b = 8, whose tiles do not fit the other kernel's registers: Gram with at most a quarter idle (8 blocks,
+//     a million rows 1745 -> 893 us); update and Gram with none (7 blocks 2490 -> 2290 us; 5 blocks, two
+//     idle, 1909 -> 2296), or up to 4 tiles from 65536 rows on;
+//   b = 4: Gram of more than 16 tiles (31 blocks 1289 -> 896 us) or with hardly any idle; update and Gram
+//     from 20 blocks on (a million rows, 17 blocks 1509 -> 1615 us, 20: 1719 -> 1616, 31: 2602 -> 2042);
+//   b = 2, more than 16 tiles: with at most 7 / 32 idle (4.2 million rows, 31 blocks 1112 -> 910 us, 20
+//     741 -> 984), or up to 2^17 rows, where the other kernel's ranges leave CTAs idle (100003 rows, 20 blocks
+//     54 -> 44 us);
+//   b = 1, more than 16 tiles: while V has at most 2^25 entries (32 blocks, a million rows 123 -> 96 us;
+//     100003 rows, 64 blocks 213 -> 34); beyond, its short loads fall behind (2.1 million, 17 blocks 113 ->
+//     148; 4.2 million, 40 blocks 384 -> 686).
 template <typename TC, int B, bool UPD>
 constexpr int kRowTilesMin = sizeof(TC) == 4   // the fewest and most tiles ever picked; 0: none are
                                  ? (B >= 4 ? 1 : (UPD ? 17 : (B == 2 ? 1 : 0)))
-                                 : (B == 8 ? 1 : (UPD ? (B == 4 ? 17 : 0) : (B == 4 ? 1 : 17)));
+                                 : (B == 8 ? 1 : (UPD ? (B == 4 ? 21 : 0) : (B == 4 ? 1 : 17)));
 template <typename TC, int B, bool UPD>
 constexpr int kRowTilesMax = sizeof(TC) == 4 && B == 2 && !UPD ? 16 : kRowBlocks<TC, B> * kRowLanesMax;
 template <typename T, typename TC, int B, bool UPD>
-static bool rows_pick(int tiles) {
+static bool rows_pick(int tiles, int64_t n) {
   if (tiles < kRowTilesMin<TC, B, UPD> || tiles > kRowTilesMax<TC, B, UPD>) return false;
   if (sizeof(TC) == 4) return true;
-  const int l = row_lanes<TC, B>(tiles), slots = (tiles + l - 1) / l * l;
-  if (B == 8) return 3 * slots <= 4 * tiles;
-  return tiles > 16 || 10 * slots <= 11 * tiles;
+  const int l = row_lanes<TC, B>(tiles), slots = (tiles + l - 1) / l * l, cap = l * kRowBlocks<TC, B>;
+  if (B == 8) return UPD ? slots == tiles || (tiles <= 4 && n >= 65536 && 3 * slots <= 4 * tiles) : 3 * slots <= 4 * tiles;
+  if (B == 4) return tiles > 16 || 10 * slots <= 11 * tiles;
+  if (B == 2) return 32 * tiles >= 25 * cap || n <= (1 << 17);
+  return n * tiles <= (1 << 25);
 }
 
 template <typename T, typename TC, int B, int L, bool UPD>
@@ -529,7 +541,7 @@ static int gram_rows(const BlockSet& V, int64_t n, const T* W, int bw, int ldw, 
                      double* scratch, size_t capacity, bool* done, cudaStream_t s, GramParts* parts = nullptr) {
   *done = false;
   if constexpr (B <= 8 && kRowTilesMin<TC, B, false> > 0) {
-    if (bw != B || V.bv != B || V.ld != B || ldw != B || !rows_pick<T, TC, B, false>(V.nv)) return FE_OK;
+    if (bw != B || V.bv != B || V.ld != B || ldw != B || !rows_pick<T, TC, B, false>(V.nv, n)) return FE_OK;
     *done = true;
     return launch_rows<T, TC, B, false>(V, n, nullptr, 0.0, 0.0, const_cast<T*>(W), alpha, G, scratch, capacity, s,
                                          parts);
@@ -1295,7 +1307,7 @@ static int launch_update_gram(const BlockSet& V, int64_t n, const double* C, dou
                               double beta, const double* M, T* W, int gram_v, const int* skip,
                               const int* vc32, double* G, cudaStream_t s) {
   if constexpr (kRowTilesMin<T, BW, true> > 0)
-    if (gram_v && !M && !skip && !vc32 && rows_pick<T, T, BW, true>(V.nv + 1))
+    if (gram_v && !M && !skip && !vc32 && rows_pick<T, T, BW, true>(V.nv + 1, n))
       return launch_rows<T, T, BW, true>(V, n, C, alpha, beta, W, 1.0, G, nullptr, 0, s);
   constexpr int NR = BV > BW ? BV : BW;
   constexpr int kRegsPerTile = NR * BW * (int)(sizeof(T) / 4);

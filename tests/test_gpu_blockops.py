@@ -313,3 +313,27 @@ def test_row_sweep_long_sums(b, nv, n, scale):
     if run:
         G = fe.block_gram(V, W, engine="fma").cpu().numpy()
         assert np.abs(G / vw - 1).max() <= (run + 1) * u
+
+
+@pytest.mark.parametrize("b,nv,n", [(2, 20, 1 << 17), (2, 20, (1 << 17) + 1), (2, 24, 140001), (2, 25, 140001), (1, 17, (1 << 25) // 17),
+                                    (1, 17, (1 << 25) // 17 + 1), (8, 3, 65535), (8, 3, 65536), (8, 5, 70001), (8, 7, 70001),
+                                    (4, 19, 70001), (4, 20, 70001)])
+def test_fp64_kernel_choice(b, nv, n):
+    """Both sides of the rules that choose between the row sweeps and the tile kernels in FP64: Gram and
+    update + Gram against torch's FP64 products of the same data.  Bounds: twice those of test_row_sweeps,
+    since both sides round."""
+    t = __import__("torch")
+    g = t.Generator(device="cuda").manual_seed(n + nv)
+    V = t.randn(nv, n, b, generator=g, device="cuda", dtype=t.float64)
+    W = t.randn(n, b, generator=g, device="cuda", dtype=t.float64)
+    C = t.randn(nv * b, b, generator=g, device="cuda", dtype=t.float64) / (nv * b) ** 0.5
+    A = V.permute(1, 0, 2).reshape(n, -1)
+    u = 2.0 ** -53
+    G = fe.block_gram(V, W, engine="fma")
+    assert ((G - A.T @ W).abs() <= 64 * u * (A.abs().T @ W.abs())).all()
+    want = 0.5 * W + A @ C
+    mag = 0.5 * W.abs() + A.abs() @ C.abs()
+    G = fe.block_update_gram(V, C, W, alpha=1.0, beta=0.5)
+    assert ((W - want).abs() <= 2 * (nv * b + 8) * u * mag).all()
+    A = t.cat([A, W], 1)
+    assert ((G - A.T @ W).abs() <= 64 * u * (A.abs().T @ W.abs())).all()
