@@ -461,7 +461,7 @@ static size_t tc_smem_bytes(int nkc, int NP) {
 
 // ---------------------------------------------------------------- pipelined form (K <= 32)
 // The same product with the phases of consecutive tiles overlapped.  One persistent CTA per SM
-// with four warp roles:
+// with four warp roles (numbers for K > 16; up to there warps 0-7, 24, 25 and 8-23, PipeRoles):
 //   warps 0-15  split V rows into digits: a unit is 8 columns of one row, thread t takes unit
 //               t = row + 128 cb (cb < ceil(K / 8)); units write the digit tiles of buffer t % 2;
 //   warp 28     (one thread) issues the TMA copies of tile t's V rows into staging buffer t % 2;
@@ -488,12 +488,18 @@ static size_t tc_smem_bytes(int nkc, int NP) {
 // assembly, 97 without the split as well; 186 with 8 assembling warps, 187 with every other result
 // normalised in integers instead of converted.
 namespace {
-constexpr int kSplitWarps = 16, kEpiWarps = 12;
-constexpr int kEpiParts = kEpiWarps / 4;                 // epilogue threads per row
-constexpr int kSplitThreads = kSplitWarps * 32;
-constexpr int kProdWarp = kSplitWarps + kEpiWarps, kMmaWarp = kProdWarp + 1;
-constexpr int kPipeWarps = kMmaWarp + 1;
-constexpr int kPipeThreads = kPipeWarps * 32;
+// Warp roles: 16 splitting and 12 assembling warps, three threads per row of results.  Up to 16 columns of V
+// (FEW) half of the splitting warps would have no unit and only meet at the barriers, and the results
+// bind: 8 and 16 there, four threads per row (4.2 million rows, 8 columns into 8 340 -> 269 us, 16 into 8
+// 356 -> 307, 16 into 32 902 -> 650 against 8 and 8 warps; 357, 380 and 801 with 16 and 12).
+template <bool FEW>
+struct PipeRoles {
+  static constexpr int kSplitWarps = FEW ? 8 : 16, kEpiWarps = FEW ? 16 : 12;
+  static constexpr int kEpiParts = kEpiWarps / 4;                 // epilogue threads per row
+  static constexpr int kSplitThreads = kSplitWarps * 32;
+  static constexpr int kProdWarp = kSplitWarps + kEpiWarps, kMmaWarp = kProdWarp + 1;
+  static constexpr int kPipeThreads = (kMmaWarp + 1) * 32;
+};
 
 struct PipeBars {
   uint64_t vfull[2], vempty[2], afull[2], mdone[2], tempty[2];
@@ -536,8 +542,12 @@ __device__ __forceinline__ bool bar_or(int id, int nthreads, bool p) {
   return r != 0;
 }
 
-template <int BV, int NP>
-__global__ void __launch_bounds__(kPipeThreads, 1) tc_combine_pipe_kernel(const TcArgs a) {
+template <int BV, int NP, bool FEW>
+__global__ void __launch_bounds__(PipeRoles<FEW>::kPipeThreads, 1) tc_combine_pipe_kernel(const TcArgs a) {
+  using PR = PipeRoles<FEW>;
+  constexpr int kSplitWarps = PR::kSplitWarps, kEpiWarps = PR::kEpiWarps, kEpiParts = PR::kEpiParts,
+                kSplitThreads = PR::kSplitThreads, kProdWarp = PR::kProdWarp, kMmaWarp = PR::kMmaWarp,
+                kPipeThreads = PR::kPipeThreads;
   constexpr uint32_t kBufCols = NP == 32 ? 256u : 128u;  // TMEM columns per buffer (7 NP used)
   constexpr size_t kBTile = (size_t)NP * kKChunk * 2;
   constexpr int kVBuf = kTileRows * kKChunk;              // doubles per V staging buffer
@@ -725,8 +735,8 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_combine_pipe_kernel(const 
     const bool add_out = a.beta != 0.0;
     constexpr int kStep = 2 * kEpiParts;
     const int ngroups = a.N > 2 * part ? (a.N - 2 * part + kStep - 1) / kStep : 0;        // this thread's groups of two results
-    // rows of Out loaded ahead of their tile: by a thread with one group (all of them: N <= 6) two tiles
-    // ahead into slot it % 2, with two groups (N <= 12) one tile ahead into slot = group
+    // rows of Out loaded ahead of their tile: by a thread with one group (three threads a row: N <= 6) two
+    // tiles ahead into slot it % 2, with two groups (N <= 12) one tile ahead into slot = group
     const int pf = !add_out ? 0 : ngroups <= 1 ? 2 : ngroups == 2 ? 1 : 0;
     double opf[2][2];
     auto load_grp = [&](int64_t it, int jj, int slot) {
@@ -844,15 +854,15 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_combine_pipe_kernel(const 
   if (warp == kMmaWarp) tc::tmem_dealloc(tbase, 2 * kBufCols);
 }
 
-template <int BV, int NP>
+template <int BV, int NP, bool FEW>
 static int launch_tc_combine_pipe_np(const TcArgs& a, cudaStream_t s) {
   static KernelSetup ks;
-  const void* fn = reinterpret_cast<const void*>(tc_combine_pipe_kernel<BV, NP>);
+  const void* fn = reinterpret_cast<const void*>(tc_combine_pipe_kernel<BV, NP, FEW>);
   constexpr size_t smem = pipe_smem_bytes(NP);
   FE_TRY(kernel_configure(ks, fn, (int)smem));
   const int64_t ntiles = ceil_div(a.n, kTileRows);
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ntiles, (int64_t)num_sms()));
-  tc_combine_pipe_kernel<BV, NP><<<(unsigned)grid, kPipeThreads, smem, s>>>(a);
+  tc_combine_pipe_kernel<BV, NP, FEW><<<(unsigned)grid, PipeRoles<FEW>::kPipeThreads, smem, s>>>(a);
   count_launch();
   FE_CUDA(cudaGetLastError());
   return FE_OK;
@@ -860,8 +870,12 @@ static int launch_tc_combine_pipe_np(const TcArgs& a, cudaStream_t s) {
 
 template <int BV>
 static int launch_tc_combine_pipe(const TcArgs& a, cudaStream_t s) {
-  if (a.NP == 16) return launch_tc_combine_pipe_np<BV, 16>(a, s);
-  return launch_tc_combine_pipe_np<BV, 32>(a, s);
+  if (a.K <= 16) {
+    if (a.NP == 16) return launch_tc_combine_pipe_np<BV, 16, true>(a, s);
+    return launch_tc_combine_pipe_np<BV, 32, true>(a, s);
+  }
+  if (a.NP == 16) return launch_tc_combine_pipe_np<BV, 16, false>(a, s);
+  return launch_tc_combine_pipe_np<BV, 32, false>(a, s);
 }
 
 bool tc_combine_supported(const BlockSet& V, const BlockSet& Out, fe_dtype dt) {
